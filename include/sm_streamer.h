@@ -339,14 +339,20 @@ int sm_set_metrics_log(sm_ctx *ctx, const char *path, double hbm_peak_gbs);
  * the fixed-point smoother, residual-restriction and prolongation kernels
  * with one thread per x row of a box (16-byte row loads, fewer
  * instructions per cell); smaller levels run the kernels with one
- * 128-thread group per box (more warps per box for latency).  Both give bit-identical results; the
- * choice is performance only.  Errors: SM_EINVAL for min_boxes < 0. */
+ * 128-thread group per box (more warps per box for latency), and those whose
+ * boxes are all resident at once (1216 on 152 SMs) a whole leg of the
+ * V-cycle per launch.  All give bit-identical results; the choice is
+ * performance only.  Errors: SM_EINVAL for min_boxes < 0. */
 int sm_set_row_kernels(sm_ctx *ctx, int min_boxes);
 
 /* Solves run as CUDA graphs (captured on first use per octree, with the
  * cycle loop and its stopping test on the device) when enabled (default),
  * or as individually launched kernels with a host loop when disabled.
- * Both paths launch the same kernels in the same order. */
+ * Both paths launch the same kernels in the same order.  On a level whose
+ * boxes are all resident on the GPU at once, each leg of an FP64 V-cycle is
+ * one cooperative launch whose blocks pass face cells to one another between
+ * colour passes; a wait that runs out (a few tenths of a second) ends the
+ * launch and the solve returns SM_ETIMEOUT. */
 int sm_set_graphs(sm_ctx *ctx, int enable);
 
 /* V-cycles run as one persistent cooperative launch when enabled (default
@@ -361,9 +367,10 @@ int sm_set_graphs(sm_ctx *ctx, int enable);
  * dropped on a change. */
 int sm_set_persistent(sm_ctx *ctx, int enable);
 
-/* Self-test of the bounded grid-barrier wait of the persistent kernel: one
- * launch whose barriers wait for one block more than the grid holds, so
- * every block's wait runs out (about a second), sets the error flag and
+/* Self-test of the bounded waits between blocks: a launch of the persistent
+ * kernel whose barriers wait for one block more than the grid holds, then
+ * one leg of level 1 whose blocks wait for words that are never published;
+ * every wait runs out (about a second), sets the error flag and the launch
  * returns.  Expected result SM_ETIMEOUT; the flag is cleared afterwards and
  * the context stays usable (the potential may have received part of a
  * V-cycle).  Errors: SM_ESTATE (no octree or a pending device error),

@@ -60,7 +60,7 @@ struct ArenaPlan {
 struct Layout {
   size_t level, ijk, parent, child, nbr, nbr6, leaf, cf_leaf, morton, scan_a, scan_b, count, flags;
   size_t phi, rhs, res, old, rho, emag, nb[3], ib[3], gh, cflux, basis, tab, dscal, hist, e32, f32, old32, gh32,
-      phx, gx, ghx, total;
+      phx, gx, ghx, xch, xseq, legr, total;
 };
 
 static Layout plan(int cap, bool mixed) {
@@ -97,6 +97,9 @@ static Layout plan(int cap, bool mixed) {
   L.phx = p.take<long long>(nc);
   L.gx = p.take<long long>(nc);
   L.ghx = p.take<long long>((size_t)cap * 6 * FACE);
+  L.xch = p.take<long long>((size_t)(cap < MAXL * LEG_CAP ? cap : MAXL * LEG_CAP) * XWORDS);
+  L.xseq = p.take<unsigned>(MAXL);
+  L.legr = p.take<int32_t>((size_t)cap * LROW);
   if (mixed) {
     L.e32 = p.take<float>(nc);
     L.f32 = p.take<float>(nc);
@@ -225,6 +228,9 @@ extern "C" int sm_bind_arena(sm_ctx *ctx, void *dev_ptr, size_t bytes) {
   ctx->phx = (long long *)(a + L.phx);
   ctx->gx = (long long *)(a + L.gx);
   ctx->ghx = (long long *)(a + L.ghx);
+  ctx->xch = (long long *)(a + L.xch);
+  ctx->xseq = (unsigned *)(a + L.xseq);
+  ctx->leg_rows = (int32_t *)(a + L.legr);
   if (ctx->cfg.precision == SM_MIXED) {
     ctx->e32 = (float *)(a + L.e32);
     ctx->f32 = (float *)(a + L.f32);
@@ -402,6 +408,39 @@ int sm_exclusive_scan(sm_ctx *ctx, const int32_t *in, int32_t *out, int n) {
   return SM_OK;
 }
 
+// What a one-launch leg needs to know of a box, one 64-byte row, so that
+// every cell it reads from memory is one dependent load away: the six face
+// neighbours, the parent, flags -- octant (bits 0-2), the box refined (3),
+// its neighbours refined (4-9), face a wall (10-15), a refinement face
+// (16-21) -- and the parent's neighbours in the octant's directions: across
+// the three faces, and across the edges that miss axis 0, 1, 2.
+__global__ void __launch_bounds__(128) k_leg_rows(int lo, int hi, const int32_t *__restrict__ nbr,
+                                                  const int32_t *__restrict__ nbr6,
+                                                  const int32_t *__restrict__ parent,
+                                                  const int32_t *__restrict__ ijk, const int32_t *__restrict__ child,
+                                                  int32_t *__restrict__ rows) {
+  const int b = lo + blockIdx.x * blockDim.x + threadIdx.x;
+  if (b >= hi) return;
+  const int P = parent[b];
+  int fl = (ijk[3 * b] & 1) | (ijk[3 * b + 1] & 1) << 1 | (ijk[3 * b + 2] & 1) << 2 | (child[8 * b] >= 0) << 3;
+  int32_t *row = rows + (size_t)LROW * b;
+  for (int f = 0; f < 6; ++f) {
+    const int q = nbr6[6 * b + f];
+    row[LR_NB + f] = q;
+    if (q >= 0 && child[8 * q] >= 0) fl |= 1 << (4 + f);
+    if (q == -1) fl |= 1 << (10 + f);
+    if (q == -2) fl |= 1 << (16 + f);
+  }
+  const int s[3] = {(fl & 1) ? 1 : -1, (fl & 2) ? 1 : -1, (fl & 4) ? 1 : -1};
+  for (int a = 0; a < 3; ++a) {
+    row[LR_PN + a] = nbr6[6 * P + 2 * a + (s[a] > 0)];
+    const int d = (a == 0 ? 1 : 1 + s[0]) + 3 * (a == 1 ? 1 : 1 + s[1]) + 9 * (a == 2 ? 1 : 1 + s[2]);
+    row[LR_PE + a] = nbr[26 * P + (d > 13 ? d - 1 : d)];
+  }
+  row[LR_P] = P;
+  row[LR_FLAGS] = fl;
+}
+
 int sm_rebuild_leaves(sm_ctx *ctx) {
   int n = ctx->n_boxes;
   k_mark_leaves<<<(n + 255) / 256, 256, 0, ctx->stream>>>(n, ctx->child, ctx->scan_a);
@@ -425,6 +464,12 @@ int sm_rebuild_leaves(sm_ctx *ctx) {
   ++ctx->n_launch;
   k_compact<<<(n + 255) / 256, 256, 0, ctx->stream>>>(n, ctx->scan_a, ctx->scan_b, ctx->cf_leaf);
   ++ctx->n_launch;
+  if (ctx->n_levels > 1) {
+    const int lo = ctx->level_off[1];
+    k_leg_rows<<<(n - lo + 127) / 128, 128, 0, ctx->stream>>>(lo, n, ctx->nbr, ctx->nbr6, ctx->parent, ctx->ijk,
+                                                              ctx->child, ctx->leg_rows);
+    ++ctx->n_launch;
+  }
   SM_CKL("refinement-face leaf list");
   SM_CK(cudaMemcpyAsync(&h[ctx->n_levels + 1], ctx->scan_b + n, sizeof(int32_t), cudaMemcpyDeviceToHost,
                         ctx->stream));

@@ -42,11 +42,27 @@ __device__ __forceinline__ bool fx_bad(long long x) {
   return (unsigned long long)(x + FX_LIM) >= (unsigned long long)(2 * FX_LIM);
 }
 
+// u / D for u < 2^63 and D = 6 or 12 on the 32-bit halves u = uh 2^32 + ul:
+// with uh = D qh + rh, ul = D ql + rl and 2^32 = D m + 4 the quotient is
+// qh 2^32 + m rh + ql + (4 rh + rl) / D -- a dozen 32-bit instructions of
+// short dependence instead of a 64-bit high product.
+template <unsigned D>
+__device__ __forceinline__ unsigned long long fx_udiv(unsigned long long u) {
+  static_assert(D == 6 || D == 12, "the small quotient's constants");
+  const unsigned uh = (unsigned)(u >> 32), ul = (unsigned)u;
+  const unsigned qh = uh / D, rh = uh - D * qh, ql = ul / D, rl = ul - D * ql;
+  const unsigned x = 4u * rh + rl;  // at most 5 (D - 1)
+  const unsigned lo = (0xffffffffu / D) * rh + ql + (D == 6 ? x * 43u >> 8 : x * 171u >> 11);
+  return (unsigned long long)qh << 32 | lo;
+}
+
 // t / D rounded to the nearest integer, ties away from zero (D constant)
 template <unsigned D>
 __device__ __forceinline__ long long fx_rdiv(long long t) {
   const unsigned long long u = t < 0 ? 0ull - (unsigned long long)t : (unsigned long long)t;
-  const unsigned long long r = (u + (D >> 1)) / D;
+  unsigned long long r;
+  if constexpr (D == 12) r = fx_udiv<12>(u + 6);
+  else r = (u + (D >> 1)) / D;
   return t < 0 ? -(long long)r : (long long)r;
 }
 
@@ -54,7 +70,7 @@ __device__ __forceinline__ long long fx_rdiv(long long t) {
 // |t| < 1.5 * 2^62: a bias that is a multiple of 6 makes the dividend
 // non-negative, so the division is an unsigned one by a constant
 __device__ __forceinline__ long long fx_div6(long long t) {
-  return (long long)(((unsigned long long)t + (6ull << 60) + 3ull) / 6ull) - (1ll << 60);
+  return (long long)fx_udiv<6>((unsigned long long)t + (6ull << 60) + 3ull) - (1ll << 60);
 }
 
 // colour-split position of cell (i,j,k) of a box, and of natural cell
@@ -693,7 +709,8 @@ __global__ void __launch_bounds__(64, 12) k_fresid_restrict_rows(int lo, long lo
                                                                  const int32_t *__restrict__ nbr6,
                                                                  const int32_t *__restrict__ parent,
                                                                  const int32_t *__restrict__ ijk, Bc bc,
-                                                                 const unsigned long long *sc) {
+                                                                 const unsigned long long *sc,
+                                                                 long long *__restrict__ oldx) {
   __shared__ longlong2 srow[4][64];  // the rows of the box, four 16-byte chunks apart
   const int r = threadIdx.x, j = r & 7, k = r >> 3;
   const int b = lo + blockIdx.x;
@@ -780,7 +797,9 @@ __global__ void __launch_bounds__(64, 12) k_fresid_restrict_rows(int lo, long lo
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       const size_t cc = pb + xpos(4 * pl.ox + c, cy, cz);
-      phx[cc] = fx_rdiv<8>(sp[c]);
+      const long long w = fx_rdiv<8>(sp[c]);
+      phx[cc] = w;
+      if (oldx) oldx[cc] = w;  // the level below starts its leg from oldx
       gx[cc] = sa[c];
     }
   }
@@ -1148,7 +1167,7 @@ __global__ void __launch_bounds__(GT) k_fresnorm(const int32_t *__restrict__ lea
 __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(64)
     k_fcoarse8(long long *__restrict__ phx, long long *__restrict__ gx, long long *__restrict__ oldx,
                const double *__restrict__ basis, Bc bc, double h2, double inv_h2, int fas,
-               unsigned long long *sc) {
+               unsigned long long *sc, unsigned *xseq, int top) {
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ double pa[64], pb[64], sd[64], se[64], V[192], lam[24];
@@ -1159,6 +1178,8 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(64)
     else lam[i - 192] = __ldg(basis + i);
   }
   pdl_wait();
+  // the exchange tags of every level of this V-cycle move on between its legs
+  if (r == 0 && t >= 1 && t <= top) ++xseq[t];
   const int E = fx_E(sc);
   const double cf = -6.0 * fx_q(E) * inv_h2;
   bool bad = false;

@@ -882,11 +882,12 @@ __global__ void k_loop_check(cudaGraphConditionalHandle h, unsigned long long *s
   sc[SC_REL] = (unsigned long long)__double_as_longlong(rel);
   if (c >= 1 && c <= (unsigned long long)SM_HIST) hist[c - 1] = rel;
   double tol = __longlong_as_double((long long)sc[SC_TOL]);
-  const bool ovf = (sc[SC_ERR] & 8ull) != 0;  // fixed-point range left: the host runs the solve again
+  const bool ovf = (sc[SC_ERR] & 12ull) != 0;  // fixed-point range left (the host runs the solve again) or a wait ran out
   cudaGraphSetConditional(h, (rel > tol && c < sc[SC_MAXC] && !ovf) ? 1u : 0u);
 }
 
 #include "mgfix.cuh"
+#include "mglevel.cuh"
 
 // ---------------------------------------------------------------------------
 // persistent V-cycle kernel
@@ -1640,7 +1641,12 @@ static int read_scalars(sm_ctx *ctx) {
   SM_CK(cudaStreamSynchronize(ctx->stream));
   unsigned long long e;
   memcpy(&e, &ctx->hscal[SC_ERR], sizeof e);
-  if (e & ERR_BARRIER) return sm_fail(ctx, SM_ETIMEOUT, "grid barrier of the persistent kernel timed out");
+  if (e & ERR_BARRIER) {
+    // the flag is cleared and the exchange words start anew, so the context stays usable
+    SM_CK(cudaMemsetAsync(ctx->dscal + SC_ERR, 0, sizeof(unsigned long long), ctx->stream));
+    ctx->xch_reset = true;
+    return sm_fail(ctx, SM_ETIMEOUT, "a wait between the blocks of a kernel ran out");
+  }
   if (e & ~fx::FX_ERR_OVF) return sm_fail(ctx, SM_ESTATE, "device consistency check failed (flags 0x%llx)", e);
   if (e) return SM_FX_RETRY;
   return SM_OK;
@@ -1686,8 +1692,83 @@ static fx::FxLev fx_levels(const sm_ctx *ctx) {
   return fl;
 }
 
-// the exponent margin of the next solve's scale (host value, not captured)
+// Boxes of the largest level whose legs run in one launch (mglevel.cuh): a
+// block per box, all resident at once.  0 when the device has no
+// cooperative launch.
+static int leg_limit(sm_ctx *ctx) {
+  if (ctx->leg_max >= 0) return ctx->leg_max;
+  int coop = 0, sms = 0, most = 1 << 30;
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, ctx->device);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device);
+  auto fits = [&](auto *k) {
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 128, 0) != cudaSuccess) per = 0;
+    if (per * sms < most) most = per * sms;
+  };
+  fits(fx::k_flevel<fx::FS_TOP>);
+  fits(fx::k_flevel<fx::FS_FAS>);
+  fits(fx::k_flevel<fx::FS_PROLONG>);
+  fits(fx::k_flevel<fx::FS_FMG>);
+  cudaGetLastError();
+  ctx->leg_max = coop ? (most < LEG_CAP ? most : LEG_CAP) : 0;
+  return ctx->leg_max;
+}
+
+// whether the legs of level l run in one launch each
+static bool leg_level(sm_ctx *ctx, int l) {
+  const int n = lvl_n(ctx, l);
+  return l >= 1 && l < ctx->n_levels && n > 0 && n <= leg_limit(ctx) && n < ctx->rows_min &&
+         ctx->cfg.nu1 <= fx::LEG_MAX_NU && ctx->cfg.nu2 <= fx::LEG_MAX_NU;
+}
+
+template <int START>
+static int fx_leg(sm_ctx *ctx, int l, unsigned skew = 0) {
+  size_t first = 0;  // boxes of the lower levels that have exchange words
+  for (int m = 1; m < l; ++m)
+    if (lvl_n(ctx, m) <= LEG_CAP) first += (size_t)lvl_n(ctx, m);
+  constexpr bool up = START == fx::FS_PROLONG;
+  fx::LevArgs a;
+  memset(&a, 0, sizeof a);
+  a.lo = ctx->level_off[l];
+  a.nu = up ? ctx->cfg.nu2 : ctx->cfg.nu1;
+  a.set_phx = START != fx::FS_FMG || l == 1;
+  a.leg = up ? 0u : 16u;
+  a.skew = skew;
+  a.phx = ctx->phx;
+  a.gx = ctx->gx;
+  a.oldx = (long long *)ctx->old;
+  a.ghx = ctx->ghx;
+  a.xch = ctx->xch + first * XWORDS;
+  a.rows = ctx->leg_rows;
+  a.seq = ctx->xseq + l;
+  a.sc = ctx->dscal;
+  a.bc = ctx->bc;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(lvl_n(ctx, l));
+  cfg.blockDim = dim3(128);
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  ++ctx->n_launch;
+  SM_CK(cudaLaunchKernelEx(&cfg, fx::k_flevel<START>, a));
+  return SM_OK;
+}
+
+// before each solve: the exponent margin of its scale (a host value, not
+// captured), and the exchange words and their counters cleared when the
+// mesh or the choice of kernels has changed
 static int fx_set_margin(sm_ctx *ctx) {
+  if (ctx->xch_reset) {
+    size_t n = 0;
+    for (int l = 1; l < ctx->n_levels; ++l)
+      if (lvl_n(ctx, l) <= LEG_CAP) n += (size_t)lvl_n(ctx, l);
+    SM_CK(cudaMemsetAsync(ctx->xch, 0, n * XWORDS * sizeof(long long), ctx->stream));
+    SM_CK(cudaMemsetAsync(ctx->xseq, 0, sizeof(unsigned) * MAXL, ctx->stream));
+    ctx->xch_reset = false;
+  }
   const unsigned long long m = (unsigned long long)ctx->fx_margin;
   memcpy(&ctx->hscal[SC_FXM], &m, sizeof m);
   SM_CK(cudaMemcpyAsync(ctx->dscal + SC_FXM, ctx->hscal + SC_FXM, sizeof(double), cudaMemcpyHostToDevice,
@@ -1756,11 +1837,11 @@ static int fx_smooth(sm_ctx *ctx, int l, int nu, bool skip_first = false) {
 
 // level-0 solve; fas: complete level 0's FAS right-hand side first (the
 // down leg of a V-cycle has restricted into it)
-static int fx_coarse(sm_ctx *ctx, bool fas = false) {
+static int fx_coarse(sm_ctx *ctx, bool fas = false, int top = 0) {
   int st = ensure_basis(ctx);
   if (st) return st;
   sm_launch(ctx, fx::k_fcoarse8, 8, 64, 0, ctx->phx, ctx->gx, (long long *)ctx->old, ctx->basis, ctx->bc,
-            ctx->lh.h2[0], ctx->lh.inv_h2[0], (int)fas, ctx->dscal);
+            ctx->lh.h2[0], ctx->lh.inv_h2[0], (int)fas, ctx->dscal, ctx->xseq, top);
   SM_CKL("coarse solve");
   return SM_OK;
 }
@@ -1801,27 +1882,48 @@ static int fx_leaf_norm(sm_ctx *ctx, int off, int n, int slot) {
 // FAS V-cycle in fixed point with `top` as finest level; with norm_slot >= 0
 // (top the finest level) max_leaf |f - L phi| is left in that slot.  The
 // Ghat values of every level <= top must match the level below on entry
-// (the prologue and every up-sweep leave them so).
-static int fx_vcycle(sm_ctx *ctx, int top, int norm_slot = -1) {
+// (the prologue and every up-sweep leave them so).  With fmg the level top
+// first takes the prolonged solution of the level below.
+//
+// A level whose boxes are all resident at once runs each leg in one launch
+// (k_flevel); a larger one runs a launch per operation.  Below a level of
+// the latter kind that is one partial wave, above another such, the FAS
+// completion also runs the first colour pass, on a copy of the whole level
+// that the restriction leaves in old.
+static int fx_vcycle(sm_ctx *ctx, int top, int norm_slot = -1, bool fmg = false) {
   int st;
   if (norm_slot >= 0)
     SM_CK(cudaMemsetAsync(ctx->dscal + norm_slot, 0, sizeof(unsigned long long), ctx->stream));
+  // a fused FMG start restricts into old alone, which only a one-launch leg
+  // (or the level-0 solve's own start) of the level below can take
+  if (fmg && !(leg_level(ctx, top) && (top == 1 || leg_level(ctx, top - 1)))) {
+    if ((st = fx_prolong(ctx, top, 1, fx::FxNorm{}))) return st;
+    fmg = false;
+  }
   bool fused = false;  // the first colour pass of level l has run (k_ffas_color0)
   for (int l = top; l >= 1; --l) {
-    if ((st = fx_smooth(ctx, l, ctx->cfg.nu1, fused))) return st;
-    // on a level of one partial wave below another, the FAS completion also
-    // runs the level's first colour pass; the restriction then copies the
-    // whole level below into old first
-    fused = l - 1 >= 1 && ctx->cfg.nu1 > 0 && lvl_n(ctx, l) < ctx->rows_min && lvl_n(ctx, l - 1) < ctx->rows_min;
-    if (lvl_n(ctx, l) >= ctx->rows_min) {
-      sm_launch(ctx, fx::k_fresid_restrict_rows, lvl_n(ctx, l), 64, 0, ctx->level_off[l], ctx->phx, ctx->gx,
-                ctx->ghx, ctx->nbr6, ctx->parent, ctx->ijk, ctx->bc, ctx->dscal);
+    if (leg_level(ctx, l)) {
+      if (l < top) st = fx_leg<fx::FS_FAS>(ctx, l);
+      else st = fmg ? fx_leg<fx::FS_FMG>(ctx, l) : fx_leg<fx::FS_TOP>(ctx, l);
+      if (st) return st;
+      fused = false;
     } else {
-      const int nl = fused ? ctx->leaf_level_off[l] - ctx->leaf_level_off[l - 1] : 0;
-      sm_launch(ctx, fx::k_fresid_restrict, lvl_n(ctx, l) + nl, GT, 0, ctx->level_off[l], lvl_n(ctx, l), ctx->phx,
-                ctx->gx, ctx->ghx, ctx->nbr6, ctx->parent, ctx->ijk, ctx->bc, ctx->dscal,
-                fused ? (long long *)ctx->old : nullptr, ctx->leaf + ctx->leaf_level_off[l - 1]);
+      if ((st = fx_smooth(ctx, l, ctx->cfg.nu1, fused))) return st;
+      const bool leg = leg_level(ctx, l - 1);
+      fused = !leg && l - 1 >= 1 && ctx->cfg.nu1 > 0 && lvl_n(ctx, l) < ctx->rows_min &&
+              lvl_n(ctx, l - 1) < ctx->rows_min;
+      if (lvl_n(ctx, l) >= ctx->rows_min) {
+        sm_launch(ctx, fx::k_fresid_restrict_rows, lvl_n(ctx, l), 64, 0, ctx->level_off[l], ctx->phx, ctx->gx,
+                  ctx->ghx, ctx->nbr6, ctx->parent, ctx->ijk, ctx->bc, ctx->dscal,
+                  leg ? (long long *)ctx->old : nullptr);
+      } else {
+        const int nl = fused ? ctx->leaf_level_off[l] - ctx->leaf_level_off[l - 1] : 0;
+        sm_launch(ctx, fx::k_fresid_restrict, lvl_n(ctx, l) + nl, GT, 0, ctx->level_off[l], lvl_n(ctx, l), ctx->phx,
+                  ctx->gx, ctx->ghx, ctx->nbr6, ctx->parent, ctx->ijk, ctx->bc, ctx->dscal,
+                  fused || leg ? (long long *)ctx->old : nullptr, ctx->leaf + ctx->leaf_level_off[l - 1]);
+      }
     }
+    if (leg_level(ctx, l - 1)) continue;  // its leg completes the FAS right-hand side
     if (fused)
       sm_launch(ctx, fx::k_ffas_color0, lvl_n(ctx, l - 1), GT, 0, ctx->level_off[l - 1], ctx->phx,
                 (const long long *)ctx->old, ctx->gx, ctx->ghx, ctx->nbr6, ctx->child, ctx->bc, ctx->dscal);
@@ -1830,14 +1932,25 @@ static int fx_vcycle(sm_ctx *ctx, int top, int norm_slot = -1) {
                 ctx->gx, ctx->ghx, ctx->nbr6, ctx->child, ctx->bc, ctx->dscal);
     SM_CKL("vcycle down");
   }
-  if ((st = fx_coarse(ctx, top >= 1))) return st;
+  if ((st = fx_coarse(ctx, top >= 1, top))) return st;
   for (int l = 1; l <= top; ++l) {
-    if ((st = fx_prolong(ctx, l, 0, fx_norm_of(ctx, norm_slot >= 0 ? l - 1 : -1, norm_slot)))) return st;
-    if ((st = fx_smooth(ctx, l, ctx->cfg.nu2))) return st;
+    if (leg_level(ctx, l)) {
+      if ((st = fx_leg<fx::FS_PROLONG>(ctx, l))) return st;
+    } else {
+      if ((st = fx_prolong(ctx, l, 0, fx_norm_of(ctx, norm_slot >= 0 ? l - 1 : -1, norm_slot)))) return st;
+      if ((st = fx_smooth(ctx, l, ctx->cfg.nu2))) return st;
+    }
   }
   if (norm_slot >= 0) {
-    const int off = ctx->leaf_level_off[top];
-    return fx_leaf_norm(ctx, off, ctx->leaf_level_off[top + 1] - off, norm_slot);
+    // the leaves no prolongation launch has measured (one launch per run of
+    // levels; leaves are listed by level)
+    for (int l = 0; l <= top;) {
+      int m = l;
+      while (m <= top && (m == top || leg_level(ctx, m + 1))) ++m;
+      const int off = ctx->leaf_level_off[l];
+      if (m > l && (st = fx_leaf_norm(ctx, off, ctx->leaf_level_off[m] - off, norm_slot))) return st;
+      l = m + 1;
+    }
   }
   return SM_OK;
 }
@@ -1849,8 +1962,7 @@ static int fx_fmg_ladder(sm_ctx *ctx, int norm_slot) {
   int st;
   if ((st = fx_coarse(ctx))) return st;
   for (int l = 1; l < ctx->n_levels; ++l) {
-    if ((st = fx_prolong(ctx, l, 1, fx::FxNorm{}))) return st;
-    if ((st = fx_vcycle(ctx, l, l == ctx->n_levels - 1 ? norm_slot : -1))) return st;
+    if ((st = fx_vcycle(ctx, l, l == ctx->n_levels - 1 ? norm_slot : -1, true))) return st;
   }
   if (ctx->n_levels == 1) {
     SM_CK(cudaMemsetAsync(ctx->dscal + norm_slot, 0, sizeof(unsigned long long), ctx->stream));
@@ -1920,6 +2032,7 @@ static sm_graph *graph_of(sm_ctx *ctx, int kind) {
 }
 
 void sm_drop_graphs(sm_ctx *ctx) {
+  ctx->xch_reset = true;
   for (auto *g : {&ctx->g_solve, &ctx->g_fmg, &ctx->g_solve32, &ctx->g_fmg32}) {
     if (g->exec) cudaGraphExecDestroy(g->exec);
     g->exec = nullptr;
@@ -2321,6 +2434,12 @@ extern "C" int sm_persist_barrier_selftest(sm_ctx *ctx) {
   // every barrier waits for one block more than the grid holds
   if ((st = persistx_launch(ctx, ctx->n_levels - 1, 0, 0, 1))) return st;
   st = read_scalars(ctx);
+  if (st == SM_ETIMEOUT && leg_level(ctx, 1)) {
+    // and every wait of a one-launch leg expects a tag that is not published
+    if ((st = fx_set_margin(ctx))) return st;
+    if ((st = fx_leg<fx::FS_TOP>(ctx, 1, 128))) return st;
+    st = read_scalars(ctx);
+  }
   // the launch ended by itself: clear its flag so the context stays usable
   SM_CK(cudaMemsetAsync(ctx->dscal + SC_ERR, 0, sizeof(unsigned long long), ctx->stream));
   SM_CK(cudaStreamSynchronize(ctx->stream));

@@ -14,6 +14,12 @@
 
 namespace sm {
 
+constexpr int LEG_CAP = 1216;      // boxes of a level that may have exchange words (8 blocks on 152 SMs)
+constexpr int XWORDS = 6 * 2 * 32; // exchange words per box
+// row of the one-launch legs' box table: face neighbours, parent, octant and
+// face flags, the parent's face and edge neighbours (k_leg_rows)
+constexpr int LROW = 16;
+enum { LR_NB = 0, LR_P = 6, LR_FLAGS = 7, LR_PN = 8, LR_PE = 11 };
 constexpr int NC = SM_BOX;         // cells per box side (Sec. 2.1.1)
 constexpr int CELLS = NC * NC * NC;
 constexpr int FACE = NC * NC;
@@ -111,6 +117,13 @@ struct sm_ctx {
   // 2c + c_t1 + c_t2, all in quanta of the solve
   long long *phx = nullptr, *gx = nullptr;                  // [max_boxes][512]
   long long *ghx = nullptr;                                 // [max_boxes][6][64]
+  // exchange words of the levels whose legs run in one launch (mglevel.cuh):
+  // [box of such a level][6][2][32], and the tag counter of every level
+  long long *xch = nullptr;
+  unsigned *xseq = nullptr;  // [MAXL]
+  int32_t *leg_rows = nullptr;  // [max_boxes][16] what a leg needs to know of a box
+  int leg_max = -1;          // boxes of the largest such level (co-resident blocks; -1: not looked up)
+  bool xch_reset = true;     // clear both before the next solve (new mesh, other kernels chosen, a wait that ran out)
   int fx_margin = 5;         // exponent margin of the fixed-point scale
   int rows_min = 2048;       // boxes of a level from which its fixed-point kernels work by rows
   // FP32 error-equation arrays of the mixed-precision solve
