@@ -91,7 +91,7 @@ static Layout plan(int cap, bool mixed) {
   L.gh = p.take<double>((size_t)cap * 6 * FACE);
   L.cflux = p.take<double>((size_t)cap * 6 * FACE);
   L.basis = p.take<double>(3 * 64 + 3 * 8);
-  L.tab = p.take<double>(6 * 4096);  // mu, D, alpha and their slopes t[i+1] - t[i]
+  L.tab = p.take<double>(12 * 4096);  // mu, D, alpha and their slopes t[i+1] - t[i]; the same packed by entry
   L.dscal = p.take<unsigned long long>(SC_N);
   L.hist = p.take<double>(SM_HIST);
   L.phx = p.take<long long>(nc);
@@ -649,12 +649,17 @@ extern "C" int sm_set_table(sm_ctx *ctx, int n, double e_max, const double *mu, 
   if (!ctx->arena) return sm_fail(ctx, SM_ESTATE, "no arena bound");
   // each table and its slopes t[i+1] - t[i] (the FP64 differences that
   // linear interpolation forms, computed once here)
-  std::vector<double> all(6 * 4096, 0.0);
+  std::vector<double> all(12 * 4096, 0.0);
   const double *src[3] = {mu, diff, alpha};
   for (int k = 0; k < 3; ++k)
     for (int i = 0; i < n; ++i) {
-      all[4096 * k + i] = src[k][i];
-      all[4096 * (3 + k) + i] = i + 1 < n ? src[k][i + 1] - src[k][i] : 0.0;
+      const double t = src[k][i], d = i + 1 < n ? src[k][i + 1] - src[k][i] : 0.0;
+      all[4096 * k + i] = t;
+      all[4096 * (3 + k) + i] = d;
+      // mu and D of an entry together, alpha apart
+      double *q = k < 2 ? &all[4096 * 6 + 4 * i + 2 * k] : &all[4096 * 10 + 2 * i];
+      q[0] = t;
+      q[1] = d;
     }
   SM_CK(cudaMemcpyAsync(ctx->tab, all.data(), sizeof(double) * all.size(), cudaMemcpyHostToDevice, ctx->stream));
   // the host arrays may be released right after the call

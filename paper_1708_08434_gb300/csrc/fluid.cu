@@ -107,12 +107,58 @@ __device__ __forceinline__ double face_flux_h(double nL2, double nL, double nR, 
   return fma(-t1, nf, -dc * dn);
 }
 
-// 2 x, exactly, on the integer pipe, for 0 <= x < 2^1023 (not NaN):
-// doubling adds one to the exponent field of a normal value and shifts the
-// bits of a subnormal one (a carry into the exponent field is the result)
-__device__ __forceinline__ double twice(double x) {
+// Half the table index of a cell, e (n-1)/(2 e_max), in units of 2^-51
+// (rounded; clamped to n - 1): the significand of e times the scale's, shifted
+// by the exponents -- integer operations only.  A face's index is then the
+// integer sum of its two cells' values, its integer part the top bits.  The
+// error, 2^-52 a cell, is below the rounding of an FP64 index once that
+// exceeds 1 (a typical index of 500 has an ulp of 2^-44).
+__device__ __forceinline__ unsigned long long half_index(double e, const Table &tb) {
+  const unsigned long long bits = (unsigned long long)dbits(e);
+  const int ex = (int)(bits >> 52);  // the sign included: negative values give a large count
+  if (ex & 0x800) return 0ull;
+  const unsigned long long A = (bits << 11) | (ex ? 1ull << 63 : 0ull);
+  const unsigned long long hi = __umul64hi(A, tb.xm);
+  const int sh = tb.xs - (ex ? ex : 1);
+  if (sh <= 0) return tb.xtop;
+  const unsigned long long x = sh > 63 ? 0ull : ((hi >> (sh - 1)) + 1ull) >> 1;
+  return x < tb.xtop ? x : tb.xtop;
+}
+
+// integer part of an index x (units of 2^-51, clamped to n - 1) and its
+// fraction as an exact double: the leading one of the 51 bits is shifted to
+// the hidden bit's place
+__device__ __forceinline__ int index_split(unsigned long long x, const Table &tb, double &w) {
+  x = x < tb.xtop ? x : tb.xtop;
+  const unsigned long long f = x & ((1ull << 51) - 1ull);
+  const int lz = __clzll((long long)f);  // 13 .. 63 when f != 0
+  const unsigned long long m = f << (lz - 11);
+  w = f ? __longlong_as_double((long long)(((unsigned long long)(1034 - lz) << 52) + m)) : 0.0;
+  return (int)(x >> 51);
+}
+
+// dx times the flux through a face (as face_flux_h) from the differences
+// n_L - n_L2, n_R - n_L and n_R2 - n_R, which a line of faces shares, and the
+// fixed-point table index of the face
+__device__ __forceinline__ double face_flux_d(double nL, double nR, double dm, double dn, double dq, double dp,
+                                              unsigned long long x, const Table &tb) {
+  double w;
+  const double2 *fc = tb.fc + 2 * index_split(x, tb, w);
+  const double2 cm = __ldg(fc), cd = __ldg(fc + 1);
+  const double t1 = fma(w, cm.y, cm.x) * dp;
+  const bool up = dbits(t1) > 0;  // v < 0: the upwind cell is R
+  const double k = koren(up ? dq : dm, dn);
+  const double nf = (up ? nR : nL) + __longlong_as_double(dbits(k) ^ (up ? (long long)0x8000000000000000ull : 0ll));
+  return fma(-t1, nf, -fma(w, cd.y, cd.x) * dn);
+}
+
+// x / 2, exactly, on the integer pipe for zeros and values whose half is a
+// normal number
+__device__ __forceinline__ double halve(double x) {
   const long long b = dbits(x);
-  return __longlong_as_double((b >> 52) ? b + (1ll << 52) : b << 1);
+  const int ex = (int)((unsigned long long)b >> 52) & 0x7ff;
+  if ((ex > 1 && ex < 0x7ff)) return __longlong_as_double(b - (1ll << 52));
+  return (b << 1) == 0 ? x : 0.5 * x;
 }
 
 // Density ghost (depth t = 1 or 2) across refinement face f of fine box b
@@ -183,6 +229,26 @@ __device__ __forceinline__ void face_loc(int f, int dep, int u, int w, int c[3])
   c[(a + 2) % 3] = w;
 }
 
+// sqrt(x) with four FP64 instructions: x = 4^k m, 1 <= m < 4, from the bits;
+// g = sqrt(m) and h = 1/(2 sqrt(m)) in single precision; two steps of
+// Newton's iteration g += (m - g^2) h (Heron's method with the division
+// replaced by the approximate reciprocal), which leave an error of 2^-65
+// beside the last rounding.  Zeros, subnormals, infinities, NaNs and negative
+// values take the library function.
+__device__ __forceinline__ double sqrt_newton(double x) {
+  const unsigned long long bits = (unsigned long long)dbits(x);
+  const int ex = (int)(bits >> 52);
+  if (ex == 0 || ex >= 0x7ff) return (bits << 1) == 0 ? x : sqrt(x);
+  const int odd = (ex - 1023) & 1, k = (ex - 1023 - odd) / 2;
+  const double m = __longlong_as_double((long long)((bits & 0x000fffffffffffffull) | (unsigned long long)(1023 + odd) << 52));
+  const float mf = __uint_as_float((unsigned)(127 + odd) << 23 | (unsigned)((bits >> 29) & 0x7fffffu));
+  const float rs = rsqrtf(mf);
+  const double g0 = cvt_f32_f64(mf * rs), h = cvt_f32_f64(0.5f * rs);
+  const double g1 = fma(fma(-g0, g0, m), h, g0);
+  const double g2 = fma(fma(-g1, g1, m), h, g1);
+  return __longlong_as_double(dbits(g2) + ((long long)k << 52));
+}
+
 // ---------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------
@@ -210,7 +276,7 @@ __global__ void __launch_bounds__(512) k_field(const int32_t *__restrict__ leaf,
   }
   // |E| = |(p_-d - p_+d)| / (2 dx) summed in quadrature: each component is
   // the mean of (p_-d - p_c)/dx and (p_c - p_+d)/dx
-  emag[(size_t)b * CELLS + t] = sqrt(fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0]))) * (0.5 * ih);
+  emag[(size_t)b * CELLS + t] = sqrt_newton(fma(d[2], d[2], fma(d[1], d[1], d[0] * d[0]))) * (0.5 * ih);
 }
 
 // Eq. 5 right-hand side on leaf cells
@@ -221,19 +287,22 @@ __global__ void __launch_bounds__(512) k_charge(const int32_t *__restrict__ leaf
   rhs[x] = use_rho ? -rho[x] * inv_eps : -q * (ni[x] - ne[x]) * inv_eps;
 }
 
-// per-cell time-step quantities at table index x of the cell's |E|:
-// sum_d mu |E_d|/dx with E_d = (p_{-d} - p_{+d})/(2 dx) (the mean of the two
-// face fields), that plus 6 D/dx^2, and mu n_e
+// Per-cell time-step quantities at (fixed-point) table index x of the cell's
+// |E|: sum_d mu |E_d| 2 dx with E_d = (p_{-d} - p_{+d})/(2 dx) (the mean of
+// the two face fields), that plus 12 D (both to be scaled by 1/(2 dx^2)),
+// and mu n_e
 __device__ __forceinline__ void dt_terms(const double *__restrict__ phi, const double *__restrict__ gh,
-                                         const int32_t *__restrict__ nbr6, const Bc &bc, int b, int t, double ih2,
-                                         double x, double ne, const Table &tb, double &adv, double &ad,
+                                         const int32_t *__restrict__ nbr6, const Bc &bc, int b, int t,
+                                         unsigned long long x, double ne, const Table &tb, double &adv, double &ad,
                                          double &drt) {
   int c[3] = {t & 7, (t >> 3) & 7, t >> 6};
   const double *p = phi + (size_t)b * CELLS;
   double pc = p[t];
   const int stride[3] = {1, NC, FACE};
-  double mu, dc;
-  lookup2x(tb.mu, tb.dmu, tb.diff, tb.ddiff, tb.n, tb.xmax, x, mu, dc);
+  double w;
+  const double2 *fc = tb.fc + 2 * index_split(x, tb, w);
+  const double2 cm = __ldg(fc), cd = __ldg(fc + 1);
+  const double mu = fma(w, cm.y, cm.x);
   double d[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -242,16 +311,18 @@ __device__ __forceinline__ void dt_terms(const double *__restrict__ phi, const d
                               : pot_ghost(phi, nbr6, gh, b, 2 * a + 1, c[0], c[1], c[2], pc, bc, 0);
     d[a] = dabs(pm - pp);
   }
-  adv = (mu * ((d[0] + d[1]) + d[2])) * (0.5 * ih2);
-  ad = fma(6.0 * ih2, dc, adv);
+  adv = mu * ((d[0] + d[1]) + d[2]);
+  ad = fma(12.0, fma(w, cd.y, cd.x), adv);
   drt = mu * ne;
 }
 
 // block maxima of three non-negative quantities (negative values count as
-// 0) into slots[0..2], compared as bit patterns on the integer pipe; red:
-// 3 * (blockDim.x / 32) words of shared memory
+// 0) into slots[0..2], compared as bit patterns on the integer pipe, the
+// first two times scale (rounding is monotonic: the maximum of the products
+// is the product of the maximum); red: 3 * (blockDim.x / 32) words of shared
+// memory
 __device__ __forceinline__ void block_max3_to(unsigned long long *slots, double a, double b, double c,
-                                              long long *red) {
+                                              long long *red, double scale) {
   long long v[3] = {max(dbits(a), 0ll), max(dbits(b), 0ll), max(dbits(c), 0ll)};
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
@@ -265,6 +336,7 @@ __device__ __forceinline__ void block_max3_to(unsigned long long *slots, double 
   if (threadIdx.x < 3) {
     long long m = 0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = max(m, red[3 * w + threadIdx.x]);
+    if (threadIdx.x < 2) m = max(dbits(__longlong_as_double(m) * scale), 0ll);
     atomicMax(slots + threadIdx.x, (unsigned long long)m);
   }
 }
@@ -279,8 +351,8 @@ __global__ void __launch_bounds__(512) k_dt(const int32_t *__restrict__ leaf, co
   int t = threadIdx.x;
   size_t x = (size_t)b * CELLS + t;
   double adv, ad, drt;
-  dt_terms(phi, gh, nbr6, bc, b, t, lh.inv_h2[level[b]], emag[x] * tb.inv_de, ne[x], tb, adv, ad, drt);
-  block_max3_to(slots + SC_ADV, adv, ad, drt, red);
+  dt_terms(phi, gh, nbr6, bc, b, t, 2 * half_index(emag[x], tb), ne[x], tb, adv, ad, drt);
+  block_max3_to(slots + SC_ADV, adv, ad, drt, red, 0.5 * lh.inv_h2[level[b]]);
 }
 
 // Fine-side fluxes through the refinement faces of leaf boxes (64 threads
@@ -319,17 +391,6 @@ __global__ void __launch_bounds__(64) k_cf_flux(const int32_t *__restrict__ leaf
   }
 }
 
-// Smem layout of one box for the update kernel
-struct UpdSmem {
-  double n[12 * 12 * 12];   // density with 2 ghost layers on faces
-  double p[10 * 10 * 10];   // potential with 1 ghost layer
-  double x[10 * 10 * 10];   // half table index |E| (n-1)/(2 e_max), 1 ghost layer
-  double F[3 * 9 * 64];     // face fluxes times dx [a][m][w][u]
-  long long red[48];
-};
-__device__ __forceinline__ int I12(int i, int j, int k) { return (i + 2) + 12 * ((j + 2) + 12 * (k + 2)); }
-__device__ __forceinline__ int I10(int i, int j, int k) { return (i + 1) + 10 * ((j + 1) + 10 * (k + 1)); }
-
 // index in a staged box of pitch P (O ghost layers) of the cell with
 // coordinate ca along axis a and u, w along axes (a+1)%3, (a+2)%3 (no
 // arrays indexed at run time: those would live in local memory)
@@ -341,129 +402,211 @@ __device__ __forceinline__ int lin_axis(int a, int ca, int u, int w) {
   return (x + O) + P * ((y + O) + P * (z + O));
 }
 
+// Shared memory of the update kernel.  Row and plane pitches make 16 lanes
+// on consecutive y (or x) of two consecutive z hit 16 different 8-byte banks.
+constexpr int UT = 192;                  // threads: one line of faces each (3 axes x 64)
+constexpr int NY = 13, NZ = 168;         // density with 2 ghost layers on faces
+constexpr int PY = 11, PZ = 120;         // potential and half index with 1 ghost layer
+constexpr int DY = 9, DZ = 72, DA = 576; // flux differences [axis][cell], over the density
+struct UpdSmem {
+  double n[12 * NZ];
+  double p[10 * PZ];
+  unsigned long long x[10 * PZ];
+  long long red[3 * (UT / 32)];
+};
+static_assert(3 * DA <= 12 * NZ, "the flux differences fit the density's place");
+__device__ __forceinline__ int iN(int x, int y, int z) { return (x + 2) + NY * (y + 2) + NZ * (z + 2); }
+__device__ __forceinline__ int iP(int x, int y, int z) { return (x + 1) + PY * (y + 1) + PZ * (z + 1); }
+
 // One forward-Euler stage on a leaf box: dst = src + dt F(src), with
 // F = -div(flux) + alpha mu |E| n_e for electrons and the same source for
-// ions.  heun != 0: dst = (n0 + src + dt F(src))/2.  Also writes the Eq. 5
-// right-hand side from dst, and with want_dt the time-step maxima of src.
-__global__ void __launch_bounds__(512, 3) k_update(
+// ions.  HEUN: dst = (n0 + src + dt F(src))/2, and the time-step maxima of
+// src.  Also writes the Eq. 5 right-hand side from dst.
+//
+// Bound by the FP64 pipe (2 instructions per clock and SM), so the work is
+// laid out to issue few of them: a thread marches one line of 9 faces along
+// an axis and forms each density difference once (three faces use it), table
+// indices and halvings are integer operations, and dt / dx^2 is one factor.  50 FP64
+// instructions per cell in stage 1 (the cell-and-face form before: 64).
+template <bool HEUN>
+__global__ void __launch_bounds__(UT, 5) k_update(
     const int32_t *__restrict__ leaf, const int32_t *__restrict__ level, const double *__restrict__ ne_src,
     const double *__restrict__ ni_src, const double *__restrict__ ne0, const double *__restrict__ ni0,
     double *__restrict__ ne_dst, double *__restrict__ ni_dst, const double *__restrict__ phi,
     const double *__restrict__ gh, const double *__restrict__ emag, const double *__restrict__ cflux,
     const int32_t *__restrict__ nbr6, const int32_t *__restrict__ child, const int32_t *__restrict__ parent,
-    const int32_t *__restrict__ ijk, Bc bc, LevelH lh, Table tb, double dt, int heun, double q, double inv_eps,
-    double *__restrict__ rhs, int want_dt, unsigned long long *slots) {
-  extern __shared__ double smraw[];
+    const int32_t *__restrict__ ijk, Bc bc, LevelH lh, Table tb, double dt, double qie, double *__restrict__ rhs,
+    unsigned long long *slots) {
+  extern __shared__ __align__(16) unsigned char smraw[];
   UpdSmem &S = *reinterpret_cast<UpdSmem *>(smraw);
-  int b = leaf[blockIdx.x];
-  int t = threadIdx.x;
-  int l = level[b];
-  const double h = lh.h[l], ih2 = lh.inv_h2[l];
-  size_t base = (size_t)b * CELLS;
-  int ci = t & 7, cj = (t >> 3) & 7, ck = t >> 6;
-  const double e = emag[base + t];
-  const double xh = e * tb.hinv_de;  // the cell's table index is 2 xh, exactly e (n-1)/e_max
-  S.n[I12(ci, cj, ck)] = ne_src[base + t];
-  S.p[I10(ci, cj, ck)] = phi[base + t];
-  S.x[I10(ci, cj, ck)] = xh;
+  const int b = leaf[blockIdx.x], t = threadIdx.x, l = level[b];
+  const double ih2 = lh.inv_h2[l];
+  const size_t base = (size_t)b * CELLS;
+  // x pairs of cells: pair t, and t + 192 for the first 64 threads
+  double2 nc[2], ec[2];
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int pi = t + UT * s;
+    if (pi >= CELLS / 2) continue;
+    const int x = 2 * (pi & 3), y = (pi >> 2) & 7, z = pi >> 5;
+    nc[s] = reinterpret_cast<const double2 *>(ne_src + base)[pi];
+    ec[s] = reinterpret_cast<const double2 *>(emag + base)[pi];
+    const double2 pc = reinterpret_cast<const double2 *>(phi + base)[pi];
+    const int q = iP(x, y, z);
+    S.n[iN(x, y, z)] = nc[s].x;
+    S.n[iN(x + 1, y, z)] = nc[s].y;
+    S.p[q] = pc.x;
+    S.p[q + 1] = pc.y;
+    S.x[q] = half_index(ec[s].x, tb);
+    S.x[q + 1] = half_index(ec[s].y, tb);
+  }
+  // fluxes known before the faces are walked: this thread's line meets the
+  // box's low and high face, whose flux at a refinement face is the fine
+  // side's (k_cf_flux), on the coarse side the mean of the four fine ones
+  const int a = t >> 6, c0 = t & 7, c1 = (t >> 3) & 7;
+  const int fu = a == 1 ? c1 : c0, fw = a == 1 ? c0 : c1;  // the line's face coordinates
+  double Fk[2] = {0.0, 0.0};
+  bool known[2] = {false, false};
+#pragma unroll
+  for (int hi = 0; hi < 2; ++hi) {
+    const int f = 2 * a + hi, nb = nbr6[6 * b + f];
+    if (nb == -2) {
+      Fk[hi] = cflux[(size_t)(6 * b + f) * FACE + fu + NC * fw] * lh.h[l];
+      known[hi] = true;
+    } else if (nb >= 0 && child[8 * nb] >= 0) {
+      const int ch = child[8 * nb + lin_axis<2, 0>(a, hi ? 0 : 1, fu >> 2, fw >> 2)];
+      const double *cf = cflux + (size_t)(6 * ch + (f ^ 1)) * FACE;
+      const int uf = 2 * (fu & 3), wf = 2 * (fw & 3);
+      double s = 0.0;
+      s += cf[uf + NC * wf];
+      s += cf[uf + 1 + NC * wf];
+      s += cf[uf + NC * (wf + 1)];
+      s += cf[uf + 1 + NC * (wf + 1)];
+      Fk[hi] = (s * 0.25) * lh.h[l];
+      known[hi] = true;
+    }
+  }
   __syncthreads();
-  // face halos: thread -> (face, face cell)
-  if (t < 6 * FACE) {
-    const int f = t >> 6, fc = t & 63;
-    const int u = fc & 7, w = fc >> 3, a = f >> 1, hi = f & 1;
+  // face halos: 6 x 64 face cells, two per thread
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int it = t + UT * s, f = it >> 6, ha = f >> 1, hi = f & 1;
+    const int x8 = it & 7, y8 = (it >> 3) & 7;
+    const int u = ha == 1 ? y8 : x8, w = ha == 1 ? x8 : y8;
     const int nb = nbr6[6 * b + f];
-    // depths 0, 1 inside the face and the ghosts -1, -2 along axis a
-    const int d0 = hi ? NC - 1 : 0, d1 = hi ? NC - 2 : 1, dg1 = hi ? NC : -1, dg2 = hi ? NC + 1 : -2;
-    const int r0 = lin_axis<10, 1>(a, d0, u, w);
-    double n0 = S.n[lin_axis<12, 2>(a, d0, u, w)], n1 = S.n[lin_axis<12, 2>(a, d1, u, w)];
-    double p0 = S.p[r0], x0 = S.x[r0];
-    double vg1, vg2, pg, xg;
+    // depths 0, 1 inside the face and the ghosts -1, -2 along the face axis
+    const int d0 = hi ? NC - 1 : 0, sg = hi ? 1 : -1;
+    const int X = ha == 0 ? d0 : x8, Y = ha == 0 ? x8 : (ha == 1 ? d0 : y8), Z = ha == 2 ? d0 : y8;
+    const int qn = iN(X, Y, Z), sn = sg * (ha == 0 ? 1 : (ha == 1 ? NY : NZ));
+    const int qp = iP(X, Y, Z), sp = sg * (ha == 0 ? 1 : (ha == 1 ? PY : PZ));
+    double vg1, vg2, pg;
+    unsigned long long xg;
     if (nb >= 0) {
       // the neighbour's cells at depths 0 and 1 of its opposite face
-      const int m0 = lin_axis<8, 0>(a, hi ? 0 : NC - 1, u, w), m1 = lin_axis<8, 0>(a, hi ? 1 : NC - 2, u, w);
-      size_t nbase = (size_t)nb * CELLS;
+      const int m0 = lin_axis<8, 0>(ha, hi ? 0 : NC - 1, u, w), m1 = lin_axis<8, 0>(ha, hi ? 1 : NC - 2, u, w);
+      const size_t nbase = (size_t)nb * CELLS;
       vg1 = ne_src[nbase + m0];
       vg2 = ne_src[nbase + m1];
       pg = phi[nbase + m0];
-      xg = child[8 * nb] < 0 ? emag[nbase + m0] * tb.hinv_de : 0.0;
+      xg = child[8 * nb] < 0 ? half_index(emag[nbase + m0], tb) : 0ull;
     } else if (nb == -1) {
-      vg1 = n0;
-      vg2 = n1;
-      pg = bc.type[f] ? 2.0 * bc.val[f] - p0 : p0;
-      xg = x0;
+      vg1 = S.n[qn];
+      vg2 = S.n[qn - sn];
+      pg = bc.type[f] ? 2.0 * bc.val[f] - S.p[qp] : S.p[qp];
+      xg = S.x[qp];
     } else {
       vg1 = density_cf_ghost(ne_src, nbr6, parent, ijk, b, f, 1, u, w, slots + SC_ERR);
       vg2 = density_cf_ghost(ne_src, nbr6, parent, ijk, b, f, 2, u, w, slots + SC_ERR);
-      pg = p0 * (1.0 / 3.0) + (2.0 / 3.0) * gh[(size_t)(6 * b + f) * FACE + u + NC * w];
-      xg = emag_cf_ghost(emag, nbr6, parent, ijk, b, f, u, w) * tb.hinv_de;
+      pg = S.p[qp] * (1.0 / 3.0) + (2.0 / 3.0) * gh[(size_t)(6 * b + f) * FACE + u + NC * w];
+      xg = half_index(emag_cf_ghost(emag, nbr6, parent, ijk, b, f, u, w), tb);
     }
-    S.n[lin_axis<12, 2>(a, dg1, u, w)] = vg1;
-    S.n[lin_axis<12, 2>(a, dg2, u, w)] = vg2;
-    const int rg = lin_axis<10, 1>(a, dg1, u, w);
-    S.p[rg] = pg;
-    S.x[rg] = xg;
+    S.n[qn + sn] = vg1;
+    S.n[qn + 2 * sn] = vg2;
+    S.p[qp + sp] = pg;
+    S.x[qp + sp] = xg;
   }
   __syncthreads();
-  // fluxes: 3 axes x 9 faces x 64
-  for (int x = t; x < 3 * 9 * FACE; x += blockDim.x) {
-    int a = x / (9 * FACE), rem = x % (9 * FACE);
-    int m = rem >> 6, u = rem & 7, w = (rem >> 3) & 7;
-    double F;
-    bool done = false;
-    if (m == 0 || m == NC) {
-      int f = 2 * a + (m == NC);
-      int nb = nbr6[6 * b + f];
-      if (nb == -2) {
-        F = cflux[(size_t)(6 * b + f) * FACE + u + NC * w] * h;
-        done = true;
-      } else if (nb >= 0 && child[8 * nb] >= 0) {
-        // coarse side of a refinement face: mean of the 4 fine fluxes
-        int ch = child[8 * nb + lin_axis<2, 0>(a, (f & 1) ? 0 : 1, u >> 2, w >> 2)];
-        const double *cf = cflux + (size_t)(6 * ch + (f ^ 1)) * FACE;
-        int uf = 2 * (u & 3), wf = 2 * (w & 3);
-        double s = 0.0;
-        s += cf[uf + NC * wf];
-        s += cf[uf + 1 + NC * wf];
-        s += cf[uf + NC * (wf + 1)];
-        s += cf[uf + 1 + NC * (wf + 1)];
-        F = (s * 0.25) * h;
-        done = true;
+  // the line's 9 faces: face m between cells m - 1 and m
+  double D[NC];
+  {
+    const int X = a == 0 ? 0 : c0, Y = a == 0 ? c0 : (a == 1 ? 0 : c1), Z = a == 2 ? 0 : c1;
+    const int sn = a == 0 ? 1 : (a == 1 ? NY : NZ), sp = a == 0 ? 1 : (a == 1 ? PY : PZ);
+    const double *n = S.n + iN(X, Y, Z), *p = S.p + iP(X, Y, Z);
+    const unsigned long long *xi = S.x + iP(X, Y, Z);
+    double nL = n[-sn], nR = n[0], dm = nL - n[-2 * sn], dn = nR - nL, pL = p[-sp], F0 = 0.0;
+    unsigned long long xL = xi[-sp];
+#pragma unroll
+    for (int m = 0; m <= NC; ++m) {
+      const double n2 = n[(m + 1) * sn], dq = n2 - nR, pR = p[m * sp];
+      const unsigned long long xR = xi[m * sp];
+      double F;
+      if (m == 0 && known[0]) F = Fk[0];
+      else if (m == NC && known[1]) F = Fk[1];
+      else F = face_flux_d(nL, nR, dm, dn, dq, pL - pR, xL + xR, tb);
+      if (m > 0) D[m - 1] = F - F0;
+      F0 = F;
+      nL = nR;
+      nR = n2;
+      dm = dn;
+      dn = dq;
+      pL = pR;
+      xL = xR;
+    }
+    __syncthreads();  // the density is no longer read: its place takes the differences
+    double *d = S.n + DA * a + X + DY * Y + DZ * Z;
+    const int sd = a == 0 ? 1 : (a == 1 ? DY : DZ);
+#pragma unroll
+    for (int m = 0; m < NC; ++m) d[m * sd] = D[m];
+  }
+  __syncthreads();
+  const double dth = -dt * ih2;
+  double m_adv = 0.0, m_ad = 0.0, m_drt = 0.0;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int pi = t + UT * s;
+    if (pi >= CELLS / 2) continue;
+    const int x0 = 2 * (pi & 3), y = (pi >> 2) & 7, z = pi >> 5;
+    const double2 ni = reinterpret_cast<const double2 *>(ni_src + base)[pi];
+    double2 e0, i0;
+    if (HEUN) {
+      e0 = reinterpret_cast<const double2 *>(ne0 + base)[pi];
+      i0 = reinterpret_cast<const double2 *>(ni0 + base)[pi];
+    }
+    double ne_new[2], ni_new[2], f[2];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const double *d = S.n + (x0 + c) + DY * y + DZ * z;
+      const double div = (d[0] + d[DA]) + d[2 * DA];  // dx^2 times the divergence
+      const double nes = c ? nc[s].y : nc[s].x, e = c ? ec[s].y : ec[s].x, nis = c ? ni.y : ni.x;
+      const int q = iP(x0 + c, y, z);
+      double w;
+      const int i = index_split(2 * S.x[q], tb, w);
+      const double2 cm = __ldg(tb.fc + 2 * i), al = __ldg(tb.al + i);
+      const double mu = fma(w, cm.y, cm.x);
+      const double src = fma(w, al.y, al.x) * mu * e * nes;
+      ne_new[c] = fma(dth, div, fma(dt, src, nes));
+      ni_new[c] = fma(dt, src, nis);
+      if (HEUN) {
+        ne_new[c] = halve((c ? e0.y : e0.x) + ne_new[c]);
+        ni_new[c] = halve((c ? i0.y : i0.x) + ni_new[c]);
+        // sum_d mu |E_d| 2 dx, that plus 12 D (both times 1/(2 dx^2) below), mu n_e
+        const double gx = dabs(S.p[q - 1] - S.p[q + 1]), gy = dabs(S.p[q - PY] - S.p[q + PY]),
+                     gz = dabs(S.p[q - PZ] - S.p[q + PZ]);
+        const double adv = mu * ((gx + gy) + gz);
+        const double2 cd = __ldg(tb.fc + 2 * i + 1);
+        const double ad = fma(12.0, fma(w, cd.y, cd.x), adv), drt = mu * nes;
+        // maxima of bit patterns, as block_max3_to compares them
+        m_adv = dbits(adv) > dbits(m_adv) ? adv : m_adv;
+        m_ad = dbits(ad) > dbits(m_ad) ? ad : m_ad;
+        m_drt = dbits(drt) > dbits(m_drt) ? drt : m_drt;
       }
+      f[c] = (ni_new[c] - ne_new[c]) * qie;
     }
-    if (!done) {
-      // cells m-2 .. m+1 along axis a
-      const int q = lin_axis<12, 2>(a, m - 2, u, w), sq = a == 0 ? 1 : (a == 1 ? 12 : 144);
-      const int r = lin_axis<10, 1>(a, m - 1, u, w), sr = a == 0 ? 1 : (a == 1 ? 10 : 100);
-      F = face_flux_h(S.n[q], S.n[q + sq], S.n[q + 2 * sq], S.n[q + 3 * sq], S.p[r], S.p[r + sr],
-                      S.x[r] + S.x[r + sr], tb);
-    }
-    S.F[(a * 9 + m) * FACE + u + NC * w] = F;
+    reinterpret_cast<double2 *>(ne_dst + base)[pi] = make_double2(ne_new[0], ne_new[1]);
+    reinterpret_cast<double2 *>(ni_dst + base)[pi] = make_double2(ni_new[0], ni_new[1]);
+    reinterpret_cast<double2 *>(rhs + base)[pi] = make_double2(f[0], f[1]);
   }
-  __syncthreads();
-  // update: div = sum over axes of the flux differences (times dx) / dx^2
-  const double *Fx = S.F + (0 * 9 + ci) * FACE + cj + NC * ck;
-  const double *Fy = S.F + (1 * 9 + cj) * FACE + ck + NC * ci;
-  const double *Fz = S.F + (2 * 9 + ck) * FACE + ci + NC * cj;
-  const double div = ((Fx[FACE] - Fx[0]) + (Fy[FACE] - Fy[0]) + (Fz[FACE] - Fz[0])) * ih2;
-  double nes = S.n[I12(ci, cj, ck)];
-  const double x = twice(xh);  // e (n-1)/e_max
-  double alpha, mu;
-  lookup2x(tb.alpha, tb.dalpha, tb.mu, tb.dmu, tb.n, tb.xmax, x, alpha, mu);
-  double src = alpha * mu * e * nes;
-  double ne_new = fma(dt, src - div, nes);
-  double ni_new = fma(dt, src, ni_src[base + t]);
-  if (heun) {
-    ne_new = 0.5 * (ne0[base + t] + ne_new);
-    ni_new = 0.5 * (ni0[base + t] + ni_new);
-  }
-  ne_dst[base + t] = ne_new;
-  ni_dst[base + t] = ni_new;
-  rhs[base + t] = (ni_new - ne_new) * (-q * inv_eps);
-  if (want_dt) {
-    double adv, ad, drt;
-    dt_terms(phi, gh, nbr6, bc, b, t, ih2, x, nes, tb, adv, ad, drt);
-    block_max3_to(slots + SC_ADV, adv, ad, drt, S.red);
-  }
+  if (HEUN) block_max3_to(slots + SC_ADV, m_adv, m_ad, m_drt, S.red, 0.5 * ih2);
 }
 
 // ---------------------------------------------------------------------------
@@ -482,6 +625,13 @@ static Table table_of(const sm_ctx *ctx) {
   tb.hinv_de = 0.5 * tb.inv_de;
   const double top = (double)(ctx->tab_n - 1);
   memcpy(&tb.xmax, &top, sizeof top);
+  tb.fc = reinterpret_cast<const double2 *>(ctx->tab + 6 * 4096);
+  tb.al = reinterpret_cast<const double2 *>(ctx->tab + 10 * 4096);
+  int p = 0;
+  const double f = frexp(tb.hinv_de, &p);  // hinv_de = xm 2^(p - 64)
+  tb.xm = (unsigned long long)ldexp(f, 64);
+  tb.xs = 1035 - p;
+  tb.xtop = (unsigned long long)(ctx->tab_n - 1) << 51;
   return tb;
 }
 
@@ -555,8 +705,9 @@ extern "C" int sm_dt_limit(sm_ctx *ctx, double q, double eps, double *dt) {
   return dt_from_slots(ctx, q, eps, dt);
 }
 
-// one stage from buffer s into buffer d (heun: averaged with buffer h0)
-static int stage(sm_ctx *ctx, int s, int d, int h0, double dt, double q, double eps, int want_dt) {
+// one stage from buffer s into buffer d; with h0 >= 0 averaged with buffer h0
+// (second Heun stage), leaving the time-step maxima of s
+static int stage(sm_ctx *ctx, int s, int d, int h0, double dt, double q, double eps) {
   int st;
   Table tb = table_of(ctx);
   if ((st = sm_fill_all_cf(ctx, ctx->phi))) return st;
@@ -567,12 +718,17 @@ static int stage(sm_ctx *ctx, int s, int d, int h0, double dt, double q, double 
     ++ctx->n_launch;
     SM_CKL("cf_flux");
   }
-  size_t smem = sizeof(UpdSmem);
-  k_update<<<ctx->n_leaves, 512, smem, ctx->stream>>>(
-      ctx->leaf, ctx->level, ctx->nbuf[s], ctx->ibuf[s], h0 >= 0 ? ctx->nbuf[h0] : nullptr,
-      h0 >= 0 ? ctx->ibuf[h0] : nullptr, ctx->nbuf[d], ctx->ibuf[d], ctx->phi, ctx->gh, ctx->emag, ctx->cflux,
-      ctx->nbr6, ctx->child, ctx->parent, ctx->ijk, ctx->bc, ctx->lh, tb, dt, h0 >= 0, q, 1.0 / eps, ctx->rhs,
-      want_dt, ctx->dscal);
+  const size_t smem = sizeof(UpdSmem);
+  // rhs = -q (n_i - n_e) / eps of the new densities; with h0 the Heun average
+  auto run = [&](auto kernel) {
+    kernel<<<ctx->n_leaves, UT, smem, ctx->stream>>>(
+        ctx->leaf, ctx->level, ctx->nbuf[s], ctx->ibuf[s], h0 >= 0 ? ctx->nbuf[h0] : nullptr,
+        h0 >= 0 ? ctx->ibuf[h0] : nullptr, ctx->nbuf[d], ctx->ibuf[d], ctx->phi, ctx->gh, ctx->emag, ctx->cflux,
+        ctx->nbr6, ctx->child, ctx->parent, ctx->ijk, ctx->bc, ctx->lh, tb, dt, -q * (1.0 / eps), ctx->rhs,
+        ctx->dscal);
+  };
+  if (h0 >= 0) run(k_update<true>);
+  else run(k_update<false>);
   ++ctx->n_launch;
   SM_CKL("update");
   return sm_restrict_pair(ctx, ctx->nbuf[d], ctx->ibuf[d]);
@@ -587,7 +743,7 @@ extern "C" int sm_fluid_stage(sm_ctx *ctx, double dt) {
   if ((st = sm_restrict_pair(ctx, ctx->nbuf[a], ctx->ibuf[a]))) return st;
   // q/eps only feed the right-hand side written alongside; a stage alone
   // uses SI values
-  if ((st = stage(ctx, a, b, -1, dt, 1.602176634e-19, 8.8541878128e-12, 0))) return st;
+  if ((st = stage(ctx, a, b, -1, dt, 1.602176634e-19, 8.8541878128e-12))) return st;
   ctx->ncur = b;
   return SM_OK;
 }
@@ -608,7 +764,7 @@ extern "C" int sm_advance_fluid(sm_ctx *ctx, double dt, double q, double eps, do
   int A = ctx->ncur, B = (A + 1) % 3, C = (A + 2) % 3;
   if ((st = sm_restrict_pair(ctx, ctx->nbuf[A], ctx->ibuf[A]))) return st;
   // stage 1: n1 = n0 + dt F(n0); new field
-  if ((st = stage(ctx, A, B, -1, dt, q, eps, 0))) return st;
+  if ((st = stage(ctx, A, B, -1, dt, q, eps))) return st;
   int c1 = 0, c2 = 0, st1, st2;
   if (ctx->pre_solve && (st = ctx->pre_solve(ctx->hook_obj, ctx))) return st;
   st1 = sm_mg_solve(ctx, tol, max_cycles, &c1, nullptr);
@@ -617,7 +773,7 @@ extern "C" int sm_advance_fluid(sm_ctx *ctx, double dt, double q, double eps, do
   if ((st = sm_compute_field(ctx))) return st;
   // stage 2: n = (n0 + n1 + dt F(n1))/2 with the time-step limits at n1
   SM_CK(cudaMemsetAsync(ctx->dscal + SC_ADV, 0, 3 * sizeof(unsigned long long), ctx->stream));
-  if ((st = stage(ctx, B, C, A, dt, q, eps, 1))) return st;
+  if ((st = stage(ctx, B, C, A, dt, q, eps))) return st;
   ctx->ncur = C;
   // the maxima go to the staged host copy without a wait: the solve below
   // synchronises before they are read
