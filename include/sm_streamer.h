@@ -557,22 +557,15 @@ const char *sm_cnn_last_error(const sm_cnn *c);
  *   f:       DEVICE double [n_problems][512] right-hand side (cell i+8j+64k)
  *   phi:     DEVICE double [n_problems][512] solution (written)
  *   stream:  cudaStream_t as void*; the call only enqueues work.
- * The library allocates nothing: its only scratch (one eigenbasis per
- * problem) is a fixed device array of SM_NOALLOC_MAX_PROBLEMS x 1728 bytes
- * (1.77 MB) that every GPU loading the library holds until exit.  The first
- * call on a device looks up that array's device address (set-up, with the
- * device current); make that first call before any stream capture.  Every
- * later call made outside a capture looks the address up again, so after a
- * device reset (cudaDeviceReset) make one uncaptured call before capturing
- * again.  Each device has its own copy of the array.  All calls on one
- * device share it and each call overwrites the slots of its problems before
- * reading them, so nothing needs clearing, but calls that overlap on the
- * same device (different streams) race on it and must be ordered; calls on
- * different devices are independent.  Device ordinals 0..63 are supported.
- * Errors: SM_ENOMEM if n_problems > SM_NOALLOC_MAX_PROBLEMS (the fixed
- * scratch is too small), SM_EINVAL (n_problems < 0, length <= 0, null
- * pointer, device ordinal above 63), SM_ECUDA (no device, first call of a
- * device inside a stream capture, address lookup or launch failed). */
+ * The library allocates nothing and keeps nothing on the device: the
+ * eigenbases travel as launch parameters, so calls on different streams are
+ * independent.  The first call on a device loads the kernels (with the
+ * device current); make that first call before any stream capture.  Device
+ * ordinals 0..63 are supported.
+ * Errors: SM_ENOMEM if n_problems > SM_NOALLOC_MAX_PROBLEMS, SM_EINVAL
+ * (n_problems < 0, length <= 0, null pointer, device ordinal above 63),
+ * SM_ECUDA (no device, first call of a device inside a stream capture,
+ * launch failed). */
 #define SM_NOALLOC_MAX_PROBLEMS 1024
 int sm_box_solve_noalloc(double length, int n_problems, const int32_t *bc_type, const double *bc_val,
                          const double *f, double *phi, void *stream);
