@@ -374,15 +374,18 @@ __global__ void __launch_bounds__(QT) k_q_prolong(int off, int n, int l, double 
   }
 }
 
+#include "quadleg.cuh"
+
 // Exact level-0 solve (one box): phi = A^-1 (f - L0), A the operator's
 // matrix with homogeneous wall ghosts (inverted on the host), L0 the
 // operator of phi = 0 with the wall values.
 __global__ void k_q_coarse(double *__restrict__ phi, const double *__restrict__ rhs, const double *__restrict__ ainv,
-                           QTabs T, const __grid_constant__ QBc bc, double inv_h2) {
+                           QTabs T, const __grid_constant__ QBc bc, double inv_h2, unsigned *xseq) {
   __shared__ double r[QC];
   const int c = threadIdx.x, i = c % QN, j = c / QN;
   const double wl = T.w[3 * i], wh = T.w[3 * i + 1];
   q_wait();
+  if (c == 0) ++*xseq;  // the exchange tags move on between the two legs of every level
   double l0 = 0.0;
   if (i == 0 && bc.type[0]) l0 += wl * bc.g2[0];
   if (i == QN - 1 && bc.type[1]) l0 += wh * bc.g2[1];
@@ -1105,6 +1108,9 @@ struct sm_quad {
   double *cflux = nullptr, *ainv = nullptr, *lut = nullptr, *d_h = nullptr;
   unsigned long long *slots = nullptr;
   unsigned *d_err = nullptr;
+  unsigned long long *xch = nullptr;      // exchange words of the one-launch legs [max_boxes][4][8][2]
+  unsigned *xseq = nullptr;               // their tag counter
+  int leg_max = -1;                       // boxes of the largest level with such legs (-1: not looked up)
   double *snap = nullptr;                 // regrid snapshot [6][max_boxes][64]
   int *d_rg = nullptr;                    // regrid move descriptors [max_boxes][10]
   unsigned long long *d_need = nullptr;   // refinement test: cells that need refinement, per box
@@ -1116,8 +1122,8 @@ struct sm_quad {
   // V-cycle graphs per top level (captured on first use, dropped when the
   // mesh changes) and the launches each holds
   cudaStream_t cap = nullptr;
-  cudaGraphExec_t vgraph[QMAXL] = {nullptr};
-  long long vgraph_launches[QMAXL] = {0};
+  cudaGraphExec_t vgraph[2 * QMAXL] = {nullptr};  // [fmg][top]
+  long long vgraph_launches[2 * QMAXL] = {0};
   bool graphs = true, pdl = true;
   ~sm_quad() {
     for (auto &g : vgraph)
@@ -1320,20 +1326,94 @@ void smooth(sm_quad *q, int l, int nu, bool skip_first = false) {
 
 void coarse_solve(sm_quad *q) {
   qlaunch(q, k_q_coarse, 1, QC, q->var[V_PHI], (const double *)q->var[V_RHS], (const double *)q->ainv, tabs(q),
-          q->bc, q->inv_h2[0]);
+          q->bc, q->inv_h2[0], q->xseq);
 }
 
-void vcycle(sm_quad *q, int top) {
+// Boxes of the largest level whose legs run in one launch (a warp per box,
+// all resident at once); 0 without cooperative launch.
+int leg_limit(sm_quad *q) {
+  if (q->leg_max >= 0) return q->leg_max;
+  int dev = 0, coop = 0, sms = 0, most = 1 << 30;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  auto fits = [&](auto *k) {
+    int per = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32, 0) != cudaSuccess) per = 0;
+    most = std::min(most, per * sms);
+  };
+  fits(k_q_leg<QL_TOP>);
+  fits(k_q_leg<QL_FAS>);
+  fits(k_q_leg<QL_PROLONG>);
+  fits(k_q_leg<QL_FMG>);
+  cudaGetLastError();
+  return q->leg_max = coop ? most : 0;
+}
+
+bool leg_level(sm_quad *q, int l) {
+  return l >= 1 && level_count(q, l) > 0 && level_count(q, l) <= leg_limit(q);
+}
+
+template <int START>
+void leg(sm_quad *q, int l, unsigned skew = 0) {
+  constexpr bool up = START == QL_PROLONG;
+  QLeg a = {};
+  a.lo = q->off[l];
+  a.nu = up ? q->nu2 : q->nu1;
+  a.leg = up ? 0u : 64u;
+  a.skew = skew;
+  a.h2 = q->h[l] * q->h[l];
+  a.inv_h2 = q->inv_h2[l];
+  a.phi = q->var[V_PHI];
+  a.rhs = q->var[V_RHS];
+  a.old = q->var[V_OLD];
+  a.xch = q->xch;
+  a.seq = q->xseq;
+  a.err = q->d_err;
+  a.lev = l;
+  a.T = tabs(q);
+  a.bc = q->bc;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(level_count(q, l));
+  cfg.blockDim = dim3(32);
+  cfg.stream = q->stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k_q_leg<START>, a);
+  ++q->launches;
+}
+
+// One V-cycle with level `top` on top; with fmg that level first takes the
+// prolonged solution of the level below.  A level whose boxes are all
+// resident at once runs each leg in one launch, a larger one a launch per
+// operation (below another such level the FAS completion also runs the first
+// colour pass, on a copy of the whole level that the restriction leaves in
+// old).
+void vcycle(sm_quad *q, int top, bool fmg = false) {
   bool fused = false;  // the first colour pass of level l has run (k_q_fas_rbgs0)
+  if (fmg && !leg_level(q, top)) {
+    const int n = level_count(q, top);
+    qlaunch(q, k_q_prolong, blocks_for(n), QT, q->off[top], n, top, q->var[V_PHI], (const double *)q->var[V_OLD], 0,
+            tabs(q), q->bc, q->d_err);
+  }
   for (int l = top; l >= 1; --l) {
-    smooth(q, l, q->nu1, fused);
     const int n = level_count(q, l), nc = level_count(q, l - 1);
-    // below the top level but above level 0 the FAS step also runs the first
-    // colour pass; the restriction then copies the level's leaves into old
-    fused = l - 1 >= 1;
-    const int ncp = fused ? nc : 0;
-    qlaunch(q, k_q_resid_restrict, blocks_for(n + ncp), QT, q->off[l], n, l, (const double *)q->var[V_PHI],
-            q->var[V_RHS], q->var[V_OLD], tabs(q), q->bc, q->inv_h2[l], q->d_err, q->off[l - 1], ncp);
+    if (leg_level(q, l)) {
+      if (l < top) leg<QL_FAS>(q, l);
+      else if (fmg) leg<QL_FMG>(q, l);
+      else leg<QL_TOP>(q, l);
+      fused = false;
+    } else {
+      smooth(q, l, q->nu1, fused);
+      fused = l - 1 >= 1 && !leg_level(q, l - 1);
+      const int ncp = fused ? nc : 0;
+      qlaunch(q, k_q_resid_restrict, blocks_for(n + ncp), QT, q->off[l], n, l, (const double *)q->var[V_PHI],
+              q->var[V_RHS], q->var[V_OLD], tabs(q), q->bc, q->inv_h2[l], q->d_err, q->off[l - 1], ncp);
+    }
+    if (leg_level(q, l - 1)) continue;  // its leg completes the FAS right-hand side
     if (fused)
       qlaunch(q, k_q_fas_rbgs0, blocks_for(nc), QT, q->off[l - 1], nc, l - 1, q->var[V_PHI], q->var[V_RHS],
               (const double *)q->var[V_OLD], tabs(q), q->bc, q->inv_h2[l - 1], q->h[l - 1] * q->h[l - 1], q->d_err);
@@ -1343,6 +1423,10 @@ void vcycle(sm_quad *q, int top) {
   }
   coarse_solve(q);
   for (int l = 1; l <= top; ++l) {
+    if (leg_level(q, l)) {
+      leg<QL_PROLONG>(q, l);
+      continue;
+    }
     const int n = level_count(q, l);
     qlaunch(q, k_q_prolong, blocks_for(n), QT, q->off[l], n, l, q->var[V_PHI], (const double *)q->var[V_OLD], 1,
             tabs(q), q->bc, q->d_err);
@@ -1351,21 +1435,22 @@ void vcycle(sm_quad *q, int top) {
 }
 
 void drop_graphs(sm_quad *q) {
-  for (int l = 0; l < QMAXL; ++l)
-    if (q->vgraph[l]) {
-      cudaGraphExecDestroy(q->vgraph[l]);
-      q->vgraph[l] = nullptr;
+  for (auto &g : q->vgraph)
+    if (g) {
+      cudaGraphExecDestroy(g);
+      g = nullptr;
     }
 }
 
 // One V-cycle with level `top` on top, as a CUDA graph captured on first
 // use (the same launches as vcycle; host launch gaps removed)
-int vcycle_g(sm_quad *q, int top) {
+int vcycle_g(sm_quad *q, int top, bool fmg = false) {
   if (!q->graphs) {
-    vcycle(q, top);
+    vcycle(q, top, fmg);
     return check(q, "V-cycle");
   }
-  if (!q->vgraph[top]) {
+  const int gi = fmg ? QMAXL + top : top;
+  if (!q->vgraph[gi]) {
     if (!q->cap && cudaStreamCreateWithFlags(&q->cap, cudaStreamNonBlocking) != cudaSuccess)
       return qfail(q, SM_ECUDA, "capture stream");
     cudaStream_t saved = q->stream;
@@ -1374,24 +1459,35 @@ int vcycle_g(sm_quad *q, int top) {
     if (cudaStreamBeginCapture(q->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
       return qfail(q, SM_ECUDA, "begin capture");
     q->stream = q->cap;
-    vcycle(q, top);
+    vcycle(q, top, fmg);
     q->stream = saved;
     const cudaError_t e = cudaStreamEndCapture(q->cap, &g);
     if (e != cudaSuccess || !g) {
       cudaGetLastError();
       return qfail(q, SM_ECUDA, "V-cycle capture");
     }
-    const cudaError_t ei = cudaGraphInstantiate(&q->vgraph[top], g, 0);
+    const cudaError_t ei = cudaGraphInstantiate(&q->vgraph[gi], g, 0);
     cudaGraphDestroy(g);
-    q->vgraph_launches[top] = q->launches - l0;
+    q->vgraph_launches[gi] = q->launches - l0;
     q->launches = l0;
     if (ei != cudaSuccess) {
-      q->vgraph[top] = nullptr;
+      q->vgraph[gi] = nullptr;
       return qfail(q, SM_ECUDA, "V-cycle instantiate");
     }
   }
-  if (cudaGraphLaunch(q->vgraph[top], q->stream) != cudaSuccess) return qfail(q, SM_ECUDA, "graph launch");
-  q->launches += q->vgraph_launches[top];
+  if (cudaGraphLaunch(q->vgraph[gi], q->stream) != cudaSuccess) return qfail(q, SM_ECUDA, "graph launch");
+  q->launches += q->vgraph_launches[gi];
+  return SM_OK;
+}
+
+// status of the device's error word (bit 2 is cleared, so the context stays
+// usable after a wait that ran out)
+int device_error(sm_quad *q, unsigned e) {
+  if (e & Q_ERR_WAIT) {
+    cudaMemsetAsync(q->d_err, 0, sizeof(unsigned), q->stream);
+    return qfail(q, SM_ETIMEOUT, "a wait between the blocks of a kernel ran out");
+  }
+  if (e) return qfail(q, SM_ESTATE, "a coarse box needed at a refinement boundary is missing");
   return SM_OK;
 }
 
@@ -1409,33 +1505,34 @@ int resmax(sm_quad *q, int v, double *out) {
       cudaMemcpyAsync(&e, q->d_err, sizeof(e), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
       cudaStreamSynchronize(q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "residual norm");
-  if (e) return qfail(q, SM_ESTATE, "a coarse box needed at a refinement boundary is missing");
+  if (int st = device_error(q, e)) return st;
   double d;
   std::memcpy(&d, &bits, sizeof(d));
   *out = d;
   return SM_OK;
 }
 
-int rel_residual(sm_quad *q, double *rel) {
-  double num = 0.0, den = 0.0;
-  if (cudaMemsetAsync(q->var[V_TMP], 0, sizeof(double) * QC * (size_t)n_boxes(q), q->stream) != cudaSuccess)
-    return qfail(q, SM_ECUDA, "memset");
+// relative residual against den, the residual of phi = 0
+int rel_residual(sm_quad *q, double den, double *rel) {
+  double num = 0.0;
   if (int st = resmax(q, V_PHI, &num)) return st;
-  if (int st = resmax(q, V_TMP, &den)) return st;
   *rel = den > 0.0 ? num / den : num;
   return SM_OK;
 }
 
 int solve_loop(sm_quad *q, double tol, int max_cycles, int c0, int *cycles, double *rel) {
   int c = c0;
-  double r = 0.0;
+  double r = 0.0, den = 0.0;
+  if (cudaMemsetAsync(q->var[V_TMP], 0, sizeof(double) * QC * (size_t)n_boxes(q), q->stream) != cudaSuccess)
+    return qfail(q, SM_ECUDA, "memset");
+  if (int st = resmax(q, V_TMP, &den)) return st;
   if (c0 > 0) {
-    if (int st = rel_residual(q, &r)) return st;
+    if (int st = rel_residual(q, den, &r)) return st;
   }
   while (c == 0 || (r > tol && c < max_cycles)) {
     if (int st = vcycle_g(q, q->nlev - 1)) return st;
     ++c;
-    if (int st = rel_residual(q, &r)) return st;
+    if (int st = rel_residual(q, den, &r)) return st;
   }
   if (cycles) *cycles = c;
   if (rel) *rel = r;
@@ -1579,7 +1676,7 @@ extern "C" int sm_quad_destroy(sm_quad *q) {
 
 namespace {
 struct QLayout {
-  size_t lev, par, chl, nbr8, pn, ref, ij, w, wv, var[NV], cflux, ainv, lut, h, slots, err, snap, rg, need, fine,
+  size_t lev, par, chl, nbr8, pn, ref, ij, w, wv, var[NV], cflux, ainv, lut, h, slots, err, xch, xseq, snap, rg, need, fine,
       total;
 };
 QLayout qlayout(const sm_quad *q) {
@@ -1607,6 +1704,8 @@ QLayout qlayout(const sm_quad *q) {
   L.h = take(sizeof(double) * 3 * QMAXL);
   L.slots = take(sizeof(unsigned long long) * 8);
   L.err = take(sizeof(unsigned));
+  L.xch = take(sizeof(unsigned long long) * 64 * nb);
+  L.xseq = take(sizeof(unsigned));
   L.snap = take(sizeof(double) * 6 * QC * nb);
   L.rg = take(sizeof(int) * 10 * nb);
   L.need = take(sizeof(unsigned long long) * nb);
@@ -1646,6 +1745,8 @@ extern "C" int sm_quad_bind_arena(sm_quad *q, void *dev_ptr, size_t bytes) {
   q->d_h = (double *)(a + L.h);
   q->slots = (unsigned long long *)(a + L.slots);
   q->d_err = (unsigned *)(a + L.err);
+  q->xch = (unsigned long long *)(a + L.xch);
+  q->xseq = (unsigned *)(a + L.xseq);
   q->snap = (double *)(a + L.snap);
   q->d_rg = (int *)(a + L.rg);
   q->d_need = (unsigned long long *)(a + L.need);
@@ -1783,13 +1884,8 @@ extern "C" int sm_quad_fmg(sm_quad *q, double tol, int max_cycles, int *cycles, 
   const int top = q->nlev - 1;
   restrict_all(q, V_RHS);
   coarse_solve(q);
-  for (int l = 1; l <= top; ++l) {
-    const int n = level_count(q, l);
-    k_q_prolong<<<blocks_for(n), QT, 0, q->stream>>>(q->off[l], n, l, q->var[V_PHI], q->var[V_OLD], 0, tabs(q),
-                                                      q->bc, q->d_err);
-    ++q->launches;
-    if (int st = vcycle_g(q, l)) return st;
-  }
+  for (int l = 1; l <= top; ++l)
+    if (int st = vcycle_g(q, l, true)) return st;
   if (int st = check(q, "FMG")) return st;
   return solve_loop(q, tol, max_cycles, 1, cycles, rel);
 }
