@@ -648,26 +648,45 @@ __global__ void __launch_bounds__(QT) k_q_update(int n, const double *__restrict
   }
 }
 
-// parents' quadrants := volume-weighted restriction of the n boxes of a level
-__global__ void __launch_bounds__(QT) k_q_restrict(int off, int n, double *__restrict__ v, QTabs T) {
-  QWARP();
-  if (k_ >= n) return;
-  const int b = off + k_;
-  load_ctx(T, b, C, lane);
-  q_wait();
-  if (lane >= 16) return;
-  const int p = C.pn[4];
-  const int2 B = make_int2(C.ix, C.iy);
-  const int ii = lane & 3, jj = lane >> 2;
-  double sum = 0.0, wsum = 0.0;
-  for (int dj = 0; dj < 2; ++dj)
-    for (int di = 0; di < 2; ++di) {
-      const int i = 2 * ii + di, j = 2 * jj + dj;
-      const double w = T.wv[(size_t)b * QN + i];
-      sum += w * v[(size_t)b * QC + i + QN * j];
-      wsum += w;
+// Volume-weighted means of the four children of one or two variables into
+// every refined box, in one launch without waiting: a warp restricts its
+// leaf box into its quadrant of the parent (lanes 0-15 the first variable,
+// 16-31 the second) and counts itself in there; the warp that completes the
+// parent's four goes on with the parent, the others end.  (A launch per level
+// and variable took 3 us each, 84 of them a Heun step on 15 levels.)  The
+// counters are zero again after the launch.
+__global__ void __launch_bounds__(QT) k_q_restrict_tree(int n, double *v, double *v2, QTabs T, int *count) {
+  const int lane = threadIdx.x & 31, k = blockIdx.x * WPB + (threadIdx.x >> 5);
+  if (k >= n || T.chl[4 * k] >= 0) return;
+  int b = k;
+  double *const x = lane < 16 ? v : v2;
+  const int ii = lane & 3, jj = (lane >> 2) & 3;
+  for (bool first = true;; first = false) {
+    const int p = T.par[b];
+    if (p < 0) return;
+    const int2 B = T.ij[b];
+    if (x) {
+      double sum = 0.0, wsum = 0.0;
+      for (int dj = 0; dj < 2; ++dj)
+        for (int di = 0; di < 2; ++di) {
+          const int i = 2 * ii + di, j = 2 * jj + dj;
+          const double w = T.wv[(size_t)b * QN + i], *c = x + (size_t)b * QC + i + QN * j;
+          sum += w * (first ? *c : __ldcg(c));  // a parent's cells were written by other warps: read them from L2
+          wsum += w;
+        }
+      x[(size_t)p * QC + 4 * (B.x & 1) + ii + QN * (4 * (B.y & 1) + jj)] = sum / wsum;
     }
-  v[(size_t)p * QC + 4 * (B.x & 1) + ii + QN * (4 * (B.y & 1) + jj)] = sum / wsum;
+    __threadfence();
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) {
+      last = atomicAdd(count + p, 1) == 3;
+      if (last) count[p] = 0;
+      __threadfence();
+    }
+    if (!__shfl_sync(0xffffffffu, last, 0)) return;
+    b = p;
+  }
 }
 
 // time-step limits: max over leaf cells of sum|v_d|/dx, that plus 4D/dx^2,
@@ -1110,6 +1129,7 @@ struct sm_quad {
   unsigned *d_err = nullptr;
   unsigned long long *xch = nullptr;      // exchange words of the one-launch legs [max_boxes][4][8][2]
   unsigned *xseq = nullptr;               // their tag counter
+  int *rcount = nullptr;                  // [max_boxes] children counted in by k_q_restrict_tree (zero between)
   int leg_max = -1;                       // boxes of the largest level with such legs (-1: not looked up)
   double *snap = nullptr;                 // regrid snapshot [6][max_boxes][64]
   int *d_rg = nullptr;                    // regrid move descriptors [max_boxes][10]
@@ -1539,12 +1559,13 @@ int solve_loop(sm_quad *q, double tol, int max_cycles, int c0, int *cycles, doub
   return r <= tol ? SM_OK : qfail(q, SM_ENOCONV, "tolerance not reached");
 }
 
-void restrict_all(sm_quad *q, int v) {
-  for (int l = q->nlev - 1; l >= 1; --l) {
-    const int n = level_count(q, l);
-    k_q_restrict<<<blocks_for(n), QT, 0, q->stream>>>(q->off[l], n, q->var[v], tabs(q));
-    ++q->launches;
-  }
+// refined boxes of variable v (and v2) := the mean of their children
+void restrict_all(sm_quad *q, int v, int v2 = -1) {
+  if (q->nlev < 2) return;
+  const int n = n_boxes(q);
+  k_q_restrict_tree<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[v], v2 >= 0 ? q->var[v2] : nullptr, tabs(q),
+                                                          q->rcount);
+  ++q->launches;
 }
 
 int euler_stage(sm_quad *q, int sne, int sni, int dne, int dni, double dt) {
@@ -1555,8 +1576,7 @@ int euler_stage(sm_quad *q, int sne, int sni, int dne, int dni, double dt) {
                                                    q->var[V_PHI], q->var[V_EMAG], q->cflux, tabs(q), q->bc, qlut(q),
                                                    q->d_h, dt, q->d_err);
   q->launches += 2;
-  restrict_all(q, dne);
-  restrict_all(q, dni);
+  restrict_all(q, dne, dni);
   return check(q, "fluid stage");
 }
 
@@ -1676,7 +1696,7 @@ extern "C" int sm_quad_destroy(sm_quad *q) {
 
 namespace {
 struct QLayout {
-  size_t lev, par, chl, nbr8, pn, ref, ij, w, wv, var[NV], cflux, ainv, lut, h, slots, err, xch, xseq, snap, rg, need, fine,
+  size_t lev, par, chl, nbr8, pn, ref, ij, w, wv, var[NV], cflux, ainv, lut, h, slots, err, xch, xseq, rcount, snap, rg, need, fine,
       total;
 };
 QLayout qlayout(const sm_quad *q) {
@@ -1706,6 +1726,7 @@ QLayout qlayout(const sm_quad *q) {
   L.err = take(sizeof(unsigned));
   L.xch = take(sizeof(unsigned long long) * 64 * nb);
   L.xseq = take(sizeof(unsigned));
+  L.rcount = take(sizeof(int) * nb);
   L.snap = take(sizeof(double) * 6 * QC * nb);
   L.rg = take(sizeof(int) * 10 * nb);
   L.need = take(sizeof(unsigned long long) * nb);
@@ -1747,6 +1768,7 @@ extern "C" int sm_quad_bind_arena(sm_quad *q, void *dev_ptr, size_t bytes) {
   q->d_err = (unsigned *)(a + L.err);
   q->xch = (unsigned long long *)(a + L.xch);
   q->xseq = (unsigned *)(a + L.xseq);
+  q->rcount = (int *)(a + L.rcount);
   q->snap = (double *)(a + L.snap);
   q->d_rg = (int *)(a + L.rg);
   q->d_need = (unsigned long long *)(a + L.need);
@@ -1926,8 +1948,7 @@ extern "C" int sm_quad_fluid_stage(sm_quad *q, double dt) {
   if (!q) return SM_EINVAL;
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
   if (!q->lut_n) return qfail(q, SM_ESTATE, "no coefficient table");
-  restrict_all(q, V_NE);
-  restrict_all(q, V_NI);
+  restrict_all(q, V_NE, V_NI);
   if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt)) return st;
   const size_t bytes = sizeof(double) * QC * (size_t)n_boxes(q);
   if (cudaMemcpyAsync(q->var[V_NE], q->var[V_NE1], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess ||
@@ -1944,8 +1965,7 @@ extern "C" int sm_quad_advance(sm_quad *q, double dt, double c, double eps, doub
   if (!q->lut_n) return qfail(q, SM_ESTATE, "no coefficient table");
   const size_t bytes = sizeof(double) * QC * (size_t)n_boxes(q);
   const long long cells = (long long)n_boxes(q) * QC;
-  restrict_all(q, V_NE);
-  restrict_all(q, V_NI);
+  restrict_all(q, V_NE, V_NI);
   if (cudaMemcpyAsync(q->var[V_NE0], q->var[V_NE], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess ||
       cudaMemcpyAsync(q->var[V_NI0], q->var[V_NI], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "copy");
@@ -2033,8 +2053,7 @@ extern "C" int sm_quad_regrid(sm_quad *q, const int8_t *flags, int *n_refined, i
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
   const int n = n_boxes(q), M = q->max_boxes, L0 = q->nlev, T = 256;
   cudaStream_t s = q->stream;
-  restrict_all(q, V_NE);
-  restrict_all(q, V_NI);
+  restrict_all(q, V_NE, V_NI);
   // scratch in the per-call work fields (V_OLD onwards: nothing there
   // outlives a call)
   char *wp = reinterpret_cast<char *>(q->var[V_OLD]);
