@@ -7,6 +7,7 @@
 
 #include <vector>
 
+#include "fluid_dev.cuh"
 #include "sm_internal.cuh"
 #include "sm_nvtx.h"
 
@@ -653,14 +654,10 @@ extern "C" int sm_set_table(sm_ctx *ctx, int n, double e_max, const double *mu, 
   const double *src[3] = {mu, diff, alpha};
   for (int k = 0; k < 3; ++k)
     for (int i = 0; i < n; ++i) {
-      const double t = src[k][i], d = i + 1 < n ? src[k][i + 1] - src[k][i] : 0.0;
-      all[4096 * k + i] = t;
-      all[4096 * (3 + k) + i] = d;
-      // mu and D of an entry together, alpha apart
-      double *q = k < 2 ? &all[4096 * 6 + 4 * i + 2 * k] : &all[4096 * 10 + 2 * i];
-      q[0] = t;
-      q[1] = d;
+      all[4096 * k + i] = src[k][i];
+      all[4096 * (3 + k) + i] = i + 1 < n ? src[k][i + 1] - src[k][i] : 0.0;
     }
+  table_pack(&all[4096 * 6], n, mu, diff, alpha);
   SM_CK(cudaMemcpyAsync(ctx->tab, all.data(), sizeof(double) * all.size(), cudaMemcpyHostToDevice, ctx->stream));
   // the host arrays may be released right after the call
   SM_CK(cudaStreamSynchronize(ctx->stream));

@@ -7,6 +7,7 @@
 #include <math.h>
 #include <string.h>
 
+#include "fluid_dev.cuh"
 #include "sm_internal.cuh"
 #include "sm_nvtx.h"
 
@@ -17,149 +18,6 @@ int sm_mg_solve_internal(sm_ctx *ctx, double tol, int max_cycles, int *cycles);
 // ---------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------
-
-// Non-negative doubles (no NaN) order as their bit patterns: clamps and
-// minima of such values are integer operations, off the FP64 pipe (2 FP64
-// instructions per clock and SM on this GPU).
-__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
-__device__ __forceinline__ double dabs(double x) { return __longlong_as_double(dbits(x) & 0x7fffffffffffffffll); }
-
-// floor(x) and x - floor(x) of a finite 0 < x < 2^30, exactly, from the bit
-// fields: the integer part is the significand shifted by the exponent, the
-// fraction the remaining significand bits renormalised (never subnormal:
-// at least 2^-52)
-__device__ __forceinline__ void split_frac(double x, int &i, double &w) {
-  const unsigned long long b = (unsigned long long)dbits(x);
-  const int e = (int)(b >> 52) - 1023;
-  if (e < 0) {
-    i = 0;
-    w = x;
-    return;
-  }
-  const unsigned long long m = (b & 0x000fffffffffffffull) | (1ull << 52);
-  const int sh = 52 - e;
-  i = (int)(m >> sh);
-  const unsigned long long fm = m & ((1ull << sh) - 1ull);
-  if (fm == 0ull) {
-    w = 0.0;
-    return;
-  }
-  const int top = 63 - __clzll((long long)fm);  // value fm 2^(e-52) = 1.f 2^(top + e - 52)
-  w = __longlong_as_double((long long)(((unsigned long long)(top + e - 52 + 1023) << 52) |
-                                       ((fm << (52 - top)) & 0x000fffffffffffffull)));
-}
-
-// Linear interpolation in two tables sampled at E_k = k e_max/(n-1) at
-// x = e (n-1)/e_max (given), clamped at both ends (Sec. 2.3): the index and
-// weight come from the bits of x; the interpolation a0 + w (a1 - a0) is one
-// FP64 FMA each, with the slope a1 - a0 stored beside the table (sa, sb).
-__device__ __forceinline__ void lookup2x(const double *__restrict__ ta, const double *__restrict__ sa,
-                                         const double *__restrict__ tb, const double *__restrict__ sb, int n,
-                                         long long xmax, double x, double &va, double &vb) {
-  const long long bx = dbits(x);
-  if (bx <= 0) {  // x <= 0 (or -0)
-    va = __ldg(ta);
-    vb = __ldg(tb);
-    return;
-  }
-  if (bx >= xmax) {  // x >= n - 1
-    va = __ldg(ta + n - 1);
-    vb = __ldg(tb + n - 1);
-    return;
-  }
-  int i;
-  double w;
-  split_frac(x, i, w);
-  va = fma(w, __ldg(sa + i), __ldg(ta + i));
-  vb = fma(w, __ldg(sb + i), __ldg(tb + i));
-}
-
-// psi(a/b) b for the Koren limiter psi(x) = max(0, min(1, (2+x)/6, x)),
-// without the division: 0 when a b <= 0 (a or b is +-0, or their signs
-// differ: tested on the bits, with no product), else
-// sign(b) min(|b|, (2|b| + |a|)/6, |a|) with the minimum taken on the bit
-// patterns
-__device__ __forceinline__ double koren(double a, double b) {
-  const long long ba = dbits(a), bb = dbits(b);
-  if ((ba ^ bb) < 0 || (ba << 1) == 0 || (bb << 1) == 0) return 0.0;
-  const double ab = dabs(b), aa = dabs(a);
-  long long m = dbits(ab);
-  m = min(m, dbits(fma(2.0, ab, aa) * (1.0 / 6.0)));
-  m = min(m, dbits(aa));
-  return __longlong_as_double(m | (dbits(b) & (long long)0x8000000000000000ull));
-}
-
-// dx times the flux through the face between cells L and R (positive
-// toward R): v = -mu(E*) E_face with E_face = (p_L - p_R)/dx,
-// E* = (|E|_L + |E|_R)/2 at table index x; advective part by Eq. 7 when
-// v >= 0 and Eq. 6 when v < 0; diffusive part -D(E*) (n_R - n_L)/dx.
-// Written as -mu dp n_f - D dn: v < 0 exactly when mu dp > 0.
-__device__ __forceinline__ double face_flux_h(double nL2, double nL, double nR, double nR2, double pL, double pR,
-                                              double x, const Table &tb) {
-  double mu, dc;
-  lookup2x(tb.mu, tb.dmu, tb.diff, tb.ddiff, tb.n, tb.xmax, x, mu, dc);
-  const double t1 = mu * (pL - pR);
-  const double dn = nR - nL;
-  const bool up = dbits(t1) > 0;  // v < 0: the upwind cell is R
-  // the operands are selected first, so each path costs one FP64 operation
-  const double k = koren((up ? nR2 : nL) - (up ? nR : nL2), dn);
-  const double nf = (up ? nR : nL) + __longlong_as_double(dbits(k) ^ (up ? (long long)0x8000000000000000ull : 0ll));
-  return fma(-t1, nf, -dc * dn);
-}
-
-// Half the table index of a cell, e (n-1)/(2 e_max), in units of 2^-51
-// (rounded; clamped to n - 1): the significand of e times the scale's, shifted
-// by the exponents -- integer operations only.  A face's index is then the
-// integer sum of its two cells' values, its integer part the top bits.  The
-// error, 2^-52 a cell, is below the rounding of an FP64 index once that
-// exceeds 1 (a typical index of 500 has an ulp of 2^-44).
-__device__ __forceinline__ unsigned long long half_index(double e, const Table &tb) {
-  const unsigned long long bits = (unsigned long long)dbits(e);
-  const int ex = (int)(bits >> 52);  // the sign included: negative values give a large count
-  if (ex & 0x800) return 0ull;
-  const unsigned long long A = (bits << 11) | (ex ? 1ull << 63 : 0ull);
-  const unsigned long long hi = __umul64hi(A, tb.xm);
-  const int sh = tb.xs - (ex ? ex : 1);
-  if (sh <= 0) return tb.xtop;
-  const unsigned long long x = sh > 63 ? 0ull : ((hi >> (sh - 1)) + 1ull) >> 1;
-  return x < tb.xtop ? x : tb.xtop;
-}
-
-// integer part of an index x (units of 2^-51, clamped to n - 1) and its
-// fraction as an exact double: the leading one of the 51 bits is shifted to
-// the hidden bit's place
-__device__ __forceinline__ int index_split(unsigned long long x, const Table &tb, double &w) {
-  x = x < tb.xtop ? x : tb.xtop;
-  const unsigned long long f = x & ((1ull << 51) - 1ull);
-  const int lz = __clzll((long long)f);  // 13 .. 63 when f != 0
-  const unsigned long long m = f << (lz - 11);
-  w = f ? __longlong_as_double((long long)(((unsigned long long)(1034 - lz) << 52) + m)) : 0.0;
-  return (int)(x >> 51);
-}
-
-// dx times the flux through a face (as face_flux_h) from the differences
-// n_L - n_L2, n_R - n_L and n_R2 - n_R, which a line of faces shares, and the
-// fixed-point table index of the face
-__device__ __forceinline__ double face_flux_d(double nL, double nR, double dm, double dn, double dq, double dp,
-                                              unsigned long long x, const Table &tb) {
-  double w;
-  const double2 *fc = tb.fc + 2 * index_split(x, tb, w);
-  const double2 cm = __ldg(fc), cd = __ldg(fc + 1);
-  const double t1 = fma(w, cm.y, cm.x) * dp;
-  const bool up = dbits(t1) > 0;  // v < 0: the upwind cell is R
-  const double k = koren(up ? dq : dm, dn);
-  const double nf = (up ? nR : nL) + __longlong_as_double(dbits(k) ^ (up ? (long long)0x8000000000000000ull : 0ll));
-  return fma(-t1, nf, -fma(w, cd.y, cd.x) * dn);
-}
-
-// x / 2, exactly, on the integer pipe for zeros and values whose half is a
-// normal number
-__device__ __forceinline__ double halve(double x) {
-  const long long b = dbits(x);
-  const int ex = (int)((unsigned long long)b >> 52) & 0x7ff;
-  if ((ex > 1 && ex < 0x7ff)) return __longlong_as_double(b - (1ll << 52));
-  return (b << 1) == 0 ? x : 0.5 * x;
-}
 
 // Density ghost (depth t = 1 or 2) across refinement face f of fine box b
 // at face cell (u,w): linear prolongation (c + c_sx + c_sy + c_sz)/4 of the
@@ -227,26 +85,6 @@ __device__ __forceinline__ void face_loc(int f, int dep, int u, int w, int c[3])
   c[a] = (f & 1) ? NC - 1 - dep : dep;
   c[(a + 1) % 3] = u;
   c[(a + 2) % 3] = w;
-}
-
-// sqrt(x) with four FP64 instructions: x = 4^k m, 1 <= m < 4, from the bits;
-// g = sqrt(m) and h = 1/(2 sqrt(m)) in single precision; two steps of
-// Newton's iteration g += (m - g^2) h (Heron's method with the division
-// replaced by the approximate reciprocal), which leave an error of 2^-65
-// beside the last rounding.  Zeros, subnormals, infinities, NaNs and negative
-// values take the library function.
-__device__ __forceinline__ double sqrt_newton(double x) {
-  const unsigned long long bits = (unsigned long long)dbits(x);
-  const int ex = (int)(bits >> 52);
-  if (ex == 0 || ex >= 0x7ff) return (bits << 1) == 0 ? x : sqrt(x);
-  const int odd = (ex - 1023) & 1, k = (ex - 1023 - odd) / 2;
-  const double m = __longlong_as_double((long long)((bits & 0x000fffffffffffffull) | (unsigned long long)(1023 + odd) << 52));
-  const float mf = __uint_as_float((unsigned)(127 + odd) << 23 | (unsigned)((bits >> 29) & 0x7fffffu));
-  const float rs = rsqrtf(mf);
-  const double g0 = cvt_f32_f64(mf * rs), h = cvt_f32_f64(0.5f * rs);
-  const double g1 = fma(fma(-g0, g0, m), h, g0);
-  const double g2 = fma(fma(-g1, g1, m), h, g1);
-  return __longlong_as_double(dbits(g2) + ((long long)k << 52));
 }
 
 // ---------------------------------------------------------------------------
@@ -355,10 +193,12 @@ __global__ void __launch_bounds__(512) k_dt(const int32_t *__restrict__ leaf, co
   block_max3_to(slots + SC_ADV, adv, ad, drt, red, 0.5 * lh.inv_h2[level[b]]);
 }
 
-// Fine-side fluxes through the refinement faces of leaf boxes (64 threads
-// per box, one per face cell, over the list of leaves that have such a
-// face); read by the box itself and averaged by its coarse neighbour, so
-// both sides use the same numbers.
+// Fine-side fluxes through the refinement faces of leaf boxes: 64 threads, a
+// face cell each, per box of the list of leaves that have such a face and
+// axis (only the face on the octant's side of an axis can be one; a block
+// per box that walked its six faces took 26 us on streamer6); read by the
+// box itself and averaged by its coarse neighbour, so both sides use the same
+// numbers.
 __global__ void __launch_bounds__(64) k_cf_flux(const int32_t *__restrict__ leaf, const int32_t *__restrict__ level,
                                                 const double *__restrict__ n, const double *__restrict__ phi,
                                                 const double *__restrict__ gh, const double *__restrict__ emag,
@@ -366,29 +206,23 @@ __global__ void __launch_bounds__(64) k_cf_flux(const int32_t *__restrict__ leaf
                                                 const int32_t *__restrict__ parent,
                                                 const int32_t *__restrict__ ijk, LevelH lh, Table tb,
                                                 double *__restrict__ cflux, unsigned long long *err) {
-  int b = leaf[blockIdx.x];
-  int u = threadIdx.x & 7, w = threadIdx.x >> 3;
-  double ih = lh.inv_h[level[b]];
-  size_t base = (size_t)b * CELLS;
-  for (int f = 0; f < 6; ++f) {
-    if (__ldg(nbr6 + 6 * b + f) != -2) continue;
-    int c0[3], c1[3];
-    face_loc(f, 0, u, w, c0);
-    face_loc(f, 1, u, w, c1);
-    int a = f >> 1;
-    double n0 = n[base + cidx(c0[0], c0[1], c0[2])], n1 = n[base + cidx(c1[0], c1[1], c1[2])];
-    double g1 = density_cf_ghost(n, nbr6, parent, ijk, b, f, 1, u, w, err);
-    double g2 = density_cf_ghost(n, nbr6, parent, ijk, b, f, 2, u, w, err);
-    double p0 = phi[base + cidx(c0[0], c0[1], c0[2])];
-    double pg = p0 * (1.0 / 3.0) + (2.0 / 3.0) * gh[(size_t)(6 * b + f) * FACE + fcell(a, c0[0], c0[1], c0[2])];
-    double e0 = emag[base + cidx(c0[0], c0[1], c0[2])];
-    double eg = emag_cf_ghost(emag, nbr6, parent, ijk, b, f, u, w);
-    const double x = (e0 + eg) * tb.hinv_de;
-    double F;
-    if (f & 1) F = face_flux_h(n1, n0, g1, g2, p0, pg, x, tb);
-    else F = face_flux_h(g2, g1, n0, n1, pg, p0, x, tb);
-    cflux[(size_t)(6 * b + f) * FACE + u + NC * w] = F * ih;
-  }
+  const int b = leaf[blockIdx.x], a = blockIdx.y, f = 2 * a + (ijk[3 * b + a] & 1);
+  if (__ldg(nbr6 + 6 * b + f) != -2) return;
+  const int u = threadIdx.x & 7, w = threadIdx.x >> 3;
+  const size_t base = (size_t)b * CELLS;
+  int c0[3], c1[3];
+  face_loc(f, 0, u, w, c0);
+  face_loc(f, 1, u, w, c1);
+  const double n0 = n[base + cidx(c0[0], c0[1], c0[2])], n1 = n[base + cidx(c1[0], c1[1], c1[2])];
+  const double g1 = density_cf_ghost(n, nbr6, parent, ijk, b, f, 1, u, w, err);
+  const double g2 = density_cf_ghost(n, nbr6, parent, ijk, b, f, 2, u, w, err);
+  const double p0 = phi[base + cidx(c0[0], c0[1], c0[2])];
+  const double pg = p0 * (1.0 / 3.0) + (2.0 / 3.0) * gh[(size_t)(6 * b + f) * FACE + fcell(a, c0[0], c0[1], c0[2])];
+  const unsigned long long x = half_index(emag[base + cidx(c0[0], c0[1], c0[2])], tb) +
+                               half_index(emag_cf_ghost(emag, nbr6, parent, ijk, b, f, u, w), tb);
+  const double F = (f & 1) ? face_flux_d(n0, g1, n0 - n1, g1 - n0, g2 - g1, p0 - pg, x, tb)
+                           : face_flux_d(g1, n0, g1 - g2, n0 - g1, n1 - n0, pg - p0, x, tb);
+  cflux[(size_t)(6 * b + f) * FACE + u + NC * w] = F * lh.inv_h[level[b]];
 }
 
 // index in a staged box of pitch P (O ghost layers) of the cell with
@@ -613,25 +447,8 @@ __global__ void __launch_bounds__(UT, 5) k_update(
 // host drivers
 // ---------------------------------------------------------------------------
 static Table table_of(const sm_ctx *ctx) {
-  Table tb;
-  tb.mu = ctx->tab;
-  tb.diff = ctx->tab + 4096;
-  tb.alpha = ctx->tab + 8192;
-  tb.dmu = ctx->tab + 3 * 4096;
-  tb.ddiff = ctx->tab + 4 * 4096;
-  tb.dalpha = ctx->tab + 5 * 4096;
-  tb.n = ctx->tab_n;
-  tb.inv_de = (ctx->tab_n - 1) / ctx->tab_emax;
-  tb.hinv_de = 0.5 * tb.inv_de;
-  const double top = (double)(ctx->tab_n - 1);
-  memcpy(&tb.xmax, &top, sizeof top);
-  tb.fc = reinterpret_cast<const double2 *>(ctx->tab + 6 * 4096);
-  tb.al = reinterpret_cast<const double2 *>(ctx->tab + 10 * 4096);
-  int p = 0;
-  const double f = frexp(tb.hinv_de, &p);  // hinv_de = xm 2^(p - 64)
-  tb.xm = (unsigned long long)ldexp(f, 64);
-  tb.xs = 1035 - p;
-  tb.xtop = (unsigned long long)(ctx->tab_n - 1) << 51;
+  Table tb = {};
+  table_index_consts(tb, ctx->tab + 6 * 4096, ctx->tab_n, ctx->tab_emax);
   return tb;
 }
 
@@ -712,7 +529,7 @@ static int stage(sm_ctx *ctx, int s, int d, int h0, double dt, double q, double 
   Table tb = table_of(ctx);
   if ((st = sm_fill_all_cf(ctx, ctx->phi))) return st;
   if (ctx->n_cf_leaves > 0) {
-    k_cf_flux<<<ctx->n_cf_leaves, 64, 0, ctx->stream>>>(ctx->cf_leaf, ctx->level, ctx->nbuf[s], ctx->phi,
+    k_cf_flux<<<dim3(ctx->n_cf_leaves, 3), 64, 0, ctx->stream>>>(ctx->cf_leaf, ctx->level, ctx->nbuf[s], ctx->phi,
                                                          ctx->gh, ctx->emag, ctx->nbr6, ctx->parent, ctx->ijk,
                                                          ctx->lh, tb, ctx->cflux, ctx->dscal + SC_ERR);
     ++ctx->n_launch;

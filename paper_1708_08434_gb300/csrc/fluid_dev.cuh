@@ -1,0 +1,138 @@
+// fluid_dev.cuh -- arithmetic of the fluid kernels (octree and quadtree):
+// the field's square root, table lookups, the Koren limiter and the flux
+// through a face, written for the FP64 pipe of this GPU (2 instructions per
+// clock and SM): whatever is exact on the bit patterns runs on the integer
+// pipe.
+#pragma once
+
+#include <math.h>
+
+#include <vector>
+
+#include "sm_internal.cuh"
+
+namespace sm {
+
+// fixed-point index constants of a table of n entries up to e_max, and its
+// packed arrays: fc entries {mu, slope, D, slope}, al {alpha, slope}
+inline void table_index_consts(Table &tb, const double *packed, int n, double e_max) {
+  tb.fc = reinterpret_cast<const double2 *>(packed);
+  tb.al = reinterpret_cast<const double2 *>(packed + 4 * 4096);
+  int p = 0;
+  const double f = frexp(0.5 * ((n - 1) / e_max), &p);  // (n-1)/(2 e_max) = xm 2^(p - 64)
+  tb.xm = (unsigned long long)ldexp(f, 64);
+  tb.xs = 1035 - p;
+  tb.xtop = (unsigned long long)(n - 1) << 51;
+}
+
+// the packed arrays of host tables (6 x 4096 doubles)
+inline void table_pack(double *out, int n, const double *mu, const double *diff, const double *alpha) {
+  const double *src[3] = {mu, diff, alpha};
+  for (int k = 0; k < 3; ++k)
+    for (int i = 0; i < n; ++i) {
+      double *q = k < 2 ? out + 4 * i + 2 * k : out + 4 * 4096 + 2 * i;
+      q[0] = src[k][i];
+      q[1] = i + 1 < n ? src[k][i + 1] - src[k][i] : 0.0;
+    }
+}
+
+// Non-negative doubles (no NaN) order as their bit patterns: clamps and
+// minima of such values are integer operations, off the FP64 pipe (2 FP64
+// instructions per clock and SM on this GPU).
+__device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
+__device__ __forceinline__ double dabs(double x) { return __longlong_as_double(dbits(x) & 0x7fffffffffffffffll); }
+
+// psi(a/b) b for the Koren limiter psi(x) = max(0, min(1, (2+x)/6, x)),
+// without the division: 0 when a b <= 0 (a or b is +-0, or their signs
+// differ: tested on the bits, with no product), else
+// sign(b) min(|b|, (2|b| + |a|)/6, |a|) with the minimum taken on the bit
+// patterns
+__device__ __forceinline__ double koren(double a, double b) {
+  const long long ba = dbits(a), bb = dbits(b);
+  if ((ba ^ bb) < 0 || (ba << 1) == 0 || (bb << 1) == 0) return 0.0;
+  const double ab = dabs(b), aa = dabs(a);
+  long long m = dbits(ab);
+  m = min(m, dbits(fma(2.0, ab, aa) * (1.0 / 6.0)));
+  m = min(m, dbits(aa));
+  return __longlong_as_double(m | (dbits(b) & (long long)0x8000000000000000ull));
+}
+
+// Half the table index of a cell, e (n-1)/(2 e_max), in units of 2^-51
+// (rounded; clamped to n - 1): the significand of e times the scale's, shifted
+// by the exponents -- integer operations only.  A face's index is then the
+// integer sum of its two cells' values, its integer part the top bits.  The
+// error, 2^-52 a cell, is below the rounding of an FP64 index once that
+// exceeds 1 (a typical index of 500 has an ulp of 2^-44).
+__device__ __forceinline__ unsigned long long half_index(double e, const Table &tb) {
+  const unsigned long long bits = (unsigned long long)dbits(e);
+  const int ex = (int)(bits >> 52);  // the sign included: negative values give a large count
+  if (ex & 0x800) return 0ull;
+  const unsigned long long A = (bits << 11) | (ex ? 1ull << 63 : 0ull);
+  const unsigned long long hi = __umul64hi(A, tb.xm);
+  const int sh = tb.xs - (ex ? ex : 1);
+  if (sh <= 0) return tb.xtop;
+  const unsigned long long x = sh > 63 ? 0ull : ((hi >> (sh - 1)) + 1ull) >> 1;
+  return x < tb.xtop ? x : tb.xtop;
+}
+
+// integer part of an index x (units of 2^-51, clamped to n - 1) and its
+// fraction as an exact double: the leading one of the 51 bits is shifted to
+// the hidden bit's place
+__device__ __forceinline__ int index_split(unsigned long long x, const Table &tb, double &w) {
+  x = x < tb.xtop ? x : tb.xtop;
+  const unsigned long long f = x & ((1ull << 51) - 1ull);
+  const int lz = __clzll((long long)f);  // 13 .. 63 when f != 0
+  const unsigned long long m = f << (lz - 11);
+  w = f ? __longlong_as_double((long long)(((unsigned long long)(1034 - lz) << 52) + m)) : 0.0;
+  return (int)(x >> 51);
+}
+
+// dx times the flux through the face between cells L and R (positive
+// toward R): v = -mu(E*) E_face with E_face = (p_L - p_R)/dx, E* = (|E|_L +
+// |E|_R)/2; advective part by Eq. 7 when v >= 0 and Eq. 6 when v < 0; diffusive
+// part -D(E*) (n_R - n_L)/dx.  Written as -mu dp n_f - D dn: v < 0 exactly when
+// mu dp > 0; from the differences
+// n_L - n_L2, n_R - n_L and n_R2 - n_R, which a line of faces shares, and the
+// fixed-point table index of the face
+__device__ __forceinline__ double face_flux_d(double nL, double nR, double dm, double dn, double dq, double dp,
+                                              unsigned long long x, const Table &tb) {
+  double w;
+  const double2 *fc = tb.fc + 2 * index_split(x, tb, w);
+  const double2 cm = __ldg(fc), cd = __ldg(fc + 1);
+  const double t1 = fma(w, cm.y, cm.x) * dp;
+  const bool up = dbits(t1) > 0;  // v < 0: the upwind cell is R
+  const double k = koren(up ? dq : dm, dn);
+  const double nf = (up ? nR : nL) + __longlong_as_double(dbits(k) ^ (up ? (long long)0x8000000000000000ull : 0ll));
+  return fma(-t1, nf, -fma(w, cd.y, cd.x) * dn);
+}
+
+// x / 2, exactly, on the integer pipe for zeros and values whose half is a
+// normal number
+__device__ __forceinline__ double halve(double x) {
+  const long long b = dbits(x);
+  const int ex = (int)((unsigned long long)b >> 52) & 0x7ff;
+  if ((ex > 1 && ex < 0x7ff)) return __longlong_as_double(b - (1ll << 52));
+  return (b << 1) == 0 ? x : 0.5 * x;
+}
+
+// sqrt(x) with four FP64 instructions: x = 4^k m, 1 <= m < 4, from the bits;
+// g = sqrt(m) and h = 1/(2 sqrt(m)) in single precision; two steps of
+// Newton's iteration g += (m - g^2) h (Heron's method with the division
+// replaced by the approximate reciprocal), which leave an error of 2^-65
+// beside the last rounding.  Zeros, subnormals, infinities, NaNs and negative
+// values take the library function.
+__device__ __forceinline__ double sqrt_newton(double x) {
+  const unsigned long long bits = (unsigned long long)dbits(x);
+  const int ex = (int)(bits >> 52);
+  if (ex == 0 || ex >= 0x7ff) return (bits << 1) == 0 ? x : sqrt(x);
+  const int odd = (ex - 1023) & 1, k = (ex - 1023 - odd) / 2;
+  const double m = __longlong_as_double((long long)((bits & 0x000fffffffffffffull) | (unsigned long long)(1023 + odd) << 52));
+  const float mf = __uint_as_float((unsigned)(127 + odd) << 23 | (unsigned)((bits >> 29) & 0x7fffffu));
+  const float rs = rsqrtf(mf);
+  const double g0 = cvt_f32_f64(mf * rs), h = cvt_f32_f64(0.5f * rs);
+  const double g1 = fma(fma(-g0, g0, m), h, g0);
+  const double g2 = fma(fma(-g1, g1, m), h, g1);
+  return __longlong_as_double(dbits(g2) + ((long long)k << 52));
+}
+
+}  // namespace sm

@@ -35,8 +35,18 @@
 #include <utility>
 #include <vector>
 
+#include "fluid_dev.cuh"
 #include "sm_quad.h"
 #include "sm_nvtx.h"
+
+using sm::Table;
+using sm::dabs;
+using sm::dbits;
+using sm::face_flux_d;
+using sm::half_index;
+using sm::halve;
+using sm::index_split;
+using sm::sqrt_newton;
 
 namespace {
 
@@ -49,7 +59,7 @@ constexpr int S1 = QN + 2;       // staged side with one ghost layer
 constexpr int S2 = QN + 4;       // staged side with two ghost layers
 
 // fields in the arena: the public sm_var numbering first
-enum { V_PHI = 0, V_RHS, V_RES, V_NE, V_NI, V_EMAG, V_RHO, V_OLD, V_TMP, V_NE0, V_NI0, V_NE1, V_NI1, NV };
+enum { V_PHI = 0, V_RHS, V_RES, V_NE, V_NI, V_EMAG, V_RHO, V_OLD, V_TMP, V_NE1, V_NI1, NV };
 
 struct QBc {
   int type[4];      // 0 Neumann zero (and the axis), 1 Dirichlet
@@ -63,12 +73,6 @@ struct QTabs {
   const int2 *ij;
   const double *w;   // [box][8][3]: w_lo, w_hi, 1/(w_lo + w_hi + 2) of column i
   const double *wv;  // [box][8]: volume (and y-face area) weight of column i
-};
-
-struct QLut {
-  const double *mu, *diff, *alpha;
-  int n;
-  double inv_de;     // (n - 1) / e_max
 };
 
 __device__ __forceinline__ int dir8(int dx, int dy) {
@@ -432,11 +436,11 @@ __global__ void __launch_bounds__(QT) k_q_resmax(int n, const double *__restrict
 // Eq. 5 on leaf cells
 __global__ void k_q_charge(int n, double *__restrict__ rhs, const double *__restrict__ ne,
                            const double *__restrict__ ni, const double *__restrict__ rho, const int *__restrict__ chl,
-                           double q, double eps, int use_rho) {
+                           double q, double inv_eps, int use_rho) {
   const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (g >= (long long)n * QC) return;
   if (chl[4 * (g / QC)] >= 0) return;
-  rhs[g] = use_rho ? -rho[g] / eps : -q * (ni[g] - ne[g]) / eps;
+  rhs[g] = use_rho ? -rho[g] * inv_eps : -q * (ni[g] - ne[g]) * inv_eps;
 }
 
 // |E| on leaf cells: face fields (phi_i - phi_{i+1})/h, cell components the
@@ -457,48 +461,30 @@ __global__ void __launch_bounds__(QT) k_q_field(int n, const double *__restrict_
   double *s = sm[wv_];
   const int l = C.lev;
   stage_phi(phi, nullptr, C, b, bc, 0, s, lane, err, v0, v1);
-  const double ih = inv_h[l];
+  const double hih = 0.5 * inv_h[l];
   for (int c = lane; c < QC; c += 32) {
-    const int i = c % QN, j = c / QN;
-    const double pc = s[(j + 1) * S1 + i + 1];
-    const double ex = ((s[(j + 1) * S1 + i] - pc) * ih + (pc - s[(j + 1) * S1 + i + 2]) * ih) / 2.0;
-    const double ey = ((s[j * S1 + i + 1] - pc) * ih + (pc - s[(j + 2) * S1 + i + 1]) * ih) / 2.0;
-    emag[(size_t)b * QC + c] = sqrt(ex * ex + ey * ey);
+    const int q = (c / QN + 1) * S1 + c % QN + 1;
+    // (the mean of a cell's two face fields is the centred difference)
+    const double dx = s[q - 1] - s[q + 1], dy = s[q - S1] - s[q + S1];
+    emag[(size_t)b * QC + c] = sqrt_newton(fma(dy, dy, dx * dx)) * hih;
   }
 }
 
-__device__ __forceinline__ double lut(const double *t, const QLut &L, double e) {
-  const double x = e * L.inv_de;
-  if (x <= 0.0) return t[0];
-  if (x >= L.n - 1) return t[L.n - 1];
-  const int i = (int)x;
-  const double w = x - i;
-  return t[i] + w * (t[i + 1] - t[i]);
-}
-
-// psi(a/b) b of the Koren limiter, division-free (Eq. 7)
-__device__ __forceinline__ double koren(double a, double b) {
-  if (a * b <= 0.0) return 0.0;
-  const double s = b > 0.0 ? 1.0 : -1.0, aa = fabs(a), bb = fabs(b);
-  double m = bb;
-  m = fmin(m, (2.0 * bb + aa) * (1.0 / 6.0));
-  m = fmin(m, aa);
-  return s * m;
-}
-
 // Stage the density n with two ghost layers (S2 x S2, interior at (i+2,
-// j+2)), the potential (S1) and |E| with one layer: density ghosts are
+// j+2)), the potential (S1) and the half table index of |E| with one layer:
+// density ghosts are
 // same-level copies, mirrors at walls and the axis, and at refinement
 // boundaries the prolongation (2c + c_x + c_y)/4 of the coarse cell
 // containing the ghost, limited to 2c; |E| ghosts the inner value at walls
 // and the coarse cell's value at refinement boundaries.
 __device__ void stage_fluid(const double *nv, const double *phi, const double *emag, const BoxCtx &C, int b,
-                            const QBc &bc, double *sn, double *sp, double *se, int lane, unsigned *err) {
+                            const QBc &bc, double *sn, double *sp, unsigned long long *se, const Table &tb, int lane,
+                            unsigned *err) {
   const int l = C.lev;
   stage_phi(phi, nullptr, C, b, bc, 0, sp, lane, err, phi[(size_t)b * QC + lane], phi[(size_t)b * QC + lane + 32]);
   for (int c = lane; c < QC; c += 32) {
     sn[(c / QN + 2) * S2 + c % QN + 2] = nv[(size_t)b * QC + c];
-    se[(c / QN + 1) * S1 + c % QN + 1] = emag[(size_t)b * QC + c];
+    se[(c / QN + 1) * S1 + c % QN + 1] = half_index(emag[(size_t)b * QC + c], tb);
   }
   __syncwarp();
   const int2 B = make_int2(C.ix, C.iy);
@@ -532,44 +518,39 @@ __device__ void stage_fluid(const double *nv, const double *phi, const double *e
     face_cell(f, 0, u, ci, cj);
     face_cell(f, -1, u, gi, gj);
     const int nb = C.nb[f];
-    double v;
+    unsigned long long v;
     if (nb >= 0) {
       int si, sj;
       face_cell(f ^ 1, 0, u, si, sj);
-      v = emag[(size_t)nb * QC + si + QN * sj];
+      v = half_index(emag[(size_t)nb * QC + si + QN * sj], tb);
     } else if (nb == -1) {
       v = se[(cj + 1) * S1 + ci + 1];
     } else {
       const int cx = (B.x * QN + gi) >> 1, cy = (B.y * QN + gj) >> 1;
-      v = coarse_val(emag, C, cx, cy, cx, cy, ncl, bc, 0, true, err);
+      v = half_index(coarse_val(emag, C, cx, cy, cx, cy, ncl, bc, 0, true, err), tb);
     }
     se[(gj + 1) * S1 + gi + 1] = v;
   }
   __syncwarp();
 }
 
-// flux through face m (between cells m-1 and m) along axis a at u
-__device__ __forceinline__ double face_flux(const double *sn, const double *sp, const double *se, int a, int m, int u,
-                                            double h, double ih, const QLut &L) {
-  auto N_ = [&](int t) { return a == 0 ? sn[(u + 2) * S2 + t + 2] : sn[(t + 2) * S2 + u + 2]; };
-  auto P_ = [&](int t) { return a == 0 ? sp[(u + 1) * S1 + t + 1] : sp[(t + 1) * S1 + u + 1]; };
-  auto E_ = [&](int t) { return a == 0 ? se[(u + 1) * S1 + t + 1] : se[(t + 1) * S1 + u + 1]; };
-  const double nL2 = N_(m - 2), nL = N_(m - 1), nR = N_(m), nR2 = N_(m + 1);
-  const double e_face = (P_(m - 1) - P_(m)) * ih, e_star = (E_(m - 1) + E_(m)) / 2.0;
-  const double mu = lut(L.mu, L, e_star), dc = lut(L.diff, L, e_star);
-  const double v = -mu * e_face;
-  const double nf = v < 0.0 ? nR - koren(nR2 - nR, nR - nL) : nL + koren(nL - nL2, nR - nL);
-  return v * nf - dc * (nR - nL) * ih;
-  (void)h;
+// dx times the flux through face m (between cells m-1 and m) along axis a at u
+__device__ __forceinline__ double face_flux(const double *sn, const double *sp, const unsigned long long *se, int a,
+                                            int m, int u, const Table &tb) {
+  const int q = a == 0 ? (u + 2) * S2 + m + 2 : (m + 2) * S2 + u + 2, sq = a == 0 ? 1 : S2;
+  const int r = a == 0 ? (u + 1) * S1 + m + 1 : (m + 1) * S1 + u + 1, sr = a == 0 ? 1 : S1;
+  const double nL = sn[q - sq], nR = sn[q];
+  return face_flux_d(nL, nR, nL - sn[q - 2 * sq], nR - nL, sn[q + sq] - nR, sp[r - sr] - sp[r], se[r - sr] + se[r], tb);
 }
 
 // Fine-side fluxes of every leaf box face that borders a coarser leaf:
 // cflux[box][face][u]
 __global__ void __launch_bounds__(QT) k_q_cf_flux(int n, const double *__restrict__ nv, const double *__restrict__ phi,
                                                   const double *__restrict__ emag, double *__restrict__ cflux,
-                                                  QTabs T, const __grid_constant__ QBc bc, QLut L, const double *__restrict__ hs,
+                                                  QTabs T, const __grid_constant__ QBc bc, Table tb, const double *__restrict__ hs,
                                                   unsigned *err) {
-  __shared__ double snm[WPB][S2 * S2], spm[WPB][S1 * S1], sem[WPB][S1 * S1];
+  __shared__ double snm[WPB][S2 * S2], spm[WPB][S1 * S1];
+  __shared__ unsigned long long sem[WPB][S1 * S1];
   QWARP();
   if (k_ >= n) return;
   const int b = k_;
@@ -580,23 +561,57 @@ __global__ void __launch_bounds__(QT) k_q_cf_flux(int n, const double *__restric
   for (int f = 0; f < 4; ++f) any |= C.nb[f] == -2;
   if (!any) return;
   const int l = C.lev;
-  stage_fluid(nv, phi, emag, C, b, bc, snm[wv_], spm[wv_], sem[wv_], lane, err);
+  stage_fluid(nv, phi, emag, C, b, bc, snm[wv_], spm[wv_], sem[wv_], tb, lane, err);
   const int f = lane >> 3, u = lane & 7;
   if (C.nb[f] == -2)
     cflux[(size_t)b * 32 + f * 8 + u] =
-        face_flux(snm[wv_], spm[wv_], sem[wv_], f >> 1, (f & 1) ? QN : 0, u, hs[l], 1.0 / hs[l], L);
+        face_flux(snm[wv_], spm[wv_], sem[wv_], f >> 1, (f & 1) ? QN : 0, u, tb) * (1.0 / hs[l]);
+}
+
+__device__ __forceinline__ void max_word(unsigned long long *slot, long long x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, o));
+  if ((threadIdx.x & 31) == 0) atomicMax(slot, (unsigned long long)max(x, 0ll));
+}
+
+// maxima over a box (a warp) of the three time-step quantities, the first two
+// times scale, into slots[0..2] (bit patterns; the products' maximum is the
+// maximum's product, rounding being monotonic)
+__device__ __forceinline__ void max3_to(unsigned long long *slots, double adv, double ad, double drt, double scale) {
+  max_word(slots, dbits(adv * scale));
+  max_word(slots + 1, dbits(ad * scale));
+  max_word(slots + 2, dbits(drt));
+}
+
+// sum_d mu |E_d| 2 dx of the staged potential at q, that plus 8 D (both to be
+// scaled by 1/(2 dx^2)), and mu n_e, as running maxima
+__device__ __forceinline__ void dt_cell(const double *sp, int q, double mu, double dc, double ne, double &m0,
+                                        double &m1, double &m2) {
+  const double adv = mu * (dabs(sp[q - 1] - sp[q + 1]) + dabs(sp[q - S1] - sp[q + S1]));
+  const double ad = fma(8.0, dc, adv), drt = mu * ne;
+  m0 = dbits(adv) > dbits(m0) ? adv : m0;
+  m1 = dbits(ad) > dbits(m1) ? ad : m1;
+  m2 = dbits(drt) > dbits(m2) ? drt : m2;
 }
 
 // One forward Euler stage on every leaf box: dst = src - dt div F + dt
 // alpha mu |E| n_e (Eq. 2-3); a face next to a refined box takes the
-// area-weighted mean of the two fine fluxes from cflux.
+// area-weighted mean of the two fine fluxes from cflux.  HEUN: dst = (n0 +
+// that)/2 (dst may be n0: a cell reads only its own), and the time-step
+// maxima of src.  With rhs also the Eq. 5 right-hand side of dst.  The box's
+// density differences are formed once and shared by the faces; bound by the
+// FP64 pipe (see fluid_dev.cuh).
+template <bool HEUN>
 __global__ void __launch_bounds__(QT) k_q_update(int n, const double *__restrict__ ne, const double *__restrict__ ni,
-                                                 double *__restrict__ ne_out, double *__restrict__ ni_out,
-                                                 const double *__restrict__ phi, const double *__restrict__ emag,
-                                                 const double *__restrict__ cflux, QTabs T, const __grid_constant__ QBc bc, QLut L,
-                                                 const double *__restrict__ hs, double dt, unsigned *err) {
-  __shared__ double snm[WPB][S2 * S2], spm[WPB][S1 * S1], sem[WPB][S1 * S1];
-  __shared__ double sf[WPB][2][(QN + 1) * QN];
+                                                 const double *ne0, const double *ni0, double *ne_out, double *ni_out,
+                                                 double *__restrict__ rhs, const double *__restrict__ phi,
+                                                 const double *__restrict__ emag, const double *__restrict__ cflux,
+                                                 QTabs T, const __grid_constant__ QBc bc, Table tb,
+                                                 const double *__restrict__ hs, double dt, double qie,
+                                                 unsigned long long *slots, unsigned *err) {
+  constexpr int DL = QN + 3;  // differences of a line: cells -2 .. 9
+  __shared__ double snm[WPB][S2 * S2], spm[WPB][S1 * S1], sf[WPB][2][(QN + 1) * QN], sdm[WPB][2][DL * QN];
+  __shared__ unsigned long long sem[WPB][S1 * S1];
   QWARP();
   if (k_ >= n) return;
   const int b = k_;
@@ -604,48 +619,67 @@ __global__ void __launch_bounds__(QT) k_q_update(int n, const double *__restrict
   q_wait();
   if (C.ref & 16) return;
   const int l = C.lev;
-  const double h = hs[l], ih = 1.0 / h;
-  stage_fluid(ne, phi, emag, C, b, bc, snm[wv_], spm[wv_], sem[wv_], lane, err);
-  for (int g = lane; g < 2 * (QN + 1) * QN; g += 32) {
-    const int a = g / ((QN + 1) * QN), r = g % ((QN + 1) * QN), m = r / QN, u = r % QN;
-    double F = face_flux(snm[wv_], spm[wv_], sem[wv_], a, m, u, h, ih, L);
-    if (m == 0 || m == QN) {
-      const int f = 2 * a + (m == QN ? 1 : 0);
-      const int nb = C.nb[f];
-      if ((C.ref >> f) & 1) {  // refined neighbour: mean of its fine fluxes
-        int cx, cy;
-        if (a == 0) {
-          cx = (f & 1) ? 0 : 1;
-          cy = u >> 2;
-        } else {
-          cx = u >> 2;
-          cy = (f & 1) ? 0 : 1;
-        }
-        const int ch = T.chl[4 * nb + cx + 2 * cy];
-        double s = 0.0, ws = 0.0;
-        for (int du = 0; du < 2; ++du) {
-          const int uf = 2 * (u & 3) + du;
-          const double w = a == 0 ? 1.0 : T.wv[(size_t)ch * QN + uf];
-          s += w * cflux[(size_t)ch * 32 + (f ^ 1) * 8 + uf];
-          ws += w;
-        }
-        F = s / ws;
-      }
-    }
-    sf[wv_][a][m * QN + u] = F;
+  const double h = hs[l], ih2 = hs[QMAXL + l];
+  const double *sn = snm[wv_], *sp = spm[wv_];
+  const unsigned long long *se = sem[wv_];
+  stage_fluid(ne, phi, emag, C, b, bc, snm[wv_], spm[wv_], sem[wv_], tb, lane, err);
+  for (int g = lane; g < 2 * DL * QN; g += 32) {
+    const int a = g / (DL * QN), r = g % (DL * QN), k = r / QN, u = r % QN;
+    const int q = a == 0 ? (u + 2) * S2 + k : k * S2 + u + 2, sq = a == 0 ? 1 : S2;  // cell k - 2 of line u
+    sdm[wv_][a][r] = sn[q + sq] - sn[q];
   }
   __syncwarp();
-  for (int c = lane; c < QC; c += 32) {
-    const int i = c % QN, j = c / QN;
-    const double wl = T.w[(size_t)b * 24 + 3 * i], wh = T.w[(size_t)b * 24 + 3 * i + 1];
-    const double div = (wh * sf[wv_][0][(i + 1) * QN + j] - wl * sf[wv_][0][i * QN + j]) * ih +
-                       (sf[wv_][1][(j + 1) * QN + i] - sf[wv_][1][j * QN + i]) * ih;
-    const double e = sem[wv_][(j + 1) * S1 + i + 1];
-    const size_t g = (size_t)b * QC + c;
-    const double src = lut(L.alpha, L, e) * lut(L.mu, L, e) * e * ne[g];
-    ne_out[g] = ne[g] - dt * div + dt * src;
-    ni_out[g] = ni[g] + dt * src;
+  for (int g = lane; g < 2 * (QN + 1) * QN; g += 32) {
+    const int a = g / ((QN + 1) * QN), r = g % ((QN + 1) * QN), m = r / QN, u = r % QN;
+    const int f = 2 * a + (m == QN ? 1 : 0);
+    double F;
+    if ((m == 0 || m == QN) && ((C.ref >> f) & 1)) {  // refined neighbour: mean of its fine fluxes
+      const int cx = a == 0 ? ((f & 1) ? 0 : 1) : u >> 2, cy = a == 0 ? u >> 2 : ((f & 1) ? 0 : 1);
+      const int ch = T.chl[4 * C.nb[f] + cx + 2 * cy];
+      double s = 0.0, ws = 0.0;
+      for (int du = 0; du < 2; ++du) {
+        const int uf = 2 * (u & 3) + du;
+        const double w = a == 0 ? 1.0 : T.wv[(size_t)ch * QN + uf];
+        s += w * cflux[(size_t)ch * 32 + (f ^ 1) * 8 + uf];
+        ws += w;
+      }
+      F = s / ws * h;
+    } else {
+      const int q = a == 0 ? (u + 2) * S2 + m + 2 : (m + 2) * S2 + u + 2, sq = a == 0 ? 1 : S2;
+      const int r1 = a == 0 ? (u + 1) * S1 + m + 1 : (m + 1) * S1 + u + 1, sr = a == 0 ? 1 : S1;
+      const double *d = sdm[wv_][a] + r;
+      F = face_flux_d(sn[q - sq], sn[q], d[0], d[QN], d[2 * QN], sp[r1 - sr] - sp[r1], se[r1 - sr] + se[r1], tb);
+    }
+    sf[wv_][a][r] = F;
   }
+  __syncwarp();
+  const double dth = -dt * ih2;
+  double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+#pragma unroll
+  for (int s2 = 0; s2 < 2; ++s2) {
+    const int c = lane + 32 * s2, i = c % QN, j = c / QN, q = (j + 1) * S1 + i + 1;
+    const double wl = T.w[(size_t)b * 24 + 3 * i], wh = T.w[(size_t)b * 24 + 3 * i + 1];
+    const double *fx = sf[wv_][0] + i * QN + j, *fy = sf[wv_][1] + j * QN + i;
+    const double div = fma(wh, fx[QN], -wl * fx[0]) + (fy[QN] - fy[0]);  // dx^2 times the divergence
+    const size_t g = (size_t)b * QC + c;
+    const double nes = sn[(j + 2) * S2 + i + 2], e = emag[g];
+    double w;
+    const int k = index_split(2 * se[q], tb, w);
+    const double2 cm = __ldg(tb.fc + 2 * k), al = __ldg(tb.al + k);
+    const double mu = fma(w, cm.y, cm.x);
+    const double src = fma(w, al.y, al.x) * mu * e * nes;
+    double a = fma(dth, div, fma(dt, src, nes)), bq = fma(dt, src, ni[g]);
+    if (HEUN) {
+      a = halve(ne0[g] + a);
+      bq = halve(ni0[g] + bq);
+      const double2 cd = __ldg(tb.fc + 2 * k + 1);
+      dt_cell(sp, q, mu, fma(w, cd.y, cd.x), nes, m0, m1, m2);
+    }
+    ne_out[g] = a;
+    ni_out[g] = bq;
+    if (rhs) rhs[g] = (bq - a) * qie;
+  }
+  if (HEUN) max3_to(slots, m0, m1, m2, 0.5 * ih2);
 }
 
 // Volume-weighted means of the four children of one or two variables into
@@ -692,7 +726,7 @@ __global__ void __launch_bounds__(QT) k_q_restrict_tree(int n, double *v, double
 // time-step limits: max over leaf cells of sum|v_d|/dx, that plus 4D/dx^2,
 // and mu n_e (slots 0..2, bit patterns of non-negative doubles)
 __global__ void __launch_bounds__(QT) k_q_dt(int n, const double *__restrict__ phi, const double *__restrict__ emag,
-                                             const double *__restrict__ ne, QTabs T, const __grid_constant__ QBc bc, QLut L,
+                                             const double *__restrict__ ne, QTabs T, const __grid_constant__ QBc bc, Table tb,
                                              const double *__restrict__ hs, unsigned long long *slots,
                                              unsigned *err) {
   __shared__ double sm[WPB][S1 * S1];
@@ -702,32 +736,19 @@ __global__ void __launch_bounds__(QT) k_q_dt(int n, const double *__restrict__ p
   double v0, v1;
   begin_box(phi, T, b, C, lane, v0, v1);
   if (C.ref & 16) return;
-  const int l = C.lev;
   double *s = sm[wv_];
   stage_phi(phi, nullptr, C, b, bc, 0, s, lane, err, v0, v1);
-  const double h = hs[l], ih = 1.0 / h;
   double m0 = 0.0, m1 = 0.0, m2 = 0.0;
-  for (int c = lane; c < QC; c += 32) {
-    const int i = c % QN, j = c / QN;
-    const double pc = s[(j + 1) * S1 + i + 1];
-    const double ex = ((s[(j + 1) * S1 + i] - pc) * ih + (pc - s[(j + 1) * S1 + i + 2]) * ih) * 0.5;
-    const double ey = ((s[j * S1 + i + 1] - pc) * ih + (pc - s[(j + 2) * S1 + i + 1]) * ih) * 0.5;
-    const double e = emag[(size_t)b * QC + c];
-    const double mu = lut(L.mu, L, e), dc = lut(L.diff, L, e);
-    const double adv = (fabs(mu * ex) + fabs(mu * ey)) * ih;
-    m0 = fmax(m0, adv);
-    m1 = fmax(m1, adv + 2.0 * 2.0 * dc * (ih * ih));
-    m2 = fmax(m2, mu * ne[(size_t)b * QC + c]);
+#pragma unroll
+  for (int s2 = 0; s2 < 2; ++s2) {
+    const int c = lane + 32 * s2;
+    const size_t g = (size_t)b * QC + c;
+    double w;
+    const int k = index_split(2 * half_index(emag[g], tb), tb, w);
+    const double2 cm = __ldg(tb.fc + 2 * k), cd = __ldg(tb.fc + 2 * k + 1);
+    dt_cell(s, (c / QN + 1) * S1 + c % QN + 1, fma(w, cm.y, cm.x), fma(w, cd.y, cd.x), ne[g], m0, m1, m2);
   }
-  max_bits(slots, m0);
-  max_bits(slots + 1, m1);
-  max_bits(slots + 2, m2);
-}
-
-__global__ void k_q_average(long long n, double *__restrict__ a, const double *__restrict__ b0,
-                            const double *__restrict__ b1) {
-  const long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (g < n) a[g] = (b0[g] + b1[g]) / 2.0;
+  max3_to(slots, m0, m1, m2, 0.5 * hs[QMAXL + C.lev]);
 }
 
 // alpha(e) from the table with every operation rounded on its own (no fused
@@ -1255,8 +1276,10 @@ int upload_tables(sm_quad *q) {
 QTabs tabs(const sm_quad *q) {
   return {q->d_lev, q->d_par, q->d_chl, q->d_nbr8, q->d_pn, q->d_ref, q->d_ij, q->d_w, q->d_wv};
 }
-QLut qlut(const sm_quad *q) {
-  return {q->lut, q->lut + q->lut_n, q->lut + 2 * q->lut_n, q->lut_n, (q->lut_n - 1) / q->lut_emax};
+Table qtable(const sm_quad *q) {
+  Table tb = {};
+  sm::table_index_consts(tb, q->lut + 3 * 4096, q->lut_n, q->lut_emax);
+  return tb;
 }
 
 // the level-0 operator with homogeneous wall ghosts (columns L e_k) and its
@@ -1568,13 +1591,21 @@ void restrict_all(sm_quad *q, int v, int v2 = -1) {
   ++q->launches;
 }
 
-int euler_stage(sm_quad *q, int sne, int sni, int dne, int dni, double dt) {
+// one Euler stage of (sne, sni) into (dne, dni); with n0e >= 0 averaged with
+// (n0e, n0i), leaving the time-step maxima in slots 0..2; with qie != 0 the
+// right-hand side (n_i - n_e) qie too
+int euler_stage(sm_quad *q, int sne, int sni, int dne, int dni, double dt, double qie, int n0e = -1, int n0i = -1) {
   const int n = n_boxes(q);
   k_q_cf_flux<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[sne], q->var[V_PHI], q->var[V_EMAG], q->cflux, tabs(q),
-                                                    q->bc, qlut(q), q->d_h, q->d_err);
-  k_q_update<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[sne], q->var[sni], q->var[dne], q->var[dni],
-                                                   q->var[V_PHI], q->var[V_EMAG], q->cflux, tabs(q), q->bc, qlut(q),
-                                                   q->d_h, dt, q->d_err);
+                                                    q->bc, qtable(q), q->d_h, q->d_err);
+  auto run = [&](auto kernel) {
+    kernel<<<blocks_for(n), QT, 0, q->stream>>>(
+        n, q->var[sne], q->var[sni], n0e >= 0 ? q->var[n0e] : nullptr, n0e >= 0 ? q->var[n0i] : nullptr, q->var[dne],
+        q->var[dni], qie != 0.0 ? q->var[V_RHS] : nullptr, q->var[V_PHI], q->var[V_EMAG], q->cflux, tabs(q), q->bc,
+        qtable(q), q->d_h, dt, qie, q->slots, q->d_err);
+  };
+  if (n0e >= 0) run(k_q_update<true>);
+  else run(k_q_update<false>);
   q->launches += 2;
   restrict_all(q, dne, dni);
   return check(q, "fluid stage");
@@ -1583,7 +1614,7 @@ int euler_stage(sm_quad *q, int sne, int sni, int dne, int dni, double dt) {
 int charge(sm_quad *q, double c, double eps, int use_rho) {
   const long long cells = (long long)n_boxes(q) * QC;
   k_q_charge<<<(int)((cells + 255) / 256), 256, 0, q->stream>>>(n_boxes(q), q->var[V_RHS], q->var[V_NE],
-                                                                  q->var[V_NI], q->var[V_RHO], q->d_chl, c, eps,
+                                                                  q->var[V_NI], q->var[V_RHO], q->d_chl, c, 1.0 / eps,
                                                                   use_rho);
   ++q->launches;
   return check(q, "charge");
@@ -1597,13 +1628,8 @@ int field(sm_quad *q) {
   return check(q, "field");
 }
 
-int dt_limit(sm_quad *q, double c, double eps, double *dt) {
-  const int n = n_boxes(q);
-  if (cudaMemsetAsync(q->slots, 0, 3 * sizeof(unsigned long long), q->stream) != cudaSuccess)
-    return qfail(q, SM_ECUDA, "memset");
-  k_q_dt<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[V_PHI], q->var[V_EMAG], q->var[V_NE], tabs(q), q->bc,
-                                               qlut(q), q->d_h, q->slots, q->d_err);
-  ++q->launches;
+// the time step from the maxima in slots 0..2 (synchronises)
+int dt_read(sm_quad *q, double c, double eps, double *dt) {
   unsigned long long bits[3];
   if (cudaMemcpyAsync(bits, q->slots, sizeof(bits), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
       cudaStreamSynchronize(q->stream) != cudaSuccess)
@@ -1616,6 +1642,16 @@ int dt_limit(sm_quad *q, double c, double eps, double *dt) {
   if (m[2] > 0.0 && eps / (c * m[2]) < d) d = eps / (c * m[2]);
   *dt = 0.9 * d;
   return SM_OK;
+}
+
+int dt_limit(sm_quad *q, double c, double eps, double *dt) {
+  const int n = n_boxes(q);
+  if (cudaMemsetAsync(q->slots, 0, 3 * sizeof(unsigned long long), q->stream) != cudaSuccess)
+    return qfail(q, SM_ECUDA, "memset");
+  k_q_dt<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[V_PHI], q->var[V_EMAG], q->var[V_NE], tabs(q), q->bc,
+                                               qtable(q), q->d_h, q->slots, q->d_err);
+  ++q->launches;
+  return dt_read(q, c, eps, dt);
 }
 
 }  // namespace
@@ -1720,7 +1756,7 @@ QLayout qlayout(const sm_quad *q) {
   for (int v = 0; v < NV; ++v) L.var[v] = take(sizeof(double) * QC * nb);
   L.cflux = take(sizeof(double) * 32 * nb);
   L.ainv = take(sizeof(double) * QC * QC);
-  L.lut = take(sizeof(double) * 3 * 4096);
+  L.lut = take(sizeof(double) * 9 * 4096);  // mu, D, alpha; the same packed by entry
   L.h = take(sizeof(double) * 3 * QMAXL);
   L.slots = take(sizeof(unsigned long long) * 8);
   L.err = take(sizeof(unsigned));
@@ -1881,11 +1917,12 @@ extern "C" int sm_quad_set_table(sm_quad *q, int n, double e_max, const double *
                                  const double *alpha) {
   if (!q || !mu || !diff || !alpha || n < 2 || n > 4096 || !(e_max > 0.0)) return SM_EINVAL;
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
-  std::vector<double> t(3 * (size_t)n);
+  std::vector<double> t(9 * 4096, 0.0);
   std::memcpy(t.data(), mu, sizeof(double) * n);
   std::memcpy(t.data() + n, diff, sizeof(double) * n);
   std::memcpy(t.data() + 2 * n, alpha, sizeof(double) * n);
-  if (cudaMemcpyAsync(q->lut, t.data(), sizeof(double) * 3 * n, cudaMemcpyHostToDevice, q->stream) != cudaSuccess ||
+  sm::table_pack(t.data() + 3 * 4096, n, mu, diff, alpha);
+  if (cudaMemcpyAsync(q->lut, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice, q->stream) != cudaSuccess ||
       cudaStreamSynchronize(q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "table upload");
   q->lut_n = n;
@@ -1949,7 +1986,7 @@ extern "C" int sm_quad_fluid_stage(sm_quad *q, double dt) {
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
   if (!q->lut_n) return qfail(q, SM_ESTATE, "no coefficient table");
   restrict_all(q, V_NE, V_NI);
-  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt)) return st;
+  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt, 0.0)) return st;
   const size_t bytes = sizeof(double) * QC * (size_t)n_boxes(q);
   if (cudaMemcpyAsync(q->var[V_NE], q->var[V_NE1], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess ||
       cudaMemcpyAsync(q->var[V_NI], q->var[V_NI1], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess)
@@ -1963,34 +2000,27 @@ extern "C" int sm_quad_advance(sm_quad *q, double dt, double c, double eps, doub
   if (!q || !(eps > 0.0) || max_cycles < 1) return SM_EINVAL;
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
   if (!q->lut_n) return qfail(q, SM_ESTATE, "no coefficient table");
-  const size_t bytes = sizeof(double) * QC * (size_t)n_boxes(q);
-  const long long cells = (long long)n_boxes(q) * QC;
+  const double qie = -c / eps;
   restrict_all(q, V_NE, V_NI);
-  if (cudaMemcpyAsync(q->var[V_NE0], q->var[V_NE], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess ||
-      cudaMemcpyAsync(q->var[V_NI0], q->var[V_NI], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess)
-    return qfail(q, SM_ECUDA, "copy");
-  if (int st = euler_stage(q, V_NE0, V_NI0, V_NE, V_NI, dt)) return st;
-  if (int st = charge(q, c, eps, 0)) return st;
+  // stage 1 into the work densities; stage 2 averages them back in place
+  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt, qie)) return st;
   int c1 = 0, c2 = 0;
   const int st1 = solve_loop(q, tol, max_cycles, 0, &c1, nullptr);
   if (st1 && st1 != SM_ENOCONV) return st1;
   if (int st = field(q)) return st;
-  double dtn = 0.0;
-  if (int st = dt_limit(q, c, eps, &dtn)) return st;
-  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt)) return st;
-  k_q_average<<<(int)((cells + 255) / 256), 256, 0, q->stream>>>(cells, q->var[V_NE], q->var[V_NE0], q->var[V_NE1]);
-  k_q_average<<<(int)((cells + 255) / 256), 256, 0, q->stream>>>(cells, q->var[V_NI], q->var[V_NI0], q->var[V_NI1]);
-  q->launches += 2;
-  if (int st = charge(q, c, eps, 0)) return st;
+  if (cudaMemsetAsync(q->slots, 0, 3 * sizeof(unsigned long long), q->stream) != cudaSuccess)
+    return qfail(q, SM_ECUDA, "memset");
+  if (int st = euler_stage(q, V_NE1, V_NI1, V_NE, V_NI, dt, qie, V_NE, V_NI)) return st;
   const int st2 = solve_loop(q, tol, max_cycles, 0, &c2, nullptr);
   if (st2 && st2 != SM_ENOCONV) return st2;
   if (int st = field(q)) return st;
+  double dtn = 0.0;
+  if (int st = dt_read(q, c, eps, &dtn)) return st;
   if (dt_next) *dt_next = dtn;
   if (cycles) {
     cycles[0] = c1;
     cycles[1] = c2;
   }
-  if (cudaStreamSynchronize(q->stream) != cudaSuccess) return qfail(q, SM_ECUDA, "advance");
   return st1 ? st1 : st2;
 }
 

@@ -60,15 +60,9 @@ struct LevelH {
 
 // transport-coefficient lookup table (device arrays)
 struct Table {
-  const double *mu, *diff, *alpha;
-  const double *dmu, *ddiff, *dalpha;  // slopes t[i+1] - t[i]
-  int n;
-  double inv_de;    // (n-1)/e_max
-  double hinv_de;   // (n-1)/(2 e_max): the index of the face value (e_L + e_R)/2 from e_L + e_R
-  long long xmax;   // bit pattern of the double n - 1 (upper clamp, compared as an integer)
   const double2 *fc;         // {mu, its slope}, {D, its slope} per entry (slopes 0 at the last)
   const double2 *al;         // {alpha, its slope}
-  unsigned long long xm;     // hinv_de = xm 2^(-64 - (xs - 1035)): significand and shift of the fixed-point index
+  unsigned long long xm;     // (n-1)/(2 e_max) = xm 2^(971 - xs): scale of the fixed-point half index
   int xs;
   unsigned long long xtop;   // n - 1 in units of 2^-51
 };
