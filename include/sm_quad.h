@@ -161,9 +161,14 @@ int sm_quad_refine_flags(sm_quad *q, double c0, double c1, double c0_deref, doub
  * unchanged), SM_ESTATE. */
 int sm_quad_regrid(sm_quad *q, const int8_t *flags, int *n_refined, int *n_derefined, int *n_dropped);
 
-/* on != 0 (the default): each V-cycle runs as a CUDA graph, captured per
- * top level on first use and dropped when the mesh or the arena changes;
- * 0: the same launches are issued from the host.  Results are identical. */
+/* on != 0 (the default): a solve runs as one CUDA graph with its cycle loop
+ * and stopping test on the device (a V-cycle of sm_quad_vcycles as a graph
+ * too), captured on first use and dropped when the mesh or the arena
+ * changes; 0: the same launches are issued from the host.  Results are
+ * identical.  On a level whose boxes are all resident at once each leg of a
+ * V-cycle is one cooperative launch whose blocks pass face cells to one
+ * another; a wait that runs out (a few tenths of a second) ends the launch
+ * and the solve returns SM_ETIMEOUT. */
 int sm_quad_set_graphs(sm_quad *q, int on);
 /* on != 0 (the default): the V-cycle kernels are launched with programmatic
  * dependent launch (each loads its box's tables while its predecessor
@@ -171,7 +176,7 @@ int sm_quad_set_graphs(sm_quad *q, int on);
  * order.  Results are identical. */
 int sm_quad_set_pdl(sm_quad *q, int on);
 /* Kernel launches issued by this context so far (a graph counts its
- * kernels). */
+ * kernels but the one-thread stopping test of a solve's loop). */
 int sm_quad_launch_count(const sm_quad *q, long long *n);
 /* One-line reason of the last error of this context ("" if none). */
 const char *sm_quad_last_error(const sm_quad *q);

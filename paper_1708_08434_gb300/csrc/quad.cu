@@ -402,6 +402,30 @@ __global__ void k_q_coarse(double *__restrict__ phi, const double *__restrict__ 
   phi[c] = acc;
 }
 
+// device slots (unsigned long long each): time-step maxima, then the solve's
+// scalars
+enum { QS_ADV = 0, QS_NUM = 4, QS_DEN, QS_CYC, QS_REL, QS_TOL, QS_MAXC, QS_N };
+
+// a solve's stopping parameters, before its graph runs
+__global__ void k_q_begin(unsigned long long *slots, double tol, int max_cycles) {
+  slots[QS_TOL] = (unsigned long long)__double_as_longlong(tol);
+  slots[QS_MAXC] = (unsigned long long)max_cycles;
+  slots[QS_CYC] = 0ull;
+}
+
+// Stopping test of the device-side cycle loop: relative residual, cycle
+// count, and whether another cycle runs (not after a device error)
+__global__ void k_q_check(cudaGraphConditionalHandle h, unsigned long long *slots, const unsigned *err) {
+  const double num = __longlong_as_double((long long)slots[QS_NUM]);
+  const double den = __longlong_as_double((long long)slots[QS_DEN]);
+  const double rel = den > 0.0 ? num / den : num;
+  const unsigned long long c = slots[QS_CYC] + 1ull;
+  slots[QS_CYC] = c;
+  slots[QS_REL] = (unsigned long long)__double_as_longlong(rel);
+  const double tol = __longlong_as_double((long long)slots[QS_TOL]);
+  cudaGraphSetConditional(h, rel > tol && c < slots[QS_MAXC] && *err == 0u ? 1u : 0u);
+}
+
 __device__ __forceinline__ void max_bits(unsigned long long *slot, double v) {
   unsigned long long x = (unsigned long long)__double_as_longlong(fabs(v));
   for (int o = 16; o > 0; o >>= 1) {
@@ -1163,13 +1187,21 @@ struct sm_quad {
   // V-cycle graphs per top level (captured on first use, dropped when the
   // mesh changes) and the launches each holds
   cudaStream_t cap = nullptr;
-  cudaGraphExec_t vgraph[2 * QMAXL] = {nullptr};  // [fmg][top]
-  long long vgraph_launches[2 * QMAXL] = {0};
+  cudaGraphExec_t vgraph[QMAXL] = {nullptr};
+  long long vgraph_launches[QMAXL] = {0};
+  // whole solves with the cycle loop on the device [fmg]: launches before the
+  // loop and per cycle
+  cudaStream_t cap2 = nullptr;
+  cudaGraphExec_t sgraph[2] = {nullptr, nullptr};
+  long long sgraph_launches[2][2] = {{0, 0}, {0, 0}};
   bool graphs = true, pdl = true;
   ~sm_quad() {
     for (auto &g : vgraph)
       if (g) cudaGraphExecDestroy(g);
+    for (auto &g : sgraph)
+      if (g) cudaGraphExecDestroy(g);
     if (cap) cudaStreamDestroy(cap);
+    if (cap2) cudaStreamDestroy(cap2);
   }
 };
 
@@ -1478,22 +1510,22 @@ void vcycle(sm_quad *q, int top, bool fmg = false) {
 }
 
 void drop_graphs(sm_quad *q) {
-  for (auto &g : q->vgraph)
-    if (g) {
-      cudaGraphExecDestroy(g);
-      g = nullptr;
-    }
+  auto drop = [](cudaGraphExec_t &g) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  };
+  for (auto &g : q->vgraph) drop(g);
+  for (auto &g : q->sgraph) drop(g);
 }
 
 // One V-cycle with level `top` on top, as a CUDA graph captured on first
 // use (the same launches as vcycle; host launch gaps removed)
-int vcycle_g(sm_quad *q, int top, bool fmg = false) {
+int vcycle_g(sm_quad *q, int top) {
   if (!q->graphs) {
-    vcycle(q, top, fmg);
+    vcycle(q, top);
     return check(q, "V-cycle");
   }
-  const int gi = fmg ? QMAXL + top : top;
-  if (!q->vgraph[gi]) {
+  if (!q->vgraph[top]) {
     if (!q->cap && cudaStreamCreateWithFlags(&q->cap, cudaStreamNonBlocking) != cudaSuccess)
       return qfail(q, SM_ECUDA, "capture stream");
     cudaStream_t saved = q->stream;
@@ -1502,26 +1534,28 @@ int vcycle_g(sm_quad *q, int top, bool fmg = false) {
     if (cudaStreamBeginCapture(q->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
       return qfail(q, SM_ECUDA, "begin capture");
     q->stream = q->cap;
-    vcycle(q, top, fmg);
+    vcycle(q, top);
     q->stream = saved;
     const cudaError_t e = cudaStreamEndCapture(q->cap, &g);
     if (e != cudaSuccess || !g) {
       cudaGetLastError();
       return qfail(q, SM_ECUDA, "V-cycle capture");
     }
-    const cudaError_t ei = cudaGraphInstantiate(&q->vgraph[gi], g, 0);
+    const cudaError_t ei = cudaGraphInstantiate(&q->vgraph[top], g, 0);
     cudaGraphDestroy(g);
-    q->vgraph_launches[gi] = q->launches - l0;
+    q->vgraph_launches[top] = q->launches - l0;
     q->launches = l0;
     if (ei != cudaSuccess) {
-      q->vgraph[gi] = nullptr;
+      q->vgraph[top] = nullptr;
       return qfail(q, SM_ECUDA, "V-cycle instantiate");
     }
   }
-  if (cudaGraphLaunch(q->vgraph[gi], q->stream) != cudaSuccess) return qfail(q, SM_ECUDA, "graph launch");
-  q->launches += q->vgraph_launches[gi];
+  if (cudaGraphLaunch(q->vgraph[top], q->stream) != cudaSuccess) return qfail(q, SM_ECUDA, "graph launch");
+  q->launches += q->vgraph_launches[top];
   return SM_OK;
 }
+
+void restrict_all(sm_quad *q, int v, int v2 = -1);
 
 // status of the device's error word (bit 2 is cleared, so the context stays
 // usable after a wait that ran out)
@@ -1534,56 +1568,161 @@ int device_error(sm_quad *q, unsigned e) {
   return SM_OK;
 }
 
-// max leaf residual of var (the potential, or the zero array)
-int resmax(sm_quad *q, int v, double *out) {
+// max leaf residual of var (the potential, or the zero array) into a slot
+void resmax(sm_quad *q, int v, int slot) {
   const int n = n_boxes(q);
-  if (cudaMemsetAsync(q->slots + 4, 0, sizeof(unsigned long long), q->stream) != cudaSuccess)
-    return qfail(q, SM_ECUDA, "memset");
+  cudaMemsetAsync(q->slots + slot, 0, sizeof(unsigned long long), q->stream);
   k_q_resmax<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[v], q->var[V_RHS], tabs(q), q->bc, q->d_h + QMAXL,
-                                                   q->slots + 4, q->d_err);
+                                                   q->slots + slot, q->d_err);
   ++q->launches;
-  unsigned long long bits = 0;
+}
+
+// the solve's scalars and the error word (synchronises)
+int read_solve(sm_quad *q, unsigned long long (&s)[QS_N]) {
   unsigned e = 0;
-  if (cudaMemcpyAsync(&bits, q->slots + 4, sizeof(bits), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
+  if (cudaMemcpyAsync(s, q->slots, sizeof(s), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
       cudaMemcpyAsync(&e, q->d_err, sizeof(e), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
       cudaStreamSynchronize(q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "residual norm");
-  if (int st = device_error(q, e)) return st;
+  return device_error(q, e);
+}
+
+double bits_of(unsigned long long b) {
   double d;
-  std::memcpy(&d, &bits, sizeof(d));
-  *out = d;
+  std::memcpy(&d, &b, sizeof(d));
+  return d;
+}
+
+// work before the cycle loop: the residual of phi = 0 (the denominator), and
+// for FMG the restricted right-hand side, the ladder and its residual
+void solve_prefix(sm_quad *q, bool fmg) {
+  cudaMemsetAsync(q->var[V_TMP], 0, sizeof(double) * QC * (size_t)n_boxes(q), q->stream);
+  resmax(q, V_TMP, QS_DEN);
+  if (!fmg) return;
+  restrict_all(q, V_RHS);
+  coarse_solve(q);
+  for (int l = 1; l < q->nlev; ++l) vcycle(q, l, true);
+  resmax(q, V_PHI, QS_NUM);
+}
+
+void solve_body(sm_quad *q) {
+  vcycle(q, q->nlev - 1);
+  resmax(q, V_PHI, QS_NUM);
+}
+
+void solve_check(sm_quad *q, cudaGraphConditionalHandle h) {
+  k_q_check<<<1, 1, 0, q->stream>>>(h, q->slots, q->d_err);  // not counted: the host loop tests without a launch
+}
+
+// Capture prefix + WHILE { cycle; check } into an executable graph (an FMG
+// result is checked once before the loop and counts as cycle 1; otherwise
+// the body runs at least once).
+int capture_solve(sm_quad *q, bool fmg) {
+  if ((!q->cap && cudaStreamCreateWithFlags(&q->cap, cudaStreamNonBlocking) != cudaSuccess) ||
+      (!q->cap2 && cudaStreamCreateWithFlags(&q->cap2, cudaStreamNonBlocking) != cudaSuccess))
+    return qfail(q, SM_ECUDA, "capture stream");
+  leg_limit(q);  // occupancy queries outside the capture
+  cudaStream_t saved = q->stream;
+  const long long l0 = q->launches;
+  long long l1 = l0, l2 = l0;
+  cudaGraph_t g = nullptr, body = nullptr, whole = nullptr;
+  bool ok = cudaStreamBeginCapture(q->cap, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
+  if (ok) {
+    q->stream = q->cap;
+    cudaStreamCaptureStatus cs;
+    cudaGraphConditionalHandle h = 0;
+    const cudaGraphNode_t *deps = nullptr;
+    size_t nd = 0;
+    cudaGraphNode_t node;
+    // the node-parameter union has no default constructor: zeroed raw storage
+    alignas(cudaGraphNodeParams) unsigned char pbuf[sizeof(cudaGraphNodeParams)];
+    std::memset(pbuf, 0, sizeof pbuf);
+    cudaGraphNodeParams &p = *reinterpret_cast<cudaGraphNodeParams *>(pbuf);
+    ok = cudaStreamGetCaptureInfo(q->cap, &cs, nullptr, &g, nullptr, nullptr, nullptr) == cudaSuccess &&
+         cudaGraphConditionalHandleCreate(&h, g, fmg ? 0u : 1u, cudaGraphCondAssignDefault) == cudaSuccess;
+    if (ok) {
+      solve_prefix(q, fmg);
+      if (fmg) solve_check(q, h);
+      l1 = q->launches;
+      p.type = cudaGraphNodeTypeConditional;
+      p.conditional.handle = h;
+      p.conditional.type = cudaGraphCondTypeWhile;
+      p.conditional.size = 1;
+      ok = cudaStreamGetCaptureInfo(q->cap, &cs, nullptr, nullptr, &deps, nullptr, &nd) == cudaSuccess &&
+           cudaGraphAddNode(&node, g, deps, nullptr, nd, &p) == cudaSuccess;
+    }
+    if (ok) {
+      body = p.conditional.phGraph_out[0];
+      ok = cudaStreamUpdateCaptureDependencies(q->cap, &node, nullptr, 1, cudaStreamSetCaptureDependencies) ==
+               cudaSuccess &&
+           cudaStreamBeginCaptureToGraph(q->cap2, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
+               cudaSuccess;
+    }
+    if (ok) {
+      q->stream = q->cap2;
+      solve_body(q);
+      solve_check(q, h);
+      l2 = q->launches;
+      ok = cudaStreamEndCapture(q->cap2, &body) == cudaSuccess;
+    }
+    q->stream = saved;
+    ok = cudaStreamEndCapture(q->cap, &whole) == cudaSuccess && ok;
+  }
+  q->launches = l0;
+  q->sgraph_launches[fmg][0] = l1 - l0;
+  q->sgraph_launches[fmg][1] = l2 - l1;
+  ok = ok && cudaGraphInstantiate(&q->sgraph[fmg], whole, 0) == cudaSuccess;
+  if (whole) cudaGraphDestroy(whole);
+  if (!ok) {
+    q->sgraph[fmg] = nullptr;
+    cudaGetLastError();
+    return qfail(q, SM_ECUDA, "solve capture");
+  }
   return SM_OK;
 }
 
-// relative residual against den, the residual of phi = 0
-int rel_residual(sm_quad *q, double den, double *rel) {
-  double num = 0.0;
-  if (int st = resmax(q, V_PHI, &num)) return st;
-  *rel = den > 0.0 ? num / den : num;
-  return SM_OK;
-}
-
-int solve_loop(sm_quad *q, double tol, int max_cycles, int c0, int *cycles, double *rel) {
-  int c = c0;
-  double r = 0.0, den = 0.0;
-  if (cudaMemsetAsync(q->var[V_TMP], 0, sizeof(double) * QC * (size_t)n_boxes(q), q->stream) != cudaSuccess)
-    return qfail(q, SM_ECUDA, "memset");
-  if (int st = resmax(q, V_TMP, &den)) return st;
-  if (c0 > 0) {
-    if (int st = rel_residual(q, den, &r)) return st;
+// FMG, or V-cycles from the current potential, until the relative residual is
+// at most tol: one graph with the loop on the device, or the same launches
+// with a read after every cycle
+int run_solve(sm_quad *q, bool fmg, double tol, int max_cycles, int *cycles, double *rel) {
+  unsigned long long s[QS_N];
+  int c = 0;
+  double r = 0.0;
+  if (q->graphs) {
+    if (!q->sgraph[fmg])
+      if (int st = capture_solve(q, fmg)) return st;
+    k_q_begin<<<1, 1, 0, q->stream>>>(q->slots, tol, max_cycles);
+    if (cudaGraphLaunch(q->sgraph[fmg], q->stream) != cudaSuccess) return qfail(q, SM_ECUDA, "graph launch");
+    if (int st = read_solve(q, s)) return st;
+    c = (int)s[QS_CYC];
+    r = bits_of(s[QS_REL]);
+    q->launches += q->sgraph_launches[fmg][0] + q->sgraph_launches[fmg][1] * (long long)(fmg ? c - 1 : c);
+  } else {
+    solve_prefix(q, fmg);
+    auto residual = [&] {
+      const int st = read_solve(q, s);
+      const double num = bits_of(s[QS_NUM]), den = bits_of(s[QS_DEN]);
+      r = den > 0.0 ? num / den : num;
+      return st;
+    };
+    if (fmg) {
+      c = 1;
+      if (int st = residual()) return st;
+    }
+    while (c == 0 || (r > tol && c < max_cycles)) {
+      solve_body(q);
+      ++c;
+      if (int st = residual()) return st;
+    }
   }
-  while (c == 0 || (r > tol && c < max_cycles)) {
-    if (int st = vcycle_g(q, q->nlev - 1)) return st;
-    ++c;
-    if (int st = rel_residual(q, den, &r)) return st;
-  }
+  if (int st = check(q, "solve")) return st;
   if (cycles) *cycles = c;
   if (rel) *rel = r;
   return r <= tol ? SM_OK : qfail(q, SM_ENOCONV, "tolerance not reached");
 }
 
 // refined boxes of variable v (and v2) := the mean of their children
-void restrict_all(sm_quad *q, int v, int v2 = -1) {
+void restrict_all(sm_quad *q, int v, int v2) {
   if (q->nlev < 2) return;
   const int n = n_boxes(q);
   k_q_restrict_tree<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[v], v2 >= 0 ? q->var[v2] : nullptr, tabs(q),
@@ -1758,7 +1897,7 @@ QLayout qlayout(const sm_quad *q) {
   L.ainv = take(sizeof(double) * QC * QC);
   L.lut = take(sizeof(double) * 9 * 4096);  // mu, D, alpha; the same packed by entry
   L.h = take(sizeof(double) * 3 * QMAXL);
-  L.slots = take(sizeof(unsigned long long) * 8);
+  L.slots = take(sizeof(unsigned long long) * QS_N);
   L.err = take(sizeof(unsigned));
   L.xch = take(sizeof(unsigned long long) * 64 * nb);
   L.xseq = take(sizeof(unsigned));
@@ -1940,20 +2079,14 @@ extern "C" int sm_quad_fmg(sm_quad *q, double tol, int max_cycles, int *cycles, 
   SM_RANGE();
   if (!q || max_cycles < 1 || !(tol >= 0.0)) return SM_EINVAL;
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
-  const int top = q->nlev - 1;
-  restrict_all(q, V_RHS);
-  coarse_solve(q);
-  for (int l = 1; l <= top; ++l)
-    if (int st = vcycle_g(q, l, true)) return st;
-  if (int st = check(q, "FMG")) return st;
-  return solve_loop(q, tol, max_cycles, 1, cycles, rel);
+  return run_solve(q, true, tol, max_cycles, cycles, rel);
 }
 
 extern "C" int sm_quad_solve(sm_quad *q, double tol, int max_cycles, int *cycles, double *rel) {
   SM_RANGE();
   if (!q || max_cycles < 1 || !(tol >= 0.0)) return SM_EINVAL;
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
-  return solve_loop(q, tol, max_cycles, 0, cycles, rel);
+  return run_solve(q, false, tol, max_cycles, cycles, rel);
 }
 
 extern "C" int sm_quad_vcycles(sm_quad *q, int n) {
@@ -2005,13 +2138,13 @@ extern "C" int sm_quad_advance(sm_quad *q, double dt, double c, double eps, doub
   // stage 1 into the work densities; stage 2 averages them back in place
   if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt, qie)) return st;
   int c1 = 0, c2 = 0;
-  const int st1 = solve_loop(q, tol, max_cycles, 0, &c1, nullptr);
+  const int st1 = run_solve(q, false, tol, max_cycles, &c1, nullptr);
   if (st1 && st1 != SM_ENOCONV) return st1;
   if (int st = field(q)) return st;
   if (cudaMemsetAsync(q->slots, 0, 3 * sizeof(unsigned long long), q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "memset");
   if (int st = euler_stage(q, V_NE1, V_NI1, V_NE, V_NI, dt, qie, V_NE, V_NI)) return st;
-  const int st2 = solve_loop(q, tol, max_cycles, 0, &c2, nullptr);
+  const int st2 = run_solve(q, false, tol, max_cycles, &c2, nullptr);
   if (st2 && st2 != SM_ENOCONV) return st2;
   if (int st = field(q)) return st;
   double dtn = 0.0;
