@@ -1175,6 +1175,7 @@ struct sm_quad {
   unsigned long long *xch = nullptr;      // exchange words of the one-launch legs [max_boxes][4][8][2]
   unsigned *xseq = nullptr;               // their tag counter
   int *rcount = nullptr;                  // [max_boxes] children counted in by k_q_restrict_tree (zero between)
+  int leg_few = 0;                        // boxes of the largest level for the form with more registers
   int leg_max = -1;                       // boxes of the largest level with such legs (-1: not looked up)
   double *snap = nullptr;                 // regrid snapshot [6][max_boxes][64]
   int *d_rg = nullptr;                    // regrid move descriptors [max_boxes][10]
@@ -1404,6 +1405,9 @@ void coarse_solve(sm_quad *q) {
           q->bc, q->inv_h2[0], q->xseq);
 }
 
+// blocks per SM of the two forms of a leg kernel (200 and 72 registers)
+constexpr int LEG_FEW = 10, LEG_MANY = 28;
+
 // Boxes of the largest level whose legs run in one launch (a warp per box,
 // all resident at once); 0 without cooperative launch.
 int leg_limit(sm_quad *q) {
@@ -1417,10 +1421,17 @@ int leg_limit(sm_quad *q) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 32, 0) != cudaSuccess) per = 0;
     most = std::min(most, per * sms);
   };
-  fits(k_q_leg<QL_TOP>);
-  fits(k_q_leg<QL_FAS>);
-  fits(k_q_leg<QL_PROLONG>);
-  fits(k_q_leg<QL_FMG>);
+  // the forms for levels of few boxes and of many
+  fits(k_q_leg<QL_TOP, LEG_FEW>);
+  fits(k_q_leg<QL_FAS, LEG_FEW>);
+  fits(k_q_leg<QL_PROLONG, LEG_FEW>);
+  fits(k_q_leg<QL_FMG, LEG_FEW>);
+  q->leg_few = most;
+  most = 1 << 30;
+  fits(k_q_leg<QL_TOP, LEG_MANY>);
+  fits(k_q_leg<QL_FAS, LEG_MANY>);
+  fits(k_q_leg<QL_PROLONG, LEG_MANY>);
+  fits(k_q_leg<QL_FMG, LEG_MANY>);
   cudaGetLastError();
   return q->leg_max = coop ? most : 0;
 }
@@ -1457,7 +1468,8 @@ void leg(sm_quad *q, int l, unsigned skew = 0) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, k_q_leg<START>, a);
+  if (level_count(q, l) <= q->leg_few) cudaLaunchKernelEx(&cfg, k_q_leg<START, LEG_FEW>, a);
+  else cudaLaunchKernelEx(&cfg, k_q_leg<START, LEG_MANY>, a);
   ++q->launches;
 }
 

@@ -25,10 +25,13 @@
 // read: phi is stored at the very end.  Restricted values go to old and rhs
 // of the level below, which the leg of that level starts from (a leaf box
 // there starts from phi); nothing in a leg writes the phi of another level.
-// The arithmetic is that of the separate kernels, in their order.
 //
-// Bound: latency of the exchange (700 to 1050 cycles a word) and of the
-// FP64 chain of a cell.
+// Bound: the exchange (700 to 1050 cycles a word) and the FP64 pipe, which
+// takes 16 cycles for a warp's instruction: with four warps on an SM each
+// waits some 64 cycles per FP64 instruction.  So instructions are counted.
+// w_lo + w_hi is 2 in both geometries, so the Gauss-Seidel division is a
+// quarter, done on the exponent; an update is four FP64 instructions before
+// the halo is awaited and two after it.
 
 enum { QL_TOP = 0, QL_FAS = 1, QL_PROLONG = 2, QL_FMG = 3 };  // how a leg starts
 
@@ -54,16 +57,28 @@ __device__ __forceinline__ void qx_put(unsigned long long *p, double v, unsigned
                "l"((b << 32) | tag)
                : "memory");
 }
-// true when both halves carry the tag
-__device__ __forceinline__ bool qx_get(const unsigned long long *p, unsigned tag, double &v) {
+struct QWord {
   unsigned long long a, b;
-  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-  v = __longlong_as_double((long long)((a & 0xffffffff00000000ull) | (b >> 32)));
-  return (unsigned)a == tag && (unsigned)b == tag;
+  __device__ __forceinline__ void load(const unsigned long long *p) {
+    asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  }
+  // 0 when both halves carry the tag
+  __device__ __forceinline__ unsigned off(unsigned tag) const { return ((unsigned)a ^ tag) | ((unsigned)b ^ tag); }
+  __device__ __forceinline__ double value() const {
+    return __longlong_as_double((long long)((a & 0xffffffff00000000ull) | (b >> 32)));
+  }
+};
+// 1/x for positive x in single precision's range: Newton's iteration from the
+// single-precision reciprocal
+__device__ __forceinline__ double q_recip(double x) {
+  double y = sm::cvt_f32_f64(__frcp_rn(sm::cvt_f64_f32_rn(x)));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
 }
 
-template <int START>
-__global__ void __launch_bounds__(32, 28) k_q_leg(const __grid_constant__ QLeg a) {
+// OCC: blocks an SM has to hold (more registers for a level of few boxes)
+template <int START, int OCC>
+__global__ void __launch_bounds__(32, OCC) k_q_leg(const __grid_constant__ QLeg a) {
   constexpr bool UP = START == QL_PROLONG, PRO = START == QL_PROLONG || START == QL_FMG;
   constexpr unsigned ALL = 0xffffffffu;
   __shared__ double sph[32];  // phihat of the refinement faces' cells [face][8]
@@ -76,12 +91,18 @@ __global__ void __launch_bounds__(32, 28) k_q_leg(const __grid_constant__ QLeg a
   const bool atx = i2 == 0 || i2 == 3, aty = j == 0 || j == QN - 1;
   const int nx = atx ? T.nbr8[8 * b + face_dir8(fx)] : -3, ny = aty ? T.nbr8[8 * b + face_dir8(fy)] : -3;
   const int pnl = lane < 9 ? T.pn[9 * b + lane] : 0;  // the parent's neighbourhood, an entry a lane
+  const int nbl = T.nbr8[8 * b + face_dir8(lane >> 3)];  // neighbour across the face of lane / 8
   const int2 ij = T.ij[b];
   const int ref = T.ref[b];
+  double wv[2] = {1.0, 1.0};
+  if (!UP) {
+    wv[0] = T.wv[(size_t)b * QN + 2 * i2];
+    wv[1] = T.wv[(size_t)b * QN + 2 * i2 + 1];
+  }
   const unsigned tag0 = (*a.seq << 7) + a.leg;
   const unsigned stop = *a.err & Q_ERR_WAIT;
   const double *wc = T.w + (size_t)b * 24 + 6 * i2;
-  const double wl[2] = {wc[0], wc[3]}, wh[2] = {wc[1], wc[4]}, wi[2] = {wc[2], wc[5]};
+  const double wl[2] = {wc[0], wc[3]}, wh[2] = {wc[1], wc[4]};
   double2 f2 = *reinterpret_cast<const double2 *>(a.rhs + g);
   double2 u2 = make_double2(0.0, 0.0);
   if (START != QL_FMG) u2 = *reinterpret_cast<const double2 *>(a.phi + g);
@@ -96,20 +117,6 @@ __global__ void __launch_bounds__(32, 28) k_q_leg(const __grid_constant__ QLeg a
   const int ncl = QN << (a.lev - 1);
   // entry of the parent's neighbourhood that holds coarse cell (cx, cy)
   auto cbox = [&](int cx, int cy) { return ((cx >> 3) - (ij.x >> 1) + 1) + 3 * ((cy >> 3) - (ij.y >> 1) + 1); };
-  // value of the level below at coarse cell (qx, qy), or across the wall from
-  // (cx, cy) inside; every lane calls it (the neighbourhood sits across lanes)
-  auto coarse = [&](auto val, int qx, int qy, int cx, int cy, bool homog) {
-    const bool out = qx < 0 || qy < 0 || qx >= ncl || qy >= ncl;
-    const int x = out ? cx : qx, y = out ? cy : qy;
-    const int q = __shfl_sync(ALL, pnl, cbox(x, y));
-    const bool ok = q >= 0;
-    if (!ok) atomicOr(a.err, 1u);  // a coarse box needed here is missing
-    const double v = ok ? val((size_t)q * QC + (x & 7) + QN * (y & 7)) : 0.0;
-    if (!out) return v;
-    const int w = qx < 0 ? 0 : (qx >= ncl ? 1 : (qy < 0 ? 2 : 3));
-    return a.bc.type[w] ? (homog ? 0.0 : a.bc.g2[w]) - v : v;
-  };
-
   const bool bx = nx >= 0, by = ny >= 0;
   auto own = [&](int c) { return ((j + c) & 1) ? u[1] : u[0]; };
   // the x face belongs to the cell of colour c: column 0 (p = 0) at -x, column 7 (p = 1) at +x
@@ -123,49 +130,118 @@ __global__ void __launch_bounds__(32, 28) k_q_leg(const __grid_constant__ QLeg a
     if (bx && xact(c)) qx_put(mx, v, tag0 + ev);
     if (by) qx_put(my + 2 * ((j + c) & 1), v, tag0 + ev);
   };
-  // halo of the lane's colour-c cell across its x and y faces
+  // Halo of the lane's colour-c cell across its x and y faces (0 where there
+  // is none).  Two polls are kept in flight: the first is issued before the
+  // arithmetic that needs no halo, so that its trip to memory is not added to
+  // it.
   double hx = 0.0, hy = 0.0;
-  auto await = [&](int c, unsigned ev) {
+  struct Poll {
+    QWord x, y;
+  };
+  auto poll = [&](int c, Poll &q) {
+    if (bx && xact(c)) q.x.load(qx_);
+    if (by) q.y.load(qy_ + 2 * ((j + c) & 1));
+  };
+  auto await = [&](int c, unsigned ev, Poll &q) {
     const unsigned tag = tag0 + ev + a.skew;
     const bool x = bx && xact(c);
+    auto off = [&](const Poll &w) { return (x ? w.x.off(tag) : 0u) | (by ? w.y.off(tag) : 0u); };
     if (x || by) {
+      Poll w = q;
       for (int it = 0;; ++it) {
-        bool ok = true;
-        if (x) ok = qx_get(qx_, tag, hx);
-        if (by) ok = qx_get(qy_ + 2 * ((j + c) & 1), tag, hy) && ok;
-        if (ok) break;
+        poll(c, w);
+        if (off(q) == 0u) break;
+        poll(c, q);
+        if (off(w) == 0u) {
+          q = w;
+          break;
+        }
         if (it > Q_SPIN) {
           atomicOr(a.err, Q_ERR_WAIT);
           break;
         }
       }
     }
+    hx = x ? q.x.value() : 0.0;
+    hy = by ? q.y.value() : 0.0;
   };
-  // the four neighbours of the lane's colour-c cell: shuffles inside the box,
-  // halos x and y from other boxes, ghosts at walls and refinement faces
-  auto around = [&](int c, double x, double y, double &L, double &R, double &S, double &N) {
-    const int p = (j + c) & 1;
-    const double me = own(c), oth = own(c ^ 1);
-    double xs = __shfl_sync(ALL, oth, p ? lane + 1 : lane - 1);
-    S = __shfl_sync(ALL, oth, lane - 4);
-    N = __shfl_sync(ALL, oth, lane + 4);
-    auto ghost = [&](int nb, int face, int at) {
-      if (nb == -1) return a.bc.type[face] ? a.bc.g2[face] - me : me;
-      return me * (1.0 / 3.0) + sph[8 * face + at] * (2.0 / 3.0);
-    };
-    if (xact(c)) xs = bx ? x : ghost(nx, fx, j);
-    if (aty) {
-      const double v = by ? y : ghost(ny, fy, 2 * i2 + p);
-      if (j == 0) S = v;
-      else N = v;
+  // The four neighbours of the lane's colour-c cell: the pair's other column,
+  // the next column beyond the pair, and the rows below and above, by
+  // shuffles; 0 where that leaves the box.
+  struct Around {
+    double me, oth, xs, S, N;
+  };
+  auto around = [&](int c) {
+    Around r;
+    r.me = own(c);
+    r.oth = own(c ^ 1);
+    r.xs = __shfl_sync(ALL, r.oth, ((j + c) & 1) ? lane + 1 : lane - 1);
+    r.S = __shfl_sync(ALL, r.oth, lane - 4);
+    r.N = __shfl_sync(ALL, r.oth, lane + 4);
+    if (xact(c)) r.xs = 0.0;
+    if (j == 0) r.S = 0.0;
+    if (j == QN - 1) r.N = 0.0;
+    return r;
+  };
+  // A ghost at a wall or refinement face is A + B own (Dirichlet 2g - own,
+  // Neumann own, 2/3 phihat + own / 3): of the x face's cell and of the y
+  // face's two (by column); no ghost: zeros
+  double gxA = 0.0, gxB = 0.0, gyA[2] = {0.0, 0.0}, gyB = 0.0;
+  const bool anyg = __any_sync(ALL, nx == -1 || nx == -2 || ny == -1 || ny == -2);
+  auto ghosts = [&] {
+    if (nx == -1) {
+      gxA = a.bc.type[fx] ? a.bc.g2[fx] : 0.0;
+      gxB = a.bc.type[fx] ? -1.0 : 1.0;
+    } else if (nx == -2) {
+      gxA = sph[8 * fx + j];
+      gxB = 1.0 / 3.0;
     }
-    L = p ? oth : xs;
-    R = p ? xs : oth;
+    if (ny == -1) {
+      gyA[0] = gyA[1] = a.bc.type[fy] ? a.bc.g2[fy] : 0.0;
+      gyB = a.bc.type[fy] ? -1.0 : 1.0;
+    } else if (ny == -2) {
+      gyA[0] = sph[8 * fy + 2 * i2];
+      gyA[1] = sph[8 * fy + 2 * i2 + 1];
+      gyB = 1.0 / 3.0;
+    }
   };
-  auto lap = [&](int c, double L, double R, double S, double N) {
+  // four times the red-black update of colour c: uA - uB own + w oth + w' xs
+  // + S + N + w' hx + hy, ghosts folded into uA and uB
+  double uA[2], uB[2] = {0.0, 0.0};
+  auto w_in = [&](int c) { return ((j + c) & 1) ? wl[1] : wh[0]; };  // the pair's other column
+  auto w_out = [&](int c) { return ((j + c) & 1) ? wh[1] : wl[0]; };  // the column beyond
+  auto update_form = [&](int c) {
     const int p = (j + c) & 1;
-    const double v = own(c);
-    return ((p ? wl[1] : wl[0]) * (L - v) + (p ? wh[1] : wh[0]) * (R - v) + (S - v) + (N - v)) * a.inv_h2;
+    uA[c] = -a.h2 * (p ? f[1] : f[0]);
+    if (anyg) {
+      const double w = xact(c) ? w_out(c) : 0.0;
+      uA[c] += fma(w, gxA, p ? gyA[1] : gyA[0]);
+      uB[c] = fma(w, gxB, gyB);
+    }
+  };
+  auto update0 = [&](int c, const Around &r) {
+    double t = fma(w_in(c), r.oth, uA[c]);
+    if (anyg) t = fma(uB[c], r.me, t);
+    return fma(w_out(c), r.xs, t) + (r.S + r.N);
+  };
+  auto update1 = [&](int c, double base) {
+    const double t = fma(w_out(c), hx, base + hy);  // hx, hy are 0 where there is no halo
+    // a quarter on the exponent (zeros, small and non-finite values multiply)
+    const long long b = __double_as_longlong(t);
+    const int ex = (int)((unsigned long long)b >> 52) & 0x7ff;
+    return ex > 2 && ex < 0x7ff ? __longlong_as_double(b - (2ll << 52)) : 0.25 * t;
+  };
+  // h^2 L phi at the lane's colour-c cell from its neighbours with the halo x,
+  // y; differences first, which keeps the rounding at that of the differences
+  auto lap = [&](int c, const Around &r, double x, double y) {
+    const int p = (j + c) & 1;
+    double X = bx ? x : 0.0, Y = by ? y : 0.0;
+    if (anyg) {
+      X = bx ? X : fma(gxB, r.me, gxA);
+      Y = by ? Y : fma(gyB, r.me, p ? gyA[1] : gyA[0]);
+    }
+    const double xs = xact(c) ? X : r.xs, S = j == 0 ? Y : r.S, N = j == QN - 1 ? Y : r.N;
+    return fma(w_in(c), r.oth - r.me, fma(w_out(c), xs - r.me, (S - r.me) + (N - r.me)));
   };
   auto set = [&](double (&d)[2], int c, double v) {
     if ((j + c) & 1) d[1] = v;
@@ -176,37 +252,61 @@ __global__ void __launch_bounds__(32, 28) k_q_leg(const __grid_constant__ QLeg a
     // (2c + c_x + c_y)/4: one coarse cell under the pair, its x neighbour for
     // each column, the y neighbour for both
     const int cx = 4 * ij.x + i2, cy = (QN * ij.y + j) >> 1, qy = cy + ((j & 1) ? 1 : -1);
-    auto cv = [&](int x, int y) {
-      const double p = coarse([&](size_t k) { return a.phi[k]; }, x, y, cx, cy, UP);
-      return UP ? p - coarse([&](size_t k) { return a.old[k]; }, x, y, cx, cy, true) : p;
-    };
-    const double c0 = 2.0 * cv(cx, cy), cl = cv(cx - 1, cy), cr = cv(cx + 1, cy), cq = cv(cx, qy);
-    const double s0 = c0 + cl + cq, s1 = c0 + cr + cq;
-    u[0] = UP ? u[0] + 0.25 * s0 : 0.25 * s0;
-    u[1] = UP ? u[1] + 0.25 * s1 : 0.25 * s1;
+    const int px[4] = {cx, cx - 1, cx + 1, cx}, py[4] = {cy, cy, cy, qy};
+    double cv[4], ov[4] = {0.0, 0.0, 0.0, 0.0};
+    bool out[4], missing = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {  // every load before any use
+      out[k] = px[k] < 0 || py[k] < 0 || px[k] >= ncl || py[k] >= ncl;
+      const int x = out[k] ? cx : px[k], y = out[k] ? cy : py[k];
+      const int q = __shfl_sync(ALL, pnl, cbox(x, y));
+      missing |= q < 0;
+      const size_t at = (size_t)(q < 0 ? 0 : q) * QC + (x & 7) + QN * (y & 7);
+      cv[k] = a.phi[at];
+      if (UP) ov[k] = a.old[at];
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      if (UP) cv[k] -= ov[k];
+      if (out[k]) {
+        const int w = px[k] < 0 ? 0 : (px[k] >= ncl ? 1 : (py[k] < 0 ? 2 : 3));
+        cv[k] = a.bc.type[w] ? (UP ? 0.0 : a.bc.g2[w]) - cv[k] : cv[k];
+      }
+    }
+    if (missing) atomicOr(a.err, 1u);  // a coarse box needed here is missing
+    const double t = fma(2.0, cv[0], cv[3]);
+    u[0] = UP ? fma(0.25, t + cv[1], u[0]) : 0.25 * (t + cv[1]);
+    u[1] = UP ? fma(0.25, t + cv[2], u[1]) : 0.25 * (t + cv[2]);
     publish(1, 0);
   }
   {
-    // phihat of the refinement faces: lane -> (face, cell)
+    // 2/3 phihat of the refinement faces: lane -> (face, cell)
     const int face = lane >> 3, at = lane & 7;
-    const int nb = T.nbr8[8 * b + face_dir8(face)];
-    if (__any_sync(ALL, nb == -2)) {
+    const bool cf = nbl == -2;
+    if (__any_sync(ALL, cf)) {
       int gi, gj;
       face_cell(face, -1, at, gi, gj);
       const int Gx = ij.x * QN + gi, Gy = ij.y * QN + gj;
-      // lanes of other faces read the cell under the box (any existing one)
-      const bool cf = nb == -2;
+      // lanes of other faces read a cell under the box
       const int cx = cf ? Gx >> 1 : 4 * ij.x, cy = cf ? Gy >> 1 : 4 * ij.y;
       int qx = cx, qy = cy;
       if (cf && face < 2) qy += (Gy & 1) ? 1 : -1;
       else if (cf) qx += (Gx & 1) ? 1 : -1;
-      auto val = [&](size_t k) { return a.phi[k]; };
-      const double c = coarse(val, cx, cy, cx, cy, false);
-      const double ct = coarse(val, qx, qy, cx, cy, false);
-      sph[lane] = 0.75 * c + 0.25 * ct;
+      const bool out = qx < 0 || qy < 0 || qx >= ncl || qy >= ncl;
+      const int x = out ? cx : qx, y = out ? cy : qy;
+      const int b0 = __shfl_sync(ALL, pnl, cbox(cx, cy)), b1 = __shfl_sync(ALL, pnl, cbox(x, y));
+      if (b0 < 0 || b1 < 0) atomicOr(a.err, 1u);
+      const double c = a.phi[(size_t)(b0 < 0 ? 0 : b0) * QC + (cx & 7) + QN * (cy & 7)];
+      double ct = a.phi[(size_t)(b1 < 0 ? 0 : b1) * QC + (x & 7) + QN * (y & 7)];
+      if (out) {
+        const int w = qx < 0 ? 0 : (qx >= ncl ? 1 : (qy < 0 ? 2 : 3));
+        ct = a.bc.type[w] ? a.bc.g2[w] - ct : ct;
+      }
+      sph[lane] = fma(1.0 / 6.0, ct, 0.5 * c);
       __syncwarp();
     }
   }
+  ghosts();
   unsigned ev = 0;
   if (!PRO) {
     // halos from the neighbours' cells (FAS start: restricted values of a
@@ -219,64 +319,66 @@ __global__ void __launch_bounds__(32, 28) k_q_leg(const __grid_constant__ QLeg a
       y[0] = v.x;
       y[1] = v.y;
     }
-    double L, R, S, N;
-    around(0, x, (j & 1) ? y[1] : y[0], L, R, S, N);
-    if (refined) {
-      double L1, R1, S1_, N1;
-      around(1, x, (j & 1) ? y[0] : y[1], L1, R1, S1_, N1);
-      const double l0 = lap(0, L, R, S, N), l1 = lap(1, L1, R1, S1_, N1);
-      const bool odd = j & 1;  // colour 0 is the odd column
-      f[0] += odd ? l1 : l0;
-      f[1] += odd ? l0 : l1;
-      *reinterpret_cast<double2 *>(a.rhs + g) = make_double2(f[0], f[1]);
+    const bool odd = j & 1;  // colour 0 is the odd column of odd rows
+    const Around r0 = around(0);
+    if (refined) {  // the FAS right-hand side f += L phi
+      const Around r1 = around(1);
+      const double t0 = lap(0, r0, x, odd ? y[1] : y[0]), t1 = lap(1, r1, x, odd ? y[0] : y[1]);
+      f[0] = fma(odd ? t1 : t0, a.inv_h2, f[0]);
+      f[1] = fma(odd ? t0 : t1, a.inv_h2, f[1]);
     }
-    const int p = j & 1;
-    set(u, 0, ((p ? wl[1] : wl[0]) * L + (p ? wh[1] : wh[0]) * R + S + N - a.h2 * (p ? f[1] : f[0])) * (p ? wi[1] : wi[0]));
+    hx = xact(0) ? x : 0.0;
+    hy = odd ? y[1] : y[0];
+    update_form(0);
+    set(u, 0, update1(0, update0(0, r0)));
     publish(0, ++ev);
+    update_form(1);
+    if (refined) *reinterpret_cast<double2 *>(a.rhs + g) = make_double2(f[0], f[1]);
+  } else {
+    update_form(0);
+    update_form(1);
+  }
+  // weights of the restriction's means
+  double w0 = 0.0, w1 = 0.0;
+  if (!UP) {
+    const double r = 0.5 * q_recip(wv[0] + wv[1]);
+    w0 = wv[0] * r;
+    w1 = wv[1] * r;
   }
   double x1 = 0.0, y1 = 0.0;  // colour 1's halo in the last pass
   for (int sweep = 0; sweep < a.nu; ++sweep) {
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       if (!PRO && c == 0 && sweep == 0) continue;
-      await(c, ev);
+      Poll q = {};
+      const Around r = around(c);
+      poll(c, q);
+      const double base = update0(c, r);
+      await(c, ev, q);
       if (!UP && c == 1) {
         x1 = hx;
         y1 = hy;
       }
-      double L, R, S, N;
-      around(c, hx, hy, L, R, S, N);
-      const int p = (j + c) & 1;
-      set(u, c, ((p ? wl[1] : wl[0]) * L + (p ? wh[1] : wh[0]) * R + S + N - a.h2 * (p ? f[1] : f[0])) * (p ? wi[1] : wi[0]));
+      set(u, c, update1(c, base));
       ++ev;
       if (!UP || c == 0 || sweep + 1 < a.nu) publish(c, ev);
     }
   }
   if (!UP) {
-    await(0, ev);  // the neighbours' last colour-1 cells
-    double L, R, S, N;
-    around(0, hx, hy, L, R, S, N);
-    const double l0 = lap(0, L, R, S, N);
-    around(1, x1, y1, L, R, S, N);
-    const double l1 = lap(1, L, R, S, N);
+    Poll q = {};
+    poll(0, q);
+    const Around n1 = around(1), n0 = around(0);
     const bool odd = j & 1;
-    const double r[2] = {f[0] - (odd ? l1 : l0), f[1] - (odd ? l0 : l1)};
-    // volume-weighted means over the 2 x 2 children: the even row's lane sums
-    // the potential, the odd row's the residual
-    const double w0 = T.wv[(size_t)b * QN + 2 * i2], w1 = T.wv[(size_t)b * QN + 2 * i2 + 1];
-    const double t0 = __shfl_xor_sync(ALL, odd ? u[0] : r[0], 4), t1 = __shfl_xor_sync(ALL, odd ? u[1] : r[1], 4);
-    const double a0 = odd ? t0 : u[0], a1 = odd ? t1 : u[1], b0 = odd ? r[0] : t0, b1 = odd ? r[1] : t1;
-    double sum = 0.0, ws = 0.0;
-    sum += w0 * a0;
-    ws += w0;
-    sum += w1 * a1;
-    ws += w1;
-    sum += w0 * b0;
-    ws += w0;
-    sum += w1 * b1;
-    ws += w1;
+    const double r1 = fma(-lap(1, n1, x1, y1), a.inv_h2, odd ? f[0] : f[1]);  // colour 1: the even column of odd rows
     const int P = __shfl_sync(ALL, pnl, 4);
-    (odd ? a.rhs : a.old)[(size_t)P * QC + 4 * (ij.x & 1) + i2 + QN * (4 * (ij.y & 1) + (j >> 1))] = sum / ws;
+    await(0, ev, q);  // the neighbours' last colour-1 cells
+    const double r0 = fma(-lap(0, n0, hx, hy), a.inv_h2, odd ? f[1] : f[0]);
+    const double r[2] = {odd ? r1 : r0, odd ? r0 : r1};
+    // volume-weighted means over the 2 x 2 children: the even row's lane forms
+    // the potential's, the odd row's the residual's
+    const double t0 = __shfl_xor_sync(ALL, odd ? u[0] : r[0], 4), t2 = __shfl_xor_sync(ALL, odd ? u[1] : r[1], 4);
+    const double m = fma(w0, t0 + (odd ? r[0] : u[0]), w1 * (t2 + (odd ? r[1] : u[1])));
+    (odd ? a.rhs : a.old)[(size_t)P * QC + 4 * (ij.x & 1) + i2 + QN * (4 * (ij.y & 1) + (j >> 1))] = m;
   }
   *reinterpret_cast<double2 *>(a.phi + g) = make_double2(u[0], u[1]);
 }
