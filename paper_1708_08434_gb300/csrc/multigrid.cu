@@ -2067,6 +2067,7 @@ static int capture_solve(sm_ctx *ctx, int kind, sm_graph *out) {
     int st = ensure_basis(ctx);  // once per context, outside any graph
     if (st) return st;
   }
+  leg_limit(ctx);  // occupancy queries outside the capture
   const int fmg = kind == 1 || kind == 3;
   if (ctx->persist) {
     int st = kind < 2 ? persistx_prepare(ctx) : persist_prepare32(ctx);
@@ -2535,6 +2536,7 @@ extern "C" int sm_kernel_bench(sm_ctx *ctx, int kclass, int reps, double *us_per
     if ((st = solve_prologue(ctx))) return st;
     if ((st = leaf_resid32(ctx))) return st;
   }
+  leg_limit(ctx);
   cudaStream_t saved = ctx->stream;
   if (!ctx->cap) SM_CK(cudaStreamCreateWithFlags(&ctx->cap, cudaStreamNonBlocking));
   SM_CK(cudaStreamBeginCapture(ctx->cap, cudaStreamCaptureModeThreadLocal));

@@ -1441,13 +1441,12 @@ bool leg_level(sm_quad *q, int l) {
 }
 
 template <int START>
-void leg(sm_quad *q, int l, unsigned skew = 0) {
+void leg(sm_quad *q, int l) {
   constexpr bool up = START == QL_PROLONG;
   QLeg a = {};
   a.lo = q->off[l];
   a.nu = up ? q->nu2 : q->nu1;
   a.leg = up ? 0u : 64u;
-  a.skew = skew;
   a.h2 = q->h[l] * q->h[l];
   a.inv_h2 = q->inv_h2[l];
   a.phi = q->var[V_PHI];
@@ -1533,6 +1532,7 @@ void drop_graphs(sm_quad *q) {
 // One V-cycle with level `top` on top, as a CUDA graph captured on first
 // use (the same launches as vcycle; host launch gaps removed)
 int vcycle_g(sm_quad *q, int top) {
+  leg_limit(q);  // occupancy queries outside the capture
   if (!q->graphs) {
     vcycle(q, top);
     return check(q, "V-cycle");
@@ -1743,16 +1743,17 @@ void restrict_all(sm_quad *q, int v, int v2) {
 }
 
 // one Euler stage of (sne, sni) into (dne, dni); with n0e >= 0 averaged with
-// (n0e, n0i), leaving the time-step maxima in slots 0..2; with qie != 0 the
-// right-hand side (n_i - n_e) qie too
-int euler_stage(sm_quad *q, int sne, int sni, int dne, int dni, double dt, double qie, int n0e = -1, int n0i = -1) {
+// (n0e, n0i), leaving the time-step maxima in slots 0..2; with `charge` the
+// right-hand side (n_i - n_e) qie too, zero where qie is
+int euler_stage(sm_quad *q, int sne, int sni, int dne, int dni, double dt, bool charge, double qie, int n0e = -1,
+                int n0i = -1) {
   const int n = n_boxes(q);
   k_q_cf_flux<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[sne], q->var[V_PHI], q->var[V_EMAG], q->cflux, tabs(q),
                                                     q->bc, qtable(q), q->d_h, q->d_err);
   auto run = [&](auto kernel) {
     kernel<<<blocks_for(n), QT, 0, q->stream>>>(
         n, q->var[sne], q->var[sni], n0e >= 0 ? q->var[n0e] : nullptr, n0e >= 0 ? q->var[n0i] : nullptr, q->var[dne],
-        q->var[dni], qie != 0.0 ? q->var[V_RHS] : nullptr, q->var[V_PHI], q->var[V_EMAG], q->cflux, tabs(q), q->bc,
+        q->var[dni], charge ? q->var[V_RHS] : nullptr, q->var[V_PHI], q->var[V_EMAG], q->cflux, tabs(q), q->bc,
         qtable(q), q->d_h, dt, qie, q->slots, q->d_err);
   };
   if (n0e >= 0) run(k_q_update<true>);
@@ -2131,7 +2132,7 @@ extern "C" int sm_quad_fluid_stage(sm_quad *q, double dt) {
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
   if (!q->lut_n) return qfail(q, SM_ESTATE, "no coefficient table");
   restrict_all(q, V_NE, V_NI);
-  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt, 0.0)) return st;
+  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt, false, 0.0)) return st;
   const size_t bytes = sizeof(double) * QC * (size_t)n_boxes(q);
   if (cudaMemcpyAsync(q->var[V_NE], q->var[V_NE1], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess ||
       cudaMemcpyAsync(q->var[V_NI], q->var[V_NI1], bytes, cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess)
@@ -2148,14 +2149,14 @@ extern "C" int sm_quad_advance(sm_quad *q, double dt, double c, double eps, doub
   const double qie = -c / eps;
   restrict_all(q, V_NE, V_NI);
   // stage 1 into the work densities; stage 2 averages them back in place
-  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt, qie)) return st;
+  if (int st = euler_stage(q, V_NE, V_NI, V_NE1, V_NI1, dt, true, qie)) return st;
   int c1 = 0, c2 = 0;
   const int st1 = run_solve(q, false, tol, max_cycles, &c1, nullptr);
   if (st1 && st1 != SM_ENOCONV) return st1;
   if (int st = field(q)) return st;
   if (cudaMemsetAsync(q->slots, 0, 3 * sizeof(unsigned long long), q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "memset");
-  if (int st = euler_stage(q, V_NE1, V_NI1, V_NE, V_NI, dt, qie, V_NE, V_NI)) return st;
+  if (int st = euler_stage(q, V_NE1, V_NI1, V_NE, V_NI, dt, true, qie, V_NE, V_NI)) return st;
   const int st2 = run_solve(q, false, tol, max_cycles, &c2, nullptr);
   if (st2 && st2 != SM_ENOCONV) return st2;
   if (int st = field(q)) return st;

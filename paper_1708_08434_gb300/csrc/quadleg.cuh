@@ -40,7 +40,7 @@ constexpr int Q_SPIN = 1 << 18;  // polls of one wait (a few tenths of a second)
 
 struct QLeg {
   int lo, nu;
-  unsigned leg, skew;  // tag offset of the leg; skew only for testing the bounded wait
+  unsigned leg;  // tag offset of the leg
   double h2, inv_h2;
   double *phi, *rhs, *old;
   unsigned long long *xch;  // [box][face][8][2]
@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(32, OCC) k_q_leg(const __grid_constant__ QLeg 
     if (by) q.y.load(qy_ + 2 * ((j + c) & 1));
   };
   auto await = [&](int c, unsigned ev, Poll &q) {
-    const unsigned tag = tag0 + ev + a.skew;
+    const unsigned tag = tag0 + ev;
     const bool x = bx && xact(c);
     auto off = [&](const Poll &w) { return (x ? w.x.off(tag) : 0u) | (by ? w.y.off(tag) : 0u); };
     if (x || by) {

@@ -48,3 +48,26 @@ def test_one_launch_legs(name, nu1, nu2, bct):
     a, b = g.download(p.PHI), o.get(quad.PHI)
     g.close()
     assert np.abs(a - b).max() <= 1e-12 * np.abs(b).max()
+
+
+def test_advance_without_charge():
+    """A Heun step with zero charge leaves a zero right-hand side behind, as
+    the separate charge kernel did, not the one of the solve before."""
+    import paper_1708_08434_gb300 as p
+    dom, st = _mesh("axi_small", None)
+    o = quad.build_mesh(dom, st)
+    t = o.tables()
+    g = p.Quad(dom, len(t["level"]))
+    synth.refine_all2(dom, st, g.level_ij, g.refine_level)
+    ne, ni = synth.streamer_densities2(dom, st, t["level"], t["ij"])
+    g.upload(p.NE, ne)
+    g.upload(p.NI, ni)
+    g.set_table(synth.coefficient_table())
+    g.charge_rhs(synth.E_CHARGE, synth.EPS0)
+    g.fmg(1e-8, 40)
+    g.compute_field()
+    assert np.abs(g.download(p.RHS)).max() > 0.0
+    g.advance(1e-13, 0.0, synth.EPS0, 1e-8, 40)
+    rhs = g.download(p.RHS)[t["child"][:, 0] < 0]
+    g.close()
+    assert np.array_equal(rhs, np.zeros_like(rhs))
