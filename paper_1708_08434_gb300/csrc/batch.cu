@@ -54,8 +54,14 @@ struct TileShape {
   int tx, ty, tz;
 };
 
+// Rows of the FP32 grids (error and its right-hand side) are padded to whole
+// 16-byte groups, so that every row of every size can be staged by 16-byte
+// copies; the pad cells of the error are never written and stay zero, like
+// the cells outside the grid.  (Element-wise staging of the sides that are
+// not a multiple of 4 took 1900 cycles a plane, a third of it now.)
+__host__ __device__ constexpr int pitch(int N) { return (N + 3) & ~3; }
 __device__ __forceinline__ long long gidx(int N, int x, int y, int z) {
-  return (long long)x + (long long)N * (y + (long long)N * z);
+  return (long long)x + (long long)pitch(N) * (y + (long long)N * z);
 }
 
 // physical-boundary ghost of `in` across face f (homogeneous for errors)
@@ -69,7 +75,7 @@ template <typename T>
 __device__ __forceinline__ T sum6(const T *__restrict__ v, int N, int x, int y, int z, T c, const Bc &bc,
                                   int homog) {
   long long i = gidx(N, x, y, z);
-  long long sy = N, sz = (long long)N * N;
+  long long sy = pitch(N), sz = sy * N;
   T s = x > 0 ? v[i - 1] : wall(bc, 0, c, homog);
   s += x < N - 1 ? v[i + 1] : wall(bc, 1, c, homog);
   s += y > 0 ? v[i - sy] : wall(bc, 2, c, homog);
@@ -110,9 +116,10 @@ constexpr int EPL = RW * ER, FPL = RW * FR;   // floats per staged plane
 constexpr int RWD = CX + 4;                   // FP64 staged row: x0-2 .. x0+33
 constexpr int DPL = RWD * FR;                 // doubles per staged potential plane
 constexpr int RING = 8;                       // staged planes per block (power of 2)
-constexpr int NRING = 2 * (CX + 2) + 2 * CY;  // cells of the one-cell ring around a column
-constexpr size_t SWEEP_SMEM = sizeof(float) * RING * (EPL + FPL);
-constexpr size_t SWEEP_SMEM_PHI = SWEEP_SMEM + sizeof(double) * RING * CX * CY;
+constexpr int ST = 128;                       // threads of a sweep block: four rows each
+constexpr int SRING = 6;                      // staged planes of a sweep (even, the colour parity unrolls)
+constexpr int SPL = EPL + FPL;                // floats of one sweep slot: an error plane and its rhs plane
+constexpr int RINGT = CX + CY;                // colour-0 cells of the one-cell ring around a column
 constexpr size_t OUTER_SMEM = sizeof(double) * RING * DPL;
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
@@ -146,202 +153,231 @@ __device__ __forceinline__ float wall_w(const Bc &bc, int a, int v, int N) {
 }
 
 // One full red-black Gauss-Seidel sweep (colour 0, then colour 1) of level
-// k on the error, column by column, from e_in into e_out (two buffers, so
+// k on the error, a block per column, from e_in into e_out (two buffers, so
 // that every column reads the sweep's starting values: a column's halo is
 // never a value another column has already swept).  Step p updates colour 0
 // on plane p over the column and the one-cell ring around it (the ring
 // repeats what the neighbouring columns compute, from the same values),
-// then colour 1 on plane p-1 over the column, which by then has all its
-// colour-0 neighbours, and stores plane p-1.  The updates use the values of
-// two separate colour passes over the level.  With zero_in the sweep starts
-// from e = 0 (the first sweep of a level in a V-cycle): e_in is not read,
-// the staged error planes are zero-filled.  With phi != nullptr (level 0,
-// last sweep of a cycle) the swept error is not stored but added to the
-// FP64 potential, phi += (double)e, and emax of the solve is raised to the
-// largest exponent field of the new values.
-// Ring use at step p: planes p-2 .. p+1 are read, p+2 .. p+4 are in flight,
-// and plane p+5 is issued into the slot of plane p-3 (last read at step p-1).
-// The slots of planes -1 and N are zero-filled, so every update adds six
-// staged neighbours (the wall ghosts come in through the coefficient w).
-__global__ void __launch_bounds__(CT) k_bt_sweep(const int4 *__restrict__ cols, int ncols, int k,
-                                                 const BSolve *__restrict__ tab,
-                                                 const unsigned char *__restrict__ active,
-                                                 const float *__restrict__ e_in, float *__restrict__ e_out,
-                                                 const float *__restrict__ f, Bc bc, double *__restrict__ phi,
-                                                 unsigned *__restrict__ emax, int zero_in) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float(*se)[EPL] = reinterpret_cast<float(*)[EPL]>(smem_raw);
-  float(*sf)[FPL] = reinterpret_cast<float(*)[FPL]>(smem_raw + sizeof(float) * RING * EPL);
-  double(*sph)[CX * CY] = reinterpret_cast<double(*)[CX * CY]>(smem_raw + SWEEP_SMEM);
-  const int t = threadIdx.x, tx = t % CX, ty2 = 2 * (t / CX);
-  constexpr int NCH = (ER + FR) * (RW / 4);  // 16-byte chunks of one staged plane pair (e, f)
-  for (int it = blockIdx.x; it < ncols; it += gridDim.x) {
-    const int4 C = cols[it];
-    if (!active[C.x]) continue;  // uniform per block
-    const int N = tab[C.x].N[k];
-    const long long off = tab[C.x].off[k], NN = (long long)N * N;
-    const float h2 = tab[C.x].h2f[k];
-    const int x0 = C.y * CX, y0 = C.z * CY;
-    const float *ev = e_in + off, *fv = f + off;
-    float *eo = e_out + off;
-    double *pv = phi ? phi + tab[C.x].off64 : nullptr;
-    const bool vec = (N & 3) == 0;
-    // this thread's 16-byte chunks (at most two): shared address in slot 0,
-    // source plane (e or f), in-plane element offset, inside the grid
-    unsigned cdst[2] = {0u, 0u};
-    int coff[2] = {0, 0};
-    bool cise[2] = {false, false}, cok[2] = {false, false}, chas[2] = {false, false};
-    if (vec) {
+// then colour 1 on plane p-1 over the column, whose colour-0 neighbours are
+// all done by then, and stores plane p-1.  The updates use the values of
+// two separate colour passes over the level.  ZERO: the sweep starts from
+// e = 0 (the first sweep of a level in a V-cycle); e_in is not read.  PHI
+// (level 0, last sweep of a cycle): the swept error is not stored but added
+// to the FP64 potential, phi += (double)e, and emax of the solve is raised
+// to the largest exponent field of the new values.
+//
+// Instruction issue bounds a sweep whose neighbours all come from shared
+// memory (150 instructions a warp for 64 cells, 0.8 issued a cycle), so a
+// thread keeps its own four rows in registers in colour order: of its two
+// colour-0 cells of plane p, U, one (o, "outer") has a y neighbour outside
+// the thread's rows and one (i, "inner") has not, and so have the colour-1
+// cells V.  The rows of U on plane p are those of V on planes p-1 and p+1,
+// so the z neighbours of Uo(p) are Vo(p-1), Vo(p+1), and only the x
+// neighbours and one y neighbour in four are read from shared memory;
+// colour-0 results alone are written back, and colour 1 of plane p-1 needs
+// of plane p only the thread's own values, so one barrier a plane is enough.
+// Slots at step p: planes p-1 .. p+1 are read, p+2 and p+3 are in flight,
+// and plane p+4 is issued into the slot of plane p-2 (last read at step
+// p-1).  Cells outside the grid are zero in the slots and in the registers;
+// the wall ghosts enter through the coefficient w of c.
+template <bool ZERO, bool PHI>
+__global__ void __launch_bounds__(ST, PHI ? 5 : 6) k_bt_sweep(const int4 *__restrict__ cols, int k,
+                                                              const BSolve *__restrict__ tab,
+                                                              const unsigned char *__restrict__ active,
+                                                              const float *__restrict__ e_in,
+                                                              float *__restrict__ e_out,
+                                                              const float *__restrict__ f, Bc bc,
+                                                              double *__restrict__ phi,
+                                                              unsigned *__restrict__ emax) {
+  __shared__ __align__(16) float sm[SRING * SPL];
+  const int t = threadIdx.x, tx = t % CX, ty = 4 * (t / CX);
+  const int4 C = cols[blockIdx.x];
+  if (!active[C.x]) return;
+  const int N = tab[C.x].N[k], P = pitch(N);
+  const long long off = tab[C.x].off[k], PL = (long long)P * N;
+  const float h2 = tab[C.x].h2f[k];
+  const int x0 = C.y * CX, y0 = C.z * CY;
+  // this thread's 16-byte chunks of a plane pair (e rows, then f rows)
+  constexpr int ECH = ER * (RW / 4), FIRST = ZERO ? ECH : 0, NCH = SPL / 4 - FIRST, U = (NCH + ST - 1) / ST;
+  const float *csrc[U];
+  bool cok[U];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int i = t + u * CT;
-        if (i >= NCH) continue;
-        const bool ise = i < ER * (RW / 4);
-        const int j = ise ? i : i - ER * (RW / 4);
-        const int r = j / (RW / 4), c4 = 4 * (j % (RW / 4));
-        const int y = y0 - (ise ? 2 : 1) + r, x = x0 - 4 + c4;
-        chas[u] = true;
-        cise[u] = ise;
-        cok[u] = y >= 0 && y < N && x >= 0 && x < N && !(ise && zero_in);
-        coff[u] = cok[u] ? y * N + x : 0;
-        cdst[u] = ise ? smem_u32(&se[0][r * RW + c4]) : smem_u32(&sf[0][r * RW + c4]);
+  for (int u = 0; u < U; ++u) {
+    const int i = FIRST + t + u * ST;
+    const bool ise = i < ECH;
+    const int j = ise ? i : i - ECH, y = y0 - (ise ? 2 : 1) + j / (RW / 4), x = x0 - 4 + 4 * (j % (RW / 4));
+    cok[u] = y >= 0 && y < N && x >= 0 && x < N;
+    csrc[u] = (ise ? e_in : f) + off + (cok[u] ? y * P + x : 0);
+  }
+  const unsigned cdst = smem_u32(sm + 4 * (FIRST + t));
+  // copies of plane z (if it exists) into slot sl as one commit group;
+  // called for z = 0, 1, 2, ... in order
+  auto issue = [&](int z, int sl) {
+    if (z < N) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if ((u + 1) * ST <= NCH || t < NCH - u * ST)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(cdst + 4u * (sl * SPL + 4 * u * ST)),
+                       "l"(csrc[u]), "r"(cok[u] ? 16 : 0)
+                       : "memory");
+        csrc[u] += PL;
       }
     }
-    // error-plane copies into slot sl that only zero-fill it (planes -1 and
-    // N, the z neighbours beyond the grid, whose terms are then exact zeros)
-    auto zero_slot = [&](int sl) {
-      if (vec) {
+    cp_commit();
+  };
+  if (ZERO) {
+    for (int i = t; i < SRING * (EPL / 4); i += ST)
+      reinterpret_cast<float4 *>(sm + (i / (EPL / 4)) * SPL)[i % (EPL / 4)] = make_float4(0.f, 0.f, 0.f, 0.f);
+  }
 #pragma unroll
-        for (int u = 0; u < 2; ++u)
-          if (chas[u] && cise[u])
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, 0;\n" ::"r"(cdst[u] + (unsigned)sl * (EPL * 4u)),
-                         "l"(ev)
-                         : "memory");
-      } else {
-        for (int i = t; i < EPL; i += CT) cp_async<4>(&se[sl][i], ev, false);
-      }
-    };
-    // this thread's chunk sources in plane z, advanced one plane per issue
-    const float *csrc[2] = {(cise[0] ? ev : fv) + coff[0], (cise[1] ? ev : fv) + coff[1]};
-    const unsigned cstr[2] = {cise[0] ? EPL * 4u : FPL * 4u, cise[1] ? EPL * 4u : FPL * 4u};
-    // copies of plane z (if it exists) into slot sl = z mod RING as one
-    // commit group; called for z = 0, 1, 2, ... in order
-    auto issue = [&](int z, int sl) {
-      if (z == N) zero_slot(sl);
-      if (z < N) {
-        const float *ez = ev + z * NN, *fz = fv + z * NN;
-        if (vec) {
+  for (int z = 0; z < SRING - 2; ++z) issue(z, z);
+  // Gauss-Seidel value of a cell holding c from its neighbours; w is the
+  // cell's wall coefficient
+  auto relax = [&](float c, float x1, float x2, float y1, float y2, float z1, float z2, float w, float fv) {
+    const float nb = ((x1 + x2) + (y1 + y2)) + (z1 + z2);
+    return (fmaf(w, c, nb) - h2 * fv) * (1.0f / 6.0f);
+  };
+  // rows ya .. ya+3 (N even: valid in pairs).  Even planes have Uo, Ui, Vo,
+  // Vi on rows a, b, c, d (0, 2, 3, 1 or, with an odd first cell, 3, 1, 0,
+  // 2), odd planes on c, d, a, b.
+  const int x = x0 + tx, ya = y0 + ty, par = (x + ya) & 1;
+  const bool warp_in = ya < N;
+  const bool in01 = x < N && ya < N, in23 = x < N && ya + 2 < N;
+  const bool inA = par ? in23 : in01, inB = par ? in01 : in23;  // rows a and d; rows b and c
+  const int q0 = (ty + 2) * RW + tx + 4;
+  const float *const qa = sm + q0 + (par ? 3 : 0) * RW, *const qb = sm + q0 + (par ? 1 : 2) * RW;
+  const float *const qc = sm + q0 + (par ? 0 : 3) * RW, *const qd = sm + q0 + (par ? 2 : 1) * RW;
+  const int fa = par ? RW : -RW;  // to the far y neighbour of row a; the other way round for c
+  const float *const ga = qa + fa, *const gc = qc - fa;
+  const float wx = wall_w(bc, 0, x, N);
+  const float wa = wx + wall_w(bc, 1, ya + (par ? 3 : 0), N), wb = wx + wall_w(bc, 1, ya + (par ? 1 : 2), N);
+  const float wc = wx + wall_w(bc, 1, ya + (par ? 0 : 3), N), wd = wx + wall_w(bc, 1, ya + (par ? 2 : 1), N);
+  // ring cells of colour 0: every other cell beside the column, the even
+  // planes' (E) and the odd planes' (O) being the two of one pair of cells
+  // (x0, y0, N even: both inside the grid or neither)
+  const float *qE = sm, *qO = sm;
+  float rwE = 0.f, rwO = 0.f;
+  bool rin = false;
+  if (t < RINGT) {
+    const bool row = t < CX;  // rows y0-1, y0+CY; else columns x0-1, x0+CX
+    const int j = row ? t % (CX / 2) : (t - CX) % (CY / 2);
+    const bool far = row ? t >= CX / 2 : t >= CX + CY / 2;
+    const int rx = row ? x0 + 2 * j : (far ? x0 + CX : x0 - 1), ry = row ? (far ? y0 + CY : y0 - 1) : y0 + 2 * j;
+    rin = rx >= 0 && rx < N && ry >= 0 && ry < N;
+    const int odd = (rx + ry) & 1, dx = row ? 1 : 0, dy = 1 - dx;
+    const float *rq = sm + (ry - y0 + 2) * RW + (rx - x0 + 4);
+    const int ps = dx + dy * RW;
+    qE = rq + odd * ps, qO = rq + (1 - odd) * ps;
+    rwE = wall_w(bc, 0, rx + odd * dx, N) + wall_w(bc, 1, ry + odd * dy, N);
+    rwO = wall_w(bc, 0, rx + (1 - odd) * dx, N) + wall_w(bc, 1, ry + (1 - odd) * dy, N);
+  }
+  const float wlo = bc.type[4] ? -1.f : 1.f, whi = bc.type[5] ? -1.f : 1.f;
+  float *eo = e_out + off + (long long)ya * P + x;  // this thread's cells of the plane stored next
+  const long long NN = (long long)N * N;
+  double *pv = PHI ? phi + tab[C.x].off64 + (long long)ya * N + x : nullptr;
+  double ph[2][4] = {};  // PHI: potential of two planes, loaded two steps ahead
+  auto load_phi = [&](int z, double(&d)[4]) {
+    if (z >= N) return;
+    const double *src = pv + (z >= 2 ? 2 : z) * NN;  // pv moves on from step 2
+    if (in01) d[0] = src[0], d[1] = src[N];
+    if (in23) d[2] = src[2 * N], d[3] = src[3 * N];
+  };
+  if (PHI) load_phi(0, ph[0]);
+  unsigned em = 0;  // PHI: largest exponent field written
+  constexpr int F = EPL - RW;  // from an error cell to its right-hand side, in a slot
+  cp_wait<SRING - 3>();        // plane 0 has landed
+  __syncthreads();
+  // U and V of planes p-2, p-1, p at the head of step p
+  float Uo2 = 0.f, Ui2 = 0.f, Uo1 = 0.f, Ui1 = 0.f, Vo1 = 0.f, Vi1 = 0.f;
+  float Uo0 = 0.f, Ui0 = 0.f, Vo0 = 0.f, Vi0 = 0.f;
+  if (!ZERO) Uo0 = qa[0], Ui0 = qb[0], Vo0 = qc[0], Vi0 = qd[0];
+  float wz = wlo, wz1 = 0.f;  // wall coefficients of planes p and p-1
+  // steps p = pb + i, unrolled by the ring size so that every slot index
+  // and colour parity is a constant (pb is a multiple of SRING)
+  for (int pb = 0; pb <= N; pb += SRING) {
 #pragma unroll
-          for (int u = 0; u < 2; ++u)
-            if (chas[u]) {
-              asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(cdst[u] + (unsigned)sl * cstr[u]),
-                           "l"(csrc[u]), "r"(cok[u] ? 16 : 0)
-                           : "memory");
-              csrc[u] += NN;
-            }
-        } else {
-          for (int i = t; i < (ER + FR) * RW; i += CT) {
-            const bool ise = i < ER * RW;
-            const int j = ise ? i : i - ER * RW;
-            const int r = j / RW, c = j % RW;
-            const int y = y0 - (ise ? 2 : 1) + r, x = x0 - 4 + c;
-            const bool ok = y >= 0 && y < N && x >= 0 && x < N && !(ise && zero_in);
-            const float *src = ise ? ez : fz;
-            float *dst = ise ? &se[sl][j] : &sf[sl][j];
-            cp_async<4>(dst, ok ? src + y * N + x : src, ok);
+    for (int i = 0; i < SRING; ++i) {
+      const int p = pb + i;
+      if (p > N) break;
+      cp_wait<SRING - 4>();  // this thread's copies of planes <= p+1 have landed
+      __syncthreads();       // everyone's have; step p-1's reads of plane p-2 are done
+      issue(p + SRING - 2, (i + SRING - 2) % SRING);
+      if (p == N - 1) wz += whi;
+      if (warp_in) {
+        const bool odd = i & 1;
+        const int S0 = i * SPL, Sp = ((i + 1) % SRING) * SPL, Sm = ((i + SRING - 1) % SRING) * SPL;
+        const float *o0 = odd ? qc : qa, *i0 = odd ? qd : qb, *g0 = odd ? gc : ga;
+        const float wo = odd ? wc : wa, wi = odd ? wd : wb;
+        const bool ino = odd ? inB : inA, ini = odd ? inA : inB;
+        float Uon = 0.f, Uin = 0.f, Von = 0.f, Vin = 0.f;  // plane p+1
+        if (p < N) {
+          if (!ZERO && p + 1 < N) {
+            Uon = (odd ? qa : qc)[Sp], Uin = (odd ? qb : qd)[Sp];
+            Von = o0[Sp], Vin = i0[Sp];
           }
-        }
-        if (pv) {  // level 0: N even, rows of the column in 16-byte pairs
-          const int r = t / (CX / 2), x = x0 + 2 * (t % (CX / 2)), y = y0 + r;
-          const bool ok = x < N && y < N;
-          cp_async<16>(&sph[sl][r * CX + 2 * (t % (CX / 2))], ok ? pv + z * NN + y * N + x : pv, ok);
-        }
-      }
-      cp_commit();
-    };
-    // Gauss-Seidel update of the staged cell at e-plane index q (rhs index
-    // qf) of the plane held in pz, with the planes below / above it in pm /
-    // pp (zero planes beyond the grid) and its rhs plane in fz; w is the
-    // cell's wall coefficient
-    auto update = [&](float *pz, const float *pm, const float *pp, const float *fz, int q, int qf, float w) {
-      const float c = pz[q];
-      float s = pz[q - 1] + pz[q + 1];
-      s += pz[q - RW];
-      s += pz[q + RW];
-      s += pm[q];
-      s += pp[q];
-      s = fmaf(w, c, s);
-      pz[q] = (s - h2 * fz[qf]) * (1.0f / 6.0f);
-    };
-    // this thread's two column cells (rows ya, ya+1) and its ring cell
-    const int x = x0 + tx, ya = y0 + ty2;
-    const bool in = x < N && ya < N;  // N even, ya even: both rows or neither
-    const int q0 = (ty2 + 2) * RW + tx + 4, qf0 = (ty2 + 1) * RW + tx + 4;
-    const float wx = wall_w(bc, 0, x, N);
-    const float w0 = wx + wall_w(bc, 1, ya, N), w1 = wx + wall_w(bc, 1, ya + 1, N);
-    int rx = -1, ry = -1;
-    if (t < NRING) {
-      if (t < CX + 2) rx = x0 - 1 + t, ry = y0 - 1;
-      else if (t < 2 * (CX + 2)) rx = x0 - 1 + t - (CX + 2), ry = y0 + CY;
-      else if (t < 2 * (CX + 2) + CY) rx = x0 - 1, ry = y0 + t - 2 * (CX + 2);
-      else rx = x0 + CX, ry = y0 + t - 2 * (CX + 2) - CY;
-    }
-    const bool rin = rx >= 0 && rx < N && ry >= 0 && ry < N;
-    const int rq = (ry - y0 + 2) * RW + (rx - x0 + 4), rqf = (ry - y0 + 1) * RW + (rx - x0 + 4);
-    const float rw = rin ? wall_w(bc, 0, rx, N) + wall_w(bc, 1, ry, N) : 0.f;
-    const long long row0 = (long long)ya * N + x;
-    float *eo_z = eo + row0;                         // this thread's cells of the plane stored next
-    double *pv_z = pv ? pv + row0 : nullptr;
-    const int par = (x + ya) & 1, rpar = (rx + ry) & 1;  // colour parities at plane 0
-    unsigned em = 0;  // with phi: largest exponent field written
-    __syncthreads();  // the previous column's planes are no longer read
-    zero_slot((-1) & (RING - 1));  // plane -1, landing with plane 0's group
-#pragma unroll
-    for (int z = 0; z < RING - 3; ++z) issue(z, z);  // planes 0 .. RING-4
-    // steps p = pb + i, unrolled by the ring size so that every slot index
-    // and colour parity is a constant (pb is a multiple of RING)
-    for (int pb = 0; pb <= N; pb += RING) {
-#pragma unroll
-      for (int i = 0; i < RING; ++i) {
-        const int p = pb + i;
-        if (p > N) break;
-        cp_wait<RING - 5>();  // this thread's copies of planes <= p+1 have landed
-        __syncthreads();      // everyone's have; step p-1's reads of plane p-3 are done
-        issue(p + RING - 3, (i + RING - 3) & (RING - 1));
-        float *Pm2 = se[(i - 2) & (RING - 1)], *Pm1 = se[(i - 1) & (RING - 1)], *P0 = se[i & (RING - 1)],
-              *Pp1 = se[(i + 1) & (RING - 1)];
-        const int o = par ^ (i & 1);  // row offset of the colour-0 cell of plane p and the colour-1 cell of p-1
-        if (p < N) {                  // colour 0 on plane p: one column cell per thread, and the ring
-          const float wz = wall_w(bc, 2, p, N);
-          const float *F0 = sf[i & (RING - 1)];
-          if (in) update(P0, Pm1, Pp1, F0, q0 + o * RW, qf0 + o * RW, (o ? w1 : w0) + wz);
-          if (rin && rpar == (i & 1)) update(P0, Pm1, Pp1, F0, rq, rqf, rw + wz);
-        }
-        __syncthreads();
-        if (p >= 1 && in) {  // colour 1 on plane p-1, then store both cells
-          update(Pm1, Pm2, P0, sf[(i - 1) & (RING - 1)], q0 + o * RW, qf0 + o * RW,
-                 (o ? w1 : w0) + wall_w(bc, 2, p - 1, N));
-          const float v0 = Pm1[q0], v1 = Pm1[q0 + RW];
-          if (pv) {
-            const double *ph = sph[(i - 1) & (RING - 1)];
-            const double n0 = ph[ty2 * CX + tx] + cvt_f32_f64(v0), n1 = ph[(ty2 + 1) * CX + tx] + cvt_f32_f64(v1);
-            pv_z[0] = n0;
-            pv_z[N] = n1;
-            pv_z += NN;
-            em = max(em, max(expo_of(n0), expo_of(n1)));
+          float ui, uo;
+          if (ZERO) {
+            ui = (0.f - h2 * i0[S0 + F]) * (1.0f / 6.0f);
+            uo = (0.f - h2 * o0[S0 + F]) * (1.0f / 6.0f);
           } else {
-            eo_z[0] = v0;
-            eo_z[N] = v1;
-            eo_z += NN;
+            ui = relax(Ui0, i0[S0 - 1], i0[S0 + 1], Vi0, Vo0, Vi1, Vin, wi + wz, i0[S0 + F]);
+            uo = relax(Uo0, o0[S0 - 1], o0[S0 + 1], Vi0, g0[S0], Vo1, Von, wo + wz, o0[S0 + F]);
+          }
+          Ui0 = ini ? ui : 0.f;
+          Uo0 = ino ? uo : 0.f;
+          const_cast<float *>(i0)[S0] = Ui0;
+          const_cast<float *>(o0)[S0] = Uo0;
+        }
+        if (p >= 1) {  // colour 1 on plane p-1, then store its four cells
+          const float nvi = relax(Vi1, i0[Sm - 1], i0[Sm + 1], Uo1, Ui1, Ui2, Ui0, wi + wz1, i0[Sm + F]);
+          const float nvo = relax(Vo1, o0[Sm - 1], o0[Sm + 1], Ui1, g0[Sm], Uo2, Uo0, wo + wz1, o0[Sm + F]);
+          const bool up = odd ? !par : par;  // rows 0 .. 3 hold U V U V (or V U V U)
+          const float r0 = up ? Uo1 : nvo, r1 = up ? nvi : Ui1, r2 = up ? Ui1 : nvi, r3 = up ? nvo : Uo1;
+          if (PHI) {
+            double(&d)[4] = ph[(i + 1) & 1];
+            const double n0 = d[0] + cvt_f32_f64(r0), n1 = d[1] + cvt_f32_f64(r1);
+            const double n2 = d[2] + cvt_f32_f64(r2), n3 = d[3] + cvt_f32_f64(r3);
+            if (in01) {
+              pv[0] = n0, pv[N] = n1;
+              em = max(em, max(expo_of(n0), expo_of(n1)));
+            }
+            if (in23) {
+              pv[2 * N] = n2, pv[3 * N] = n3;
+              em = max(em, max(expo_of(n2), expo_of(n3)));
+            }
+          } else {
+            if (in01) eo[0] = r0, eo[P] = r1;
+            if (in23) eo[2 * P] = r2, eo[3 * P] = r3;
+            eo += PL;
           }
         }
+        if (PHI) {  // plane p+1, used at step p+2
+          load_phi(p + 1, ph[(i + 1) & 1]);
+          if (p >= 1) pv += NN;
+        }
+        Uo2 = Uo1, Ui2 = Ui1, Uo1 = Uo0, Ui1 = Ui0, Uo0 = Uon, Ui0 = Uin;
+        Vo1 = Vo0, Vi1 = Vi0, Vo0 = Von, Vi0 = Vin;
       }
+      if (rin && p < N) {
+        const int S0 = i * SPL, Sp = ((i + 1) % SRING) * SPL, Sm = ((i + SRING - 1) % SRING) * SPL;
+        const float *r = (i & 1) ? qO : qE;
+        float v;
+        if (ZERO) {
+          v = (0.f - h2 * r[S0 + F]) * (1.0f / 6.0f);
+        } else {
+          const float zm = p > 0 ? r[Sm] : 0.f, zp = p + 1 < N ? r[Sp] : 0.f;
+          v = relax(r[S0], r[S0 - 1], r[S0 + 1], r[S0 - RW], r[S0 + RW], zm, zp, ((i & 1) ? rwO : rwE) + wz, r[S0 + F]);
+        }
+        const_cast<float *>(r)[S0] = v;
+      }
+      wz1 = wz;
+      wz = 0.f;
     }
-    cp_wait<0>();
-    if (pv) {  // uniform per block
-      em = __reduce_max_sync(0xffffffffu, em);
-      if ((t & 31) == 0 && em) atomicMax(emax + C.x, em);
-    }
+  }
+  cp_wait<0>();
+  if (PHI) {
+    em = __reduce_max_sync(0xffffffffu, em);
+    if ((t & 31) == 0 && em) atomicMax(emax + C.x, em);
   }
 }
 
@@ -420,40 +456,32 @@ __global__ void __launch_bounds__(CT, 6) k_bt_restrict_col(const int4 *__restric
     if (!active[C.x]) continue;  // uniform per block
     const BSolve &S = tab[C.x];
     const int N = S.N[k], Nc = S.N[k + 1];  // N = 2 Nc
-    const long long NN = (long long)N * N;
+    const int P = pitch(N), Pc = pitch(Nc);
+    const long long NN = (long long)P * N;
     const float *ef = e + S.off[k], *ff = f + S.off[k];
     float *fc = f + S.off[k + 1];
     const float inv_h2 = 1.0f / S.h2f[k];
     const int x0 = C.y * CX, y0 = C.z * CY, x = x0 + tx, ya = y0 + ty2;
     const bool in = x < N && ya < N;  // N even, ya even: both rows or neither
-    const bool vec = (N & 3) == 0;
-    // this thread's 16-byte chunk of a staged plane (vec grids): slot-0
-    // offset, in-plane element offset, inside the grid
+    // this thread's 16-byte chunk of a staged plane: slot-0 offset, in-plane
+    // element offset, inside the grid
     int cdst = -1, coff = 0;
     bool cok = false;
-    if (vec && t < RFR * (RRW / 4)) {
+    if (t < RFR * (RRW / 4)) {
       const int r = t / (RRW / 4), c4 = 4 * (t % (RRW / 4)), y = y0 - 1 + r, xx = x0 - 4 + c4;
       cok = y >= 0 && y < N && xx >= 0 && xx < N;
-      coff = cok ? y * N + xx : 0;
+      coff = cok ? y * P + xx : 0;
       cdst = r * RRW + c4;
     }
-    // this thread's chunk source in plane z (vec grids), advanced one plane
-    // per issue of a plane of the grid
+    // this thread's chunk source in plane z, advanced one plane per issue of
+    // a plane of the grid
     const float *csrc = ef + coff;
     // copies of plane z into slot sl = z mod RING (zero planes outside the
     // grid); called for z = -1, 0, 1, ... in order
     auto issue = [&](int z, int sl) {
       const bool zin = z >= 0 && z < N;
-      if (vec) {
-        if (cdst >= 0) cp_async<16>(&se[sl][cdst], zin ? csrc : ef, cok && zin);
-        if (zin) csrc += NN;
-      } else {
-        for (int i = t; i < RPL; i += CT) {
-          const int y = y0 - 1 + i / RRW, xx = x0 - 4 + i % RRW;
-          const bool ok = zin && y >= 0 && y < N && xx >= 0 && xx < N;
-          cp_async<4>(&se[sl][i], ok ? ef + z * NN + y * N + xx : ef, ok);
-        }
-      }
+      if (cdst >= 0) cp_async<16>(&se[sl][cdst], zin ? csrc : ef, cok && zin);
+      if (zin) csrc += NN;
       cp_commit();
     };
     const int q0 = (ty2 + 1) * RRW + tx + 4;
@@ -461,14 +489,14 @@ __global__ void __launch_bounds__(CT, 6) k_bt_restrict_col(const int4 *__restric
     const float w0 = wx + wall_w(bc, 1, ya, N), w1 = wx + wall_w(bc, 1, ya + 1, N);
     // this thread's two f values of planes z (fa) and z+1 (fb), loaded two
     // planes ahead of their use
-    const float *frow = ff + (in ? (long long)ya * N + x : 0);
+    const float *frow = ff + (in ? (long long)ya * P + x : 0);
     float fa0 = 0.f, fa1 = 0.f, fb0 = 0.f, fb1 = 0.f;
     if (in) {
-      fa0 = __ldg(frow), fa1 = __ldg(frow + N);
-      if (N > 1) fb0 = __ldg(frow + NN), fb1 = __ldg(frow + NN + N);
+      fa0 = __ldg(frow), fa1 = __ldg(frow + P);
+      if (N > 1) fb0 = __ldg(frow + NN), fb1 = __ldg(frow + NN + P);
     }
     const float *fnext = frow + 2 * NN;  // f of plane z+2 at step z
-    float *fcz = fc + (long long)(ya >> 1) * Nc + (x >> 1);  // this thread's coarse cell, coarse plane z/2
+    float *fcz = fc + (long long)(ya >> 1) * Pc + (x >> 1);  // this thread's coarse cell, coarse plane z/2
     float acc = 0.f;
     __syncthreads();  // the previous column's planes are no longer read
 #pragma unroll
@@ -481,7 +509,7 @@ __global__ void __launch_bounds__(CT, 6) k_bt_restrict_col(const int4 *__restric
         const int z = zb + i;
         if (z >= N) break;
         float fn0 = 0.f, fn1 = 0.f;
-        if (in && z + 2 < N) fn0 = __ldg(fnext), fn1 = __ldg(fnext + N);
+        if (in && z + 2 < N) fn0 = __ldg(fnext), fn1 = __ldg(fnext + P);
         fnext += NN;
         cp_wait<2>();     // this thread's copies of planes <= z+1 have landed
         __syncthreads();  // everyone's have; step z-1's reads are done
@@ -508,7 +536,7 @@ __global__ void __launch_bounds__(CT, 6) k_bt_restrict_col(const int4 *__restric
         acc = (i & 1) ? acc + rs : rs;
         if (i & 1) {
           if (in && !(tx & 1)) *fcz = acc * 0.125f;
-          fcz += (long long)Nc * Nc;
+          fcz += (long long)Pc * Nc;
         }
       }
     }
@@ -536,7 +564,8 @@ __global__ void __launch_bounds__(CT) k_bt_prolong(const int4 *__restrict__ cols
     if (!active[C.x]) continue;  // uniform per block
     const BSolve &S = tab[C.x];
     const int N = S.N[k], Nc = S.N[k + 1];  // N = 2 Nc
-    const long long NN = (long long)N * N, NNc = (long long)Nc * Nc;
+    const int P = pitch(N), Pc = pitch(Nc);
+    const long long NN = (long long)P * N, NNc = (long long)Pc * Nc;
     float *ef = e + S.off[k];
     const float *ec = e + S.off[k + 1];
     const int x0 = C.y * CX, y0 = C.z * CY, X0 = x0 / 2 - 1, Y0 = y0 / 2 - 1;
@@ -557,17 +586,17 @@ __global__ void __launch_bounds__(CT) k_bt_prolong(const int4 *__restrict__ cols
       float v = 0.f;
       if (t < PPL && Z < Nc) {
         const int X = X0 + t % PX, Y = Y0 + t / PX;
-        if (X >= 0 && X < Nc && Y >= 0 && Y < Nc) v = ec[Z * NNc + (long long)Y * Nc + X];
+        if (X >= 0 && X < Nc && Y >= 0 && Y < Nc) v = ec[Z * NNc + (long long)Y * Pc + X];
       }
       return v;
     };
-    const long long row0 = (long long)ya * N + x;
+    const long long row0 = (long long)ya * P + x;
     // fine values (rows ya, ya+1) of planes 2Z, 2Z+1 (f) and 2Z+2, 2Z+3 (g);
     // those of step Z+2 are loaded during step Z
     float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f, g0 = 0.f, g1 = 0.f, g2 = 0.f, g3 = 0.f;
     if (in) {
-      f0 = ef[row0], f1 = ef[row0 + N], f2 = ef[NN + row0], f3 = ef[NN + row0 + N];
-      if (Nc > 1) g0 = ef[2 * NN + row0], g1 = ef[2 * NN + row0 + N], g2 = ef[3 * NN + row0], g3 = ef[3 * NN + row0 + N];
+      f0 = ef[row0], f1 = ef[row0 + P], f2 = ef[NN + row0], f3 = ef[NN + row0 + P];
+      if (Nc > 1) g0 = ef[2 * NN + row0], g1 = ef[2 * NN + row0 + P], g2 = ef[3 * NN + row0], g3 = ef[3 * NN + row0 + P];
     }
     const float *enext = ef + 4 * NN + row0;  // plane 2Z+4 at step Z
     float *eout = ef + row0;                  // plane 2Z at step Z
@@ -586,7 +615,7 @@ __global__ void __launch_bounds__(CT) k_bt_prolong(const int4 *__restrict__ cols
         const int Z = Zb + i;
         if (Z >= Nc) break;
         float h0 = 0.f, h1 = 0.f, h2 = 0.f, h3 = 0.f;
-        if (in && Z + 2 < Nc) h0 = enext[0], h1 = enext[N], h2 = enext[NN], h3 = enext[NN + N];
+        if (in && Z + 2 < Nc) h0 = enext[0], h1 = enext[P], h2 = enext[NN], h3 = enext[NN + P];
         enext += 2 * NN;
         if (in) {
           const float *cz = sc[i & 3];
@@ -597,9 +626,9 @@ __global__ void __launch_bounds__(CT) k_bt_prolong(const int4 *__restrict__ cols
           const float cym = cz[qc - PX], cyp = cz[qc + PX];
           // (c + c_x + c_y + c_z) with the wall ghosts, for the four fine cells
           eout[0] = f0 + 0.25f * fmaf(wxy0 + wz_lo, c, ((c + cxn) + cym) + c_lo);
-          eout[N] = f1 + 0.25f * fmaf(wxy1 + wz_lo, c, ((c + cxn) + cyp) + c_lo);
+          eout[P] = f1 + 0.25f * fmaf(wxy1 + wz_lo, c, ((c + cxn) + cyp) + c_lo);
           eout[NN] = f2 + 0.25f * fmaf(wxy0 + wz_hi, c, ((c + cxn) + cym) + c_hi);
-          eout[NN + N] = f3 + 0.25f * fmaf(wxy1 + wz_hi, c, ((c + cxn) + cyp) + c_hi);
+          eout[NN + P] = f3 + 0.25f * fmaf(wxy1 + wz_hi, c, ((c + cxn) + cyp) + c_hi);
         }
         eout += 2 * NN;
         __syncthreads();  // plane Z-2's slot is free
@@ -651,7 +680,8 @@ __global__ void __launch_bounds__(512) k_bt_coarse(const int *__restrict__ solve
     lam[a * BMAXC + m] = -4.0 * sn * sn;
   }
   const float *fv = f + S.off[k];
-  for (int c = t; c < n3; c += blockDim.x) x[c] = (double)fv[c];
+  const int P = pitch(n);
+  for (int c = t; c < n3; c += blockDim.x) x[c] = (double)fv[c % n + P * (c / n)];
   __syncthreads();
   // forward along x, y, z; divide; backward along x, y, z
   for (int pass = 0; pass < 6; ++pass) {
@@ -686,7 +716,7 @@ __global__ void __launch_bounds__(512) k_bt_coarse(const int *__restrict__ solve
     if ((t & 31) == 0 && em) atomicMax(emax + s, em);
   } else {
     float *ev = e + S.off[k];
-    for (int c = t; c < n3; c += blockDim.x) ev[c] = (float)x[c];
+    for (int c = t; c < n3; c += blockDim.x) ev[c % n + P * (c / n)] = (float)x[c];
   }
 }
 
@@ -730,7 +760,7 @@ __global__ void __launch_bounds__(CT, 5) k_bt_outer(const int4 *__restrict__ col
     if (!active[C.x]) continue;  // uniform per block
     const BSolve &S = tab[C.x];
     const int N = S.N[0];
-    const long long o64 = S.off64, o32 = S.off[0], NN = (long long)N * N;
+    const long long o64 = S.off64, NN = (long long)N * N;
     const int E = max(max((int)emax[C.x], ebc), 123);
     const bool finite = E < 0x7ff;
     // 2^(E-1080) h^-2, exact: a power of two (exponent field E - 57 >= 66)
@@ -794,6 +824,8 @@ __global__ void __launch_bounds__(CT, 5) k_bt_outer(const int4 *__restrict__ col
       return bc.type[f] ? fix_of_bits((unsigned long long)__double_as_longlong(bc.g2[f]), E) - c : c;
     };
     const long long row0 = (long long)ya * N + x;
+    const int P = pitch(N);
+    float *const rz = f32 + S.off[0] + (long long)ya * P + x;
     // f of planes p (set A for even p, B for odd p): loaded two steps ahead
     double fa0 = 0.0, fa1 = 0.0, fb0 = 0.0, fb1 = 0.0;
     if (in0) fa0 = fv[row0];
@@ -839,7 +871,7 @@ __global__ void __launch_bounds__(CT, 5) k_bt_outer(const int4 *__restrict__ col
         const long long sx = ((xm + xp) + (ym + yp)) + (zm + zp) - 6 * c;  // exact
         const double r = fma(-__ll2double_rn(sx), kk, o ? f1 : f0);
         const unsigned long long rb = finite ? (unsigned long long)__double_as_longlong(r) : 0x7ff8000000000000ull;
-        f32[o32 + p * NN + row0 + o * N] = cvt_bits_f32_rn(rb);
+        rz[(long long)p * P * N + o * P] = cvt_bits_f32_rn(rb);
         const unsigned long long a = rb & 0x7fffffffffffffffull;
         m = a > m ? a : m;
       }
@@ -902,7 +934,7 @@ __global__ void __launch_bounds__(CT, OUTER0_BLOCKS) k_bt_outer0(const int4 *__r
     if (!active[C.x]) continue;  // uniform per block
     const BSolve &S = tab[C.x];
     const int N = S.N[0];
-    const long long o64 = S.off64, o32 = S.off[0], NN = (long long)N * N;
+    const long long o64 = S.off64, NN = (long long)N * N;
     const double inv_h2 = S.inv_h2;
     // this thread's cells: (x, y) and (x+1, y) of every plane
     const int x = C.y * CX + 2 * (t % (CX / 2)), y = C.z * CY + t / (CX / 2);
@@ -923,7 +955,8 @@ __global__ void __launch_bounds__(CT, OUTER0_BLOCKS) k_bt_outer0(const int4 *__r
     }
     const bool in = x < N && y < N, vec = (N & 1) == 0;  // N even: both cells or neither, 16-byte aligned
     const double *pz = phi + o64 + (long long)y * N + x, *fz = f64 + o64 + (long long)y * N + x;
-    float *rz = f32 + o32 + (long long)y * N + x;
+    const int P = pitch(N);
+    float *rz = f32 + S.off[0] + (long long)y * P + x;
     // r of one cell from f, with the plane's wall terms (w4, w5)
     auto resid = [&](int u, double f, bool w4, bool w5) {
       double r = f;
@@ -945,12 +978,12 @@ __global__ void __launch_bounds__(CT, OUTER0_BLOCKS) k_bt_outer0(const int4 *__r
 #pragma unroll 4
       for (int p = 0; p < N; ++p) {
         const bool w4 = p == 0 && bc.type[4], w5 = p == N - 1 && bc.type[5];
-        const long long at = p * NN;
+        const long long at = p * NN, at32 = (long long)p * P * N;
         if (vec) {
           const double2 v = *reinterpret_cast<const double2 *>(pz + at);
           const double2 f = *reinterpret_cast<const double2 *>(fz + at);
           const unsigned long long r0 = resid(0, f.x, w4, w5), r1 = resid(1, f.y, w4, w5);
-          *reinterpret_cast<float2 *>(rz + at) = make_float2(cvt_bits_f32_rn(r0), cvt_bits_f32_rn(r1));
+          *reinterpret_cast<float2 *>(rz + at32) = make_float2(cvt_bits_f32_rn(r0), cvt_bits_f32_rn(r1));
           take(v.x, r0);
           take(v.y, r1);
         } else {
@@ -958,7 +991,7 @@ __global__ void __launch_bounds__(CT, OUTER0_BLOCKS) k_bt_outer0(const int4 *__r
           for (int u = 0; u < 2; ++u)
             if (x + u < N) {
               const unsigned long long r = resid(u, fz[at + u], w4, w5);
-              rz[at + u] = cvt_bits_f32_rn(r);
+              rz[at32 + u] = cvt_bits_f32_rn(r);
               take(pz[at + u], r);
             }
         }
@@ -1155,7 +1188,7 @@ extern "C" int sm_batch_create(sm_batch **out, int n_solves, const int *cells_pe
     for (int s = 0; s < n_solves; ++s)
       if (k < S[s].nlev) {
         S[s].off[k] = pool;
-        pool += pad_grid((long long)S[s].N[k] * S[s].N[k] * S[s].N[k]);
+        pool += pad_grid((long long)pitch(S[s].N[k]) * S[s].N[k] * S[s].N[k]);
       }
   int ndev = 0;
   if (cudaGetDeviceCount(&ndev) != cudaSuccess || ndev < 1) {
@@ -1413,8 +1446,13 @@ static int smooth_level(sm_batch *b, int k, int nu, bool from_zero, bool add_phi
     const float *in = (s & 1) ? b->e32b : b->e32;
     float *out = (s & 1) ? b->e32 : b->e32b;
     double *phi = (add_phi && s == nu - 1) ? b->phi : nullptr;
-    k_bt_sweep<<<grid_for(b, n), CT, phi ? SWEEP_SMEM_PHI : SWEEP_SMEM, b->stream>>>(
-        cols, (int)n, k, b->d_tab, b->d_active, in, out, b->f32, b->bc, phi, b->d_emax, (from_zero && s == 0) ? 1 : 0);
+    auto run = [&](auto kernel) {
+      kernel<<<(unsigned)n, ST, 0, b->stream>>>(cols, k, b->d_tab, b->d_active, in, out, b->f32, b->bc, phi,
+                                                b->d_emax);
+    };
+    if (phi) run(k_bt_sweep<false, true>);
+    else if (from_zero && s == 0) run(k_bt_sweep<true, false>);
+    else run(k_bt_sweep<false, false>);
     ++b->n_launch;
   }
   if ((nu & 1) && !add_phi) {
@@ -1442,7 +1480,6 @@ static int set_attrs(sm_batch *b) {
     if (!b->ev_fork[k]) BCK(cudaEventCreateWithFlags(&b->ev_fork[k], cudaEventDisableTiming));
     if (!b->ev_join[k]) BCK(cudaEventCreateWithFlags(&b->ev_join[k], cudaEventDisableTiming));
   }
-  BCK(cudaFuncSetAttribute(k_bt_sweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SWEEP_SMEM_PHI));
   BCK(cudaFuncSetAttribute(k_bt_outer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OUTER_SMEM));
   BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->rcol_per_sm, k_bt_restrict_col, CT, 0));
   b->rcol_per_sm = std::max(1, b->rcol_per_sm);
@@ -1782,9 +1819,9 @@ extern "C" int sm_batch_kernel_bench(sm_batch *b, int kclass, int reps, double *
   auto launch = [&]() {
     switch (kclass) {
       case 0:
-        k_bt_sweep<<<grid_for(b, nsw), CT, SWEEP_SMEM, b->stream>>>(b->d_tiles + b->scol_off[0], (int)nsw, 0,
-                                                                     b->d_tab, b->d_active, b->e32, b->e32b,
-                                                                     b->f32, b->bc, nullptr, nullptr, 0);
+        k_bt_sweep<false, false><<<(unsigned)nsw, ST, 0, b->stream>>>(b->d_tiles + b->scol_off[0], 0, b->d_tab,
+                                                                      b->d_active, b->e32, b->e32b, b->f32, b->bc,
+                                                                      nullptr, nullptr);
         break;
       case 1:
         k_bt_outer<<<grid_for(b, b->fine_cnt), CT, OUTER_SMEM, b->stream>>>(
