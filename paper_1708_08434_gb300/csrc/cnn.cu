@@ -507,15 +507,18 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
   TrainS &S = *reinterpret_cast<TrainS *>(smraw + o2);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   TcState tc;
+  // what needs nothing of the launch before it runs while that one ends
+  zero_acts(F);
+  zero16(S.d2, sizeof(S.d2));
+  for (int i = t; i < NG; i += TT) S.grad[i] = 0.0f;
+  pdl_wait();
+  if (*err) return;  // a wait of an earlier pass ran out: the results are void
   tc_begin(tc, &mbar, &tslot, err, TRAIN_COLS);
   load_net(N, w);
   for (int i = t; i < 27 * 256; i += TT) {
     const int tp = i / 256, co = (i / 16) % 16, ci = i % 16;
     S.w2t[W2Ti(tp, co, ci)] = __float2bfloat16_rn(w[O_W2 + (co * 16 + ci) * 27 + tp]);
   }
-  zero_acts(F);
-  zero16(S.d2, sizeof(S.d2));
-  for (int i = t; i < NG; i += TT) S.grad[i] = 0.0f;
   float my_loss = 0.0f;
   bool wg_acc = false;  // the backward-weight accumulators hold a sum
   __syncthreads();
@@ -758,34 +761,63 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
   }
 }
 
-// gradient = sum of the CTA partials in CTA order (deterministic)
-__global__ void k_cnn_reduce(const float *__restrict__ partial, int nblk, float *__restrict__ grad,
-                             const float *__restrict__ loss_partial, float *__restrict__ loss) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < NP) {
-    float s = 0.0f;
-    for (int b = 0; b < nblk; ++b) s += partial[(size_t)b * NP + i];
-    grad[i] = s;
-  }
-  if (i == 0) {
-    float s = 0.0f;
-    for (int b = 0; b < nblk; ++b) s += loss_partial[b];
-    *loss = s;
-  }
+// One Adam step of a parameter on the FP32 master weights (bias-corrected moments)
+struct AdamStep {
+  float *w, *m, *v;
+  float lr, c1, c2;
+};
+__device__ __forceinline__ void adam_update(const AdamStep &A, int i, float gi) {
+  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  float mi = b1 * A.m[i] + (1.0f - b1) * gi;
+  float vi = b2 * A.v[i] + (1.0f - b2) * gi * gi;
+  A.m[i] = mi;
+  A.v[i] = vi;
+  A.w[i] -= A.lr * (mi / A.c1) / (sqrtf(vi / A.c2) + eps);
 }
 
-// Adam on the FP32 master weights (bias-corrected moments)
-__global__ void k_cnn_adam(float *__restrict__ w, float *__restrict__ m, float *__restrict__ v,
-                           const float *__restrict__ g, float lr, float c1, float c2) {
+__global__ void k_cnn_adam(AdamStep A, const float *__restrict__ g) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NP) return;
-  const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
-  float gi = g[i];
-  float mi = b1 * m[i] + (1.0f - b1) * gi;
-  float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  if (i < NP) adam_update(A, i, g[i]);
+}
+
+// gradient = sum of the CTA partials in CTA order (deterministic), the loss
+// likewise (the last block); ADAM: followed by the Adam step of the same
+// parameter, unless a completion wait of the gradient pass ran out.  Latency
+// bounds it: 5 MB from L2 in one chain of adds per parameter, so a warp a
+// block spreads the parameters over all SMs and 19 loads of a chain are in
+// flight (152 CTAs: eight rounds).  12.6 us as blocks of 256 with one load
+// at a time, and 3.6 us for Adam as its own launch.
+constexpr int RED_T = 32, RED_BLOCKS = (NP + RED_T - 1) / RED_T + 1;
+__device__ __forceinline__ float ordered_sum(const float *__restrict__ p, int n, int stride) {
+  constexpr int U = 19;
+  float s = 0.0f;
+  int b = 0;
+  for (; b + U <= n; b += U) {
+    float v[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = p[(size_t)(b + u) * stride];
+#pragma unroll
+    for (int u = 0; u < U; ++u) s += v[u];
+  }
+  for (; b < n; ++b) s += p[(size_t)b * stride];
+  return s;
+}
+template <bool ADAM>
+__global__ void __launch_bounds__(RED_T) k_cnn_reduce(const float *__restrict__ partial, int nblk,
+                                                      float *__restrict__ grad,
+                                                      const float *__restrict__ loss_partial,
+                                                      float *__restrict__ loss, AdamStep A,
+                                                      const unsigned *__restrict__ err) {
+  pdl_wait();
+  const int i = blockIdx.x * RED_T + threadIdx.x;
+  if (blockIdx.x == gridDim.x - 1) {
+    if (threadIdx.x == 0) *loss = ordered_sum(loss_partial, nblk, 1);
+  } else if (i < NP) {
+    const bool ok = !ADAM || *err == 0;
+    const float g = ordered_sum(partial + i, nblk, NP);
+    grad[i] = g;
+    if (ADAM && ok) adam_update(A, i, g);
+  }
 }
 
 // Inputs of the listed boxes from the solver state, on the 10^3 box-with-
@@ -941,7 +973,7 @@ static CLayout clayout(int max_samples, int max_boxes, int sms) {
   L.grad = take(4 * NP);
   L.partial = take(4 * (size_t)NP * sms);
   L.lossp = take(4 * (size_t)sms);
-  L.loss = take(4);
+  L.loss = take(4 * (size_t)max_samples);  // per minibatch of an epoch
   L.derr = take(4);
   L.X = take(2 * (size_t)NPOS * 2 * max_samples);
   L.target = take(4 * (size_t)512 * max_samples);
@@ -1070,20 +1102,44 @@ extern "C" int sm_cnn_forward(sm_cnn *c, const float *x_host, int n, float *out_
   return check_derr(c);
 }
 
-static int grad_step(sm_cnn *c, int n, const int *ids_host) {
-  CCK(cudaMemcpyAsync(c->ids, ids_host, 4 * (size_t)n, cudaMemcpyHostToDevice, c->stream));
-  int nblk = std::min(n, c->sms);
-  k_cnn_train<<<nblk, TT, train_smem(), c->stream>>>(c->X, c->target, c->ids, n, 1.0f / (512.0f * n), c->w,
-                                                     c->partial, c->lossp, c->derr);
-  k_cnn_reduce<<<(NP + 255) / 256, 256, 0, c->stream>>>(c->partial, nblk, c->grad, c->lossp, c->loss);
-  CCK(cudaGetLastError());
+static AdamStep adam_next(sm_cnn *c, float lr) {
+  ++c->adam_step;
+  return {c->w, c->m, c->v, lr, 1.0f - powf(0.9f, (float)c->adam_step), 1.0f - powf(0.999f, (float)c->adam_step)};
+}
+
+// Gradient (and loss, to loss[0]) of the n samples whose slots are listed at
+// ids (device); with lr the Adam step too.  Both kernels may be launched
+// while their predecessor ends and wait for it before they read anything.
+static int grad_step(sm_cnn *c, int n, const int *ids, float *loss, const float *lr) {
+  const int nblk = std::min(n, c->sms);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cfg.stream = c->stream;
+  cfg.gridDim = dim3(nblk);
+  cfg.blockDim = dim3(TT);
+  cfg.dynamicSmemBytes = train_smem();
+  CCK(cudaLaunchKernelEx(&cfg, k_cnn_train, (const bf16 *)c->X, (const float *)c->target, ids, n,
+                         1.0f / (512.0f * n), (const float *)c->w, c->partial, c->lossp, c->derr));
+  cfg.gridDim = dim3(RED_BLOCKS);
+  cfg.blockDim = dim3(RED_T);
+  cfg.dynamicSmemBytes = 0;
+  CCK(cudaLaunchKernelEx(&cfg, lr ? k_cnn_reduce<true> : k_cnn_reduce<false>, (const float *)c->partial, nblk, c->grad,
+                         (const float *)c->lossp, loss, lr ? adam_next(c, *lr) : AdamStep{},
+                         (const unsigned *)c->derr));
+  return SM_OK;
+}
+
+static int load_ids(sm_cnn *c, const int *ids, int n) {
+  CCK(cudaMemcpyAsync(c->ids, ids, 4 * (size_t)n, cudaMemcpyHostToDevice, c->stream));
   return SM_OK;
 }
 
 static int adam(sm_cnn *c, float lr) {
-  ++c->adam_step;
-  float c1 = 1.0f - powf(0.9f, (float)c->adam_step), c2 = 1.0f - powf(0.999f, (float)c->adam_step);
-  k_cnn_adam<<<(NP + 255) / 256, 256, 0, c->stream>>>(c->w, c->m, c->v, c->grad, lr, c1, c2);
+  k_cnn_adam<<<(NP + 255) / 256, 256, 0, c->stream>>>(adam_next(c, lr), c->grad);
   CCK(cudaGetLastError());
   return SM_OK;
 }
@@ -1099,8 +1155,8 @@ extern "C" int sm_cnn_gradient(sm_cnn *c, const float *x_host, const float *t_ho
   CCK(cudaMemcpyAsync(c->target, t_host, 4 * (size_t)512 * n, cudaMemcpyHostToDevice, c->stream));
   std::vector<int> ids(n);
   for (int i = 0; i < n; ++i) ids[i] = i;
-  int st = grad_step(c, n, ids.data());
-  if (st) return st;
+  int st = load_ids(c, ids.data(), n);
+  if (st || (st = grad_step(c, n, c->ids, c->loss, nullptr))) return st;
   CCK(cudaMemcpyAsync(grad_host, c->grad, 4 * NP, cudaMemcpyDeviceToHost, c->stream));
   float l = 0.0f;
   CCK(cudaMemcpyAsync(&l, c->loss, 4, cudaMemcpyDeviceToHost, c->stream));
@@ -1148,25 +1204,24 @@ extern "C" int sm_cnn_train(sm_cnn *c, int epochs, int batch, float lr, unsigned
   if (c->n_samples < 1) return cfail(c, SM_ESTATE, "no recorded samples");
   int n = c->n_samples;
   std::vector<int> order(n);
+  std::vector<float> losses;
   double last = 0.0;
   for (int ep = 0; ep < epochs; ++ep) {
     std::vector<std::pair<uint64_t, int>> key(n);
     for (int i = 0; i < n; ++i) key[i] = {splitmix(seed ^ ((uint64_t)ep << 32) ^ (uint64_t)i), i};
     std::sort(key.begin(), key.end());
     for (int i = 0; i < n; ++i) order[i] = key[i].second;
+    // the whole epoch is enqueued; its losses and the error word are read
+    // once at its end (after an error the later steps change nothing)
+    int st = load_ids(c, order.data(), n), nb = 0;
+    if (st) return st;
+    for (int s = 0; s < n; s += std::min(batch, n - s))
+      if ((st = grad_step(c, std::min(batch, n - s), c->ids + s, c->loss + nb++, &lr))) return st;
+    losses.resize(nb);
+    CCK(cudaMemcpyAsync(losses.data(), c->loss, 4 * (size_t)nb, cudaMemcpyDeviceToHost, c->stream));
+    if ((st = check_derr(c))) return st;
     double acc = 0.0;
-    int nb = 0;
-    for (int s = 0; s < n; s += batch) {
-      int k = std::min(batch, n - s);
-      int st = grad_step(c, k, order.data() + s);
-      if (st) return st;
-      if ((st = adam(c, lr))) return st;
-      float l = 0.0f;
-      CCK(cudaMemcpyAsync(&l, c->loss, 4, cudaMemcpyDeviceToHost, c->stream));
-      if ((st = check_derr(c))) return st;
-      acc += l;
-      ++nb;
-    }
+    for (float l : losses) acc += l;
     last = acc / nb;
   }
   if (loss) *loss = (float)last;
@@ -1186,7 +1241,7 @@ extern "C" int sm_cnn_kernel_bench(sm_cnn *c, int kind, int n, int reps, double 
   if (kind == 0 && n > c->max_boxes) return SM_EINVAL;
   std::vector<int> ids(n);
   for (int i = 0; i < n; ++i) ids[i] = i;
-  CCK(cudaMemcpyAsync(c->ids, ids.data(), 4 * (size_t)n, cudaMemcpyHostToDevice, c->stream));
+  if (int st = load_ids(c, ids.data(), n)) return st;
   auto launch = [&]() -> int {
     if (kind == 0) {
       k_cnn_forward<<<std::min(n, 4 * c->sms), CT, fwd_smem(), c->stream>>>(c->X, n, c->w, c->out, nullptr,
@@ -1194,7 +1249,7 @@ extern "C" int sm_cnn_kernel_bench(sm_cnn *c, int kind, int n, int reps, double 
       CCK(cudaGetLastError());
       return SM_OK;
     }
-    return grad_step(c, n, ids.data());
+    return grad_step(c, n, c->ids, c->loss, nullptr);
   };
   int st = launch();  // warm-up
   if (st) return st;
