@@ -245,18 +245,42 @@ __device__ __forceinline__ int W2i(int t, int co, int ci) {
   return t * 256 + (ci >> 3) * 128 + (co >> 3) * 64 + (co & 7) * 8 + (ci & 7);
 }
 
-__device__ void load_net(NetS &N, const float *__restrict__ w) {
-  for (int i = threadIdx.x; i < NW1; i += blockDim.x) N.w1[(i % 27) * 32 + i / 27] = rbf(w[O_W1 + i]);
-  for (int i = threadIdx.x; i < NW3; i += blockDim.x) N.w3[(i % 27) * 16 + i / 27] = rbf(w[O_W3 + i]);
-  for (int i = threadIdx.x; i < 27 * 256; i += blockDim.x) {
-    int t = i / 256, co = (i / 16) % 16, ci = i % 16;
-    N.w2[W2i(t, co, ci)] = __float2bfloat16_rn(w[O_W2 + (co * 16 + ci) * 27 + t]);
+// position of W2[co][ci][t] in TrainS::w2t (ci is the N index, co the K index)
+__device__ __forceinline__ int W2Ti(int t, int co, int ci) {
+  return t * 256 + (co >> 3) * 128 + (ci >> 3) * 64 + (ci & 7) * 8 + (co & 7);
+}
+
+// The parameters in the layouts of the kernels (w2t only for training),
+// read in order with all of a thread's loads in flight (18000 cycles as
+// strided reads of one layout after the other, 1500 like this).
+template <int NT>
+__device__ void load_net(NetS &N, bf16 *w2t, const float *__restrict__ w) {
+  constexpr int IT = (NP + NT - 1) / NT;
+  const int t0 = threadIdx.x;
+  float v[IT];
+#pragma unroll
+  for (int k = 0; k < IT; ++k) v[k] = t0 + k * NT < NP ? w[t0 + k * NT] : 0.0f;
+#pragma unroll
+  for (int k = 0; k < IT; ++k) {
+    const int i = t0 + k * NT;
+    if (i < O_B1) {
+      N.w1[(i % 27) * 32 + i / 27] = rbf(v[k]);
+    } else if (i < O_W2) {
+      N.b1[i - O_B1] = v[k];
+    } else if (i < O_B2) {
+      const int j = i - O_W2, t = j % 27, ci = (j / 27) % 16, co = j / 432;
+      const bf16 x = __float2bfloat16_rn(v[k]);
+      N.w2[W2i(t, co, ci)] = x;
+      if (w2t) w2t[W2Ti(t, co, ci)] = x;
+    } else if (i < O_W3) {
+      N.b2[i - O_B2] = v[k];
+    } else if (i < O_B3) {
+      const int j = i - O_W3;
+      N.w3[(j % 27) * 16 + j / 27] = rbf(v[k]);
+    } else if (i == O_B3) {
+      N.b3 = v[k];
+    }
   }
-  if (threadIdx.x < 16) {
-    N.b1[threadIdx.x] = w[O_B1 + threadIdx.x];
-    N.b2[threadIdx.x] = w[O_B2 + threadIdx.x];
-  }
-  if (threadIdx.x == 0) N.b3 = w[O_B3];
 }
 
 // the 16 channels at slot s of an array in a1's layout, as floats
@@ -290,6 +314,30 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// The same sums of N values (16 or 32) in N - 1 (+ 1) exchanges instead of 5 N:
+// every exchange halves the values a lane still carries.  Lane l returns the
+// total of value l (N = 32) or l / 2 (N = 16), with the additions of
+// warp_sum.
+template <int N>
+__device__ __forceinline__ float warp_sums(float (&v)[N]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    const int o = 16 >> k, n = N >> (k + 1);  // n values are kept
+    if (n >= 1) {
+      const bool hi = lane & o;
+#pragma unroll
+      for (int i = 0; i < n; ++i) {
+        const float send = hi ? v[i] : v[i + n], keep = hi ? v[i + n] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      }
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+    }
+  }
+  return v[0];
+}
+
 __device__ __forceinline__ uint32_t pack2(bf16 lo, bf16 hi) {
   return (uint32_t)__bfloat16_as_ushort(lo) | ((uint32_t)__bfloat16_as_ushort(hi) << 16);
 }
@@ -313,47 +361,56 @@ __device__ bool forward_box(const NetS &N, FwdS &F, TcState &tc, float *z1d, flo
                             float *a2d) {
   constexpr int VPT = 512 / NT;
   const int t = threadIdx.x;
-  // layer 1: valid 3^3 conv 2 -> 16 on CUDA cores, voxels t + r NT per
-  // thread (the 32 weights of a tap are broadcast 16-byte loads)
+  // layer 1: valid 3^3 conv 2 -> 16 on CUDA cores, four voxels (t % 128 +
+  // 128 r) and NC channels per thread.  A 16-byte load takes four cycles of
+  // the SM's shared-memory path even when it is a broadcast, so the weights
+  // of a tap are shared by four voxels: one voxel and all 16 channels per
+  // thread took 14300 cycles a box.
   {
-    int pv[VPT];
-    float acc[VPT][16];
+    constexpr int NC = 16 * 128 / NT;  // channels per thread, a warp's group c0 .. c0+NC-1
+    const int vt = t & 127, c0 = NC * (t >> 7);
+    const bf16 *xp = F.x + 2 * Pos(vt);
+    float acc[4][NC];
 #pragma unroll
-    for (int r = 0; r < VPT; ++r) {
-      pv[r] = Pos(t + r * NT);
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int co = 0; co < 16; ++co) acc[r][co] = N.b1[co];
-    }
+      for (int c = 0; c < NC; ++c) acc[r][c] = N.b1[c0 + c];
+#pragma unroll 3
     for (int tp = 0; tp < 27; ++tp) {
       const int off = Off(tp);
-      float2 xv[VPT];
+      float2 xv[4];
 #pragma unroll
-      for (int r = 0; r < VPT; ++r)
-        xv[r] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(F.x + 2 * (pv[r] + off)));
-      const float4 *wt = reinterpret_cast<const float4 *>(N.w1 + 32 * tp);
+      for (int r = 0; r < 4; ++r)
+        xv[r] = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(xp + 2 * (200 * r + off)));
+      const float4 *wt = reinterpret_cast<const float4 *>(N.w1 + 32 * tp + 2 * c0);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const float4 wv = wt[k];  // W1[2k][0], W1[2k][1], W1[2k+1][0], W1[2k+1][1]
+      for (int k = 0; k < NC / 2; ++k) {
+        const float4 wv = wt[k];  // W1[c][0], W1[c][1], W1[c+1][0], W1[c+1][1], c = c0 + 2k
 #pragma unroll
-        for (int r = 0; r < VPT; ++r) {
+        for (int r = 0; r < 4; ++r) {
           acc[r][2 * k] += wv.x * xv[r].x + wv.y * xv[r].y;
           acc[r][2 * k + 1] += wv.z * xv[r].x + wv.w * xv[r].y;
         }
       }
     }
 #pragma unroll
-    for (int r = 0; r < VPT; ++r) {
-      const int v = t + r * NT;
-      bf16 *a1v = F.a1 + 8 * A1S((v & 7) + 1, 0, ((v >> 3) & 7) + 1 + 10 * ((v >> 6) + 1));
+    for (int r = 0; r < 4; ++r) {
+      const int v = vt + 128 * r;
+      uint32_t pk[NC / 2];
 #pragma unroll
-      for (int co = 0; co < 16; ++co) {
-        bf16 a = __float2bfloat16_rn(fmaxf(acc[r][co], 0.0f));
-        a1v[co < 8 ? co : 80 + (co - 8)] = a;
+      for (int c = 0; c < NC; c += 2) {
+        const bf16 a0 = __float2bfloat16_rn(fmaxf(acc[r][c], 0.0f)), a1 = __float2bfloat16_rn(fmaxf(acc[r][c + 1], 0.0f));
+        pk[c >> 1] = pack2(a0, a1);
         if (z1d) {
-          z1d[co * 512 + v] = acc[r][co];
-          a1d[co * 512 + v] = bf(a);
+          z1d[(c0 + c) * 512 + v] = acc[r][c];
+          z1d[(c0 + c + 1) * 512 + v] = acc[r][c + 1];
+          a1d[(c0 + c) * 512 + v] = bf(a0);
+          a1d[(c0 + c + 1) * 512 + v] = bf(a1);
         }
       }
+      bf16 *a1v = F.a1 + 8 * (VS(v) + 10 * (c0 >> 3)) + (c0 & 7);
+#pragma unroll
+      for (int c = 0; c < NC / 4; ++c) reinterpret_cast<uint2 *>(a1v)[c] = make_uint2(pk[2 * c], pk[2 * c + 1]);
     }
   }
   // the tensor cores read a1 (and the weights) through the async proxy
@@ -366,10 +423,11 @@ __device__ bool forward_box(const NetS &N, FwdS &F, TcState &tc, float *z1d, flo
     tc_fence_after();
     const int j = t >> 5, R0 = 11 + 16 * j;
     const uint32_t a0 = smem_u32(F.a1), b0 = smem_u32(N.w2);
+    const uint64_t ad = tc_desc(a0 + 16 * A1S(0, 0, R0 - 11), 160, 320), bd = tc_desc(b0, 256, 128);
+#pragma unroll
     for (int tp = 0; tp < 27; ++tp) {
       const int dx = tp % 3 - 1, dy = (tp / 3) % 3 - 1, dz = tp / 9 - 1;
-      tc_mma(tc.taddr + 16 * j, tc_desc(a0 + 16 * A1S(1 + dx, 0, R0 + dy + 10 * dz), 160, 320),
-             tc_desc(b0 + 512 * tp, 256, 128), TC_IDESC, tp > 0);
+      tc_mma(tc.taddr + 16 * j, ad + A1S(1 + dx, 0, 11 + dy + 10 * dz), bd + 32 * tp, TC_IDESC, tp > 0);
     }
     tc_commit(tc.mbar);
   }
@@ -451,7 +509,7 @@ __global__ void __launch_bounds__(CT) k_cnn_forward(const bf16 *__restrict__ X, 
   FwdS &F = *reinterpret_cast<FwdS *>(smraw + ((sizeof(NetS) + 127) & ~(size_t)127));
   TcState tc;
   tc_begin(tc, &mbar, &tslot, err, FWD_COLS);
-  load_net(N, w);
+  load_net<CT>(N, nullptr, w);
   zero_acts(F);
   __syncthreads();
   for (int b = blockIdx.x; b < n; b += gridDim.x) {
@@ -475,7 +533,7 @@ __device__ __forceinline__ int g_to_param(int i) { return i < G_B2 ? i : i + NW2
 struct TrainS {
   bf16 w2t[27 * 256];     // backward-data B operand: [t][co/8][ci/8][ci%8][co%8]
   bf16 d2[D2_SLOTS * 8];  // dL/dz2 as three BF16 terms, zero outside the box interior
-  float g3[512];          // dL/d out
+  float g3[NPOS];         // dL/d out on the 10^3 positions, zero outside the box interior
   float grad[NG];
   float part[TT];         // per-thread partial sums of the bias gradients
   float red[TT / 32];
@@ -486,13 +544,8 @@ static_assert(offsetof(FwdS, a1) % 16 == 0 && offsetof(TrainS, d2) % 16 == 0 && 
 static_assert(((sizeof(NetS) + 127) & ~(size_t)127) + ((sizeof(FwdS) + 127) & ~(size_t)127) + sizeof(TrainS) <=
                   227 * 1024,
               "training shared memory");
-static_assert(sizeof(NetS) == 19140 && sizeof(FwdS) == 71456 && sizeof(TrainS) == 121220,
+static_assert(sizeof(NetS) == 19140 && sizeof(FwdS) == 71456 && sizeof(TrainS) == 123172,
               "layout the operand ranges were checked against");
-
-// position of W2[co][ci][t] in TrainS::w2t (ci is the N index, co the K index)
-__device__ __forceinline__ int W2Ti(int t, int co, int ci) {
-  return t * 256 + (co >> 3) * 128 + (ci >> 3) * 64 + (ci & 7) * 8 + (co & 7);
-}
 
 __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X, const float *__restrict__ target,
                                                   const int *__restrict__ ids, int n, float inv_count,
@@ -510,15 +563,12 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
   // what needs nothing of the launch before it runs while that one ends
   zero_acts(F);
   zero16(S.d2, sizeof(S.d2));
+  for (int i = t; i < NPOS; i += TT) S.g3[i] = 0.0f;
   for (int i = t; i < NG; i += TT) S.grad[i] = 0.0f;
   pdl_wait();
   if (*err) return;  // a wait of an earlier pass ran out: the results are void
   tc_begin(tc, &mbar, &tslot, err, TRAIN_COLS);
-  load_net(N, w);
-  for (int i = t; i < 27 * 256; i += TT) {
-    const int tp = i / 256, co = (i / 16) % 16, ci = i % 16;
-    S.w2t[W2Ti(tp, co, ci)] = __float2bfloat16_rn(w[O_W2 + (co * 16 + ci) * 27 + tp]);
-  }
+  load_net<TT>(N, S.w2t, w);
   float my_loss = 0.0f;
   bool wg_acc = false;  // the backward-weight accumulators hold a sum
   __syncthreads();
@@ -530,92 +580,70 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
     for (int v = t; v < 512; v += TT) {
       const float e = F.out[v] - tg[v];
       my_loss += e * e * inv_count;
-      S.g3[v] = 2.0f * inv_count * e;
+      S.g3[Pos(v)] = 2.0f * inv_count * e;
     }
     __syncthreads();
-    // layer 3 weights: warp w takes taps w, w + 8, ...; lane l the voxels
-    // l + 32k, whose sums the warp then adds (fixed order); bias: warp 7
-    for (int tp = warp; tp < 27; tp += TT / 32) {
-      const int so = SOff(tp);
-      float acc[16];
-#pragma unroll
-      for (int ci = 0; ci < 16; ++ci) acc[ci] = 0.0f;
-      for (int v = lane; v < 512; v += 32) {
-        float a[16];
-        row16(F.a2, VS(v) + so, a);
-        const float g = S.g3[v];
-#pragma unroll
-        for (int ci = 0; ci < 16; ++ci) acc[ci] += a[ci] * g;
-      }
-#pragma unroll
-      for (int ci = 0; ci < 16; ++ci) acc[ci] = warp_sum(acc[ci]);
-      if (lane == 0)
-#pragma unroll
-        for (int ci = 0; ci < 16; ++ci) S.grad[G_W3 + ci * 27 + tp] += acc[ci];
-    }
-    if (warp == TT / 32 - 1) {
-      float acc = 0.0f;
-      for (int v = lane; v < 512; v += 32) acc += S.g3[v];
-      acc = warp_sum(acc);
-      if (lane == 0) S.grad[G_B3] += acc;
-    }
-    // dL/dz2[u][c] = relu'(a2[u][c]) sum_t W3[c][t] g3[u - d_t] for voxels
-    // t + r TT, stored as three BF16 terms h0 + h1 + h2 equal to the
-    // FP32 value (each remainder is exact in FP32 and the last has at most 8
-    // significant bits)
+    // dL/dz2[u][c] = relu'(a2[u][c]) sum_t W3[c][t] g3[u - d_t], stored as
+    // three BF16 terms h0 + h1 + h2 equal to the FP32 value (each remainder
+    // is exact in FP32 and the last has at most 8 significant bits): four
+    // voxels (t % 128 + 128 r) and four channels per thread, the weights of
+    // a tap shared by the voxels (9100 cycles a box with all 16 channels of
+    // one voxel per thread)
     {
+      const int vt = t & 127, c0 = 4 * (t >> 7), pu = Pos(vt);
+      float acc[4][4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0.0f;
+#pragma unroll 3
+      for (int tp = 0; tp < 27; ++tp) {
+        const float4 wv = *reinterpret_cast<const float4 *>(N.w3 + 16 * tp + c0);
+        const float *g = S.g3 + pu - Off(tp);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const float gv = g[200 * r];
+          acc[r][0] += wv.x * gv;
+          acc[r][1] += wv.y * gv;
+          acc[r][2] += wv.z * gv;
+          acc[r][3] += wv.w * gv;
+        }
+      }
       float bsum[16];
 #pragma unroll
-      for (int c = 0; c < 16; ++c) bsum[c] = 0.0f;
-#pragma unroll 1
-      for (int r = 0; r < 512 / TT; ++r) {
-        const int u = t + r * TT, ux = u & 7, uy = (u >> 3) & 7, uz = u >> 6;
-        float acc[16];
+      for (int r = 0; r < 4; ++r) {
+        const int u = vt + 128 * r, ux = u & 7, R = ((u >> 3) & 7) + 1 + 10 * ((u >> 6) + 1), h = c0 >> 3;
+        const uint2 aw = *reinterpret_cast<const uint2 *>(F.a2 + 8 * (VS(u) + 10 * h) + (c0 & 7));
+        const uint32_t av[2] = {aw.x, aw.y};
+        uint32_t t0[2], t1[2], t2[2];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) acc[c] = 0.0f;
-        for (int tp = 0; tp < 27; ++tp) {
-          const int vx = ux - (tp % 3 - 1), vy = uy - ((tp / 3) % 3 - 1), vz = uz - (tp / 9 - 1);
-          if (vx < 0 || vx > 7 || vy < 0 || vy > 7 || vz < 0 || vz > 7) continue;
-          const float g = S.g3[vx + 8 * vy + 64 * vz];
-          float wv[16];
-          w16(N.w3 + 16 * tp, wv);
+        for (int k = 0; k < 2; ++k) {
+          const float2 a2v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&av[k]));
+          bf16 hv[3][2];
 #pragma unroll
-          for (int c = 0; c < 16; ++c) acc[c] += wv[c] * g;
-        }
-        float a2v[16];
-        row16(F.a2, VS(u), a2v);
-        const int R = (uy + 1) + 10 * (uz + 1);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          uint32_t t0[4], t1[4], t2[4];
-#pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            bf16 hv[3][2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              const int c = 8 * h + 2 * k + e;
-              const float d = a2v[c] > 0.0f ? acc[c] : 0.0f;
-              bsum[c] += d;
-              hv[0][e] = __float2bfloat16_rn(d);
-              const float r1 = d - bf(hv[0][e]);
-              hv[1][e] = __float2bfloat16_rn(r1);
-              hv[2][e] = __float2bfloat16_rn(r1 - bf(hv[1][e]));
-            }
-            t0[k] = pack2(hv[0][0], hv[0][1]);
-            t1[k] = pack2(hv[1][0], hv[1][1]);
-            t2[k] = pack2(hv[2][0], hv[2][1]);
+          for (int e = 0; e < 2; ++e) {
+            const float d = (e ? a2v.y : a2v.x) > 0.0f ? acc[r][2 * k + e] : 0.0f;
+            bsum[4 * r + 2 * k + e] = d;
+            hv[0][e] = __float2bfloat16_rn(d);
+            const float r1 = d - bf(hv[0][e]);
+            hv[1][e] = __float2bfloat16_rn(r1);
+            hv[2][e] = __float2bfloat16_rn(r1 - bf(hv[1][e]));
           }
-          *reinterpret_cast<uint4 *>(S.d2 + 8 * D2S(ux + 1, 0, h, R)) = make_uint4(t0[0], t0[1], t0[2], t0[3]);
-          *reinterpret_cast<uint4 *>(S.d2 + 8 * D2S(ux + 1, 1, h, R)) = make_uint4(t1[0], t1[1], t1[2], t1[3]);
-          *reinterpret_cast<uint4 *>(S.d2 + 8 * D2S(ux + 1, 2, h, R)) = make_uint4(t2[0], t2[1], t2[2], t2[3]);
+          t0[k] = pack2(hv[0][0], hv[0][1]);
+          t1[k] = pack2(hv[1][0], hv[1][1]);
+          t2[k] = pack2(hv[2][0], hv[2][1]);
         }
+        bf16 *d = S.d2 + 8 * D2S(ux + 1, 0, h, R) + (c0 & 7);
+        *reinterpret_cast<uint2 *>(d) = make_uint2(t0[0], t0[1]);
+        *reinterpret_cast<uint2 *>(d + 8 * 20) = make_uint2(t1[0], t1[1]);
+        *reinterpret_cast<uint2 *>(d + 8 * 40) = make_uint2(t2[0], t2[1]);
       }
-      // layer-2 bias: per warp, then the warps in order (below)
-#pragma unroll
-      for (int c = 0; c < 16; ++c) bsum[c] = warp_sum(bsum[c]);
-      if (lane == 0)
-#pragma unroll
-        for (int c = 0; c < 16; ++c) S.part[16 * warp + c] = bsum[c];
+      // layer-2 bias: sums of 32 voxels, added in voxel order below
+      const float b = warp_sums(bsum);
+      if (!(lane & 1)) {  // value lane / 2 = 4 r + c: voxels 32 (warp % 4 + 4 r) ..
+        const int i = lane >> 1;
+        S.part[16 * ((warp & 3) + 4 * (i >> 2)) + c0 + (i & 3)] = b;
+      }
     }
     async_proxy_fence();
     tc_fence_before();
@@ -627,24 +655,55 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
       tc_fence_after();
       const int j = t >> 5, R0 = 11 + 16 * j;
       const uint32_t a0 = smem_u32(F.a1), d0 = smem_u32(S.d2), b0 = smem_u32(S.w2t);
+      const uint64_t dd = tc_desc(d0 + 16 * D2S(0, 0, 0, R0 - 11), 160, 960), bd = tc_desc(b0, 256, 128);
+#pragma unroll
       for (int tp = 0; tp < 27; ++tp) {
         const int dx = tp % 3 - 1, dy = (tp / 3) % 3 - 1, dz = tp / 9 - 1;
-        const uint64_t bd = tc_desc(b0 + 512 * tp, 256, 128);
+#pragma unroll
         for (int m = 0; m < 3; ++m)
-          tc_mma(tc.taddr + 16 * j, tc_desc(d0 + 16 * D2S(1 - dx, m, 0, R0 - dy - 10 * dz), 160, 960), bd,
-                 TC_IDESC, tp > 0 || m > 0);
+          tc_mma(tc.taddr + 16 * j, dd + D2S(1 - dx, m, 0, 11 - dy - 10 * dz), bd + 32 * tp, TC_IDESC,
+                 tp > 0 || m > 0);
       }
+      const uint64_t db = tc_desc(d0, 960, 160);
       for (int c = j; c < 9; c += TC_TILES) {
         const int dy = c % 3 - 1, dz = c / 3 - 1;
+        const uint64_t ad = tc_desc(a0 + 16 * A1S(0, 0, 11 + dy + 10 * dz), 320, 16);
+#pragma unroll
         for (int p = 0; p < 32; ++p) {
           const int R = (2 * (p & 3) + 1) + 10 * ((p >> 2) + 1);  // x rows y = 2 (p % 4), +1 of plane z = p / 4
-          tc_mma(tc.taddr + WG_COL0 + 48 * c, tc_desc(a0 + 16 * A1S(0, 0, R + dy + 10 * dz), 320, 16),
-                 tc_desc(d0 + 16 * D2S(1, 0, 0, R), 960, 160), TC_IDESC_WG, wg_acc || p > 0);
+          tc_mma(tc.taddr + WG_COL0 + 48 * c, ad + A1S(0, 0, R - 11), db + D2S(1, 0, 0, R), TC_IDESC_WG,
+                 wg_acc || p > 0);
         }
       }
       tc_commit(tc.mbar);
     }
     wg_acc = true;
+    __syncwarp();
+    // layer 3 weights, while the tensor cores work: warp w takes taps w and
+    // w + 16, lane l the voxels l + 32k, whose sums the warp then adds (fixed
+    // order); bias: the last warp
+    for (int tp = warp; tp < 27; tp += TT / 32) {
+      const int so = SOff(tp);
+      float acc[16];
+#pragma unroll
+      for (int ci = 0; ci < 16; ++ci) acc[ci] = 0.0f;
+#pragma unroll 4
+      for (int v = lane; v < 512; v += 32) {
+        float a[16];
+        row16(F.a2, VS(v) + so, a);
+        const float g = S.g3[Pos(v)];
+#pragma unroll
+        for (int ci = 0; ci < 16; ++ci) acc[ci] += a[ci] * g;
+      }
+      const float sum = warp_sums(acc);
+      if (!(lane & 1)) S.grad[G_W3 + (lane >> 1) * 27 + tp] += sum;
+    }
+    if (warp == TT / 32 - 1) {
+      float acc = 0.0f;
+      for (int v = lane; v < 512; v += 32) acc += S.g3[Pos(v)];
+      acc = warp_sum(acc);
+      if (lane == 0) S.grad[G_B3] += acc;
+    }
     if (t < 16) {
       float acc = 0.0f;
       for (int i = 0; i < TT / 32; ++i) acc += S.part[16 * i + t];
@@ -669,8 +728,10 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
     }
     tc_fence_before();
     __syncthreads();
-    // layer 1 weights (valid conv on the 10^3 input): warp w takes taps
-    // w, w + 8, ...; lane l the voxels l + 32k, whose sums the warp adds
+    // layer 1 weights (valid conv on the 10^3 input): warp w takes taps w
+    // and w + 16, lane l the voxels l + 32k, whose sums the warp adds (16300
+    // cycles a box with five exchanges a sum, 9800 with one; both taps at
+    // once, to read dL/dz1 once, took 26000)
     {
       const float *d1 = reinterpret_cast<const float *>(F.a2);
       for (int tp = warp; tp < 27; tp += TT / 32) {
@@ -678,22 +739,18 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
         float acc[32];  // [co][ci]
 #pragma unroll
         for (int i = 0; i < 32; ++i) acc[i] = 0.0f;
+#pragma unroll 2
         for (int v = lane; v < 512; v += 32) {
           const float2 xv = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(F.x + 2 * (Pos(v) + off)));
-          float dv[16];
-#pragma unroll
-          for (int co = 0; co < 16; ++co) dv[co] = d1[co * 512 + v];
 #pragma unroll
           for (int co = 0; co < 16; ++co) {
-            acc[2 * co] += xv.x * dv[co];
-            acc[2 * co + 1] += xv.y * dv[co];
+            const float dv = d1[co * 512 + v];
+            acc[2 * co] += xv.x * dv;
+            acc[2 * co + 1] += xv.y * dv;
           }
         }
-#pragma unroll
-        for (int i = 0; i < 32; ++i) acc[i] = warp_sum(acc[i]);
-        if (lane == 0)
-#pragma unroll
-          for (int i = 0; i < 32; ++i) S.grad[G_W1 + i * 27 + tp] += acc[i];
+        const float sum = warp_sums(acc);
+        S.grad[G_W1 + lane * 27 + tp] += sum;
       }
       // layer-1 bias: thread t sums channel t / G over the voxels t % G +
       // G i (G = TT / 16), then the G partial sums of a channel in order
@@ -717,17 +774,17 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
   }
   float *dst = partial + (size_t)blockIdx.x * NP;
   // W2 gradient: the three terms' columns of the useful rows of each
-  // backward-weight accumulator (lanes 0-23 and 80-103: warps 0, 2, 3)
+  // backward-weight accumulator (lanes 0-23 and 80-103: the warps of quarters 0, 2, 3)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   {
     const int q = warp & 3;
-    if (warp < 4 && q != 1) {
+    if (q != 1) {
       const int L = 32 * q + lane, g = L >> 3, c8 = L & 7;
       const bool use = g <= 2 || (g >= 10 && g <= 12);
       const int ci = g <= 2 ? c8 : 8 + c8, dx = g <= 2 ? g - 1 : g - 11;
-      for (int c = 0; c < 9; ++c) {
+      for (int c = warp >> 2; c < 9; c += TT / 128) {
         float sum[16];
 #pragma unroll
         for (int co = 0; co < 16; ++co) sum[co] = 0.0f;
