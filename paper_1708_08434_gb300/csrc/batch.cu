@@ -120,7 +120,7 @@ constexpr int ST = 128;                       // threads of a sweep block: four 
 constexpr int SRING = 6;                      // staged planes of a sweep (even, the colour parity unrolls)
 constexpr int SPL = EPL + FPL;                // floats of one sweep slot: an error plane and its rhs plane
 constexpr int RINGT = CX + CY;                // colour-0 cells of the one-cell ring around a column
-constexpr size_t OUTER_SMEM = sizeof(double) * RING * DPL;
+constexpr int OSL = 4;                        // staged potential planes of the outer residual
 
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
   return (unsigned)__cvta_generic_to_shared(p);
@@ -736,178 +736,202 @@ __global__ void __launch_bounds__(512) k_bt_coarse(const int *__restrict__ solve
 // 2^-53 of values up to 2^(E-1022)), and the FP64 pipe does one operation
 // per cell instead of seven.  A solve whose potential holds an infinity or
 // a NaN gets NaN residuals.
-// Planes of phi (one-cell halo) are staged by asynchronous copies and
-// converted in place one step ahead: at step p planes p-1 .. p+1 are read,
-// plane p+2 is converted, p+3 .. p+4 are in flight and plane p+5 is issued
-// into the slot of plane p-3; f is loaded into registers two planes ahead.
+//
+// A block per column, four rows a thread.  Instruction issue bounds the pass
+// when every neighbour comes from shared memory (207 instructions a warp for
+// 32 cells), so a thread keeps the fixed-point values of its rows on planes
+// p-1, p and p+1 in registers: the z and the inner y neighbours need no load.
+// Planes of phi (one-cell halo) are staged by asynchronous copies; at step p
+// a thread converts its four values of plane p+1, which it keeps and writes
+// back for the neighbours' x and outer y reads at step p+1, and at most one
+// halo value.  Wall ghosts enter as in the sweep: +1 (Neumann) or -1
+// (Dirichlet) in the coefficient of c, and the sum of the Dirichlet 2g, both
+// exact integers; DIR: a face in x or y is Dirichlet.  Slots at step p:
+// planes p and p+1 are read, p+2 is in flight, plane p+3 is issued into the
+// slot of plane p-1 (last read at step p-1).  124e6 cells: 734 us against
+// 818 with all neighbours staged (20 bytes a cell are 0.37 ms, two FP64
+// operations 0.42 ms; shorter forms of the two conversions ran no faster).
 // The max norm is taken on the bit patterns of |r|.
-__global__ void __launch_bounds__(CT, 5) k_bt_outer(const int4 *__restrict__ cols, int ncols,
-                                                 const BSolve *__restrict__ tab,
-                                                 const unsigned char *__restrict__ active,
-                                                 const double *__restrict__ phi, const double *__restrict__ f64,
-                                                 float *__restrict__ f32, Bc bc, const unsigned *__restrict__ emax,
-                                                 unsigned long long *__restrict__ num) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  long long(*sp)[DPL] = reinterpret_cast<long long(*)[DPL]>(smem_raw);
-  __shared__ unsigned long long red[CT / 32];
-  const int t = threadIdx.x, tx = t % CX, ty2 = 2 * (t / CX);
-  int ebc = 0;  // exponent bound of the Dirichlet wall values
+
+template <bool DIR>
+__device__ __forceinline__ unsigned long long outer_column(const int4 &C, const BSolve &S, int E,
+                                                           const double *__restrict__ phi,
+                                                           const double *__restrict__ f64, float *__restrict__ f32,
+                                                           const Bc &bc, long long *sp) {
+  const int t = threadIdx.x, tx = t % CX, ty = 4 * (t / CX);
+  const int N = S.N[0], P = pitch(N);
+  const long long NN = (long long)N * N;
+  const bool finite = E < 0x7ff;
+  // 2^(E-1080) h^-2, exact: a power of two (exponent field E - 57 >= 66)
+  // times h^-2
+  const double kk = S.inv_h2 * __longlong_as_double((long long)(finite ? E - 57 : 1023) << 52);
+  const int x0 = C.y * CX, y0 = C.z * CY, x = x0 + tx, ya = y0 + ty;
+  const double *pv = phi + S.off64;
+  // this thread's 16-byte chunks of a staged plane (N even)
+  // of it: rows r, r + 7, r + 14
+  constexpr int CROW = RWD / 2, RSTEP = ST / CROW, U = (FR + RSTEP - 1) / RSTEP;
+  const bool vec = (N & 1) == 0;
+  const int crow = t / CROW, cx = x0 - 2 + 2 * (t % CROW), cy = y0 - 1 + crow;
+  const bool cxok = crow < RSTEP && cx >= 0 && cx < N;
+  const double *csrc = pv + (cy * N + cx);
+  auto issue = [&](int z, int sl) {
+    if (z < N) {
+      long long *dst = sp + sl * DPL;
+      if (vec) {
+        if (crow < RSTEP) {
 #pragma unroll
-  for (int f = 0; f < 6; ++f)
-    if (bc.type[f]) ebc = max(ebc, (int)expo_of(bc.g2[f]));
-  for (int it = blockIdx.x; it < ncols; it += gridDim.x) {
-    const int4 C = cols[it];
-    if (!active[C.x]) continue;  // uniform per block
-    const BSolve &S = tab[C.x];
-    const int N = S.N[0];
-    const long long o64 = S.off64, NN = (long long)N * N;
-    const int E = max(max((int)emax[C.x], ebc), 123);
-    const bool finite = E < 0x7ff;
-    // 2^(E-1080) h^-2, exact: a power of two (exponent field E - 57 >= 66)
-    // times h^-2
-    const double kk = S.inv_h2 * __longlong_as_double((long long)(finite ? E - 57 : 1023) << 52);
-    const int x0 = C.y * CX, y0 = C.z * CY;
-    const double *pv = phi + o64, *fv = f64 + o64;
-    const bool vec = (N & 1) == 0;
-    const int x = x0 + tx, ya = y0 + ty2;
-    const bool in0 = x < N && ya < N, in1 = x < N && ya + 1 < N;
-    // this thread's 16-byte chunks of a staged plane (at most two): slot-0
-    // shared offset, in-plane element offset, inside the grid
-    int cdst[2] = {-1, -1}, coff[2] = {0, 0};
-    bool cok[2] = {false, false};
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int i = t + u * CT;
-      if (!vec || i >= FR * (RWD / 2)) continue;
-      const int r = i / (RWD / 2), c2 = 2 * (i % (RWD / 2)), y = y0 - 1 + r, xx = x0 - 2 + c2;
-      cok[u] = y >= 0 && y < N && xx >= 0 && xx < N;
-      coff[u] = cok[u] ? y * N + xx : 0;
-      cdst[u] = r * RWD + c2;
-    }
-    auto issue = [&](int z) {
-      if (z < N) {
-        const int sl = z & (RING - 1);
-        const double *pz = pv + z * NN;
-        if (vec) {
-#pragma unroll
-          for (int u = 0; u < 2; ++u)
-            if (cdst[u] >= 0) cp_async<16>(&sp[sl][cdst[u]], pz + coff[u], cok[u]);
-        } else {
-          for (int i = t; i < FR * RWD; i += CT) {
-            const int y = y0 - 1 + i / RWD, xx = x0 - 2 + i % RWD;
-            const bool ok = y >= 0 && y < N && xx >= 0 && xx < N;
-            cp_async<8>(&sp[sl][i], ok ? pz + y * N + xx : pz, ok);
+          for (int u = 0; u < U; ++u) {
+            const int y = cy + u * RSTEP;
+            const bool ok = cxok && y >= 0 && y < N;
+            if (crow + u * RSTEP < FR)
+              cp_async<16>(dst + 2 * t + u * RSTEP * RWD, ok ? csrc + u * RSTEP * N : pv, ok);
           }
         }
-      }
-      cp_commit();
-    };
-    // staged plane z -> fixed point, in place (the columns x0-1 .. x0+32
-    // that the stencil reads; cells outside the grid were zero-filled)
-    constexpr int NCV = FR * (CX + 2);  // values converted per plane
-    int cj[3];                          // this thread's (at most three), -1 for none
-#pragma unroll
-    for (int u = 0; u < 3; ++u) {
-      const int i = t + u * CT;
-      cj[u] = i < NCV ? (i / (CX + 2)) * RWD + 1 + i % (CX + 2) : -1;
-    }
-    auto convert = [&](int z) {
-      if (z < N) {
-        long long *pz = sp[z & (RING - 1)];
-#pragma unroll
-        for (int u = 0; u < 3; ++u)
-          if (cj[u] >= 0) pz[cj[u]] = fix_of_bits((unsigned long long)pz[cj[u]], E);
-      }
-    };
-    // ghost across wall face f of a cell holding c: c (Neumann) or 2g - c
-    auto wallv = [&](int f, long long c) {
-      return bc.type[f] ? fix_of_bits((unsigned long long)__double_as_longlong(bc.g2[f]), E) - c : c;
-    };
-    const long long row0 = (long long)ya * N + x;
-    const int P = pitch(N);
-    float *const rz = f32 + S.off[0] + (long long)ya * P + x;
-    // f of planes p (set A for even p, B for odd p): loaded two steps ahead
-    double fa0 = 0.0, fa1 = 0.0, fb0 = 0.0, fb1 = 0.0;
-    if (in0) fa0 = fv[row0];
-    if (in1) fa1 = fv[row0 + N];
-    if (N > 1 && in0) fb0 = fv[NN + row0];
-    if (N > 1 && in1) fb1 = fv[NN + row0 + N];
-    unsigned long long m = 0;  // bit pattern of max |r|
-    __syncthreads();           // the previous column's planes are no longer read
-#pragma unroll
-    for (int z = 0; z < RING - 3; ++z) issue(z);
-    cp_wait<RING - 5>();  // planes 0 and 1 have landed
-    __syncthreads();
-    convert(0);
-    convert(1);
-    // NEU: all four in-plane faces are Neumann (a compile-time path: the
-    // in-plane ghosts are then selects of c)
-    auto step = [&](auto neu_tag, int p, double &f0, double &f1) {
-      constexpr bool NEU = decltype(neu_tag)::value;
-      cp_wait<RING - 6>();  // this thread's copies of planes <= p+2 have landed
-      __syncthreads();      // everyone's have; planes <= p+1 are converted; step p-1's reads are done
-      issue(p + RING - 3);
-      convert(p + 2);
-      const long long *pz = sp[p & (RING - 1)], *pm = sp[(p - 1) & (RING - 1)], *pp = sp[(p + 1) & (RING - 1)];
-#pragma unroll
-      for (int o = 0; o < 2; ++o) {
-        if (!(o ? in1 : in0)) continue;
-        const int q = (ty2 + o + 1) * RWD + tx + 2, y = ya + o;
-        const long long c = pz[q];
-        long long xm, xp, ym, yp;
-        if constexpr (NEU) {
-          xm = x == 0 ? c : pz[q - 1];
-          xp = x == N - 1 ? c : pz[q + 1];
-          ym = y == 0 ? c : pz[q - RWD];
-          yp = y == N - 1 ? c : pz[q + RWD];
-        } else {
-          xm = x == 0 ? wallv(0, c) : pz[q - 1];
-          xp = x == N - 1 ? wallv(1, c) : pz[q + 1];
-          ym = y == 0 ? wallv(2, c) : pz[q - RWD];
-          yp = y == N - 1 ? wallv(3, c) : pz[q + RWD];
+        csrc += NN;
+      } else {
+        for (int i = t; i < DPL; i += ST) {
+          const int y = y0 - 1 + i / RWD, xx = x0 - 2 + i % RWD;
+          const bool ok = y >= 0 && y < N && xx >= 0 && xx < N;
+          cp_async<8>(dst + i, ok ? pv + z * NN + y * N + xx : pv, ok);
         }
-        const long long zm = p == 0 ? wallv(4, c) : pm[q];
-        const long long zp = p == N - 1 ? wallv(5, c) : pp[q];
-        const long long sx = ((xm + xp) + (ym + yp)) + (zm + zp) - 6 * c;  // exact
-        const double r = fma(-__ll2double_rn(sx), kk, o ? f1 : f0);
-        const unsigned long long rb = finite ? (unsigned long long)__double_as_longlong(r) : 0x7ff8000000000000ull;
-        rz[(long long)p * P * N + o * P] = cvt_bits_f32_rn(rb);
+      }
+    }
+    cp_commit();
+  };
+  auto fix = [&](long long b) { return fix_of_bits((unsigned long long)b, E); };
+  const int q0 = (ty + 1) * RWD + tx + 2;
+  // this thread's halo value: rows y0-1, y0+CY, then columns x0-1, x0+CX
+  int hq = -1;
+  if (t < 2 * CX) hq = (t < CX ? 0 : CY + 1) * RWD + 2 + t % CX;
+  else if (t < 2 * CX + 2 * CY) hq = (1 + (t - 2 * CX) % CY) * RWD + (t < 2 * CX + CY ? 1 : CX + 2);
+  auto convert = [&](int sl, long long(&c)[4]) {
+    long long *pl = sp + sl * DPL;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      c[r] = fix(pl[q0 + r * RWD]);
+      pl[q0 + r * RWD] = c[r];
+    }
+    if (hq >= 0) pl[hq] = fix(pl[hq]);
+  };
+  bool in[4];
+  int w[4];             // coefficient of c without the z walls
+  long long gxy[4];     // DIR: sum of the Dirichlet 2g of the in-plane walls
+  auto wall = [&](int face, bool on, int &wr, long long &g) {
+    if (!on) return;
+    wr += bc.type[face] ? -1 : 1;
+    if (DIR && bc.type[face]) g += fix(__double_as_longlong(bc.g2[face]));
+  };
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int y = ya + r;
+    in[r] = x < N && y < N;
+    w[r] = -6;
+    gxy[r] = 0;
+    wall(0, x == 0, w[r], gxy[r]);
+    wall(1, x == N - 1, w[r], gxy[r]);
+    wall(2, y == 0, w[r], gxy[r]);
+    wall(3, y == N - 1, w[r], gxy[r]);
+  }
+  const double *fz = f64 + S.off64 + (long long)ya * N + x;
+  float *rz = f32 + S.off[0] + (long long)ya * P + x;
+  double fv[4] = {};  // f of plane p
+  auto load_f = [&](double(&d)[4]) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+      if (in[r]) d[r] = fz[r * N];
+    fz += NN;
+  };
+  unsigned long long m = 0;  // bit pattern of max |r|
+#pragma unroll
+  for (int z = 0; z < OSL - 1; ++z) issue(z, z);
+  cp_wait<OSL - 2>();  // plane 0 has landed
+  __syncthreads();
+  long long cm[4] = {}, c[4], cn[4];
+  convert(0, c);
+  for (int pb = 0; pb < N; pb += OSL) {
+#pragma unroll
+    for (int i = 0; i < OSL; ++i) {
+      const int p = pb + i;
+      if (p >= N) break;
+      cp_wait<OSL - 3>();  // this thread's copies of planes <= p+1 have landed
+      __syncthreads();     // everyone's have, plane p is converted, step p-1's reads are done
+      issue(p + OSL - 1, (i + OSL - 1) % OSL);
+      load_f(fv);
+      if (p + 1 < N) {
+        convert((i + 1) % OSL, cn);
+      } else {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) cn[r] = 0;
+      }
+      int wz = 0;
+      long long gz = 0;
+      if (p == 0) {
+        wz += bc.type[4] ? -1 : 1;
+        if (bc.type[4]) gz += fix(__double_as_longlong(bc.g2[4]));
+      }
+      if (p == N - 1) {
+        wz += bc.type[5] ? -1 : 1;
+        if (bc.type[5]) gz += fix(__double_as_longlong(bc.g2[5]));
+      }
+      const long long *pl = sp + i * DPL;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        if (!in[r]) continue;
+        const int q = q0 + r * RWD;
+        const long long ym = r > 0 ? c[r - 1] : pl[q - RWD], yp = r < 3 ? c[r + 1] : pl[q + RWD];
+        long long sx = ((pl[q - 1] + pl[q + 1]) + (ym + yp)) + (cm[r] + cn[r]) + (long long)(w[r] + wz) * c[r] + gz;
+        if (DIR) sx += gxy[r];  // exact
+        const double res = fma(-__ll2double_rn(sx), kk, fv[r]);
+        const unsigned long long rb = finite ? (unsigned long long)__double_as_longlong(res) : 0x7ff8000000000000ull;
+        rz[r * P] = cvt_bits_f32_rn(rb);
         const unsigned long long a = rb & 0x7fffffffffffffffull;
         m = a > m ? a : m;
       }
-      if (p + 2 < N) {  // this set's next plane
-        if (in0) f0 = fv[(p + 2) * NN + row0];
-        if (in1) f1 = fv[(p + 2) * NN + row0 + N];
-      }
-    };
-    if (!(bc.type[0] | bc.type[1] | bc.type[2] | bc.type[3])) {
-      for (int p = 0; p < N; p += 2) {
-        step(std::true_type{}, p, fa0, fa1);
-        if (p + 1 < N) step(std::true_type{}, p + 1, fb0, fb1);
-      }
-    } else {
-      for (int p = 0; p < N; p += 2) {
-        step(std::false_type{}, p, fa0, fa1);
-        if (p + 1 < N) step(std::false_type{}, p + 1, fb0, fb1);
-      }
-    }
-    cp_wait<0>();
-    // one max per column and solve
+      rz += (long long)P * N;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
-      m = v > m ? v : m;
+      for (int r = 0; r < 4; ++r) cm[r] = c[r], c[r] = cn[r];
     }
-    if ((t & 31) == 0) red[t >> 5] = m;
-    __syncthreads();
-    if (t == 0) {
-      unsigned long long x2 = red[0];
-      for (int i = 1; i < CT / 32; ++i) x2 = red[i] > x2 ? red[i] : x2;
-      atomicMax(num + C.x, x2);
-    }
+  }
+  cp_wait<0>();
+  return m;
+}
+
+template <bool DIR>
+__global__ void __launch_bounds__(ST, DIR ? 6 : 8) k_bt_outer(const int4 *__restrict__ cols, const BSolve *__restrict__ tab,
+                                                    const unsigned char *__restrict__ active,
+                                                    const double *__restrict__ phi, const double *__restrict__ f64,
+                                                    float *__restrict__ f32, Bc bc,
+                                                    const unsigned *__restrict__ emax,
+                                                    unsigned long long *__restrict__ num) {
+  __shared__ __align__(16) long long sp[OSL * DPL];
+  __shared__ unsigned long long red[ST / 32];
+  const int4 C = cols[blockIdx.x];
+  if (!active[C.x]) return;
+  int E = max((int)emax[C.x], 123);  // and bound of the Dirichlet wall values
+#pragma unroll
+  for (int f = 0; f < 6; ++f)
+    if (bc.type[f]) E = max(E, (int)expo_of(bc.g2[f]));
+  unsigned long long m = outer_column<DIR>(C, tab[C.x], E, phi, f64, f32, bc, sp);
+  // one max per column and solve
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long v = __shfl_xor_sync(0xffffffffu, m, o);
+    m = v > m ? v : m;
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < ST / 32; ++i) m = red[i] > m ? red[i] : m;
+    atomicMax(num + C.x, m);
   }
 }
 
+// residual of a cell of a zero potential whose wall ghosts sum to sw.  Not
+// inlined: as predicated instructions its FP64 operations take the pipe for
+// every cell (83% of the pass), as a call only for warps with a wall cell.
+__device__ __noinline__ double wall_resid(double sw, double inv_h2, double f) {
+  return fma(-fma(-6.0, 0.0, sw), inv_h2, f);
+}
 constexpr int OUTER0_BLOCKS = 4;  // resident blocks per SM (64 registers a thread)
 // Residual of phi = 0 on the finest grid of every solve flagged in `active`
 // (the denominators of the relative residual): r0 = f - L0, where L0 has
@@ -962,8 +986,7 @@ __global__ void __launch_bounds__(CT, OUTER0_BLOCKS) k_bt_outer0(const int4 *__r
       double r = f;
       if (wxy[u] | w4 | w5) {
         const double g4 = w4 ? bc.g2[4] - 0.0 : 0.0, g5 = w5 ? bc.g2[5] - 0.0 : 0.0;
-        const double sw = sxy[u] + (g4 + g5);
-        r = fma(-fma(-6.0, 0.0, sw), inv_h2, f);
+        r = wall_resid(sxy[u] + (g4 + g5), inv_h2, f);
       }
       return (unsigned long long)__double_as_longlong(r);
     };
@@ -1418,6 +1441,13 @@ static BState bstate(sm_batch *b) {
   return {b->d_num, b->d_den, b->d_rel, b->d_cycles, b->d_active, b->d_any, b->d_nz, b->d_work};
 }
 
+static void launch_outer(sm_batch *b, const unsigned char *mask) {
+  const bool dir = b->bc.type[0] | b->bc.type[1] | b->bc.type[2] | b->bc.type[3];
+  auto kernel = dir ? k_bt_outer<true> : k_bt_outer<false>;
+  kernel<<<(unsigned)b->fine_cnt, ST, 0, b->stream>>>(b->d_tiles + b->fine_off, b->d_tab, mask, b->phi, b->f64, b->f32,
+                                                      b->bc, b->d_emax, b->d_num);
+}
+
 // residual of the solves flagged in `mask`; zero_phi: of phi = 0, also
 // flagging (d_nz) the solves whose stored potential is not all +0 and
 // setting their exponent bounds (d_emax, zeroed before)
@@ -1427,8 +1457,7 @@ static int outer(sm_batch *b, int zero_phi, const unsigned char *mask) {
     k_bt_outer0<<<grid_for(b, n0), CT, 0, b->stream>>>(b->d_tiles + b->fine_off, (int)n0, b->d_tab, mask, b->phi,
                                                        b->f64, b->f32, b->bc, b->d_num, b->d_nz, b->d_emax);
   else
-    k_bt_outer<<<grid_for(b, n0), CT, OUTER_SMEM, b->stream>>>(b->d_tiles + b->fine_off, (int)n0, b->d_tab, mask,
-                                                      b->phi, b->f64, b->f32, b->bc, b->d_emax, b->d_num);
+    launch_outer(b, mask);
   ++b->n_launch;
   return cudaGetLastError() == cudaSuccess ? SM_OK : bfail(b, SM_ECUDA, "outer residual launch");
 }
@@ -1480,7 +1509,6 @@ static int set_attrs(sm_batch *b) {
     if (!b->ev_fork[k]) BCK(cudaEventCreateWithFlags(&b->ev_fork[k], cudaEventDisableTiming));
     if (!b->ev_join[k]) BCK(cudaEventCreateWithFlags(&b->ev_join[k], cudaEventDisableTiming));
   }
-  BCK(cudaFuncSetAttribute(k_bt_outer, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OUTER_SMEM));
   BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->rcol_per_sm, k_bt_restrict_col, CT, 0));
   b->rcol_per_sm = std::max(1, b->rcol_per_sm);
   return SM_OK;
@@ -1824,9 +1852,7 @@ extern "C" int sm_batch_kernel_bench(sm_batch *b, int kclass, int reps, double *
                                                                       nullptr, nullptr);
         break;
       case 1:
-        k_bt_outer<<<grid_for(b, b->fine_cnt), CT, OUTER_SMEM, b->stream>>>(
-            b->d_tiles + b->fine_off, (int)b->fine_cnt, b->d_tab, b->d_active, b->phi, b->f64, b->f32, b->bc,
-            b->d_emax, b->d_num);
+        launch_outer(b, b->d_active);
         break;
       case 2:
         k_bt_prolong<<<grid_for(b, nsw), CT, 0, b->stream>>>(b->d_tiles + b->scol_off[0], (int)nsw, 0, b->d_tab,
