@@ -526,24 +526,108 @@ __device__ __forceinline__ void coarse_box(int t0, Sync sync, double *sm, T *phi
 }
 
 // FP64 residual f - L v of the cells of this thread in leaf box b; the
-// largest magnitude is returned, r is stored to r32 when given
+// largest magnitude is returned, r is stored to r32 when given.
+// The FP64 pipe bounds it when the stencil sum is formed in FP64 (eight
+// operations a cell with the maximum).  Here the sum is exact in 64-bit
+// fixed point on the integer pipe: every staged value is mapped to the
+// nearest multiple of 2^(E - 1080), E (at least 123) the largest exponent
+// field among the box's values and ghosts, which leaves two FP64 operations
+// a cell, the conversion of the sum and r = f - S 2^(E-1080) h^-2; the
+// maximum is taken on bit patterns.  The error of the map, 6.5 2^(E-1080)
+// h^-2 at most, is below the roundings of the plain sum (2^-53 of values up
+// to 2^(E-1022)).  A box that holds an infinity or a NaN takes the plain sum.
+// NaN residuals do not enter the maximum.
 __device__ __forceinline__ double resid_box(const Grp &g, double *s, int b, const double *v, const double *rhs,
-                                            const double *gh, const Nb &nb, const Bc &bc, double inv_h2,
+                                            const double *gh, const Nb &nbv, const Bc &bc, double inv_h2,
                                             float *r32) {
   const size_t base = (size_t)b * CELLS;
-  double f[CPT];
+  const double *p = v + base;
+  double f[CPT], x[CPT], hv[FPS];
 #pragma unroll
   for (int h = 0; h < CPT; ++h) f[h] = rhs[base + g.t + h * GT];
-  stage_box(g, s, v, nb, gh, b, bc, 0);
-  double m = 0.0;
+#pragma unroll
+  for (int h = 0; h < CPT; ++h) x[h] = p[g.t + h * GT];
+  // the staging of stage_box, with the values also kept by their threads
+  const int slice = g.t >> 6, u = g.t & 7, w = (g.t >> 3) & 7;
+#pragma unroll
+  for (int fc = 0; fc < 6; ++fc) {
+    if (fc % NSL != slice) continue;
+    const int r = fc / NSL, nb = nbv.v[r];
+    if (nb >= 0) hv[r] = v[(size_t)nb * CELLS + face_cell(fc ^ 1, u, w)];
+    else if (nb == -2) hv[r] = gh[(size_t)(6 * b + fc) * FACE + u + NC * w];
+    else hv[r] = 0.0;
+  }
+  unsigned e = 123;
+#pragma unroll
+  for (int h = 0; h < CPT; ++h) e = max(e, expo_of(x[h]));
+  g.sync();  // earlier users of s are done
+#pragma unroll
+  for (int h = 0; h < CPT; ++h) s[s10(g.t + h * GT)] = x[h];
+  g.sync();
+#pragma unroll
+  for (int fc = 0; fc < 6; ++fc) {
+    if (fc % NSL != slice) continue;
+    const int r = fc / NSL;
+    if (nbv.v[r] < 0) {
+      const double inner = s[s10(face_cell(fc, u, w))];
+      if (nbv.v[r] == -1) hv[r] = bc.type[fc] ? bc_g2<double>(bc, fc) - inner : inner;
+      else hv[r] = inner * (1.0 / 3.0) + (2.0 / 3.0) * hv[r];
+    }
+    e = max(e, expo_of(hv[r]));
+  }
+  // largest exponent of the box, through four edge cells (which no stencil reads)
+  unsigned *const es = reinterpret_cast<unsigned *>(s);
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((g.t & 31) == 0) es[2 + (g.t >> 5)] = e;
+  g.sync();
+#pragma unroll
+  for (int i = 0; i < GT / 32; ++i) e = max(e, es[2 + i]);
+  const int E = (int)e;
+  if (E == 0x7ff) {
+#pragma unroll
+    for (int fc = 0; fc < 6; ++fc) {
+      if (fc % NSL != slice) continue;
+      const int stride = fc < 2 ? 1 : (fc < 4 ? 10 : 100);
+      s[s10(face_cell(fc, u, w)) + ((fc & 1) ? stride : -stride)] = hv[fc / NSL];
+    }
+    g.sync();
+    double m = 0.0;
+    for (int h = 0; h < CPT; ++h) {
+      const int q = s10(g.t + h * GT);
+      const double r = rhs[base + g.t + h * GT] - (staged_sum(s, q) - 6.0 * s[q]) * inv_h2;
+      if (r32) r32[base + g.t + h * GT] = cvt_f64_f32_rn(r);
+      m = fmax(m, fabs(r));
+    }
+    return m;
+  }
+  const double kk = inv_h2 * __longlong_as_double((long long)(E - 57) << 52);  // 2^(E-1080) h^-2
+  long long *const si = reinterpret_cast<long long *>(s);
+  long long c[CPT];
+#pragma unroll
+  for (int h = 0; h < CPT; ++h) {
+    c[h] = fix_of_bits((unsigned long long)__double_as_longlong(x[h]), E);
+    si[s10(g.t + h * GT)] = c[h];
+  }
+#pragma unroll
+  for (int fc = 0; fc < 6; ++fc) {
+    if (fc % NSL != slice) continue;
+    const int stride = fc < 2 ? 1 : (fc < 4 ? 10 : 100);
+    si[s10(face_cell(fc, u, w)) + ((fc & 1) ? stride : -stride)] =
+        fix_of_bits((unsigned long long)__double_as_longlong(hv[fc / NSL]), E);
+  }
+  g.sync();
+  unsigned long long m = 0;
 #pragma unroll
   for (int h = 0; h < CPT; ++h) {
     const int q = s10(g.t + h * GT);
-    const double r = f[h] - (staged_sum(s, q) - 6.0 * s[q]) * inv_h2;
-    if (r32) r32[base + g.t + h * GT] = cvt_f64_f32_rn(r);
-    m = fmax(m, fabs(r));
+    const long long S = ((si[q - 1] + si[q + 1]) + (si[q - 10] + si[q + 10])) + (si[q - 100] + si[q + 100]) - 6 * c[h];
+    const double r = fma(-__ll2double_rn(S), kk, f[h]);
+    const unsigned long long rb = (unsigned long long)__double_as_longlong(r);
+    if (r32) r32[base + g.t + h * GT] = cvt_bits_f32_rn(rb);
+    const unsigned long long a = rb & 0x7fffffffffffffffull;
+    m = a > m && a <= 0x7ff0000000000000ull ? a : m;
   }
-  return m;
+  return __longlong_as_double((long long)m);
 }
 
 // max over a box group, pushed to *slot by thread 0 (red: GT/32 doubles
