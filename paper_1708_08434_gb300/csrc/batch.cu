@@ -56,9 +56,9 @@ struct TileShape {
 
 // Rows of the FP32 grids (error and its right-hand side) are padded to whole
 // 16-byte groups, so that every row of every size can be staged by 16-byte
-// copies; the pad cells of the error are never written and stay zero, like
-// the cells outside the grid.  (Element-wise staging of the sides that are
-// not a multiple of 4 took 1900 cycles a plane, a third of it now.)
+// copies (element by element a plane of a side that is not a multiple of 4
+// took 1900 cycles); the pad cells of the error are never written and stay
+// zero, like the cells outside the grid.
 __host__ __device__ constexpr int pitch(int N) { return (N + 3) & ~3; }
 __device__ __forceinline__ long long gidx(int N, int x, int y, int z) {
   return (long long)x + (long long)pitch(N) * (y + (long long)N * z);
@@ -96,18 +96,19 @@ __device__ __forceinline__ bool tile_cell(const int4 &T, TileShape sh, int N, in
 
 // ---- z-marching columns -------------------------------------------------
 //
-// The smoother and the outer residual walk columns of CX x CY cells in x, y
-// through the whole grid in z: one block of CT threads per column, thread t
-// owning x = x0 + t % 32 and the two rows y = y0 + 2 (t / 32) + {0, 1}.
-// Planes of the column, with an x/y halo, are staged in a ring of RING
-// shared-memory slots by asynchronous copies (cp.async) issued several
-// planes ahead.  Staged rows start 16 bytes before x0 so that rows of grids
-// with N % 4 == 0 (FP32) or N even (FP64) are copied in aligned 16-byte
-// chunks; other grids are copied element by element.  Halo cells outside
-// the grid are zero-filled by the copy (source size 0), so in-plane
-// neighbour sums need no tests; the wall ghosts enter through one
-// coefficient per cell: the homogeneous ghost is +c (Neumann) or -c
-// (Dirichlet), the inhomogeneous one c or 2g - c.
+// The smoother, the outer residual, the restriction and the prolongation
+// walk columns of CX x CY cells in x, y through the whole grid in z, a block
+// per column: the first three with ST threads of four rows each (thread t
+// owns x = x0 + t % 32 and the rows y0 + 4 (t / 32) ..), the prolongation
+// with CT threads of two.  Planes of the column, with an x/y halo, are
+// staged in a ring of shared-memory slots by asynchronous copies (cp.async)
+// issued several planes ahead.  Staged rows start 16 bytes before x0, so
+// that rows are copied in aligned 16-byte chunks (FP64 grids of odd N, which
+// are not padded, element by element).  Halo cells outside the grid are
+// zero-filled by the copy (source size 0), so in-plane neighbour sums need no
+// tests; the wall ghosts enter through one coefficient per cell: the
+// homogeneous ghost is +c (Neumann) or -c (Dirichlet), the inhomogeneous one
+// c or 2g - c.
 
 constexpr int CX = 32, CY = 16, CT = 256;
 constexpr int RW = CX + 8;                    // FP32 staged row: x0-4 .. x0+35
@@ -115,7 +116,6 @@ constexpr int ER = CY + 4, FR = CY + 2;       // staged rows: error halo 2, rhs 
 constexpr int EPL = RW * ER, FPL = RW * FR;   // floats per staged plane
 constexpr int RWD = CX + 4;                   // FP64 staged row: x0-2 .. x0+33
 constexpr int DPL = RWD * FR;                 // doubles per staged potential plane
-constexpr int RING = 8;                       // staged planes per block (power of 2)
 constexpr int ST = 128;                       // threads of a sweep block: four rows each
 constexpr int SRING = 6;                      // staged planes of a sweep (even, the colour parity unrolls)
 constexpr int SPL = EPL + FPL;                // floats of one sweep slot: an error plane and its rhs plane
@@ -175,7 +175,8 @@ __device__ __forceinline__ float wall_w(const Bc &bc, int a, int v, int N) {
 // so the z neighbours of Uo(p) are Vo(p-1), Vo(p+1), and only the x
 // neighbours and one y neighbour in four are read from shared memory;
 // colour-0 results alone are written back, and colour 1 of plane p-1 needs
-// of plane p only the thread's own values, so one barrier a plane is enough.
+// of plane p only the thread's own values, so one barrier a plane is enough:
+// 286 us for 124e6 cells (5.2 TB/s), 376 before.
 // Slots at step p: planes p-1 .. p+1 are read, p+2 and p+3 are in flight,
 // and plane p+4 is issued into the slot of plane p-2 (last read at step
 // p-1).  Cells outside the grid are zero in the slots and in the registers;
@@ -432,116 +433,121 @@ __global__ void __launch_bounds__(TILE_CELLS) k_bt_restrict(const int4 *__restri
 }
 
 // Restriction of the error equation's residual r = f - A e from level k to
-// f of level k+1, on the sweep columns of level k (the solves for which
-// level k is not the coarsest), marching the fine planes: each thread's two
-// rows (one coarse row) are summed, then x pairs by a lane shuffle, then the
-// two fine planes of a coarse plane in a register; the even lanes write 1/8
-// of the sum.  The error planes (one-cell halo, zero outside the grid, the
-// planes -1 and N zero) are staged in a ring of eight shared-memory slots by
-// 16-byte asynchronous copies issued four planes ahead, and each thread's
-// two f values are loaded two planes ahead into registers; walls enter
-// through the homogeneous ghost coefficient (+1 Neumann, -1 Dirichlet per
-// wall face).
-constexpr int RRW = CX + 8;     // staged row: x0-4 .. x0+35, whole 16-byte chunks
-constexpr int RFR = CY + 2;     // staged rows: y0-1 .. y0+16
-constexpr int RPL = RRW * RFR;  // floats per staged plane
-__global__ void __launch_bounds__(CT, 6) k_bt_restrict_col(const int4 *__restrict__ cols, int ncols, int k,
-                                                        const BSolve *__restrict__ tab,
-                                                        const unsigned char *__restrict__ active,
-                                                        const float *__restrict__ e, float *__restrict__ f, Bc bc) {
-  __shared__ __align__(16) float se[RING][RPL];
-  const int t = threadIdx.x, tx = t % CX, ty2 = 2 * (t / CX);
-  for (int it = blockIdx.x; it < ncols; it += gridDim.x) {
-    const int4 C = cols[it];
-    if (!active[C.x]) continue;  // uniform per block
-    const BSolve &S = tab[C.x];
-    const int N = S.N[k], Nc = S.N[k + 1];  // N = 2 Nc
-    const int P = pitch(N), Pc = pitch(Nc);
-    const long long NN = (long long)P * N;
-    const float *ef = e + S.off[k], *ff = f + S.off[k];
-    float *fc = f + S.off[k + 1];
-    const float inv_h2 = 1.0f / S.h2f[k];
-    const int x0 = C.y * CX, y0 = C.z * CY, x = x0 + tx, ya = y0 + ty2;
-    const bool in = x < N && ya < N;  // N even, ya even: both rows or neither
-    // this thread's 16-byte chunk of a staged plane: slot-0 offset, in-plane
-    // element offset, inside the grid
-    int cdst = -1, coff = 0;
-    bool cok = false;
-    if (t < RFR * (RRW / 4)) {
-      const int r = t / (RRW / 4), c4 = 4 * (t % (RRW / 4)), y = y0 - 1 + r, xx = x0 - 4 + c4;
-      cok = y >= 0 && y < N && xx >= 0 && xx < N;
-      coff = cok ? y * P + xx : 0;
-      cdst = r * RRW + c4;
-    }
-    // this thread's chunk source in plane z, advanced one plane per issue of
-    // a plane of the grid
-    const float *csrc = ef + coff;
-    // copies of plane z into slot sl = z mod RING (zero planes outside the
-    // grid); called for z = -1, 0, 1, ... in order
-    auto issue = [&](int z, int sl) {
-      const bool zin = z >= 0 && z < N;
-      if (cdst >= 0) cp_async<16>(&se[sl][cdst], zin ? csrc : ef, cok && zin);
-      if (zin) csrc += NN;
-      cp_commit();
-    };
-    const int q0 = (ty2 + 1) * RRW + tx + 4;
-    const float wx = wall_w(bc, 0, x, N);
-    const float w0 = wx + wall_w(bc, 1, ya, N), w1 = wx + wall_w(bc, 1, ya + 1, N);
-    // this thread's two f values of planes z (fa) and z+1 (fb), loaded two
-    // planes ahead of their use
-    const float *frow = ff + (in ? (long long)ya * P + x : 0);
-    float fa0 = 0.f, fa1 = 0.f, fb0 = 0.f, fb1 = 0.f;
-    if (in) {
-      fa0 = __ldg(frow), fa1 = __ldg(frow + P);
-      if (N > 1) fb0 = __ldg(frow + NN), fb1 = __ldg(frow + NN + P);
-    }
-    const float *fnext = frow + 2 * NN;  // f of plane z+2 at step z
-    float *fcz = fc + (long long)(ya >> 1) * Pc + (x >> 1);  // this thread's coarse cell, coarse plane z/2
-    float acc = 0.f;
-    __syncthreads();  // the previous column's planes are no longer read
+// f of level k+1, a block per sweep column of level k (the solves for which
+// level k is not the coarsest), marching the fine planes with four rows a
+// thread: two rows (one coarse row) are summed, then x pairs by a lane
+// shuffle, then the two fine planes of a coarse plane in a register; the
+// even lanes write 1/8 of the sum.  As in the sweep a thread keeps its rows
+// of planes p-1, p and p+1 in registers, so that only x neighbours and one y
+// neighbour in four are read from shared memory (213 us for 124e6 cells, 380
+// with all neighbours staged and two rows a thread).  Error planes (one-cell halo, zero
+// outside the grid) are staged by 16-byte copies: at step p planes p and p+1
+// are read, p+2 is in flight, p+3 is issued into the slot of p-1; f is loaded
+// one plane ahead.  Walls enter through the homogeneous ghost coefficient
+// (+1 Neumann, -1 Dirichlet per wall face).
+constexpr int RFR = CY + 2;    // staged rows: y0-1 .. y0+16 of x0-4 .. x0+35
+constexpr int RPL = RW * RFR;  // floats per staged plane
+__global__ void __launch_bounds__(ST, 8) k_bt_restrict_col(const int4 *__restrict__ cols, int k,
+                                                           const BSolve *__restrict__ tab,
+                                                           const unsigned char *__restrict__ active,
+                                                           const float *__restrict__ e, float *__restrict__ f,
+                                                           Bc bc) {
+  __shared__ __align__(16) float se[OSL * RPL];
+  const int t = threadIdx.x, tx = t % CX, ty = 4 * (t / CX);
+  const int4 C = cols[blockIdx.x];
+  if (!active[C.x]) return;
+  const BSolve &S = tab[C.x];
+  const int N = S.N[k], Nc = S.N[k + 1], P = pitch(N), Pc = pitch(Nc);  // N = 2 Nc
+  const long long PL = (long long)P * N;
+  const float inv_h2 = 1.0f / S.h2f[k];
+  const int x0 = C.y * CX, y0 = C.z * CY, x = x0 + tx, ya = y0 + ty;
+  constexpr int CH = RPL / 4, U = (CH + ST - 1) / ST;  // 16-byte chunks of a staged plane
+  const float *csrc[U];
+  bool cok[U];
 #pragma unroll
-    for (int z = -1; z <= 3; ++z) issue(z, z & (RING - 1));
-    // steps z = zb + i, unrolled by the ring size so that every slot index
-    // is a constant (zb is a multiple of RING)
-    for (int zb = 0; zb < N; zb += RING) {
+  for (int u = 0; u < U; ++u) {
+    const int i = t + u * ST, y = y0 - 1 + i / (RW / 4), xx = x0 - 4 + 4 * (i % (RW / 4));
+    cok[u] = y >= 0 && y < N && xx >= 0 && xx < N;
+    csrc[u] = e + S.off[k] + (cok[u] ? y * P + xx : 0);
+  }
+  auto issue = [&](int z, int sl) {
+    if (z < N) {
 #pragma unroll
-      for (int i = 0; i < RING; ++i) {
-        const int z = zb + i;
-        if (z >= N) break;
-        float fn0 = 0.f, fn1 = 0.f;
-        if (in && z + 2 < N) fn0 = __ldg(fnext), fn1 = __ldg(fnext + P);
-        fnext += NN;
-        cp_wait<2>();     // this thread's copies of planes <= z+1 have landed
-        __syncthreads();  // everyone's have; step z-1's reads are done
-        issue(z + 4, (i + 4) & (RING - 1));  // into the slot of plane z-4, last read at step z-3
-        const float *pm = se[(i - 1) & (RING - 1)], *pz = se[i & (RING - 1)], *pp = se[(i + 1) & (RING - 1)];
-        const float wz = wall_w(bc, 2, z, N);
-        float rs = 0.f;
-        if (in) {
-#pragma unroll
-          for (int o = 0; o < 2; ++o) {
-            const int q = q0 + o * RRW;
-            const float c = pz[q];
-            float sum = pz[q - 1] + pz[q + 1];
-            sum += pz[q - RRW];
-            sum += pz[q + RRW];
-            sum += pm[q];
-            sum += pp[q];
-            sum = fmaf((o ? w1 : w0) + wz, c, sum);
-            rs += (o ? fa1 : fa0) - (sum - 6.0f * c) * inv_h2;
-          }
-        }
-        fa0 = fb0, fa1 = fb1, fb0 = fn0, fb1 = fn1;
-        rs += __shfl_xor_sync(0xffffffffu, rs, 1);
-        acc = (i & 1) ? acc + rs : rs;
-        if (i & 1) {
-          if (in && !(tx & 1)) *fcz = acc * 0.125f;
-          fcz += (long long)Pc * Nc;
-        }
+      for (int u = 0; u < U; ++u) {
+        if ((u + 1) * ST <= CH || t < CH - u * ST) cp_async<16>(se + sl * RPL + 4 * (t + u * ST), csrc[u], cok[u]);
+        csrc[u] += PL;
       }
     }
-    cp_wait<0>();
+    cp_commit();
+  };
+  const bool in01 = x < N && ya < N, in23 = x < N && ya + 2 < N;  // N even: rows valid in pairs
+  const float *const q0 = se + (ty + 1) * RW + tx + 4;
+  const float wx = wall_w(bc, 0, x, N);
+  float w[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) w[r] = wx + wall_w(bc, 1, ya + r, N);
+  const float *fz = f + S.off[k] + (long long)ya * P + x;
+  float fn[4] = {}, fv[4];  // f of planes p+1 and p
+  auto load_f = [&]() {
+    if (in01) fn[0] = __ldg(fz), fn[1] = __ldg(fz + P);
+    if (in23) fn[2] = __ldg(fz + 2 * P), fn[3] = __ldg(fz + 3 * P);
+    fz += PL;
+  };
+  load_f();
+  float *fc = f + S.off[k + 1] + (long long)(ya >> 1) * Pc + (x >> 1);  // this thread's coarse cells
+#pragma unroll
+  for (int z = 0; z < OSL - 1; ++z) issue(z, z);
+  cp_wait<OSL - 2>();  // plane 0 has landed
+  __syncthreads();
+  float cm[4] = {}, c[4], cn[4], acc0 = 0.f, acc1 = 0.f;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) c[r] = q0[r * RW];
+  for (int pb = 0; pb < N; pb += OSL) {
+#pragma unroll
+    for (int i = 0; i < OSL; ++i) {
+      const int p = pb + i;
+      if (p >= N) break;
+      cp_wait<OSL - 3>();  // this thread's copies of planes <= p+1 have landed
+      __syncthreads();     // everyone's have; step p-1's reads are done
+      issue(p + OSL - 1, (i + OSL - 1) % OSL);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        fv[r] = fn[r];
+        cn[r] = p + 1 < N ? q0[((i + 1) % OSL) * RPL + r * RW] : 0.f;
+      }
+      if (p + 1 < N) load_f();
+      const float *pz = q0 + i * RPL;
+      const float wz = wall_w(bc, 2, p, N);
+      float rs[2] = {0.f, 0.f};
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        float sum = pz[r * RW - 1] + pz[r * RW + 1];
+        sum += r > 0 ? c[r - 1] : pz[-RW];
+        sum += r < 3 ? c[r + 1] : pz[4 * RW];
+        sum += cm[r];
+        sum += cn[r];
+        sum = fmaf(w[r] + wz, c[r], sum);
+        rs[r >> 1] += fv[r] - (sum - 6.0f * c[r]) * inv_h2;
+      }
+      rs[0] += __shfl_xor_sync(0xffffffffu, rs[0], 1);
+      rs[1] += __shfl_xor_sync(0xffffffffu, rs[1], 1);
+      if (i & 1) {
+        acc0 += rs[0];
+        acc1 += rs[1];
+        if (!(tx & 1)) {
+          if (in01) fc[0] = acc0 * 0.125f;
+          if (in23) fc[Pc] = acc1 * 0.125f;
+        }
+        fc += (long long)Pc * Nc;
+      } else {
+        acc0 = rs[0];
+        acc1 = rs[1];
+      }
+#pragma unroll
+      for (int r = 0; r < 4; ++r) cm[r] = c[r], c[r] = cn[r];
+    }
   }
+  cp_wait<0>();
 }
 
 // e_k += (c + c_sx + c_sy + c_sz)/4 from level k+1 (homogeneous walls), on
@@ -1129,7 +1135,6 @@ struct sm_batch {
   cudaStream_t side[BMAXL] = {};
   cudaEvent_t ev_fork[BMAXL] = {}, ev_join[BMAXL] = {};
   unsigned pending = 0;  // levels whose coarse solve is not joined yet
-  int rcol_per_sm = 1;  // resident column-restriction blocks per SM: its one-wave grid
   std::vector<size_t> restr_off, restr_cnt;  // per level index: restriction tiles
   std::vector<size_t> coarse_off, coarse_cnt;
   std::vector<size_t> scol_off, scol_cnt;  // per level index: sweep columns
@@ -1509,27 +1514,15 @@ static int set_attrs(sm_batch *b) {
     if (!b->ev_fork[k]) BCK(cudaEventCreateWithFlags(&b->ev_fork[k], cudaEventDisableTiming));
     if (!b->ev_join[k]) BCK(cudaEventCreateWithFlags(&b->ev_join[k], cudaEventDisableTiming));
   }
-  BCK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->rcol_per_sm, k_bt_restrict_col, CT, 0));
-  b->rcol_per_sm = std::max(1, b->rcol_per_sm);
   return SM_OK;
 }
 
-// the column restriction runs as one wave of at most RCOL_PER_SM resident
-// blocks per SM whatever the grid multiplier: its blocks march whole
-// columns, longest first, and a second partial wave leaves SMs idle at the
-// end; four per SM (about five columns per block on the 256-solve
-// workload) balanced better than six (370 against 405 us)
-constexpr int RCOL_PER_SM = 4;
-static size_t rcol_wave(const sm_batch *b) { return (size_t)std::min(RCOL_PER_SM, b->rcol_per_sm) * b->sms; }
-static int rcol_grid(const sm_batch *b, size_t ncols) {
-  return (int)std::max<size_t>(1, std::min(rcol_wave(b), ncols));
-}
 // the column restriction of level k -> k+1 under the column schedule, on
-// levels with a full wave of columns (on the coarser ones one thread per
-// coarse cell keeps more SMs busy: 17 against 25 us on the third level of
-// the 256-solve workload)
+// levels with four columns per SM (on the coarser ones one thread per coarse
+// cell keeps more SMs busy: 17 against 25 us on the third level of the
+// 256-solve workload)
 static bool rcol_use(const sm_batch *b, int k) {
-  return b->shape == SHAPE_COLS && b->scol_cnt[k] >= rcol_wave(b);
+  return b->shape == SHAPE_COLS && b->scol_cnt[k] >= 4 * (size_t)b->sms;
 }
 
 // exact solves of the solves whose coarsest grid is level k.  Level 0 runs
@@ -1575,8 +1568,8 @@ static int bvcycle(sm_batch *b) {
     if (rcol_use(b, k)) {
       const size_t nc = b->scol_cnt[k];
       if (nc) {
-        k_bt_restrict_col<<<rcol_grid(b, nc), CT, 0, b->stream>>>(b->d_tiles + b->scol_off[k], (int)nc, k, b->d_tab,
-                                                                 b->d_active, b->e32, b->f32, b->bc);
+        k_bt_restrict_col<<<(unsigned)nc, ST, 0, b->stream>>>(b->d_tiles + b->scol_off[k], k, b->d_tab, b->d_active,
+                                                              b->e32, b->f32, b->bc);
         ++b->n_launch;
       }
     } else {
@@ -1860,8 +1853,8 @@ extern "C" int sm_batch_kernel_bench(sm_batch *b, int kclass, int reps, double *
         break;
       default:
         if (rcol)
-          k_bt_restrict_col<<<rcol_grid(b, nr), CT, 0, b->stream>>>(b->d_tiles + b->scol_off[0], (int)nr, 0, b->d_tab,
-                                                                   b->d_active, b->e32, b->f32, b->bc);
+          k_bt_restrict_col<<<(unsigned)nr, ST, 0, b->stream>>>(b->d_tiles + b->scol_off[0], 0, b->d_tab, b->d_active,
+                                                                b->e32, b->f32, b->bc);
         else
           k_bt_restrict<<<grid_for(b, nr), TILE_CELLS, 0, b->stream>>>(b->d_tiles + b->restr_off[1], (int)nr, 0,
                                                                        b->d_tab, b->d_active, b->e32, b->f32, b->bc,
