@@ -98,10 +98,28 @@ __global__ void k_ref_flags(const int32_t *__restrict__ leaf, int n_leaves, cons
   flags[b] = f;
 }
 
-__global__ void __launch_bounds__(512) k_regrid_gather(const int32_t *__restrict__ src, const double *__restrict__ x,
-                                                       double *__restrict__ y) {
-  const int s = src[blockIdx.x];
-  y[(size_t)blockIdx.x * CELLS + threadIdx.x] = s >= 0 ? x[(size_t)s * CELLS + threadIdx.x] : 0.0;
+// Three fields to a new numbering through scratch arrays: GATHER takes box b
+// of y from box src[b] of x (zero for a new box), the other form copies the
+// scratch back.  Boxes that keep their number are left alone: levels below
+// the first changed one, and that level up to its first change.  Bytes bound
+// it; a launch and a device copy of every box per field took 23 us each.
+struct Fields3 {
+  const double *x[3];
+  double *y[3];
+};
+template <bool GATHER>
+__global__ void __launch_bounds__(256) k_regrid_move(const int32_t *__restrict__ src, Fields3 F) {
+  const int b = blockIdx.x, s = src[b];
+  if (s == b) return;
+  const size_t to = (size_t)b * (CELLS / 2) + threadIdx.x, from = GATHER ? (size_t)max(s, 0) * (CELLS / 2) + threadIdx.x : to;
+  double2 v[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    v[k] = make_double2(0.0, 0.0);
+    if (!GATHER || s >= 0) v[k] = reinterpret_cast<const double2 *>(F.x[k])[from];
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) reinterpret_cast<double2 *>(F.y[k])[to] = v[k];
 }
 
 // New boxes: (c + c_sx + c_sy + c_sz)/4 of the parent's cells, s the
@@ -393,18 +411,15 @@ int sm_regrid_impl(sm_ctx *ctx, const int8_t *flags, int *n_refined, int *n_dere
   k_rg_keep<<<gb, T, 0, ctx->stream>>>(n, ctx->parent, derv, keepv);
   ctx->n_launch += 3;
   SM_CKL("regrid decisions");
-  if ((st = sm_exclusive_scan(ctx, refv, ref_pos, n))) return st;
-  if ((st = sm_exclusive_scan(ctx, keepv, keep_pos, n))) return st;
-  // counts: dropped, derefined, and the list offsets at the old level offsets
+  // the counters and the sums at the old level offsets, read in one copy
   const int L0 = ctx->n_levels;
-  std::vector<int32_t> hk(L0 + 1), hr(L0 + 1);
-  int32_t hc[2];
-  SM_CK(cudaMemcpyAsync(hc, cnt, sizeof hc, cudaMemcpyDeviceToHost, ctx->stream));
-  for (int l = 0; l <= L0; ++l) {
-    SM_CK(cudaMemcpyAsync(&hk[l], keep_pos + ctx->level_off[l], 4, cudaMemcpyDeviceToHost, ctx->stream));
-    SM_CK(cudaMemcpyAsync(&hr[l], ref_pos + ctx->level_off[l], 4, cudaMemcpyDeviceToHost, ctx->stream));
-  }
+  if ((st = sm_exclusive_scan(ctx, refv, ref_pos, n, sm_level_pick(ctx, cnt + 2)))) return st;
+  if ((st = sm_exclusive_scan(ctx, keepv, keep_pos, n, sm_level_pick(ctx, cnt + 2 + (L0 + 1))))) return st;
+  // counts: dropped, derefined, and the list offsets at the old level offsets
+  int32_t hc[2 + 2 * (SM_MAX_LEVELS + 1)];
+  SM_CK(cudaMemcpyAsync(hc, cnt, 4 * (size_t)(2 + 2 * (L0 + 1)), cudaMemcpyDeviceToHost, ctx->stream));
   SM_CK(cudaStreamSynchronize(ctx->stream));
+  const int32_t *hr = hc + 2, *hk = hr + (L0 + 1);
   const int nref = hr[L0], nder = hc[1];
   if (n_refined) *n_refined = nref;
   if (n_derefined) *n_derefined = nder;
@@ -434,15 +449,23 @@ int sm_regrid_impl(sm_ctx *ctx, const int8_t *flags, int *n_refined, int *n_dere
   k_rg_compact<<<(m + T - 1) / T, T, 0, ctx->stream>>>(m, ff, fpos, ctx->scan_a);
   ++ctx->n_launch;
   sm_drop_graphs(ctx);
-  // fields to the new numbering (new boxes zero), through the scratch array
-  // of the previous cycle's potential
-  double *vars[6] = {ctx->phi, ctx->rhs, ctx->emag, ctx->rho, ctx->nbuf[ctx->ncur], ctx->ibuf[ctx->ncur]};
-  for (double *x : vars) {
-    k_regrid_gather<<<m, CELLS, 0, ctx->stream>>>(nsrc, x, ctx->old);
-    ++ctx->n_launch;
-    SM_CK(cudaMemcpyAsync(x, ctx->old, sizeof(double) * CELLS * (size_t)m, cudaMemcpyDeviceToDevice, ctx->stream));
+  // fields to the new numbering (new boxes zero), through the scratch arrays
+  // of the previous cycle's potential and of the densities' other stage
+  double *const ne = ctx->nbuf[ctx->ncur], *const ni = ctx->ibuf[ctx->ncur];
+  double *vars[6] = {ctx->phi, ctx->rhs, ctx->emag, ctx->rho, ne, ni};
+  double *tmp[3] = {ctx->old, ctx->nbuf[ctx->ncur ? 0 : 1], ctx->ibuf[ctx->ncur ? 0 : 1]};
+  for (int h = 0; h < 6; h += 3) {
+    Fields3 there, back;
+    for (int k = 0; k < 3; ++k) {
+      there.x[k] = back.y[k] = vars[h + k];
+      there.y[k] = tmp[k];
+      back.x[k] = tmp[k];
+    }
+    k_regrid_move<true><<<m, 256, 0, ctx->stream>>>(nsrc, there);
+    k_regrid_move<false><<<m, 256, 0, ctx->stream>>>(nsrc, back);
+    ctx->n_launch += 2;
   }
-  SM_CKL("regrid gather");
+  SM_CKL("regrid fields");
   // tables of the new mesh; neighbours and the leaf list from them
   SM_CK(cudaMemcpyAsync(ctx->level, nlev, 4 * (size_t)m, cudaMemcpyDeviceToDevice, ctx->stream));
   SM_CK(cudaMemcpyAsync(ctx->ijk, nijk, 12 * (size_t)m, cudaMemcpyDeviceToDevice, ctx->stream));
@@ -452,8 +475,7 @@ int sm_regrid_impl(sm_ctx *ctx, const int8_t *flags, int *n_refined, int *n_dere
   ctx->n_boxes = m;
   ctx->n_levels = nlevels;
   for (int l = 0; l <= SM_MAX_LEVELS; ++l) ctx->level_off[l] = L.nw[l];
-  for (int l = 0; l < nlevels; ++l)
-    if ((st = sm_build_neighbours(ctx, l))) return st;
+  if ((st = sm_build_neighbours(ctx, 0, m))) return st;
   // the fresh-box list (scan_a) is read before the leaf rebuild reuses it
   if (nref > 0) {
     k_regrid_prolong<<<8 * nref, CELLS, 0, ctx->stream>>>(ctx->scan_a, ctx->parent, ctx->ijk, ctx->nbr6, ctx->bc,

@@ -417,8 +417,15 @@ inline cudaError_t sm_launch(sm_ctx *ctx, void (*k)(KArgs...), dim3 grid, dim3 b
 // entry points implemented in the other translation units
 int sm_mg_fill_cf(sm_ctx *ctx, double *var, int level, int homog);
 int sm_fill_all_cf(sm_ctx *ctx, double *var);
-int sm_exclusive_scan(sm_ctx *ctx, const int32_t *in, int32_t *out, int n);
+// positions of a prefix sum copied to `to` (device) by the scan itself
+struct ScanPick {
+  int n;
+  int at[SM_MAX_LEVELS + 1];
+  int32_t *to;
+};
+ScanPick sm_level_pick(const sm_ctx *ctx, int32_t *to);
+int sm_exclusive_scan(sm_ctx *ctx, const int32_t *in, int32_t *out, int n, const ScanPick &pick = {});
 int sm_restrict_pair(sm_ctx *ctx, double *a, double *b);
 void sm_drop_graphs(sm_ctx *ctx);
 int sm_rebuild_leaves(sm_ctx *ctx);
-int sm_build_neighbours(sm_ctx *ctx, int level);
+int sm_build_neighbours(sm_ctx *ctx, int first, int last);
