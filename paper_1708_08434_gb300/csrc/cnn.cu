@@ -546,12 +546,16 @@ static_assert(((sizeof(NetS) + 127) & ~(size_t)127) + ((sizeof(FwdS) + 127) & ~(
 static_assert(sizeof(NetS) == 19140 && sizeof(FwdS) == 71456 && sizeof(TrainS) == 123172,
               "layout the operand ranges were checked against");
 
+// the warps of the training kernel that issue no backward MMAs
+constexpr int WORKERS = TT / 32 - TC_TILES;
+__device__ __forceinline__ void worker_sync() { asm volatile("bar.sync 1, %0;" ::"n"(32 * WORKERS) : "memory"); }
+
 __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X, const float *__restrict__ target,
                                                   const int *__restrict__ ids, int n, float inv_count,
                                                   const float *__restrict__ w, float *__restrict__ partial,
                                                   float *__restrict__ loss_partial, unsigned *__restrict__ err) {
   extern __shared__ __align__(128) unsigned char smraw[];
-  __shared__ uint64_t mbar;
+  __shared__ uint64_t mbar, mbar_wg;  // completion of forward / backward-data, of backward-weight
   __shared__ uint32_t tslot;
   const size_t o1 = (sizeof(NetS) + 127) & ~(size_t)127, o2 = o1 + ((sizeof(FwdS) + 127) & ~(size_t)127);
   NetS &N = *reinterpret_cast<NetS *>(smraw);
@@ -566,7 +570,10 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
   for (int i = t; i < NG; i += TT) S.grad[i] = 0.0f;
   pdl_wait();
   if (*err) return;  // a wait of an earlier pass ran out: the results are void
+  const uint32_t wg_bar = smem_u32(&mbar_wg);
+  if (t == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(wg_bar), "r"(TC_TILES) : "memory");
   tc_begin(tc, &mbar, &tslot, err, TRAIN_COLS);
+  uint32_t wg_phase = 0;
   load_net<TT>(N, S.w2t, w);
   float my_loss = 0.0f;
   bool wg_acc = false;  // the backward-weight accumulators hold a sum
@@ -648,8 +655,11 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
     tc_fence_before();
     __syncthreads();
     // backward-data and backward-weight of layer 2 on tcgen05 (described
-    // above TC_TILES): lane 0 of warp j issues backward-data tile j and the
-    // backward-weight accumulators j and j + 5, then commits
+    // above TC_TILES): lane 0 of warp j issues backward-data tile j, commits,
+    // then the backward-weight accumulators j and j + 5, committed to their
+    // own barrier.  The queue of MMAs holds the issuing warps until nearly its
+    // end, so the other warps do the layer 3 weights meanwhile, and dL/dz1
+    // and the layer 1 weights under the backward-weight MMAs
     if ((t & 31) == 0 && (t >> 5) < TC_TILES) {
       tc_fence_after();
       const int j = t >> 5, R0 = 11 + 16 * j;
@@ -663,6 +673,7 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
           tc_mma(tc.taddr + 16 * j, dd + D2S(1 - dx, m, 0, 11 - dy - 10 * dz), bd + 32 * tp, TC_IDESC,
                  tp > 0 || m > 0);
       }
+      tc_commit(tc.mbar);
       const uint64_t db = tc_desc(d0, 960, 160);
       for (int c = j; c < 9; c += TC_TILES) {
         const int dy = c % 3 - 1, dz = c / 3 - 1;
@@ -674,66 +685,70 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
                  wg_acc || p > 0);
         }
       }
-      tc_commit(tc.mbar);
+      tc_commit(wg_bar);
     }
     wg_acc = true;
     __syncwarp();
-    // layer 3 weights, while the tensor cores work: warp w takes taps w and
-    // w + 16, lane l the voxels l + 32k, whose sums the warp then adds (fixed
-    // order); bias: the last warp
-    for (int tp = warp; tp < 27; tp += TT / 32) {
-      const int so = SOff(tp);
-      float acc[16];
-#pragma unroll
-      for (int ci = 0; ci < 16; ++ci) acc[ci] = 0.0f;
-#pragma unroll 4
-      for (int v = lane; v < 512; v += 32) {
-        float a[16];
-        row16(F.a2, VS(v) + so, a);
-        const float g = S.g3[Pos(v)];
-#pragma unroll
-        for (int ci = 0; ci < 16; ++ci) acc[ci] += a[ci] * g;
-      }
-      const float sum = warp_sums(acc);
-      if (!(lane & 1)) S.grad[G_W3 + (lane >> 1) * 27 + tp] += sum;
-    }
-    if (warp == TT / 32 - 1) {
-      float acc = 0.0f;
-      for (int v = lane; v < 512; v += 32) acc += S.g3[Pos(v)];
-      acc = warp_sum(acc);
-      if (lane == 0) S.grad[G_B3] += acc;
-    }
-    if (t < 16) {
-      float acc = 0.0f;
-      for (int i = 0; i < TT / 32; ++i) acc += S.part[16 * i + t];
-      S.grad[G_B2 + t] += acc;
-    }
-    if (!tc_wait_all(tc)) break;
-    // dL/dz1 = relu'(a1) dA1 on the interior voxels, into the a2 space
-    // ([channel][voxel]: the lanes of a warp touch consecutive words)
-    {
-      float *d1 = reinterpret_cast<float *>(F.a2);
-      const int q = warp & 3, r = 32 * q + lane;
-      for (int j = warp >> 2; j < TC_TILES; j += TT / 128) {
+    bool ok = true;
+    if (warp >= TC_TILES) {
+      const int wk = warp - TC_TILES;  // one of the WORKERS warps
+      // layer 3 weights: a tap a warp, lane l the voxels l + 32k, whose sums
+      // the warp then adds (fixed order); biases: the last two warps
+      for (int tp = wk; tp < 27; tp += WORKERS) {
+        const int so = SOff(tp);
         float acc[16];
-        tc_ld16(tc.taddr + ((uint32_t)(32 * q) << 16) + 16 * j, acc);
-        const int R = 11 + 16 * j + (r >> 3), x = r & 7, y = R % 10 - 1, z = R / 10 - 1;
-        if (y < 0 || y > 7 || z < 0 || z > 7) continue;
-        const int v = x + 8 * y + 64 * z;
-        const bf16 *a1v = F.a1 + 8 * A1S(x + 1, 0, R);
 #pragma unroll
-        for (int ci = 0; ci < 16; ++ci) d1[ci * 512 + v] = bf(a1v[ci < 8 ? ci : 80 + (ci - 8)]) > 0.0f ? acc[ci] : 0.0f;
+        for (int ci = 0; ci < 16; ++ci) acc[ci] = 0.0f;
+#pragma unroll 4
+        for (int v = lane; v < 512; v += 32) {
+          float a[16];
+          row16(F.a2, VS(v) + so, a);
+          const float g = S.g3[Pos(v)];
+#pragma unroll
+          for (int ci = 0; ci < 16; ++ci) acc[ci] += a[ci] * g;
+        }
+        const float sum = warp_sums(acc);
+        if (!(lane & 1)) S.grad[G_W3 + (lane >> 1) * 27 + tp] += sum;
       }
-    }
-    tc_fence_before();
-    __syncthreads();
-    // layer 1 weights (valid conv on the 10^3 input): warp w takes taps w
-    // and w + 16, lane l the voxels l + 32k, whose sums the warp adds (16300
-    // cycles a box with five exchanges a sum, 9800 with one; both taps at
-    // once, to read dL/dz1 once, took 26000)
-    {
-      const float *d1 = reinterpret_cast<const float *>(F.a2);
-      for (int tp = warp; tp < 27; tp += TT / 32) {
+      if (warp == TT / 32 - 1) {
+        float acc = 0.0f;
+        for (int v = lane; v < 512; v += 32) acc += S.g3[Pos(v)];
+        acc = warp_sum(acc);
+        if (lane == 0) S.grad[G_B3] += acc;
+      }
+      if (warp == TT / 32 - 2 && lane < 16) {
+        float acc = 0.0f;
+        for (int i = 0; i < TT / 32; ++i) acc += S.part[16 * i + lane];
+        S.grad[G_B2 + lane] += acc;
+      }
+      ok = __all_sync(0xffffffffu, mbar_wait(tc.mbar, tc.phase));
+      tc_fence_after();
+      worker_sync();  // the layer 3 weights have read a2, whose space dL/dz1 takes
+      // dL/dz1 = relu'(a1) dA1 on the interior voxels, into the a2 space
+      // ([channel][voxel]: the lanes of a warp touch consecutive words); the
+      // workers of tensor-memory quarter q share its rows of the tiles
+      float *d1 = reinterpret_cast<float *>(F.a2);
+      if (ok) {
+        const int q = warp & 3, r = 32 * q + lane, first = TC_TILES + ((q - TC_TILES) & 3);
+        const int share = (TT / 32 - first + 3) / 4;
+        for (int j = (warp - first) / 4; j < TC_TILES; j += share) {
+          __syncwarp();
+          float acc[16];
+          tc_ld16(tc.taddr + ((uint32_t)(32 * q) << 16) + 16 * j, acc);
+          const int R = 11 + 16 * j + (r >> 3), x = r & 7, y = R % 10 - 1, z = R / 10 - 1;
+          if (y < 0 || y > 7 || z < 0 || z > 7) continue;
+          const int v = x + 8 * y + 64 * z;
+          const bf16 *a1v = F.a1 + 8 * A1S(x + 1, 0, R);
+#pragma unroll
+          for (int ci = 0; ci < 16; ++ci)
+            d1[ci * 512 + v] = bf(a1v[ci < 8 ? ci : 80 + (ci - 8)]) > 0.0f ? acc[ci] : 0.0f;
+        }
+      }
+      tc_fence_before();
+      worker_sync();
+      // layer 1 weights (valid conv on the 10^3 input): a tap a warp, lane l
+      // the voxels l + 32k, whose sums the warp adds
+      for (int tp = wk; tp < 27; tp += WORKERS) {
         const int off = Off(tp);
         float acc[32];  // [co][ci]
 #pragma unroll
@@ -751,23 +766,31 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
         const float sum = warp_sums(acc);
         S.grad[G_W1 + lane * 27 + tp] += sum;
       }
-      // layer-1 bias: thread t sums channel t / G over the voxels t % G +
-      // G i (G = TT / 16), then the G partial sums of a channel in order
-      {
-        constexpr int G = TT / 16;
-        const int c = t / G, g = t % G;
+      // layer-1 bias: 32 partial sums a channel (voxels g + 32 i), added in order
+      for (int i = t - 32 * TC_TILES; i < 512; i += 32 * WORKERS) {
+        const int c = i >> 5, g = i & 31;
         float acc = 0.0f;
-        for (int v = g; v < 512; v += G) acc += d1[c * 512 + v];
-        S.part[t] = acc;
+        for (int v = g; v < 512; v += 32) acc += d1[c * 512 + v];
+        S.part[i] = acc;
       }
-      __syncthreads();
-      if (t < 16) {
+      worker_sync();
+      if (wk == 0 && lane < 16) {
         float acc = 0.0f;
-        for (int g = 0; g < TT / 16; ++g) acc += S.part[(TT / 16) * t + g];
-        S.grad[G_B1 + t] += acc;
+        for (int g = 0; g < 32; ++g) acc += S.part[32 * lane + g];
+        S.grad[G_B1 + lane] += acc;
       }
     }
-    __syncthreads();
+    // both barriers' phases are over, or a wait ran out: the whole block stops
+    ok = ok && mbar_wait(wg_bar, wg_phase);
+    if (!__syncthreads_and(ok)) {
+      if (t == 0) atomicOr(tc.err, 1u);
+      mbar_wait(tc.mbar, tc.phase);
+      mbar_wait(wg_bar, wg_phase);
+      break;
+    }
+    tc.phase ^= 1;
+    wg_phase ^= 1;
+    tc_fence_after();
     zero16(F.a2, sizeof(F.a2));  // layer 3 of the next box reads zeros outside the interior
     __syncthreads();
   }
