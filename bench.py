@@ -524,9 +524,9 @@ def run_gpu(args):
     e2e_ms = max_over_ranks(e2e_ms, dev)
     # roofline of the dominant kernel: a colour pass of the red-black
     # smoother (k_fcolor), timed with CUDA events around a graph of its
-    # launches in the V-cycle mix (every level, both colours), or with
+    # launches on every level, both colours, or with
     # --persistent the persistent V-cycle kernel (one cooperative launch per
-    # V-cycle); beside it the whole FP64 V-cycle of the per-level path
+    # V-cycle); beside it the whole FP64 V-cycle of the captured path
     roof = None
     f64 = None
     if not args.no_profile:
@@ -547,8 +547,9 @@ def run_gpu(args):
                                 "and this colour's G read (4 + 4), this colour written (4); int64 fixed point"
                                 if not PERSIST else "V-cycle model, 24 B per cell and sweep"),
                 "fp64_instr_per_launch": round(kflops),
-                "note": ("mean over %d graph-launched colour passes of every level "
-                         "(the V-cycle mix), CUDA events on the launching stream; the level "
+                "note": ("mean over %d graph-launched colour passes of every level, one launch each "
+                         "(a V-cycle runs the visits of levels of at most 1216 boxes as one launch per "
+                         "leg), CUDA events on the launching stream; the level "
                          "kernels use no FP64 instruction" % kn) if not PERSIST else
                         ("mean over %d launches, each one whole V-cycle, CUDA events on the "
                          "launching stream; bytes from the per-level model" % kn)}
@@ -559,7 +560,8 @@ def run_gpu(args):
                               "hbm_frac": round(vbytes / (vus * 1e-6) / 1e9 / peak, 4),
                               "fp64_instr": round(vinstr),
                               "note": "whole FP64 V-cycle (fixed-point level kernels, FP64 level-0 solve), "
-                                      "per-level launches in a CUDA graph, bytes from the per-level model"}
+                                      "one launch per leg of a small level, in a CUDA graph, bytes from the "
+                                      "per-level model"}
     # the same step with the mixed-precision solve (FP32 error equation in an
     # FP64 defect-correction loop) on a second solver of the same workload
     mixed = None
@@ -629,10 +631,10 @@ def run_gpu(args):
         sus = per_call(lambda: g.fluid_stage(dt))
         fluid = {"fp64_peak": f64}
         # FP64 instructions per leaf cell as counted by ncu on this workload
-        # (32 x smsp__inst_executed_pipe_fp64 / leaf cells: k_field 17.4 with
-        # the FP64 square root of |E|, stage-1 k_update 64.0); bytes:
-        # compulsory traffic
-        for name, us, bpc, ipc in (("field (k_field)", fus, 16.0, 17.4), ("euler stage (k_update)", sus, 72.0, 64.0)):
+        # (32 x smsp__inst_executed_pipe_fp64 / leaf cells: k_field 13.1 with
+        # the square root of |E|, stage-1 k_update 52.7); bytes: compulsory
+        # traffic
+        for name, us, bpc, ipc in (("field (k_field)", fus, 16.0, 13.1), ("euler stage (k_update)", sus, 72.0, 52.7)):
             fluid[name] = {"us": round(us, 2), "gbs": round(leaf_cells * bpc / (us * 1e-6) / 1e9, 1),
                            "hbm_frac": round(leaf_cells * bpc / (us * 1e-6) / 1e9 / peak, 4),
                            "fp64_ginstr": round(leaf_cells * ipc / (us * 1e-6) / 1e9, 1),
@@ -1039,8 +1041,8 @@ def bench_axisymmetric(args, dev, world):
            "workload": "axi_streamer", "geometry": "axisymmetric (r, z)", "boxes": len(t["level"]),
            "leaf_cells": leaf_cells, "levels": int(len(t["level_offset"]) - 1), "tol": TOL,
            "dtype": "f64", "l2": "flushed between steps",
-           "note": "per-level launches, each V-cycle a CUDA graph (one per top level), one residual "
-                   "read per V-cycle", "paper_schedule": paper, "regrid": regrid}
+           "note": "one launch per leg of a level; a solve is one CUDA graph with the cycle loop on the device",
+           "paper_schedule": paper, "regrid": regrid}
     g.close()
     return res
 

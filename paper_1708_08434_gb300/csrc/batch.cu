@@ -6,9 +6,9 @@
 // N halved while it is even and larger than 8; the coarsest grid (at most
 // 16 per side) is solved exactly in FP64 by separable eigenbases.  The work
 // of all solves at one level index is one work list, processed by one
-// grid-stride ("persistent") launch per level and phase: z-marching columns
-// for the smoother (a whole red-black sweep per launch), the prolongation
-// and the FP64 outer residual, small 3-D tiles for the restriction.  The
+// launch per level and phase: z-marching columns for the smoother (a whole
+// red-black sweep per launch), the prolongation, the FP64 outer residual and
+// the restriction of large levels, small 3-D tiles for that of the others.  The
 // cycle is a correction-scheme V(nu1,nu2) in FP32 on the error equation
 // inside a per-solve FP64 defect-correction loop (residual and
 // accumulation in FP64); converged solves are masked out.  A whole batched solve is one
@@ -36,9 +36,11 @@ constexpr int SHAPE_COLS = 4;
 // candidate tile shapes (x, y, z), x fastest in memory; the column schedule
 // uses 8x8x8 tiles on the levels with less than a wave of columns
 constexpr int SHAPES[NSHAPES][3] = {{8, 8, 8}, {16, 8, 4}, {32, 4, 4}, {32, 8, 2}, {8, 8, 8}};
-// blocks per SM tried by the autotuner; past the resident count the hardware
-// hands out the remaining columns as blocks finish, which evens out columns
-// of uneven length (256-solve batch: 38.6 ms at 8, 37.7 ms at 32)
+// blocks per SM tried by the autotuner for the grid-stride launches (the
+// residual of phi = 0, the prolongation, the restriction tiles); past the
+// resident count the hardware hands out the remaining columns as blocks
+// finish, which evens out columns of uneven length.  The sweep, the outer
+// residual and the column restriction launch a block per column.
 constexpr int GRID_MULTS[5] = {2, 4, 8, 16, 32};
 
 struct BSolve {
@@ -182,7 +184,7 @@ __device__ __forceinline__ float wall_w(const Bc &bc, int a, int v, int N) {
 // p-1).  Cells outside the grid are zero in the slots and in the registers;
 // the wall ghosts enter through the coefficient w of c.
 template <bool ZERO, bool PHI>
-__global__ void __launch_bounds__(ST, PHI ? 5 : 6) k_bt_sweep(const int4 *__restrict__ cols, int k,
+__global__ void __launch_bounds__(ST, 6) k_bt_sweep(const int4 *__restrict__ cols, int k,
                                                               const BSolve *__restrict__ tab,
                                                               const unsigned char *__restrict__ active,
                                                               const float *__restrict__ e_in,
