@@ -921,7 +921,7 @@ struct FxNorm {
 // boxes of level l-1 (final once level l is prolonged into) to nm.slot.
 // The same integer sums as fx_prolong_box (the persistent kernel's): the
 // same bits.
-__global__ void __launch_bounds__(128) k_fprolong_rows(int lo, int n, int mode, long long *__restrict__ phx,
+__global__ void __launch_bounds__(128, 12) k_fprolong_rows(int lo, int n, int mode, long long *__restrict__ phx,
                                                        const long long *__restrict__ oldx,
                                                        long long *__restrict__ ghx,
                                                        const int32_t *__restrict__ nbr6,
