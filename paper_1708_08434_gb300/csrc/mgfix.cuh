@@ -1160,10 +1160,10 @@ __global__ void __launch_bounds__(GT) k_fresnorm(const int32_t *__restrict__ lea
 // eigenvalue scaling, x backward), then the x-slab r (y backward from the 8
 // y-slabs, z backward, store).
 // With fas != 0 it first completes the FAS right-hand side of the level-0
-// box (the work of k_ffas on it: every face is a wall), each block for its
-// plane from the whole box staged with its wall ghosts; the box's potential
-// is only written after the last cluster barrier, when every block has
-// read it.
+// box (the work of k_ffas on it: every face is a wall), each thread from its
+// cell's neighbours, whose loads are in flight together; the box's potential
+// is only written after the first cluster barrier, when every block has
+// read it.  Latency bounds it: a V-cycle waits for this one launch.
 __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(64)
     k_fcoarse8(long long *__restrict__ phx, long long *__restrict__ gx, long long *__restrict__ oldx,
                const double *__restrict__ basis, Bc bc, double h2, double inv_h2, int fas,
@@ -1171,7 +1171,6 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(64)
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
   __shared__ double pa[64], pb[64], sd[64], se[64], V[192], lam[24];
-  __shared__ long long sx[1000];
   const int r = (int)cl.block_rank(), t = threadIdx.x, lo = t & 7, hi = t >> 3;
   for (int i = t; i < 216; i += 64) {
     if (i < 192) V[i] = __ldg(basis + i);
@@ -1186,18 +1185,20 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(64)
   const int pp = xsplit(cidx(lo, hi, r));
   long long G;
   if (fas) {
-    for (int i = t; i < CELLS; i += 64) sx[s10(i)] = phx[xsplit(i)];
-    __syncthreads();
-    for (int i = t; i < 6 * FACE; i += 64) {
-      const int f = i >> 6, u = i & 7, w = (i >> 3) & 7, a = f >> 1;
-      const int q = s10(face_cell(f, u, w)), stride = a == 0 ? 1 : (a == 1 ? 10 : 100);
-      const long long inner = sx[q];
-      sx[q + ((f & 1) ? stride : -stride)] = bc.type[f] ? fx_2g(sc, f) - inner : inner;
+    const int c[3] = {lo, hi, r};
+    const long long own = phx[pp], g0 = gx[pp];
+    long long nb[6];
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      int q[3] = {lo, hi, r};
+      q[f >> 1] += (f & 1) ? 1 : -1;
+      const bool wall = c[f >> 1] == ((f & 1) ? NC - 1 : 0);
+      nb[f] = wall ? (bc.type[f] ? fx_2g(sc, f) : 0) : phx[xsplit(cidx(q[0], q[1], q[2]))];
+      if (wall) nb[f] += bc.type[f] ? -own : own;
     }
-    __syncthreads();
-    const int q = s10(cidx(lo, hi, r));
-    oldx[pp] = sx[q];
-    G = fx_rdiv<12>(gx[pp] - 2 * fx_T(sx, q));
+    oldx[pp] = own;
+    const long long T = ((nb[0] + nb[1]) + (nb[2] + nb[3])) + (nb[4] + nb[5]) - 6 * own;
+    G = fx_rdiv<12>(g0 - 2 * T);
     bad |= fx_bad(G);
     gx[pp] = G;
   } else {
@@ -1249,13 +1250,16 @@ __global__ void __cluster_dims__(8, 1, 1) __launch_bounds__(64)
     }
     se[t] = acc;
   }
-  cl.sync();  // the other blocks' reads of sd are done; se is complete
+  // this block's reads of the others' sd are done; sd is kept until theirs are
+  auto token = cl.barrier_arrive();
+  __syncthreads();  // se is complete
   {
     double acc = 0.0;
     for (int m = 0; m < NC; ++m) acc += V[2 * 64 + hi * 8 + m] * se[lo + 8 * m];
     phx[xsplit(cidx(r, lo, hi))] = fx_of(acc, E, bad);
   }
   fx_flag(bad, sc);
+  cl.barrier_wait(std::move(token));
 }
 
 // per-level constants of the scale computation: exponent bound of h_l^2
