@@ -1180,6 +1180,7 @@ struct sm_quad {
   double *snap = nullptr;                 // regrid snapshot [6][max_boxes][64]
   int *d_rg = nullptr;                    // regrid move descriptors [max_boxes][10]
   unsigned long long *d_need = nullptr;   // refinement test: cells that need refinement, per box
+  char *rgw = nullptr;                    // scratch of a regrid (QRgScratch)
   unsigned char *d_fine = nullptr;        // refinement test: derefinable, per box
   int lut_n = 0;
   double lut_emax = 0.0;
@@ -1885,16 +1886,61 @@ extern "C" int sm_quad_destroy(sm_quad *q) {
 namespace {
 struct QLayout {
   size_t lev, par, chl, nbr8, pn, ref, ij, w, wv, var[NV], cflux, ainv, lut, h, slots, err, xch, xseq, rcount, snap, rg, need, fine,
-      total;
+      rgw, total;
 };
-QLayout qlayout(const sm_quad *q) {
-  QLayout L{};
+
+// hands out 256-byte aligned parts of a range, and counts them when there is
+// no range yet
+struct Parts {
+  char *base = nullptr;
   size_t t = 0;
-  auto take = [&](size_t bytes) {
+  size_t take(size_t bytes) {
     const size_t at = t;
     t = (t + bytes + 255) & ~(size_t)255;
     return at;
-  };
+  }
+  template <typename T>
+  T *of(size_t n) {
+    const size_t at = take(sizeof(T) * n);
+    return base ? reinterpret_cast<T *>(base + at) : nullptr;
+  }
+};
+
+// scratch of a regrid on at most M boxes; at(nullptr, M) gives its size alone
+struct QRgScratch {
+  int8_t *flags;
+  int *refv, *keepv, *derv, *ref_pos, *keep_pos;
+  uint64_t *ref_keys, *kept_keys;
+  int *nlev;
+  int2 *nij;
+  uint64_t *nkey;
+  int *cnt, *counts;
+  size_t bytes;
+  static QRgScratch at(char *base, size_t M) {
+    QRgScratch S;
+    Parts p{base};
+    S.flags = p.of<int8_t>(M);
+    S.refv = p.of<int>(M);
+    S.keepv = p.of<int>(M);
+    S.derv = p.of<int>(M);
+    S.ref_pos = p.of<int>(M + 1);
+    S.keep_pos = p.of<int>(M + 1);
+    S.ref_keys = p.of<uint64_t>(M);
+    S.kept_keys = p.of<uint64_t>(M);
+    S.nlev = p.of<int>(M);
+    S.nij = p.of<int2>(M);
+    S.nkey = p.of<uint64_t>(M);
+    S.cnt = p.of<int>(2);
+    S.counts = p.of<int>(2 * QMAXL + 8);
+    S.bytes = p.t;
+    return S;
+  }
+};
+
+QLayout qlayout(const sm_quad *q) {
+  QLayout L{};
+  Parts p;
+  auto take = [&](size_t bytes) { return p.take(bytes); };
   const size_t nb = (size_t)q->max_boxes;
   L.lev = take(sizeof(int) * nb);
   L.par = take(sizeof(int) * nb);
@@ -1919,7 +1965,8 @@ QLayout qlayout(const sm_quad *q) {
   L.rg = take(sizeof(int) * 10 * nb);
   L.need = take(sizeof(unsigned long long) * nb);
   L.fine = take(nb);
-  L.total = t;
+  L.rgw = take(QRgScratch::at(nullptr, nb).bytes);
+  L.total = p.t;
   return L;
 }
 }  // namespace
@@ -1961,6 +2008,7 @@ extern "C" int sm_quad_bind_arena(sm_quad *q, void *dev_ptr, size_t bytes) {
   q->d_rg = (int *)(a + L.rg);
   q->d_need = (unsigned long long *)(a + L.need);
   q->d_fine = (unsigned char *)(a + L.fine);
+  q->rgw = a + L.rgw;
   std::vector<double> hs(3 * QMAXL);
   for (int l = 0; l < QMAXL; ++l) {
     hs[l] = q->h[l];
@@ -2230,22 +2278,12 @@ extern "C" int sm_quad_regrid(sm_quad *q, const int8_t *flags, int *n_refined, i
   const int n = n_boxes(q), M = q->max_boxes, L0 = q->nlev, T = 256;
   cudaStream_t s = q->stream;
   restrict_all(q, V_NE, V_NI);
-  // scratch in the per-call work fields (V_OLD onwards: nothing there
-  // outlives a call)
-  char *wp = reinterpret_cast<char *>(q->var[V_OLD]);
-  auto take = [&](size_t bytes) {
-    char *p = wp;
-    wp += (bytes + 255) & ~(size_t)255;
-    return p;
-  };
-  int8_t *dflags = (int8_t *)take((size_t)n);
-  int *refv = (int *)take(4 * (size_t)n), *keepv = (int *)take(4 * (size_t)n), *derv = (int *)take(4 * (size_t)n);
-  int *ref_pos = (int *)take(4 * ((size_t)n + 1)), *keep_pos = (int *)take(4 * ((size_t)n + 1));
-  uint64_t *ref_keys = (uint64_t *)take(8 * (size_t)n), *kept_keys = (uint64_t *)take(8 * (size_t)n);
-  int *nlev = (int *)take(4 * (size_t)M);
-  int2 *nij = (int2 *)take(8 * (size_t)M);
-  uint64_t *nkey = (uint64_t *)take(8 * (size_t)M);
-  int *cnt = (int *)take(8), *counts = (int *)take(4 * (2 * QMAXL + 8));
+  const QRgScratch S = QRgScratch::at(q->rgw, (size_t)M);
+  int8_t *const dflags = S.flags;
+  int *const refv = S.refv, *const keepv = S.keepv, *const derv = S.derv, *const ref_pos = S.ref_pos;
+  int *const keep_pos = S.keep_pos, *const nlev = S.nlev, *const cnt = S.cnt, *const counts = S.counts;
+  uint64_t *const ref_keys = S.ref_keys, *const kept_keys = S.kept_keys, *const nkey = S.nkey;
+  int2 *const nij = S.nij;
   const int gb = (n + T - 1) / T;
   if (cudaMemcpyAsync(dflags, flags, (size_t)n, cudaMemcpyHostToDevice, s) != cudaSuccess ||
       cudaMemsetAsync(cnt, 0, 8, s) != cudaSuccess)
