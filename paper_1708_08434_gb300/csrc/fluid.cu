@@ -149,19 +149,19 @@ __device__ __forceinline__ void dt_terms(const double *__restrict__ phi, const d
                               : pot_ghost(phi, nbr6, gh, b, 2 * a + 1, c[0], c[1], c[2], pc, bc, 0);
     d[a] = dabs(pm - pp);
   }
-  adv = mu * ((d[0] + d[1]) + d[2]);
+  adv = dabs(mu) * ((d[0] + d[1]) + d[2]);
   ad = fma(12.0, fma(w, cd.y, cd.x), adv);
   drt = mu * ne;
 }
 
-// block maxima of three non-negative quantities (negative values count as
-// 0) into slots[0..2], compared as bit patterns on the integer pipe, the
+// block maxima of three non-negative quantities (negative values and NaNs
+// count as 0) into slots[0..2], compared as bit patterns on the integer pipe, the
 // first two times scale (rounding is monotonic: the maximum of the products
 // is the product of the maximum); red: 3 * (blockDim.x / 32) words of shared
 // memory
 __device__ __forceinline__ void block_max3_to(unsigned long long *slots, double a, double b, double c,
                                               long long *red, double scale) {
-  long long v[3] = {max(dbits(a), 0ll), max(dbits(b), 0ll), max(dbits(c), 0ll)};
+  long long v[3] = {size_bits(a), size_bits(b), size_bits(c)};
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(UT, 5) k_update(
   }
   __syncthreads();
   const double dth = -dt * ih2;
-  double m_adv = 0.0, m_ad = 0.0, m_drt = 0.0;
+  long long m_adv = 0, m_ad = 0, m_drt = 0;  // maxima of bit patterns, as block_max3_to compares them
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
     const int pi = t + UT * s;
@@ -426,13 +426,12 @@ __global__ void __launch_bounds__(UT, 5) k_update(
         // sum_d mu |E_d| 2 dx, that plus 12 D (both times 1/(2 dx^2) below), mu n_e
         const double gx = dabs(S.p[q - 1] - S.p[q + 1]), gy = dabs(S.p[q - PY] - S.p[q + PY]),
                      gz = dabs(S.p[q - PZ] - S.p[q + PZ]);
-        const double adv = mu * ((gx + gy) + gz);
+        const double adv = dabs(mu) * ((gx + gy) + gz);
         const double2 cd = __ldg(tb.fc + 2 * i + 1);
         const double ad = fma(12.0, fma(w, cd.y, cd.x), adv), drt = mu * nes;
-        // maxima of bit patterns, as block_max3_to compares them
-        m_adv = dbits(adv) > dbits(m_adv) ? adv : m_adv;
-        m_ad = dbits(ad) > dbits(m_ad) ? ad : m_ad;
-        m_drt = dbits(drt) > dbits(m_drt) ? drt : m_drt;
+        m_adv = max(m_adv, size_bits(adv));
+        m_ad = max(m_ad, size_bits(ad));
+        m_drt = max(m_drt, size_bits(drt));
       }
       f[c] = (ni_new[c] - ne_new[c]) * qie;
     }
@@ -440,7 +439,9 @@ __global__ void __launch_bounds__(UT, 5) k_update(
     reinterpret_cast<double2 *>(ni_dst + base)[pi] = make_double2(ni_new[0], ni_new[1]);
     reinterpret_cast<double2 *>(rhs + base)[pi] = make_double2(f[0], f[1]);
   }
-  if (HEUN) block_max3_to(slots + SC_ADV, m_adv, m_ad, m_drt, S.red, 0.5 * ih2);
+  if (HEUN)
+    block_max3_to(slots + SC_ADV, __longlong_as_double(m_adv), __longlong_as_double(m_ad),
+                  __longlong_as_double(m_drt), S.red, 0.5 * ih2);
 }
 
 // ---------------------------------------------------------------------------

@@ -42,6 +42,13 @@ inline void table_pack(double *out, int n, const double *mu, const double *diff,
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 __device__ __forceinline__ double dabs(double x) { return __longlong_as_double(dbits(x) & 0x7fffffffffffffffll); }
 
+// bits of a non-negative number (infinity included), 0 for anything else: as
+// integers a maximum of these leaves NaNs and negative values out
+__device__ __forceinline__ long long size_bits(double x) {
+  const unsigned long long b = (unsigned long long)dbits(x);
+  return b <= 0x7ff0000000000000ull ? (long long)b : 0ll;
+}
+
 // psi(a/b) b for the Koren limiter psi(x) = max(0, min(1, (2+x)/6, x)),
 // without the division: 0 when a b <= 0 (a or b is +-0, or their signs
 // differ: tested on the bits, with no product), else

@@ -46,6 +46,7 @@ using sm::face_flux_d;
 using sm::half_index;
 using sm::halve;
 using sm::index_split;
+using sm::size_bits;
 using sm::sqrt_newton;
 
 namespace {
@@ -598,24 +599,23 @@ __device__ __forceinline__ void max_word(unsigned long long *slot, long long x) 
   if ((threadIdx.x & 31) == 0) atomicMax(slot, (unsigned long long)max(x, 0ll));
 }
 
-// maxima over a box (a warp) of the three time-step quantities, the first two
-// times scale, into slots[0..2] (bit patterns; the products' maximum is the
+// maxima over a box (a warp) of the three time-step quantities (bit patterns),
+// the first two times scale, into slots[0..2] (the products' maximum is the
 // maximum's product, rounding being monotonic)
-__device__ __forceinline__ void max3_to(unsigned long long *slots, double adv, double ad, double drt, double scale) {
-  max_word(slots, dbits(adv * scale));
-  max_word(slots + 1, dbits(ad * scale));
-  max_word(slots + 2, dbits(drt));
+__device__ __forceinline__ void max3_to(unsigned long long *slots, const long long (&m)[3], double scale) {
+  max_word(slots, dbits(__longlong_as_double(m[0]) * scale));
+  max_word(slots + 1, dbits(__longlong_as_double(m[1]) * scale));
+  max_word(slots + 2, m[2]);
 }
 
-// sum_d mu |E_d| 2 dx of the staged potential at q, that plus 8 D (both to be
-// scaled by 1/(2 dx^2)), and mu n_e, as running maxima
-__device__ __forceinline__ void dt_cell(const double *sp, int q, double mu, double dc, double ne, double &m0,
-                                        double &m1, double &m2) {
-  const double adv = mu * (dabs(sp[q - 1] - sp[q + 1]) + dabs(sp[q - S1] - sp[q + S1]));
-  const double ad = fma(8.0, dc, adv), drt = mu * ne;
-  m0 = dbits(adv) > dbits(m0) ? adv : m0;
-  m1 = dbits(ad) > dbits(m1) ? ad : m1;
-  m2 = dbits(drt) > dbits(m2) ? drt : m2;
+// sum_d |mu E_d| 2 dx of the staged potential at q, that plus 8 D (both to be
+// scaled by 1/(2 dx^2)), and mu n_e, as running maxima of bit patterns
+// without negative values and NaNs
+__device__ __forceinline__ void dt_cell(const double *sp, int q, double mu, double dc, double ne, long long (&m)[3]) {
+  const double adv = dabs(mu) * (dabs(sp[q - 1] - sp[q + 1]) + dabs(sp[q - S1] - sp[q + S1]));
+  m[0] = max(m[0], size_bits(adv));
+  m[1] = max(m[1], size_bits(fma(8.0, dc, adv)));
+  m[2] = max(m[2], size_bits(mu * ne));
 }
 
 // One forward Euler stage on every leaf box: dst = src - dt div F + dt
@@ -678,7 +678,7 @@ __global__ void __launch_bounds__(QT) k_q_update(int n, const double *__restrict
   }
   __syncwarp();
   const double dth = -dt * ih2;
-  double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+  long long m[3] = {0, 0, 0};
 #pragma unroll
   for (int s2 = 0; s2 < 2; ++s2) {
     const int c = lane + 32 * s2, i = c % QN, j = c / QN, q = (j + 1) * S1 + i + 1;
@@ -697,13 +697,13 @@ __global__ void __launch_bounds__(QT) k_q_update(int n, const double *__restrict
       a = halve(ne0[g] + a);
       bq = halve(ni0[g] + bq);
       const double2 cd = __ldg(tb.fc + 2 * k + 1);
-      dt_cell(sp, q, mu, fma(w, cd.y, cd.x), nes, m0, m1, m2);
+      dt_cell(sp, q, mu, fma(w, cd.y, cd.x), nes, m);
     }
     ne_out[g] = a;
     ni_out[g] = bq;
     if (rhs) rhs[g] = (bq - a) * qie;
   }
-  if (HEUN) max3_to(slots, m0, m1, m2, 0.5 * ih2);
+  if (HEUN) max3_to(slots, m, 0.5 * ih2);
 }
 
 // Volume-weighted means of the four children of one or two variables into
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(QT) k_q_dt(int n, const double *__restrict__ p
   if (C.ref & 16) return;
   double *s = sm[wv_];
   stage_phi(phi, nullptr, C, b, bc, 0, s, lane, err, v0, v1);
-  double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+  long long m[3] = {0, 0, 0};
 #pragma unroll
   for (int s2 = 0; s2 < 2; ++s2) {
     const int c = lane + 32 * s2;
@@ -770,9 +770,9 @@ __global__ void __launch_bounds__(QT) k_q_dt(int n, const double *__restrict__ p
     double w;
     const int k = index_split(2 * half_index(emag[g], tb), tb, w);
     const double2 cm = __ldg(tb.fc + 2 * k), cd = __ldg(tb.fc + 2 * k + 1);
-    dt_cell(s, (c / QN + 1) * S1 + c % QN + 1, fma(w, cm.y, cm.x), fma(w, cd.y, cd.x), ne[g], m0, m1, m2);
+    dt_cell(s, (c / QN + 1) * S1 + c % QN + 1, fma(w, cm.y, cm.x), fma(w, cd.y, cd.x), ne[g], m);
   }
-  max3_to(slots, m0, m1, m2, 0.5 * hs[QMAXL + C.lev]);
+  max3_to(slots, m, 0.5 * hs[QMAXL + C.lev]);
 }
 
 // alpha(e) from the table with every operation rounded on its own (no fused
