@@ -559,10 +559,13 @@ const char *sm_cnn_last_error(const sm_cnn *c);
  *   stream:  cudaStream_t as void*; the call only enqueues work.
  * The library allocates nothing and keeps nothing on the device: the
  * eigenbases travel as launch parameters, so calls on different streams are
- * independent.  The first call on a device loads the kernels (with the
- * device current); make that first call before any stream capture.  Device
- * ordinals 0..63 are supported.
- * Errors: SM_ENOMEM if n_problems > SM_NOALLOC_MAX_PROBLEMS, SM_EINVAL
+ * independent.  The first call on a device, of any problem count (0 too),
+ * loads the kernels of all counts (with the device current); make that first
+ * call before any stream capture.  After a device reset (cudaDeviceReset)
+ * the kernels are loaded again as they are launched.  Device ordinals 0..63
+ * are supported.
+ * Errors: SM_ENOMEM if n_problems > SM_NOALLOC_MAX_PROBLEMS (the largest
+ * call this entry point has always taken; nothing is sized by it), SM_EINVAL
  * (n_problems < 0, length <= 0, null pointer, device ordinal above 63),
  * SM_ECUDA (no device, first call of a device inside a stream capture,
  * launch failed). */

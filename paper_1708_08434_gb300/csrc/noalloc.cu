@@ -47,29 +47,6 @@ struct Bases {
   }
 };
 
-// The first call on a device loads the kernels, which a stream capture does
-// not allow: it has to be made outside one.
-constexpr int MAX_DEVICES = 64;
-std::mutex g_ready_mtx;
-bool g_ready[MAX_DEVICES];
-
-int device_ready(cudaStream_t stream) {
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) {
-    cudaGetLastError();
-    return SM_ECUDA;
-  }
-  if (dev < 0 || dev >= MAX_DEVICES) return SM_EINVAL;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) {
-    cudaGetLastError();
-    return SM_ECUDA;
-  }
-  std::lock_guard<std::mutex> lock(g_ready_mtx);
-  if (cs == cudaStreamCaptureStatusNone) g_ready[dev] = true;
-  return g_ready[dev] ? SM_OK : SM_ECUDA;
-}
-
 // a / d for |d| between 2^-100 and 2^100 and normal a: a single-precision
 // reciprocal, one Newton step, and the quotient corrected by its remainder
 // (five FP64 instructions)
@@ -160,6 +137,41 @@ __global__ void __launch_bounds__(CELLS / C) k_box_solve(const double *__restric
   for (int m = 0; m < NC; ++m) acc = fma(V[1][j * 8 + m], of(pb, m / S)[i + 8 * z + 64 * (m % S)], acc);
   phi[(size_t)p * CELLS + 64 * S * r + t] = acc;
   if constexpr (C > 1) cl.sync();  // no block leaves while its shared memory is read
+}
+
+// The first call on a device loads the kernels, all of them whatever its
+// problem count: CUDA would load each when it is first launched (10 us for a
+// kernel, 110 for the module), inside a stream capture or where nothing may
+// be loaded or allocated.  So that call has to be made outside a capture.
+constexpr int MAX_DEVICES = 64;
+std::mutex g_ready_mtx;
+bool g_ready[MAX_DEVICES];
+
+int device_ready(cudaStream_t stream) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return SM_ECUDA;
+  }
+  if (dev < 0 || dev >= MAX_DEVICES) return SM_EINVAL;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &cs) != cudaSuccess) {
+    cudaGetLastError();
+    return SM_ECUDA;
+  }
+  std::lock_guard<std::mutex> lock(g_ready_mtx);
+  if (g_ready[dev]) return SM_OK;
+  if (cs != cudaStreamCaptureStatusNone) return SM_ECUDA;
+  cudaFuncAttributes a;  // asking for them loads the kernel
+  if (cudaFuncGetAttributes(&a, k_box_solve<1>) != cudaSuccess ||
+      cudaFuncGetAttributes(&a, k_box_solve<2>) != cudaSuccess ||
+      cudaFuncGetAttributes(&a, k_box_solve<4>) != cudaSuccess ||
+      cudaFuncGetAttributes(&a, k_box_solve<8>) != cudaSuccess) {
+    cudaGetLastError();
+    return SM_ECUDA;
+  }
+  g_ready[dev] = true;
+  return SM_OK;
 }
 
 template <int C>
