@@ -37,6 +37,7 @@ constexpr long long FX_LIM = 1ll << 55;     // |stored value| < FX_LIM quanta
 constexpr int FX_MARGIN = 5;                // E = exponent bound + margin
 constexpr int FX_EMIN = 64;                 // keeps q and q/h^2 normal
 constexpr unsigned long long FX_ERR_OVF = 8ull;
+constexpr unsigned long long ERR_WAIT = 4ull;  // a wait between blocks ran out (ERR_BARRIER of the persistent kernel)
 
 __device__ __forceinline__ bool fx_bad(long long x) {
   return (unsigned long long)(x + FX_LIM) >= (unsigned long long)(2 * FX_LIM);
@@ -1365,12 +1366,13 @@ __global__ void __launch_bounds__(GT) k_fx_init(const int32_t *__restrict__ leve
   group_umax_to(block_grp(), den, m, red);
 }
 
-// phi = phx q for every box, unless the solve left the fixed-point range
-// (its FP64 inputs then stay as they were for the next attempt)
+// phi = phx q for every box, unless the solve left the fixed-point range or a
+// wait between blocks ran out (its FP64 inputs then stay as they were for the
+// next attempt)
 __global__ void __launch_bounds__(GT) k_fx_final(const long long *__restrict__ phx, double *__restrict__ phi,
                                                  const unsigned long long *__restrict__ sc) {
   pdl_wait();
-  if (sc[SC_ERR] & FX_ERR_OVF) return;
+  if (sc[SC_ERR] & (FX_ERR_OVF | ERR_WAIT)) return;
   const double q = fx_q(fx_E(sc));
   const size_t base = (size_t)blockIdx.x * CELLS;
 #pragma unroll

@@ -34,8 +34,9 @@
 // that very word, so it cannot be overwritten unread.
 //
 // The launch is cooperative: all blocks are resident, so every awaited
-// block runs.  A poll gives up after WAIT_SPIN tries (ERR_WAIT, the solve
-// returns SM_ETIMEOUT); later launches of the solve then return at once.
+// block runs.  A poll gives up after WAIT_SPIN tries (ERR_WAIT); the launch's
+// other waits run to their own limits, later launches of the solve return at
+// once, and the solve runs again with a launch per operation.
 //
 // What a block reads of its neighbours' cells in memory, at the start of a
 // down leg, they overwrite only after awaiting words whose values depend on
@@ -54,14 +55,13 @@ namespace fx {
 
 enum { FS_TOP = 0, FS_FAS = 1, FS_PROLONG = 2, FS_FMG = 3 };  // how a leg starts
 
-constexpr unsigned long long ERR_WAIT = 4ull;  // also the persistent kernel's barrier flag
-constexpr int WAIT_SPIN = 1 << 18;             // polls of one wait (a few tenths of a second)
+constexpr int WAIT_SPIN = 1 << 18;             // polls of one wait (0.06 s)
 constexpr int LEG_MAX_NU = 7;                  // 2 nu + 1 publications fit the tag's 16
 
 struct LevArgs {
   int lo, nu;            // first box, sweeps
   int set_phx;           // down leg: restricted values also go to phx (else to oldx alone)
-  unsigned leg, skew;    // tag offset of the leg; skew != 0 only in the self-test
+  unsigned leg, skew;    // tag offset of the leg; skew != 0 only in the self-tests
   long long *phx, *gx, *oldx, *ghx, *xch;  // xch: words of box lo
   const int32_t *rows;  // k_leg_rows
   const unsigned *seq;  // xseq of the level

@@ -1801,7 +1801,7 @@ static int leg_limit(sm_ctx *ctx) {
 // whether the legs of level l run in one launch each
 static bool leg_level(sm_ctx *ctx, int l) {
   const int n = lvl_n(ctx, l);
-  return l >= 1 && l < ctx->n_levels && n > 0 && n <= leg_limit(ctx) && n < ctx->rows_min &&
+  return !ctx->legs_off && l >= 1 && l < ctx->n_levels && n > 0 && n <= leg_limit(ctx) && n < ctx->rows_min &&
          ctx->cfg.nu1 <= fx::LEG_MAX_NU && ctx->cfg.nu2 <= fx::LEG_MAX_NU;
 }
 
@@ -1817,7 +1817,7 @@ static int fx_leg(sm_ctx *ctx, int l, unsigned skew = 0) {
   a.nu = up ? ctx->cfg.nu2 : ctx->cfg.nu1;
   a.set_phx = START != fx::FS_FMG || l == 1;
   a.leg = up ? 0u : 16u;
-  a.skew = skew;
+  a.skew = skew ? skew : ctx->leg_skew;
   a.phx = ctx->phx;
   a.gx = ctx->gx;
   a.oldx = (long long *)ctx->old;
@@ -2117,6 +2117,7 @@ static sm_graph *graph_of(sm_ctx *ctx, int kind) {
 
 void sm_drop_graphs(sm_ctx *ctx) {
   ctx->xch_reset = true;
+  ctx->legs_off = false;
   for (auto *g : {&ctx->g_solve, &ctx->g_fmg, &ctx->g_solve32, &ctx->g_fmg32}) {
     if (g->exec) cudaGraphExecDestroy(g->exec);
     g->exec = nullptr;
@@ -2241,8 +2242,9 @@ static int capture_solve(sm_ctx *ctx, int kind, sm_graph *out) {
 }
 
 // One attempt of a solve: SM_OK with the cycle count and relative
-// residual, SM_FX_RETRY when the fixed-point potential left its range (phi
-// is then unchanged), or an error.
+// residual, SM_FX_RETRY when the fixed-point potential left its range,
+// SM_ETIMEOUT when a wait between blocks ran out (phi is unchanged after
+// either), or an error.
 static int run_solve_once(sm_ctx *ctx, int kind, double tol, int max_cycles, int *cycles, double *rel_res) {
   int st;
   int c = 0;
@@ -2306,6 +2308,30 @@ static int fx_widen(sm_ctx *ctx, bool *again) {
   *again = ctx->fx_margin < 5 + 4 * 8;
   if (*again) ctx->fx_margin += 8;
   return SM_OK;
+}
+
+// After an attempt that ended with `st`: whether the work runs again, with
+// st = SM_OK then.  After SM_FX_RETRY with a wider scale; after a wait of a
+// one-launch leg that ran out (the blocks of a leg got no turn on the GPU for
+// that long) with a launch per operation, which holds until the mesh or the
+// choice of kernels changes.
+static bool fx_again(sm_ctx *ctx, int &st, bool legs) {
+  bool again = false;
+  if (st == SM_FX_RETRY) {
+    if ((st = fx_widen(ctx, &again))) return false;
+    if (!again)
+      st = sm_fail(ctx, SM_ENOCONV, "potential or right-hand side not finite or beyond 2^%d of its scale",
+                   ctx->fx_margin);
+  } else if (st == SM_ETIMEOUT && legs) {
+    for (int l = 1; l < ctx->n_levels; ++l) again = again || leg_level(ctx, l);
+    if (again) {
+      sm_drop_graphs(ctx);
+      ctx->leg_skew = 0;
+      ctx->legs_off = true;
+      st = SM_OK;
+    }
+  }
+  return again;
 }
 
 static void vcycle_model(const sm_ctx *ctx, int top, bool fixed, double *bytes, double *ops);
@@ -2399,13 +2425,8 @@ static int run_solve_logged(sm_ctx *ctx, int fmg, double tol, int max_cycles, in
   memcpy(&ctx->hscal[SC_MAXC], &mc, sizeof mc);
   SM_CK(cudaMemcpyAsync(ctx->dscal + SC_TOL, ctx->hscal + SC_TOL, 2 * sizeof(double), cudaMemcpyHostToDevice,
                         ctx->stream));
-  while ((st = run_solve_once(ctx, kind, tol, max_cycles, &c, &rel)) == SM_FX_RETRY) {
-    bool again = false;
-    if ((st = fx_widen(ctx, &again))) return st;
-    if (!again)
-      return sm_fail(ctx, SM_ENOCONV, "potential or right-hand side not finite or beyond 2^%d of its scale",
-                     ctx->fx_margin);
-  }
+  do st = run_solve_once(ctx, kind, tol, max_cycles, &c, &rel);
+  while (fx_again(ctx, st, kind < 2 && !ctx->persist));
   if (st) return st;
   if (cycles) *cycles = c;
   if (rel_res) *rel_res = rel;
@@ -2470,17 +2491,14 @@ extern "C" int sm_mg_vcycle(sm_ctx *ctx, int n_cycles, double *rel_res) {
   if (n_cycles < 0) return SM_EINVAL;
   if ((st = ensure_basis(ctx))) return st;
   const int top = ctx->n_levels - 1;
-  for (;;) {
+  do {
     if ((st = fx_set_margin(ctx))) return st;
     if ((st = fx_solve_prefix(ctx, 0, false))) return st;
     for (int c = 0; c < n_cycles; ++c)
       if ((st = ctx->persist ? persistx_launch(ctx, top, 0, 0) : fx_vcycle(ctx, top))) return st;
     if ((st = fx_epilogue(ctx))) return st;
-    if ((st = read_scalars(ctx)) != SM_FX_RETRY) break;
-    bool again = false;
-    if ((st = fx_widen(ctx, &again))) return st;
-    if (!again) return sm_fail(ctx, SM_ENOCONV, "potential or right-hand side beyond the fixed-point range");
-  }
+    st = read_scalars(ctx);
+  } while (fx_again(ctx, st, !ctx->persist));
   if (st) return st;
   double rel = 0.0;
   if ((st = rel_residual(ctx, &rel))) return st;
@@ -2529,6 +2547,15 @@ extern "C" int sm_persist_barrier_selftest(sm_ctx *ctx) {
   SM_CK(cudaMemsetAsync(ctx->dscal + SC_ERR, 0, sizeof(unsigned long long), ctx->stream));
   SM_CK(cudaStreamSynchronize(ctx->stream));
   return st;
+}
+
+extern "C" int sm_leg_wait_selftest(sm_ctx *ctx) {
+  int st = check_ready(ctx);
+  if (st) return st;
+  if (!leg_level(ctx, 1)) return sm_fail(ctx, SM_ESTATE, "no level runs in one-launch legs");
+  sm_drop_graphs(ctx);  // captured legs hold their waits' tags
+  ctx->leg_skew = 128;
+  return SM_OK;
 }
 
 extern "C" int sm_set_persistent(sm_ctx *ctx, int enable) {

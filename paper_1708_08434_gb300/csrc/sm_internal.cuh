@@ -122,6 +122,8 @@ struct sm_ctx {
   unsigned *xseq = nullptr;  // [MAXL]
   int32_t *leg_rows = nullptr;  // [max_boxes][16] what a leg needs to know of a box
   int leg_max = -1;          // boxes of the largest such level (co-resident blocks; -1: not looked up)
+  bool legs_off = false;     // a wait ran out on this mesh: every level by separate launches
+  unsigned leg_skew = 0;     // != 0: the legs' waits run out (sm_leg_wait_selftest)
   bool xch_reset = true;     // clear both before the next solve (new mesh, other kernels chosen, a wait that ran out)
   int fx_margin = 5;         // exponent margin of the fixed-point scale
   int rows_min = 2048;       // boxes of a level from which its fixed-point kernels work by rows
