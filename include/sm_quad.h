@@ -115,8 +115,16 @@ int sm_quad_fmg(sm_quad *q, double tol, int max_cycles, int *cycles, double *rel
 int sm_quad_solve(sm_quad *q, double tol, int max_cycles, int *cycles, double *rel);
 
 /* n V-cycles from the current potential with no residual evaluation
- * (enqueue only; for timing and fixed schedules). */
+ * (enqueue only; for timing and fixed schedules).  A wait between blocks
+ * that ran out in them (see sm_quad_set_graphs) is reported as SM_ETIMEOUT by
+ * the next sm_quad_download, sm_quad_dt_limit or sm_quad_regrid, whose results
+ * are then void (a regrid changes nothing); a solve goes on from the potential
+ * as they left it. */
 int sm_quad_vcycles(sm_quad *q, int n);
+/* Self-test: in the next V-cycles every wait between the blocks of a
+ * one-launch leg expects a word that is never published and runs out.
+ * Errors: SM_ESTATE (no arena, or no level that has such legs). */
+int sm_quad_leg_wait_selftest(sm_quad *q);
 
 /* |E| on leaf cells from the current potential (zero on refined boxes). */
 int sm_quad_compute_field(sm_quad *q);
@@ -167,8 +175,9 @@ int sm_quad_regrid(sm_quad *q, const int8_t *flags, int *n_refined, int *n_deref
  * changes; 0: the same launches are issued from the host.  Results are
  * identical.  On a level whose boxes are all resident at once each leg of a
  * V-cycle is one cooperative launch whose blocks pass face cells to one
- * another; a wait that runs out (a few tenths of a second) ends the launch
- * and the solve returns SM_ETIMEOUT. */
+ * another; a wait that runs out (0.11 s each) ends the launch, and the
+ * solve runs again from the potential it started with in a launch per
+ * operation, as the following ones do until the mesh changes. */
 int sm_quad_set_graphs(sm_quad *q, int on);
 /* on != 0 (the default): the V-cycle kernels are launched with programmatic
  * dependent launch (each loads its box's tables while its predecessor

@@ -76,7 +76,7 @@ EXPORTS = ["sm_create", "sm_destroy", "sm_arena_size", "sm_bind_arena", "sm_buil
            "sm_quad_create", "sm_quad_destroy", "sm_quad_arena_size", "sm_quad_bind_arena",
            "sm_quad_refine_level", "sm_quad_get_tables", "sm_quad_var_ptr", "sm_quad_upload",
            "sm_quad_download", "sm_quad_set_table", "sm_quad_charge_rhs", "sm_quad_fmg",
-           "sm_quad_solve", "sm_quad_vcycles", "sm_quad_compute_field", "sm_quad_dt_limit", "sm_quad_fluid_stage",
+           "sm_quad_solve", "sm_quad_vcycles", "sm_quad_leg_wait_selftest", "sm_quad_compute_field", "sm_quad_dt_limit", "sm_quad_fluid_stage",
            "sm_quad_advance", "sm_quad_refine_flags", "sm_quad_regrid", "sm_quad_set_graphs", "sm_quad_set_pdl", "sm_quad_launch_count", "sm_quad_last_error"]
 
 
@@ -189,6 +189,7 @@ def signatures() -> dict:
         "sm_quad_fmg": [P, D, I, pI, pD],
         "sm_quad_solve": [P, D, I, pI, pD],
         "sm_quad_vcycles": [P, I],
+        "sm_quad_leg_wait_selftest": [P],
         "sm_quad_compute_field": [P],
         "sm_quad_dt_limit": [P, D, D, pD],
         "sm_quad_fluid_stage": [P, D],
@@ -831,6 +832,10 @@ class Quad:
     def vcycles(self, n: int):
         """n V-cycles, enqueued on the stream (no residual evaluation)."""
         self._ck(self._lib.sm_quad_vcycles(self._h, int(n)))
+
+    def leg_wait_selftest(self):
+        """Let the waits of the next V-cycles' one-launch legs run out."""
+        self._ck(self._lib.sm_quad_leg_wait_selftest(self._h))
 
     def compute_field(self):
         self._ck(self._lib.sm_quad_compute_field(self._h))

@@ -59,8 +59,9 @@ constexpr int QMAXL = SM_MAX_LEVELS;
 constexpr int S1 = QN + 2;       // staged side with one ghost layer
 constexpr int S2 = QN + 4;       // staged side with two ghost layers
 
-// fields in the arena: the public sm_var numbering first
-enum { V_PHI = 0, V_RHS, V_RES, V_NE, V_NI, V_EMAG, V_RHO, V_OLD, V_TMP, V_NE1, V_NI1, NV };
+// fields in the arena: the public sm_var numbering first (V_ZERO is never
+// written: the potential of the residuals' denominator)
+enum { V_PHI = 0, V_RHS, V_RES, V_NE, V_NI, V_EMAG, V_RHO, V_OLD, V_ZERO, V_NE1, V_NI1, NV };
 
 struct QBc {
   int type[4];      // 0 Neumann zero (and the axis), 1 Dirichlet
@@ -437,17 +438,23 @@ __device__ __forceinline__ void max_bits(unsigned long long *slot, double v) {
 }
 
 // max |f - L var| over the leaf cells of all boxes (var = a zero array for
-// the denominator)
+// the denominator); with `keep` every box of src is also copied there (a copy
+// of its own costs a solve 3 us)
 __global__ void __launch_bounds__(QT) k_q_resmax(int n, const double *__restrict__ var,
                                                  const double *__restrict__ rhs, QTabs T, const __grid_constant__ QBc bc,
                                                  const double *__restrict__ inv_h2, unsigned long long *slot,
-                                                 unsigned *err) {
+                                                 unsigned *err, const double *__restrict__ src,
+                                                 double *__restrict__ keep) {
   __shared__ double sm[WPB][S1 * S1];
   QWARP();
   if (k_ >= n) return;
   const int b = k_;
   double v0, v1;
   begin_box(var, T, b, C, lane, v0, v1);
+  if (keep) {
+    keep[(size_t)b * QC + lane] = src[(size_t)b * QC + lane];
+    keep[(size_t)b * QC + lane + 32] = src[(size_t)b * QC + lane + 32];
+  }
   if (C.ref & 16) return;
   double *s = sm[wv_];
   const int l = C.lev;
@@ -1177,7 +1184,9 @@ struct sm_quad {
   int *rcount = nullptr;                  // [max_boxes] children counted in by k_q_restrict_tree (zero between)
   int leg_few = 0;                        // boxes of the largest level for the form with more registers
   int leg_max = -1;                       // boxes of the largest level with such legs (-1: not looked up)
-  double *snap = nullptr;                 // regrid snapshot [6][max_boxes][64]
+  bool legs_off = false;                  // a wait ran out on this mesh: every level by separate launches
+  unsigned leg_skew = 0;                  // != 0: the legs' waits run out (sm_quad_leg_wait_selftest)
+  double *snap = nullptr;                 // snapshot of a regrid [6][max_boxes][64]; of a solve's first potential
   int *d_rg = nullptr;                    // regrid move descriptors [max_boxes][10]
   unsigned long long *d_need = nullptr;   // refinement test: cells that need refinement, per box
   char *rgw = nullptr;                    // scratch of a regrid (QRgScratch)
@@ -1438,7 +1447,13 @@ int leg_limit(sm_quad *q) {
 }
 
 bool leg_level(sm_quad *q, int l) {
-  return l >= 1 && level_count(q, l) > 0 && level_count(q, l) <= leg_limit(q);
+  return !q->legs_off && l >= 1 && level_count(q, l) > 0 && level_count(q, l) <= leg_limit(q);
+}
+
+bool any_leg(sm_quad *q) {
+  for (int l = 1; l < q->nlev; ++l)
+    if (leg_level(q, l)) return true;
+  return false;
 }
 
 template <int START>
@@ -1448,6 +1463,7 @@ void leg(sm_quad *q, int l) {
   a.lo = q->off[l];
   a.nu = up ? q->nu2 : q->nu1;
   a.leg = up ? 0u : 64u;
+  a.skew = q->leg_skew;
   a.h2 = q->h[l] * q->h[l];
   a.inv_h2 = q->inv_h2[l];
   a.phi = q->var[V_PHI];
@@ -1528,6 +1544,7 @@ void drop_graphs(sm_quad *q) {
   };
   for (auto &g : q->vgraph) drop(g);
   for (auto &g : q->sgraph) drop(g);
+  q->legs_off = false;
 }
 
 // One V-cycle with level `top` on top, as a CUDA graph captured on first
@@ -1570,23 +1587,35 @@ int vcycle_g(sm_quad *q, int top) {
 
 void restrict_all(sm_quad *q, int v, int v2 = -1);
 
-// status of the device's error word (bit 2 is cleared, so the context stays
-// usable after a wait that ran out)
+// Status of a wait of a one-launch leg that ran out, from the device's error
+// word (the stream is idle): its bit is cleared and the following V-cycles run
+// in a launch per operation, until the mesh changes.
+int wait_error(sm_quad *q, unsigned e) {
+  if (!(e & Q_ERR_WAIT)) return SM_OK;
+  const unsigned rest = e & ~Q_ERR_WAIT;
+  if (cudaMemcpyAsync(q->d_err, &rest, sizeof(rest), cudaMemcpyHostToDevice, q->stream) != cudaSuccess ||
+      cudaStreamSynchronize(q->stream) != cudaSuccess)
+    return qfail(q, SM_ECUDA, "error word");
+  drop_graphs(q);
+  q->leg_skew = 0;
+  q->legs_off = true;
+  return qfail(q, SM_ETIMEOUT, "a wait between the blocks of a kernel ran out");
+}
+
+// status of the device's error word
 int device_error(sm_quad *q, unsigned e) {
-  if (e & Q_ERR_WAIT) {
-    cudaMemsetAsync(q->d_err, 0, sizeof(unsigned), q->stream);
-    return qfail(q, SM_ETIMEOUT, "a wait between the blocks of a kernel ran out");
-  }
+  if (int st = wait_error(q, e)) return st;
   if (e) return qfail(q, SM_ESTATE, "a coarse box needed at a refinement boundary is missing");
   return SM_OK;
 }
 
-// max leaf residual of var (the potential, or the zero array) into a slot
-void resmax(sm_quad *q, int v, int slot) {
+// max leaf residual of var (the potential, or the zero array) into a slot;
+// with `keep` the potential is copied there
+void resmax(sm_quad *q, int v, int slot, double *keep = nullptr) {
   const int n = n_boxes(q);
   cudaMemsetAsync(q->slots + slot, 0, sizeof(unsigned long long), q->stream);
   k_q_resmax<<<blocks_for(n), QT, 0, q->stream>>>(n, q->var[v], q->var[V_RHS], tabs(q), q->bc, q->d_h + QMAXL,
-                                                   q->slots + slot, q->d_err);
+                                                   q->slots + slot, q->d_err, q->var[V_PHI], keep);
   ++q->launches;
 }
 
@@ -1607,10 +1636,11 @@ double bits_of(unsigned long long b) {
 }
 
 // work before the cycle loop: the residual of phi = 0 (the denominator), and
-// for FMG the restricted right-hand side, the ladder and its residual
+// for FMG the restricted right-hand side, the ladder and its residual; with
+// one-launch legs the potential the cycles start from is kept, for the case
+// that a wait runs out (FMG does not read it)
 void solve_prefix(sm_quad *q, bool fmg) {
-  cudaMemsetAsync(q->var[V_TMP], 0, sizeof(double) * QC * (size_t)n_boxes(q), q->stream);
-  resmax(q, V_TMP, QS_DEN);
+  resmax(q, V_ZERO, QS_DEN, !fmg && any_leg(q) ? q->snap : nullptr);
   if (!fmg) return;
   restrict_all(q, V_RHS);
   coarse_solve(q);
@@ -1697,10 +1727,10 @@ int capture_solve(sm_quad *q, bool fmg) {
 // FMG, or V-cycles from the current potential, until the relative residual is
 // at most tol: one graph with the loop on the device, or the same launches
 // with a read after every cycle
-int run_solve(sm_quad *q, bool fmg, double tol, int max_cycles, int *cycles, double *rel) {
+int run_solve_once(sm_quad *q, bool fmg, double tol, int max_cycles, int &c, double &r) {
   unsigned long long s[QS_N];
-  int c = 0;
-  double r = 0.0;
+  c = 0;
+  r = 0.0;
   if (q->graphs) {
     if (!q->sgraph[fmg])
       if (int st = capture_solve(q, fmg)) return st;
@@ -1728,7 +1758,22 @@ int run_solve(sm_quad *q, bool fmg, double tol, int max_cycles, int *cycles, dou
       if (int st = residual()) return st;
     }
   }
-  if (int st = check(q, "solve")) return st;
+  return check(q, "solve");
+}
+
+// The solve; when a wait of a one-launch leg ran out (its blocks got no turn
+// on the GPU for that long) once more from the potential it started with, in
+// a launch per operation.
+int run_solve(sm_quad *q, bool fmg, double tol, int max_cycles, int *cycles, double *rel) {
+  int c, st;
+  double r;
+  if ((st = run_solve_once(q, fmg, tol, max_cycles, c, r)) == SM_ETIMEOUT) {
+    if (!fmg && cudaMemcpyAsync(q->var[V_PHI], q->snap, sizeof(double) * QC * (size_t)n_boxes(q),
+                                cudaMemcpyDeviceToDevice, q->stream) != cudaSuccess)
+      return qfail(q, SM_ECUDA, "potential");
+    st = run_solve_once(q, fmg, tol, max_cycles, c, r);
+  }
+  if (st) return st;
   if (cycles) *cycles = c;
   if (rel) *rel = r;
   return r <= tol ? SM_OK : qfail(q, SM_ENOCONV, "tolerance not reached");
@@ -1784,9 +1829,12 @@ int field(sm_quad *q) {
 // the time step from the maxima in slots 0..2 (synchronises)
 int dt_read(sm_quad *q, double c, double eps, double *dt) {
   unsigned long long bits[3];
+  unsigned e = 0;
   if (cudaMemcpyAsync(bits, q->slots, sizeof(bits), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
+      cudaMemcpyAsync(&e, q->d_err, sizeof(e), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
       cudaStreamSynchronize(q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "dt limit");
+  if (int st = wait_error(q, e)) return st;
   double m[3];
   std::memcpy(m, bits, sizeof(m));
   double d = 1e300;
@@ -2106,11 +2154,13 @@ extern "C" int sm_quad_upload(sm_quad *q, int v, const double *host) {
 extern "C" int sm_quad_download(sm_quad *q, int v, double *host) {
   if (!q || !host || v < 0 || v > V_RHO) return SM_EINVAL;
   if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
+  unsigned e = 0;
   if (cudaMemcpyAsync(host, q->var[v], sizeof(double) * QC * (size_t)n_boxes(q), cudaMemcpyDeviceToHost,
                       q->stream) != cudaSuccess ||
+      cudaMemcpyAsync(&e, q->d_err, sizeof(e), cudaMemcpyDeviceToHost, q->stream) != cudaSuccess ||
       cudaStreamSynchronize(q->stream) != cudaSuccess)
     return qfail(q, SM_ECUDA, "download");
-  return SM_OK;
+  return wait_error(q, e);
 }
 
 extern "C" int sm_quad_set_table(sm_quad *q, int n, double e_max, const double *mu, const double *diff,
@@ -2157,6 +2207,15 @@ extern "C" int sm_quad_vcycles(sm_quad *q, int n) {
   for (int c = 0; c < n; ++c)
     if (int st = vcycle_g(q, q->nlev - 1)) return st;
   return check(q, "V-cycle");
+}
+
+extern "C" int sm_quad_leg_wait_selftest(sm_quad *q) {
+  if (!q) return SM_EINVAL;
+  if (!q->arena) return qfail(q, SM_ESTATE, "no arena bound");
+  if (!any_leg(q)) return qfail(q, SM_ESTATE, "no level runs in one-launch legs");
+  drop_graphs(q);  // captured legs hold their waits' tags
+  q->leg_skew = 1u << 30;
+  return SM_OK;
 }
 
 extern "C" int sm_quad_compute_field(sm_quad *q) {
@@ -2297,10 +2356,13 @@ extern "C" int sm_quad_regrid(sm_quad *q, const int8_t *flags, int *n_refined, i
   k_qrg_counts<<<1, 32, 0, s>>>(cnt, keep_pos, ref_pos, off, L0, counts);
   q->launches += 5;
   std::vector<int> hc(3 + 2 * L0 + 1);
+  unsigned ev = 0;
   if (int st = check(q, "regrid decisions")) return st;
   if (cudaMemcpyAsync(hc.data(), counts, sizeof(int) * hc.size(), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+      cudaMemcpyAsync(&ev, q->d_err, sizeof(ev), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaStreamSynchronize(s) != cudaSuccess)
     return qfail(q, SM_ECUDA, "regrid counts");
+  if (int st = wait_error(q, ev)) return st;  // of V-cycles enqueued before: the mesh is unchanged
   const int *hk = &hc[2], *hr = &hc[3 + L0];
   const int nref = hr[L0], nder = hc[1];
   if (n_refined) *n_refined = nref;
@@ -2353,7 +2415,6 @@ extern "C" int sm_quad_regrid(sm_quad *q, const int8_t *flags, int *n_refined, i
   q->chl.resize(4 * (size_t)m);
   q->nbr8.resize(8 * (size_t)m);
   q->mort.resize(m);
-  unsigned ev = 0;
   if (cudaMemcpyAsync(q->lev.data(), q->d_lev, sizeof(int) * m, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaMemcpyAsync(hij.data(), q->d_ij, sizeof(int2) * m, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
       cudaMemcpyAsync(q->par.data(), q->d_par, sizeof(int) * m, cudaMemcpyDeviceToHost, s) != cudaSuccess ||

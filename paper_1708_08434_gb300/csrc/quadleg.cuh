@@ -18,7 +18,8 @@
 // word is overwritten two publications later by the lane whose own halo came
 // from that word's reader, so it cannot be overwritten unread.  All blocks
 // of the cooperative launch are resident; a poll gives up after Q_SPIN tries
-// (err bit 2, the solve returns SM_ETIMEOUT).
+// (Q_ERR_WAIT): later legs return at once, and the solve runs again with a
+// launch per operation.
 //
 // What a warp reads of its neighbours' cells in memory, at the start of a
 // down leg, they store only after awaiting words that depend on what was
@@ -36,11 +37,11 @@
 enum { QL_TOP = 0, QL_FAS = 1, QL_PROLONG = 2, QL_FMG = 3 };  // how a leg starts
 
 constexpr unsigned Q_ERR_WAIT = 2u;
-constexpr int Q_SPIN = 1 << 18;  // polls of one wait (a few tenths of a second)
+constexpr int Q_SPIN = 1 << 18;  // pairs of polls of one wait (0.11 s)
 
 struct QLeg {
   int lo, nu;
-  unsigned leg;  // tag offset of the leg
+  unsigned leg, skew;  // tag offset of the leg; skew != 0 only in the self-test
   double h2, inv_h2;
   double *phi, *rhs, *old;
   unsigned long long *xch;  // [box][face][8][2]
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(32, OCC) k_q_leg(const __grid_constant__ QLeg 
     if (by) q.y.load(qy_ + 2 * ((j + c) & 1));
   };
   auto await = [&](int c, unsigned ev, Poll &q) {
-    const unsigned tag = tag0 + ev;
+    const unsigned tag = tag0 + ev + a.skew;
     const bool x = bx && xact(c);
     auto off = [&](const Poll &w) { return (x ? w.x.off(tag) : 0u) | (by ? w.y.off(tag) : 0u); };
     if (x || by) {
