@@ -569,7 +569,10 @@ __global__ void __launch_bounds__(TT, 1) k_cnn_train(const bf16 *__restrict__ X,
   for (int i = t; i < NPOS; i += TT) S.g3[i] = 0.0f;
   for (int i = t; i < NG; i += TT) S.grad[i] = 0.0f;
   pdl_wait();
-  if (*err) return;  // a wait of an earlier pass ran out: the results are void
+  // a wait of an earlier pass ran out: the results are void.  One answer for
+  // the block, whose warps wait for one another below: another block of this
+  // launch may set the word meanwhile
+  if (__syncthreads_or(*err != 0)) return;
   const uint32_t wg_bar = smem_u32(&mbar_wg);
   if (t == 0) asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(wg_bar), "r"(TC_TILES) : "memory");
   tc_begin(tc, &mbar, &tslot, err, TRAIN_COLS);
