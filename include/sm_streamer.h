@@ -516,8 +516,13 @@ int sm_cnn_load_samples(sm_cnn *c, const float *x_host, const float *t_host, int
 int sm_cnn_adam_step(sm_cnn *c, const float *grad_host, float lr);
 /* `epochs` passes over the recorded samples in minibatches of `batch`, an
  * Adam step after each; sample order shuffled per epoch from `seed`.  Out:
- * mean loss of the last epoch.  Synchronises. */
+ * mean loss of the last epoch.  Synchronises.  SM_ETIMEOUT: a wait for the
+ * tensor cores ran out; the weights and Adam's step count are those of the
+ * steps before. */
 int sm_cnn_train(sm_cnn *c, int epochs, int batch, float lr, unsigned long long seed, float *loss);
+/* Self-test: in the next epoch the device's error word is set before step
+ * `step` (from 0), as a wait that ran out in it would.  Errors: SM_EINVAL. */
+int sm_cnn_wait_selftest(sm_cnn *c, int step);
 /* Timing of the network kernels (build form, no paper passage): the mean
  * duration of `reps` launches (CUDA events on the network's stream, after
  * one warm-up) over the first n recorded samples; kind 0: the forward

@@ -67,7 +67,7 @@ EXPORTS = ["sm_create", "sm_destroy", "sm_arena_size", "sm_bind_arena", "sm_buil
            "sm_batch_ptrs", "sm_batch_solve", "sm_batch_tune", "sm_batch_set_schedule", "sm_batch_info",
            "sm_batch_set_graphs", "sm_batch_kernel_bench", "sm_cnn_create", "sm_cnn_destroy", "sm_cnn_arena_size",
            "sm_cnn_bind_arena", "sm_cnn_set_params", "sm_cnn_get_params", "sm_cnn_forward",
-           "sm_cnn_gradient", "sm_cnn_adam_step", "sm_cnn_train", "sm_cnn_attach", "sm_cnn_stats",
+           "sm_cnn_gradient", "sm_cnn_adam_step", "sm_cnn_train", "sm_cnn_wait_selftest", "sm_cnn_attach", "sm_cnn_stats",
            "sm_cnn_kernel_bench", "sm_cnn_load_samples", "sm_set_metrics_log",
            "sm_set_row_kernels", "sm_var_layout", "sm_fill_ghosts_range", "sm_get_ghosts", "sm_refine",
            "sm_advance_fluid_coeffs",
@@ -162,6 +162,7 @@ def signatures() -> dict:
         "sm_cnn_gradient": [P, P, P, I, P, C.POINTER(C.c_float)],
         "sm_cnn_adam_step": [P, P, C.c_float],
         "sm_cnn_train": [P, I, I, C.c_float, C.c_ulonglong, C.POINTER(C.c_float)],
+        "sm_cnn_wait_selftest": [P, I],
         "sm_cnn_attach": [P, P, I, I, I, I, D],
         "sm_cnn_stats": [P, pI, C.POINTER(C.c_longlong), C.POINTER(C.c_longlong), pD],
         "sm_cnn_kernel_bench": [P, I, I, I, pD, pD, pD],
@@ -687,6 +688,10 @@ class Network:
         loss = C.c_float()
         self._ck(self._lib.sm_cnn_train(self._h, epochs, batch, lr, seed, C.byref(loss)))
         return loss.value
+
+    def wait_selftest(self, step):
+        """Set the error word of a wait that ran out before step `step` of the next epoch."""
+        self._ck(self._lib.sm_cnn_wait_selftest(self._h, int(step)))
 
     def attach(self, solver, mode, per_solve=512, stride=1, taper=False, accept=1.0):
         self._ck(self._lib.sm_cnn_attach(solver._h, self._h, mode, per_solve, stride, int(taper), accept))

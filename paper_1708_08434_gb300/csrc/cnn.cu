@@ -864,7 +864,8 @@ __global__ void k_cnn_adam(AdamStep A, const float *__restrict__ g) {
 
 // gradient = sum of the CTA partials in CTA order (deterministic), the loss
 // likewise (the last block); ADAM: followed by the Adam step of the same
-// parameter, unless a completion wait of the gradient pass ran out.  Latency
+// parameter, unless a completion wait of the gradient pass ran out (the loss
+// of a step that is left out so is -1: the host counts Adam's steps).  Latency
 // bounds it: 5 MB from L2 in one chain of adds per parameter, so a warp a
 // block spreads the parameters over all SMs and 19 loads of a chain are in
 // flight (152 CTAs: eight rounds).  12.6 us as blocks of 256 with one load
@@ -893,7 +894,7 @@ __global__ void __launch_bounds__(RED_T) k_cnn_reduce(const float *__restrict__ 
   pdl_wait();
   const int i = blockIdx.x * RED_T + threadIdx.x;
   if (blockIdx.x == gridDim.x - 1) {
-    if (threadIdx.x == 0) *loss = ordered_sum(loss_partial, nblk, 1);
+    if (threadIdx.x == 0) *loss = ADAM && *err ? -1.0f : ordered_sum(loss_partial, nblk, 1);
   } else if (i < NP) {
     const bool ok = !ADAM || *err == 0;
     const float g = ordered_sum(partial + i, nblk, NP);
@@ -1013,6 +1014,7 @@ struct sm_cnn {
   float *dbg = nullptr;         // [MAX_DEBUG][4][16][512]
   int *ids = nullptr, *boxes = nullptr;
   int adam_step = 0;
+  int fail_step = -1;           // sm_cnn_wait_selftest
   // attached solver
   int mode = 0, stride = 1, per_solve = 0, taper = 0;
   double accept = 1.0;  // keep a prediction when rel_cnn < accept * rel_plain
@@ -1297,16 +1299,28 @@ extern "C" int sm_cnn_train(sm_cnn *c, int epochs, int batch, float lr, unsigned
     // once at its end (after an error the later steps change nothing)
     int st = load_ids(c, order.data(), n), nb = 0;
     if (st) return st;
-    for (int s = 0; s < n; s += std::min(batch, n - s))
+    for (int s = 0; s < n; s += std::min(batch, n - s)) {
+      if (nb == c->fail_step) CCK(cudaMemsetAsync(c->derr, 1, 1, c->stream));
       if ((st = grad_step(c, std::min(batch, n - s), c->ids + s, c->loss + nb++, &lr))) return st;
+    }
+    c->fail_step = -1;
     losses.resize(nb);
     CCK(cudaMemcpyAsync(losses.data(), c->loss, 4 * (size_t)nb, cudaMemcpyDeviceToHost, c->stream));
-    if ((st = check_derr(c))) return st;
+    if ((st = check_derr(c))) {
+      for (float l : losses) c->adam_step -= l < 0.0f;  // steps that changed nothing
+      return st;
+    }
     double acc = 0.0;
     for (float l : losses) acc += l;
     last = acc / nb;
   }
   if (loss) *loss = (float)last;
+  return SM_OK;
+}
+
+extern "C" int sm_cnn_wait_selftest(sm_cnn *c, int step) {
+  if (!c || step < 0) return SM_EINVAL;
+  c->fail_step = step;
   return SM_OK;
 }
 
