@@ -139,10 +139,7 @@ __global__ void __launch_bounds__(128, 8) k_flevel(const __grid_constant__ LevAr
   const int nz = (k == 0 || k == NC - 1) ? __ldg(row + LR_NB + fz) : -3;
   const int P = __ldg(row + LR_P), flags = __ldg(row + LR_FLAGS);
   const bool refined = START == FS_FAS && (flags & 8);
-  // a wait of an earlier launch ran out: the launch ends at its first barrier,
-  // which makes one answer of what the warps read (another block of this
-  // launch may set the bit meanwhile)
-  const bool stop = (sc[SC_ERR] & ERR_WAIT) != 0;
+  const unsigned long long stop = sc[SC_ERR] & ERR_WAIT;  // a wait of an earlier launch ran out
   const unsigned tag0 = (*a.seq << 5) + a.leg;
   int pn[3] = {0, 0, 0}, pe[3] = {0, 0, 0};
   if (PRO) {
@@ -173,6 +170,11 @@ __global__ void __launch_bounds__(128, 8) k_flevel(const __grid_constant__ LevAr
   }
   if (t < 6) swall[t] = a.bc.type[t] ? fx_2g(sc, t) : 0;
   if (t < 4) sv[t >> 1][64][t & 1] = make_longlong2(0, 0);
+  // (another block of this launch may set the bit between the reads of two
+  // warps: the part of a block that stays then works on what the other part
+  // has not staged.  Barriers count the warps that are left, waits end by
+  // themselves, and the launch's results are void)
+  if (stop) return;
 
   const int cf = (h + par) & 1, oct = flags & 7;  // cf: colour of the row's cell at x face h
   const bool bx = nx >= 0, by = ny >= 0, bz = nz >= 0;  // a box across the face
@@ -327,7 +329,7 @@ __global__ void __launch_bounds__(128, 8) k_flevel(const __grid_constant__ LevAr
       }
       sp[reg(rx, ry, rz)] = w0;
     }
-    if (__syncthreads_or(stop)) return;
+    __syncthreads();
     {
       const int y = (j >> 1) + 1, z = (k >> 1) + 1, sy = (j & 1) ? 6 : -6, sz = (k & 1) ? 36 : -36;
 #pragma unroll
@@ -373,8 +375,7 @@ __global__ void __launch_bounds__(128, 8) k_flevel(const __grid_constant__ LevAr
   }
   stage(0);
   stage(1);
-  if (PRO) __syncthreads();
-  else if (__syncthreads_or(stop)) return;
+  __syncthreads();
   if (flags & GHOSTS) {
     make_ghosts(0);
     if (!PRO) make_ghosts(1);
