@@ -747,28 +747,33 @@ __global__ void __launch_bounds__(512) k_bt_coarse(const int *__restrict__ solve
 // per cell instead of seven.  A solve whose potential holds an infinity or
 // a NaN gets NaN residuals.
 //
-// A block per column, four rows a thread.  Instruction issue bounds the pass
+// A block per column, R rows a thread.  Instruction issue bounds the pass
 // when every neighbour comes from shared memory (207 instructions a warp for
 // 32 cells), so a thread keeps the fixed-point values of its rows on planes
 // p-1, p and p+1 in registers: the z and the inner y neighbours need no load.
 // Planes of phi (one-cell halo) are staged by asynchronous copies; at step p
-// a thread converts its four values of plane p+1, which it keeps and writes
+// a thread converts its values of plane p+1, which it keeps and writes
 // back for the neighbours' x and outer y reads at step p+1, and at most one
 // halo value.  Wall ghosts enter as in the sweep: +1 (Neumann) or -1
 // (Dirichlet) in the coefficient of c, and the sum of the Dirichlet 2g, both
 // exact integers; DIR: a face in x or y is Dirichlet.  Slots at step p:
 // planes p and p+1 are read, p+2 is in flight, plane p+3 is issued into the
-// slot of plane p-1 (last read at step p-1).  124e6 cells: 734 us against
-// 818 with all neighbours staged (20 bytes a cell are 0.37 ms, two FP64
+// slot of plane p-1 (last read at step p-1).  124e6 cells, R = 4: 734 us
+// against 818 with all neighbours staged (20 bytes a cell are 0.37 ms, two FP64
 // operations 0.42 ms; shorter forms of the two conversions ran no faster).
+// With a few blocks an SM the chain of a plane bounds it, so fewer rows a
+// thread (more warps a column) and f two planes ahead: 4 solves of 64^3 in 47
+// us at R = 1, 49 at 2, 94 at 4 (the rule is in launch_outer).
 // The max norm is taken on the bit patterns of |r|.
 
-template <bool DIR>
+template <bool DIR, int R>
 __device__ __forceinline__ unsigned long long outer_column(const int4 &C, const BSolve &S, int E,
                                                            const double *__restrict__ phi,
                                                            const double *__restrict__ f64, float *__restrict__ f32,
                                                            const Bc &bc, long long *sp) {
-  const int t = threadIdx.x, tx = t % CX, ty = 4 * (t / CX);
+  constexpr int T = CX * CY / R;  // threads
+  constexpr bool AHEAD = R < 4;
+  const int t = threadIdx.x, tx = t % CX, ty = R * (t / CX);
   const int N = S.N[0], P = pitch(N);
   const long long NN = (long long)N * N;
   const bool finite = E < 0x7ff;
@@ -778,8 +783,8 @@ __device__ __forceinline__ unsigned long long outer_column(const int4 &C, const 
   const int x0 = C.y * CX, y0 = C.z * CY, x = x0 + tx, ya = y0 + ty;
   const double *pv = phi + S.off64;
   // this thread's 16-byte chunks of a staged plane (N even)
-  // of it: rows r, r + 7, r + 14
-  constexpr int CROW = RWD / 2, RSTEP = ST / CROW, U = (FR + RSTEP - 1) / RSTEP;
+  // of it: rows r, r + RSTEP, ...
+  constexpr int CROW = RWD / 2, RSTEP = T / CROW, U = (FR + RSTEP - 1) / RSTEP;
   const bool vec = (N & 1) == 0;
   const int crow = t / CROW, cx = x0 - 2 + 2 * (t % CROW), cy = y0 - 1 + crow;
   const bool cxok = crow < RSTEP && cx >= 0 && cx < N;
@@ -799,7 +804,7 @@ __device__ __forceinline__ unsigned long long outer_column(const int4 &C, const 
         }
         csrc += NN;
       } else {
-        for (int i = t; i < DPL; i += ST) {
+        for (int i = t; i < DPL; i += T) {
           const int y = y0 - 1 + i / RWD, xx = x0 - 2 + i % RWD;
           const bool ok = y >= 0 && y < N && xx >= 0 && xx < N;
           cp_async<8>(dst + i, ok ? pv + z * NN + y * N + xx : pv, ok);
@@ -814,25 +819,25 @@ __device__ __forceinline__ unsigned long long outer_column(const int4 &C, const 
   int hq = -1;
   if (t < 2 * CX) hq = (t < CX ? 0 : CY + 1) * RWD + 2 + t % CX;
   else if (t < 2 * CX + 2 * CY) hq = (1 + (t - 2 * CX) % CY) * RWD + (t < 2 * CX + CY ? 1 : CX + 2);
-  auto convert = [&](int sl, long long(&c)[4]) {
+  auto convert = [&](int sl, long long(&c)[R]) {
     long long *pl = sp + sl * DPL;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < R; ++r) {
       c[r] = fix(pl[q0 + r * RWD]);
       pl[q0 + r * RWD] = c[r];
     }
     if (hq >= 0) pl[hq] = fix(pl[hq]);
   };
-  bool in[4];
-  int w[4];             // coefficient of c without the z walls
-  long long gxy[4];     // DIR: sum of the Dirichlet 2g of the in-plane walls
+  bool in[R];
+  int w[R];             // coefficient of c without the z walls
+  long long gxy[R];     // DIR: sum of the Dirichlet 2g of the in-plane walls
   auto wall = [&](int face, bool on, int &wr, long long &g) {
     if (!on) return;
     wr += bc.type[face] ? -1 : 1;
     if (DIR && bc.type[face]) g += fix(__double_as_longlong(bc.g2[face]));
   };
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < R; ++r) {
     const int y = ya + r;
     in[r] = x < N && y < N;
     w[r] = -6;
@@ -844,19 +849,23 @@ __device__ __forceinline__ unsigned long long outer_column(const int4 &C, const 
   }
   const double *fz = f64 + S.off64 + (long long)ya * N + x;
   float *rz = f32 + S.off[0] + (long long)ya * P + x;
-  double fv[4] = {};  // f of plane p
-  auto load_f = [&](double(&d)[4]) {
+  double fv[AHEAD ? 2 : 1][R] = {};  // f of plane p; AHEAD: of planes p and p+1
+  auto load_f = [&](double(&d)[R]) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r)
+    for (int r = 0; r < R; ++r)
       if (in[r]) d[r] = fz[r * N];
     fz += NN;
   };
   unsigned long long m = 0;  // bit pattern of max |r|
 #pragma unroll
   for (int z = 0; z < OSL - 1; ++z) issue(z, z);
+  if (AHEAD) {
+    load_f(fv[0]);
+    if (N > 1) load_f(fv[1]);
+  }
   cp_wait<OSL - 2>();  // plane 0 has landed
   __syncthreads();
-  long long cm[4] = {}, c[4], cn[4];
+  long long cm[R] = {}, c[R], cn[R];
   convert(0, c);
   for (int pb = 0; pb < N; pb += OSL) {
 #pragma unroll
@@ -866,12 +875,13 @@ __device__ __forceinline__ unsigned long long outer_column(const int4 &C, const 
       cp_wait<OSL - 3>();  // this thread's copies of planes <= p+1 have landed
       __syncthreads();     // everyone's have, plane p is converted, step p-1's reads are done
       issue(p + OSL - 1, (i + OSL - 1) % OSL);
-      load_f(fv);
+      double(&f)[R] = fv[AHEAD ? i & 1 : 0];
+      if (!AHEAD) load_f(f);
       if (p + 1 < N) {
         convert((i + 1) % OSL, cn);
       } else {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) cn[r] = 0;
+        for (int r = 0; r < R; ++r) cn[r] = 0;
       }
       int wz = 0;
       long long gz = 0;
@@ -885,43 +895,44 @@ __device__ __forceinline__ unsigned long long outer_column(const int4 &C, const 
       }
       const long long *pl = sp + i * DPL;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
+      for (int r = 0; r < R; ++r) {
         if (!in[r]) continue;
         const int q = q0 + r * RWD;
-        const long long ym = r > 0 ? c[r - 1] : pl[q - RWD], yp = r < 3 ? c[r + 1] : pl[q + RWD];
+        const long long ym = r > 0 ? c[r - 1] : pl[q - RWD], yp = r < R - 1 ? c[r + 1] : pl[q + RWD];
         long long sx = ((pl[q - 1] + pl[q + 1]) + (ym + yp)) + (cm[r] + cn[r]) + (long long)(w[r] + wz) * c[r] + gz;
         if (DIR) sx += gxy[r];  // exact
-        const double res = fma(-__ll2double_rn(sx), kk, fv[r]);
+        const double res = fma(-__ll2double_rn(sx), kk, f[r]);
         const unsigned long long rb = finite ? (unsigned long long)__double_as_longlong(res) : 0x7ff8000000000000ull;
         rz[r * P] = cvt_bits_f32_rn(rb);
         const unsigned long long a = rb & 0x7fffffffffffffffull;
         m = a > m ? a : m;
       }
+      if (AHEAD && p + 2 < N) load_f(f);
       rz += (long long)P * N;
 #pragma unroll
-      for (int r = 0; r < 4; ++r) cm[r] = c[r], c[r] = cn[r];
+      for (int r = 0; r < R; ++r) cm[r] = c[r], c[r] = cn[r];
     }
   }
   cp_wait<0>();
   return m;
 }
 
-template <bool DIR>
-__global__ void __launch_bounds__(ST, DIR ? 6 : 8) k_bt_outer(const int4 *__restrict__ cols, const BSolve *__restrict__ tab,
+template <bool DIR, int R>
+__global__ void __launch_bounds__(CX *CY / R, R == 1 ? 2 : (R == 2 ? 3 : (DIR ? 6 : 8))) k_bt_outer(const int4 *__restrict__ cols, const BSolve *__restrict__ tab,
                                                     const unsigned char *__restrict__ active,
                                                     const double *__restrict__ phi, const double *__restrict__ f64,
                                                     float *__restrict__ f32, Bc bc,
                                                     const unsigned *__restrict__ emax,
                                                     unsigned long long *__restrict__ num) {
   __shared__ __align__(16) long long sp[OSL * DPL];
-  __shared__ unsigned long long red[ST / 32];
+  __shared__ unsigned long long red[CX * CY / R / 32];
   const int4 C = cols[blockIdx.x];
   if (!active[C.x]) return;
   int E = max((int)emax[C.x], 123);  // and bound of the Dirichlet wall values
 #pragma unroll
   for (int f = 0; f < 6; ++f)
     if (bc.type[f]) E = max(E, (int)expo_of(bc.g2[f]));
-  unsigned long long m = outer_column<DIR>(C, tab[C.x], E, phi, f64, f32, bc, sp);
+  unsigned long long m = outer_column<DIR, R>(C, tab[C.x], E, phi, f64, f32, bc, sp);
   // one max per column and solve
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -931,7 +942,7 @@ __global__ void __launch_bounds__(ST, DIR ? 6 : 8) k_bt_outer(const int4 *__rest
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int i = 1; i < ST / 32; ++i) m = red[i] > m ? red[i] : m;
+    for (int i = 1; i < CX * CY / R / 32; ++i) m = red[i] > m ? red[i] : m;
     atomicMax(num + C.x, m);
   }
 }
@@ -1452,9 +1463,19 @@ static BState bstate(sm_batch *b) {
 
 static void launch_outer(sm_batch *b, const unsigned char *mask) {
   const bool dir = b->bc.type[0] | b->bc.type[1] | b->bc.type[2] | b->bc.type[3];
-  auto kernel = dir ? k_bt_outer<true> : k_bt_outer<false>;
-  kernel<<<(unsigned)b->fine_cnt, ST, 0, b->stream>>>(b->d_tiles + b->fine_off, b->d_tab, mask, b->phi, b->f64, b->f32,
-                                                      b->bc, b->d_emax, b->d_num);
+  // Rows a thread by the columns on an SM, so that they are resident together
+  // (2 blocks of 512 threads, 3 of 256): 256 columns of 64^3 took 66, 70 and
+  // 116 us with 1, 2 and 4 rows, 400 columns 108, 84 and 125, 800 columns 184,
+  // 162 and 171 (in-plane Dirichlet walls: 187, 167, 157).
+  const size_t n = b->fine_cnt, sms = (size_t)b->sms;
+  const int rows = n <= 2 * sms ? 1 : (n <= 3 * sms ? 2 : 4);
+  auto run = [&](auto kernel, int threads) {
+    kernel<<<(unsigned)b->fine_cnt, threads, 0, b->stream>>>(b->d_tiles + b->fine_off, b->d_tab, mask, b->phi, b->f64,
+                                                             b->f32, b->bc, b->d_emax, b->d_num);
+  };
+  if (rows == 1) dir ? run(k_bt_outer<true, 1>, CX * CY) : run(k_bt_outer<false, 1>, CX * CY);
+  else if (rows == 2) dir ? run(k_bt_outer<true, 2>, CX * CY / 2) : run(k_bt_outer<false, 2>, CX * CY / 2);
+  else dir ? run(k_bt_outer<true, 4>, CX * CY / 4) : run(k_bt_outer<false, 4>, CX * CY / 4);
 }
 
 // residual of the solves flagged in `mask`; zero_phi: of phi = 0, also
