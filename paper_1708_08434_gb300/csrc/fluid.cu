@@ -125,10 +125,10 @@ __global__ void __launch_bounds__(512) k_charge(const int32_t *__restrict__ leaf
   rhs[x] = use_rho ? -rho[x] * inv_eps : -q * (ni[x] - ne[x]) * inv_eps;
 }
 
-// Per-cell time-step quantities at (fixed-point) table index x of the cell's
-// |E|: sum_d mu |E_d| 2 dx with E_d = (p_{-d} - p_{+d})/(2 dx) (the mean of
-// the two face fields), that plus 12 D (both to be scaled by 1/(2 dx^2)),
-// and mu n_e
+// Per-cell time-step quantities at the table index of the cell's |E| (x: half
+// of it): sum_d |mu E_d| 2 dx with E_d = (p_{-d} - p_{+d})/(2 dx) (the mean of
+// the two face fields), that plus 12 D (both to be scaled by 1/(2 dx^2)), and
+// mu n_e
 __device__ __forceinline__ void dt_terms(const double *__restrict__ phi, const double *__restrict__ gh,
                                          const int32_t *__restrict__ nbr6, const Bc &bc, int b, int t,
                                          unsigned long long x, double ne, const Table &tb, double &adv, double &ad,
@@ -138,7 +138,7 @@ __device__ __forceinline__ void dt_terms(const double *__restrict__ phi, const d
   double pc = p[t];
   const int stride[3] = {1, NC, FACE};
   double w;
-  const double2 *fc = tb.fc + 2 * index_split(x, tb, w);
+  const double2 *fc = tb.fc + 2 * index_split(x, x, tb, w);
   const double2 cm = __ldg(fc), cd = __ldg(fc + 1);
   const double mu = fma(w, cm.y, cm.x);
   double d[3];
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(512) k_dt(const int32_t *__restrict__ leaf, co
   int t = threadIdx.x;
   size_t x = (size_t)b * CELLS + t;
   double adv, ad, drt;
-  dt_terms(phi, gh, nbr6, bc, b, t, 2 * half_index(emag[x], tb), ne[x], tb, adv, ad, drt);
+  dt_terms(phi, gh, nbr6, bc, b, t, half_index(emag[x], tb), ne[x], tb, adv, ad, drt);
   block_max3_to(slots + SC_ADV, adv, ad, drt, red, 0.5 * lh.inv_h2[level[b]]);
 }
 
@@ -218,10 +218,10 @@ __global__ void __launch_bounds__(64) k_cf_flux(const int32_t *__restrict__ leaf
   const double g2 = density_cf_ghost(n, nbr6, parent, ijk, b, f, 2, u, w, err);
   const double p0 = phi[base + cidx(c0[0], c0[1], c0[2])];
   const double pg = p0 * (1.0 / 3.0) + (2.0 / 3.0) * gh[(size_t)(6 * b + f) * FACE + fcell(a, c0[0], c0[1], c0[2])];
-  const unsigned long long x = half_index(emag[base + cidx(c0[0], c0[1], c0[2])], tb) +
-                               half_index(emag_cf_ghost(emag, nbr6, parent, ijk, b, f, u, w), tb);
-  const double F = (f & 1) ? face_flux_d(n0, g1, n0 - n1, g1 - n0, g2 - g1, p0 - pg, x, tb)
-                           : face_flux_d(g1, n0, g1 - g2, n0 - g1, n1 - n0, pg - p0, x, tb);
+  const unsigned long long x0 = half_index(emag[base + cidx(c0[0], c0[1], c0[2])], tb),
+                           xg = half_index(emag_cf_ghost(emag, nbr6, parent, ijk, b, f, u, w), tb);
+  const double F = (f & 1) ? face_flux_d(n0, g1, n0 - n1, g1 - n0, g2 - g1, p0 - pg, x0, xg, tb)
+                           : face_flux_d(g1, n0, g1 - g2, n0 - g1, n1 - n0, pg - p0, xg, x0, tb);
   cflux[(size_t)(6 * b + f) * FACE + u + NC * w] = F * lh.inv_h[level[b]];
 }
 
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(UT, 5) k_update(
       double F;
       if (m == 0 && known[0]) F = Fk[0];
       else if (m == NC && known[1]) F = Fk[1];
-      else F = face_flux_d(nL, nR, dm, dn, dq, pL - pR, xL + xR, tb);
+      else F = face_flux_d(nL, nR, dm, dn, dq, pL - pR, xL, xR, tb);
       if (m > 0) D[m - 1] = F - F0;
       F0 = F;
       nL = nR;
@@ -414,7 +414,7 @@ __global__ void __launch_bounds__(UT, 5) k_update(
       const double nes = c ? nc[s].y : nc[s].x, e = c ? ec[s].y : ec[s].x, nis = c ? ni.y : ni.x;
       const int q = iP(x0 + c, y, z);
       double w;
-      const int i = index_split(2 * S.x[q], tb, w);
+      const int i = index_split(S.x[q], S.x[q], tb, w);
       const double2 cm = __ldg(tb.fc + 2 * i), al = __ldg(tb.al + i);
       const double mu = fma(w, cm.y, cm.x);
       const double src = fma(w, al.y, al.x) * mu * e * nes;

@@ -23,6 +23,7 @@ inline void table_index_consts(Table &tb, const double *packed, int n, double e_
   tb.xm = (unsigned long long)ldexp(f, 64);
   tb.xs = 1035 - p;
   tb.xtop = (unsigned long long)(n - 1) << 51;
+  tb.hscale = 0.5 * ((n - 1) / e_max);
 }
 
 // the packed arrays of host tables (6 x 4096 doubles)
@@ -64,28 +65,59 @@ __device__ __forceinline__ double koren(double a, double b) {
   return __longlong_as_double(m | (dbits(b) & (long long)0x8000000000000000ull));
 }
 
-// Half the table index of a cell, e (n-1)/(2 e_max), in units of 2^-51
-// (rounded; clamped to n - 1): the significand of e times the scale's, shifted
-// by the exponents -- integer operations only.  A face's index is then the
-// integer sum of its two cells' values, its integer part the top bits.  The
-// error, 2^-52 a cell, is below the rounding of an FP64 index once that
-// exceeds 1 (a typical index of 500 has an ulp of 2^-44).
+// Half the table index of a cell, e (n-1)/(2 e_max).  From 2 on in units of
+// 2^-51 (rounded; clamped to n - 1): the significand of e times the scale's,
+// shifted by the exponents -- integer operations only.  A face's index is then
+// the integer sum of its two cells' values, its integer part the top bits; its
+// error, 2^-51, is the rounding of an FP64 index from 4 on (a typical index
+// of 500 has an ulp of 2^-44).  Below 2, where FP64 is the finer one, the FP64
+// product itself with LOW_HALF set in place of its sign.  The FP64 operations
+// of such cells are calls: as predicated instructions they take the FP64 pipe
+// for every cell (streamer6 field, time step and stage 569 us; 549 as calls).
+constexpr unsigned long long LOW_HALF = 1ull << 63;
+static __device__ __noinline__ unsigned long long low_half(double e, double scale) {
+  return LOW_HALF | (unsigned long long)dbits(e * scale);
+}
+struct LowIndex {
+  double w;
+  int i;
+};
+static __device__ __noinline__ LowIndex low_split(double yL, double yR, int top) {
+  const double y = yL + yR;  // below 4
+  const int i = min((int)y, top);
+  return {i < top ? y - i : 0.0, i};
+}
 __device__ __forceinline__ unsigned long long half_index(double e, const Table &tb) {
   const unsigned long long bits = (unsigned long long)dbits(e);
   const int ex = (int)(bits >> 52);  // the sign included: negative values give a large count
-  if (ex & 0x800) return 0ull;
+  if (ex & 0x800) return LOW_HALF;
   const unsigned long long A = (bits << 11) | (ex ? 1ull << 63 : 0ull);
   const unsigned long long hi = __umul64hi(A, tb.xm);
   const int sh = tb.xs - (ex ? ex : 1);
   if (sh <= 0) return tb.xtop;
   const unsigned long long x = sh > 63 ? 0ull : ((hi >> (sh - 1)) + 1ull) >> 1;
-  return x < tb.xtop ? x : tb.xtop;
+  if (x >= tb.xtop) return tb.xtop;
+  return x < (2ull << 51) ? low_half(e, tb.hscale) : x;
 }
 
-// integer part of an index x (units of 2^-51, clamped to n - 1) and its
-// fraction as an exact double: the leading one of the 51 bits is shifted to
-// the hidden bit's place
-__device__ __forceinline__ int index_split(unsigned long long x, const Table &tb, double &w) {
+// Integer part of the index xL + xR of a face (of a cell: twice its own half),
+// clamped to n - 1, and its fraction as an exact double: the leading one of
+// the 51 bits is shifted to the hidden bit's place.
+__device__ __forceinline__ int index_split(unsigned long long xL, unsigned long long xR, const Table &tb, double &w) {
+  unsigned long long x = xL + xR;
+  if ((xL | xR) & LOW_HALF) {
+    const double yL = __longlong_as_double((long long)(xL & ~LOW_HALF)), yR = __longlong_as_double((long long)(xR & ~LOW_HALF));
+    if (xL & xR & LOW_HALF) {  // both in FP64
+      const LowIndex r = low_split(yL, yR, (int)(tb.xtop >> 51));
+      w = r.w;
+      return r.i;
+    }
+    // the FP64 half to units of 2^-51 (below 2: the shift is at least 0)
+    const unsigned long long bits = (xL & LOW_HALF ? xL : xR) & ~LOW_HALF;
+    const int sh = 1024 - (int)(bits >> 52);
+    const unsigned long long m = (bits & 0x000fffffffffffffull) | 1ull << 52;
+    x = (xL & LOW_HALF ? xR : xL) + (sh > 54 ? 0ull : ((m << 1 >> sh) + 1ull) >> 1);
+  }
   x = x < tb.xtop ? x : tb.xtop;
   const unsigned long long f = x & ((1ull << 51) - 1ull);
   const int lz = __clzll((long long)f);  // 13 .. 63 when f != 0
@@ -100,11 +132,11 @@ __device__ __forceinline__ int index_split(unsigned long long x, const Table &tb
 // part -D(E*) (n_R - n_L)/dx.  Written as -mu dp n_f - D dn: v < 0 exactly when
 // mu dp > 0; from the differences
 // n_L - n_L2, n_R - n_L and n_R2 - n_R, which a line of faces shares, and the
-// fixed-point table index of the face
+// half table indices of the two cells
 __device__ __forceinline__ double face_flux_d(double nL, double nR, double dm, double dn, double dq, double dp,
-                                              unsigned long long x, const Table &tb) {
+                                              unsigned long long xL, unsigned long long xR, const Table &tb) {
   double w;
-  const double2 *fc = tb.fc + 2 * index_split(x, tb, w);
+  const double2 *fc = tb.fc + 2 * index_split(xL, xR, tb, w);
   const double2 cm = __ldg(fc), cd = __ldg(fc + 1);
   const double t1 = fma(w, cm.y, cm.x) * dp;
   const bool up = dbits(t1) > 0;  // v < 0: the upwind cell is R

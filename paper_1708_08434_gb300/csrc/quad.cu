@@ -572,7 +572,7 @@ __device__ __forceinline__ double face_flux(const double *sn, const double *sp, 
   const int q = a == 0 ? (u + 2) * S2 + m + 2 : (m + 2) * S2 + u + 2, sq = a == 0 ? 1 : S2;
   const int r = a == 0 ? (u + 1) * S1 + m + 1 : (m + 1) * S1 + u + 1, sr = a == 0 ? 1 : S1;
   const double nL = sn[q - sq], nR = sn[q];
-  return face_flux_d(nL, nR, nL - sn[q - 2 * sq], nR - nL, sn[q + sq] - nR, sp[r - sr] - sp[r], se[r - sr] + se[r], tb);
+  return face_flux_d(nL, nR, nL - sn[q - 2 * sq], nR - nL, sn[q + sq] - nR, sp[r - sr] - sp[r], se[r - sr], se[r], tb);
 }
 
 // Fine-side fluxes of every leaf box face that borders a coarser leaf:
@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(QT) k_q_update(int n, const double *__restrict
       const int q = a == 0 ? (u + 2) * S2 + m + 2 : (m + 2) * S2 + u + 2, sq = a == 0 ? 1 : S2;
       const int r1 = a == 0 ? (u + 1) * S1 + m + 1 : (m + 1) * S1 + u + 1, sr = a == 0 ? 1 : S1;
       const double *d = sdm[wv_][a] + r;
-      F = face_flux_d(sn[q - sq], sn[q], d[0], d[QN], d[2 * QN], sp[r1 - sr] - sp[r1], se[r1 - sr] + se[r1], tb);
+      F = face_flux_d(sn[q - sq], sn[q], d[0], d[QN], d[2 * QN], sp[r1 - sr] - sp[r1], se[r1 - sr], se[r1], tb);
     }
     sf[wv_][a][r] = F;
   }
@@ -695,7 +695,7 @@ __global__ void __launch_bounds__(QT) k_q_update(int n, const double *__restrict
     const size_t g = (size_t)b * QC + c;
     const double nes = sn[(j + 2) * S2 + i + 2], e = emag[g];
     double w;
-    const int k = index_split(2 * se[q], tb, w);
+    const int k = index_split(se[q], se[q], tb, w);
     const double2 cm = __ldg(tb.fc + 2 * k), al = __ldg(tb.al + k);
     const double mu = fma(w, cm.y, cm.x);
     const double src = fma(w, al.y, al.x) * mu * e * nes;
@@ -775,7 +775,8 @@ __global__ void __launch_bounds__(QT) k_q_dt(int n, const double *__restrict__ p
     const int c = lane + 32 * s2;
     const size_t g = (size_t)b * QC + c;
     double w;
-    const int k = index_split(2 * half_index(emag[g], tb), tb, w);
+    const unsigned long long x = half_index(emag[g], tb);
+    const int k = index_split(x, x, tb, w);
     const double2 cm = __ldg(tb.fc + 2 * k), cd = __ldg(tb.fc + 2 * k + 1);
     dt_cell(s, (c / QN + 1) * S1 + c % QN + 1, fma(w, cm.y, cm.x), fma(w, cd.y, cd.x), ne[g], m);
   }

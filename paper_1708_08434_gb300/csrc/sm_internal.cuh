@@ -65,6 +65,7 @@ struct Table {
   unsigned long long xm;     // (n-1)/(2 e_max) = xm 2^(971 - xs): scale of the fixed-point half index
   int xs;
   unsigned long long xtop;   // n - 1 in units of 2^-51
+  double hscale;             // (n-1)/(2 e_max)
 };
 
 // kernel classes for sm_kernel_bench
