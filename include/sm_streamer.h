@@ -616,6 +616,21 @@ int sm_fp64_probe(long long iters, unsigned long long *d_scratch, double *fma_pe
 int sm_check_conversions(long long n, unsigned long long seed, unsigned long long *d_scratch,
                          unsigned long long *mismatches, void *stream);
 
+/* Check of the FP64 kernels' square root, division, reciprocal and halving
+ * (not in the paper), which save instructions of the narrow FP64 pipe,
+ * against the library's on n seeded patterns.
+ *   d_scratch:  DEVICE uint64 [5], overwritten.
+ *   out:        HOST uint64 [5]: largest distance in units in the last place
+ *               of the square root of positive normal numbers; patterns of
+ *               all other kinds (zeros, subnormals, infinities, NaNs,
+ *               negative numbers) whose root differs; largest distance of a/d
+ *               (|a| 2^-823 to 2^823, |d| 2^-100 to 2^100) and of 1/x (x
+ *               2^-120 to 2^120); patterns whose half differs.
+ * Synchronises the stream.  Errors: SM_EINVAL (n < 0, null pointer),
+ * SM_ECUDA. */
+int sm_check_arithmetic(long long n, unsigned long long seed, unsigned long long *d_scratch,
+                        unsigned long long *out, void *stream);
+
 /* Human-readable reason of the last error on this context. */
 const char *sm_last_error(const sm_ctx *ctx);
 

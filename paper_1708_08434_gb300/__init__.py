@@ -61,7 +61,8 @@ EXPORTS = ["sm_create", "sm_destroy", "sm_arena_size", "sm_bind_arena", "sm_buil
            "sm_mg_vcycle", "sm_mg_solve", "sm_mg_fmg", "sm_compute_field", "sm_dt_limit",
            "sm_fluid_stage", "sm_advance_fluid", "sm_kernel_bench", "sm_set_graphs", "sm_set_pdl",
            "sm_set_persistent", "sm_persist_barrier_selftest", "sm_leg_wait_selftest",
-           "sm_launch_count", "sm_last_error", "sm_box_solve_noalloc", "sm_check_conversions", "sm_fp64_probe",
+           "sm_launch_count", "sm_last_error", "sm_box_solve_noalloc", "sm_check_conversions", "sm_check_arithmetic",
+           "sm_fp64_probe",
            "sm_refine_flags", "sm_regrid",
            "sm_batch_create", "sm_batch_destroy", "sm_batch_arena_size", "sm_batch_bind_arena",
            "sm_batch_ptrs", "sm_batch_solve", "sm_batch_tune", "sm_batch_set_schedule", "sm_batch_info",
@@ -137,6 +138,7 @@ def signatures() -> dict:
         "sm_launch_count": [P, C.POINTER(C.c_longlong)],
         "sm_box_solve_noalloc": [D, I, P, P, P, P, P],
         "sm_check_conversions": [C.c_longlong, C.c_ulonglong, P, P, P],
+        "sm_check_arithmetic": [C.c_longlong, C.c_ulonglong, P, P, P],
         "sm_fp64_probe": [C.c_longlong, P, pD, pD, P],
         "sm_refine_flags": [P, D, D, D, D, I, P],
         "sm_regrid": [P, P, pI, pI, pI],
@@ -222,6 +224,22 @@ def check_conversions(n: int, seed: int = 0x5EED):
                                   C.c_void_p(stream.cuda_stream))
     if rc != SM_OK:
         raise SmError(rc, "sm_check_conversions failed")
+    return tuple(int(v) for v in out)
+
+
+def check_arithmetic(n: int, seed: int = 0x5EED):
+    """The FP64 kernels' square root, division, reciprocal and halving
+    against the library's on n seeded patterns: (largest distance of the root
+    in units in the last place, special values whose root differs, largest
+    distance of the quotient, of the reciprocal, halves that differ)."""
+    import torch
+    lib = load()
+    scratch = torch.zeros(5, dtype=torch.int64, device="cuda")
+    out = np.zeros(5, np.uint64)
+    rc = lib.sm_check_arithmetic(int(n), int(seed), C.c_void_p(scratch.data_ptr()), _hp(out),
+                                 C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    if rc != SM_OK:
+        raise SmError(rc, "sm_check_arithmetic failed")
     return tuple(int(v) for v in out)
 
 

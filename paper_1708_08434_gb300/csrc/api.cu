@@ -744,6 +744,44 @@ __global__ void k_check_cvt(long long n, unsigned long long seed, unsigned long 
   if (bad_x) atomicAdd(count + 2, bad_x);
 }
 
+// a significand and sign at random under an exponent field in [lo, hi]
+__device__ __forceinline__ double with_exponent(unsigned long long x, int lo, int hi) {
+  const unsigned long long ex = (unsigned long long)lo + (splitmix64(x) >> 16) % (unsigned long long)(hi - lo + 1);
+  return __longlong_as_double((long long)((x & 0x800fffffffffffffull) | ex << 52));
+}
+__device__ __forceinline__ unsigned long long ulps(double a, double b) {  // of the same sign
+  const long long d = dbits(a) - dbits(b);
+  return (unsigned long long)(d < 0 ? -d : d);
+}
+
+__global__ void k_check_arith(long long n, unsigned long long seed, unsigned long long *__restrict__ out) {
+  unsigned long long m[5] = {0, 0, 0, 0, 0};
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const unsigned long long r = splitmix64(seed + (unsigned long long)i), r2 = splitmix64(r);
+    unsigned long long x = r;  // any pattern
+    if ((i & 3) == 1) x = r & 0x800fffffffffffffull;  // zeros and subnormals
+    if ((i & 3) == 2)  // around a power of 2, four ulps to each side
+      x = ((((r >> 52) & 0x7ffull) << 52) + ((r2 >> 20) & 7ull) - 4ull) | (r & 1ull) << 63;
+    if ((i & 31) == 1) x = (r & 1ull) << 63 | ((r & 2ull) ? 0x7ff0000000000000ull : 0ull);  // zeros, infinities
+    const double d = __longlong_as_double((long long)x);
+    const double s = sqrt_newton(d), t = __dsqrt_rn(d);
+    const int ex = (int)(x >> 52);
+    if (ex > 0 && ex < 0x7ff) m[0] = max(m[0], ulps(s, t));
+    else if (dbits(s) != dbits(t) && !(isnan(s) && isnan(t))) ++m[1];
+    const double h = halve(d), h2 = __dmul_rn(0.5, d);
+    if (dbits(h) != dbits(h2) && !(isnan(h) && isnan(h2))) ++m[4];
+    const double a = with_exponent(r, 200, 1846), b = with_exponent(r2, 923, 1123);
+    m[2] = max(m[2], ulps(quotient(a, b), __ddiv_rn(a, b)));
+    const double c = dabs(with_exponent(r2, 903, 1143));
+    m[3] = max(m[3], ulps(recip(c), __ddiv_rn(1.0, c)));
+  }
+  for (int k = 0; k < 5; ++k) {
+    if (!m[k]) continue;
+    if (k == 1 || k == 4) atomicAdd(out + k, m[k]);
+    else atomicMax(out + k, m[k]);
+  }
+}
+
 }  // namespace
 
 // FP64 pipe throughput probe: FP64_CHAINS independent fused multiply-add
@@ -809,3 +847,15 @@ extern "C" int sm_check_conversions(long long n, unsigned long long seed, unsign
   return SM_OK;
 }
 
+extern "C" int sm_check_arithmetic(long long n, unsigned long long seed, unsigned long long *d_scratch,
+                                   unsigned long long *out, void *stream) {
+  if (n < 0 || !d_scratch || !out) return SM_EINVAL;
+  cudaStream_t st = (cudaStream_t)stream;
+  if (cudaMemsetAsync(d_scratch, 0, 5 * sizeof(unsigned long long), st) != cudaSuccess) return SM_ECUDA;
+  if (n > 0) k_check_arith<<<1216, 256, 0, st>>>(n, seed, d_scratch);
+  if (cudaGetLastError() != cudaSuccess) return SM_ECUDA;
+  if (cudaMemcpyAsync(out, d_scratch, 5 * sizeof(unsigned long long), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+      cudaStreamSynchronize(st) != cudaSuccess)
+    return SM_ECUDA;
+  return SM_OK;
+}

@@ -47,16 +47,6 @@ struct Bases {
   }
 };
 
-// a / d for |d| between 2^-100 and 2^100 and normal a: a single-precision
-// reciprocal, one Newton step, and the quotient corrected by its remainder
-// (five FP64 instructions)
-__device__ __forceinline__ double quotient(double a, double d) {
-  const double y0 = cvt_f32_f64(__frcp_rn(cvt_f64_f32_rn(d)));
-  const double y = fma(fma(-d, y0, 1.0), y0, y0);
-  const double q = a * y;
-  return fma(fma(-q, d, a), y, q);
-}
-
 // One problem per cluster of C blocks of 512 / C threads, a cell each.  The
 // solve is FP64-pipe work (six 8-term transforms a cell, 2 instructions per
 // clock and SM), so a call of few problems spreads each over several SMs:

@@ -69,13 +69,6 @@ struct QWord {
     return __longlong_as_double((long long)((a & 0xffffffff00000000ull) | (b >> 32)));
   }
 };
-// 1/x for positive x in single precision's range: Newton's iteration from the
-// single-precision reciprocal
-__device__ __forceinline__ double q_recip(double x) {
-  double y = sm::cvt_f32_f64(__frcp_rn(sm::cvt_f64_f32_rn(x)));
-  y = fma(fma(-x, y, 1.0), y, y);
-  return fma(fma(-x, y, 1.0), y, y);
-}
 
 // OCC: blocks an SM has to hold (more registers for a level of few boxes)
 template <int START, int OCC>
@@ -342,7 +335,7 @@ __global__ void __launch_bounds__(32, OCC) k_q_leg(const __grid_constant__ QLeg 
   // weights of the restriction's means
   double w0 = 0.0, w1 = 0.0;
   if (!UP) {
-    const double r = 0.5 * q_recip(wv[0] + wv[1]);
+    const double r = 0.5 * sm::recip(wv[0] + wv[1]);
     w0 = wv[0] * r;
     w1 = wv[1] * r;
   }

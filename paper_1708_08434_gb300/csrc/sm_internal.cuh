@@ -303,6 +303,25 @@ __device__ __forceinline__ double cvt_f32_f64(float f) {
   return __hiloint2double((int)hi, (int)lo);
 }
 
+// 1/x for positive x between 2^-120 and 2^120: two steps of Newton's iteration
+// for the reciprocal, y += (1 - x y) y, from the single-precision one
+__device__ __forceinline__ double recip(double x) {
+  double y = cvt_f32_f64(__frcp_rn(cvt_f64_f32_rn(x)));
+  y = fma(fma(-x, y, 1.0), y, y);
+  return fma(fma(-x, y, 1.0), y, y);
+}
+
+// a / d for |d| between 2^-100 and 2^100 and normal a and quotient: one such
+// step, and the quotient corrected by its remainder, which the fused
+// multiply-add gives exactly (Markstein, IBM J. Res. Dev. 34, 1990): five FP64
+// instructions
+__device__ __forceinline__ double quotient(double a, double d) {
+  const double y0 = cvt_f32_f64(__frcp_rn(cvt_f64_f32_rn(d)));
+  const double y = fma(fma(-d, y0, 1.0), y0, y0);
+  const double q = a * y;
+  return fma(fma(-q, d, a), y, q);
+}
+
 // Exact stencil sums in 64-bit fixed point (integer pipe).  A finite
 // binary64 value with biased exponent field e <= E is mapped to the nearest
 // multiple of 2^(E - 1080), ties away from zero, as a signed integer: its
