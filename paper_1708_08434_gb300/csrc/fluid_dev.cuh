@@ -82,10 +82,17 @@ struct LowIndex {
   double w;
   int i;
 };
+// (the split itself on the integer pipe: the significand above and below the
+// binary point)
 static __device__ __noinline__ LowIndex low_split(double yL, double yR, int top) {
-  const double y = yL + yR;  // below 4
-  const int i = min((int)y, top);
-  return {i < top ? y - i : 0.0, i};
+  const double y = yL + yR;  // 0 to 4
+  const unsigned long long bits = (unsigned long long)dbits(y);
+  const int e = (int)(bits >> 52) - 1023;
+  if (e < 0) return {y, 0};
+  const unsigned long long m = (bits & 0x000fffffffffffffull) | 1ull << 52, f = m << (12 + e);
+  const int i = (int)(m >> (52 - e)), lz = __clzll((long long)f);
+  if (i >= top) return {0.0, top};
+  return {f ? __longlong_as_double((long long)(((unsigned long long)(1021 - lz) << 52) + (f << lz >> 11))) : 0.0, i};
 }
 __device__ __forceinline__ unsigned long long half_index(double e, const Table &tb) {
   const unsigned long long bits = (unsigned long long)dbits(e);
