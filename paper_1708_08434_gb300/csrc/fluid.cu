@@ -260,8 +260,8 @@ __device__ __forceinline__ int iP(int x, int y, int z) { return (x + 1) + PY * (
 // Bound by the FP64 pipe (2 instructions per clock and SM), so the work is
 // laid out to issue few of them: a thread marches one line of 9 faces along
 // an axis and forms each density difference once (three faces use it), table
-// indices and halvings are integer operations, and dt / dx^2 is one factor.  50 FP64
-// instructions per cell in stage 1 (the cell-and-face form before: 64).
+// indices and halvings are integer operations, and dt / dx^2 is one factor.  52.7
+// FP64 instructions per cell in stage 1 (the cell-and-face form before: 64).
 template <bool HEUN>
 __global__ void __launch_bounds__(UT, 5) k_update(
     const int32_t *__restrict__ leaf, const int32_t *__restrict__ level, const double *__restrict__ ne_src,
